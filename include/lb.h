@@ -133,9 +133,9 @@ int lb_init(lb_handle *h, int mode, uint64_t seed, double rho_mean,
 /* Advance by nsteps >= 0 time steps of Eq. (evoleq) -- propagation,
  * density (n-hat on wall rows), forces of Eq. (force2) + Eq.
  * (periodicforce), wall rule, u* of Eq. (newvel), equilibrium Eq.
- * (eqfunc), forcing Eqs. (forceterm, coeff), BGK collision -- one fused
- * kernel launch per step, enqueued on the handle's stream without
- * synchronising.  Errors: LB_ERR_STATE (not initialised), LB_ERR_CUDA.     */
+ * (eqfunc), forcing Eqs. (forceterm, coeff), BGK collision -- in one fused
+ * kernel (strip-sweep handles: one launch for many steps), enqueued on the
+ * handle's stream without synchronising.  Errors: LB_ERR_STATE (not initialised), LB_ERR_CUDA.     */
 int lb_step(lb_handle *h, int64_t nsteps);
 
 /* Density n (n-hat on wall rows) and physical velocity u* of Eq. (newvel)
@@ -205,10 +205,9 @@ int lb_set_state(lb_handle *h, const void *buf, size_t bytes, int64_t step);
 
 /* Tiling autotuner (a performance control of this library; the paper has
  * no counterpart).  Times `steps` steps of the strip-sweep kernel for each
- * candidate tiling -- segment height (rows per CTA, which trades CTAs per SM
- * against re-read warm-up rows) and strip count (the fewest strips and up
- * to three more of at least 64 columns, which changes how the tiles fill
- * the GPU) -- times the three fastest twice more and keeps the one with
+ * candidate segment height (which trades how the tiles fill the GPU against
+ * repeated warm-up rows) that gives other tiles than the ones before, times
+ * the three fastest twice more and keeps the one with
  * the smallest of its three timings for later lb_step calls, and writes its
  * segment height to *seg_h (may be NULL; 0 when the handle uses the tile
  * kernel, which has no tiling choice; lb_get_tiling gives both).  The state and the step counter are restored
@@ -218,11 +217,14 @@ int lb_set_state(lb_handle *h, const void *buf, size_t bytes, int64_t step);
  * LB_ERR_OOM.                                                              */
 int lb_autotune(lb_handle *h, int steps, int32_t *seg_h);
 
-/* Set the strip-sweep kernel's segment height (rows per CTA) without
+/* Set the strip-sweep kernel's segment height without
  * tuning, e.g. to a value an earlier lb_autotune chose; clamped to
- * [1, ny].  The trajectory does not depend on it beyond FP32 rounding
+ * [1, ny].  The kernel's tiles are one strip wide and one segment high; a
+ * strip wider than a tile can be (56 columns) is replaced by the fewest
+ * narrower ones, and segments that would leave the GPU partly idle are cut
+ * into lower tiles.  The trajectory does not depend on it beyond FP32 rounding
  * order.  No-op (LB_OK) for a handle on the tile kernel.  Host-side only
- * (may grow the per-CTA record array).  Errors: LB_ERR_ARG (seg_h < 1),
+ * (may grow the per-tile record array).  Errors: LB_ERR_ARG (seg_h < 1),
  * LB_ERR_CUDA, LB_ERR_OOM.                                                 */
 int lb_set_seg_h(lb_handle *h, int32_t seg_h);
 
@@ -252,7 +254,9 @@ int lb_set_tiling(lb_handle *h, int32_t nstrips, int32_t seg_h);
  * launch, for every tile in idx[ofs[t] .. ofs[t + 1]) to have finished the
  * previous step: the tiles that write a site (or a periodic image of one)
  * that its TMA window reads -- rows ya - 4 .. yb + 4, columns from x0 - 4
- * over the window's width -- and the tiles whose windows read its sites.
+ * over 128 columns -- and the tiles whose windows read its sites.  (Where
+ * the kernel cuts a tiling further, see lb_set_seg_h, it builds the lists of
+ * its own tiles the same way, over the 64 columns each of them reads.)
  * ofs: ntiles + 1 entries (HOST); idx: up to cap entries (HOST, may be
  * NULL when cap = 0); *count receives the number of entries.  Errors:
  * LB_ERR_ARG (a lattice or tiling the sweep does not take, or cap below
@@ -262,9 +266,9 @@ int lb_sweep_dependencies(int32_t precision, int32_t nx, int32_t ny, int32_t wal
 
 /* ------------------------------------------------------------------------
  * Batched solver: many independent lattices (different sizes and physical
- * parameters) advanced together, one kernel launch per step over a work
- * list of every instance's strips and segments (longest first), pairs of
- * steps replayed as a CUDA graph.  The paper solves one lattice at a time;
+ * parameters) advanced together, over a work
+ * list of every instance's tiles (longest first), any number of steps in one
+ * launch.  The paper solves one lattice at a time;
  * this is a throughput layer for parameter sweeps (e.g. over T, A0, lambda
  * and the wall velocity).
  * ------------------------------------------------------------------------ */

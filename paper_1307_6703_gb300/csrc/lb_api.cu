@@ -31,7 +31,13 @@ struct lb_handle {
   float ref_ax = 0.f, ref_dg = 0.f;  // reference populations of 16-bit storage
   float *wide = nullptr;         // 16-bit storage: nine float planes (moments, reductions, init)
   size_t sweep_smem = 0;
-  int sweep_seg = 64, sweep_nstrips = 0, sweep_nseg = 0, sweep_base = 0, sweep_extra = 0;
+  // The tiling as lb_set_tiling names it, and the tiles the kernel runs on
+  // (set_tiles): tile_cols columns of tiles, base_w wide (the first `extra`
+  // one quantum wider), by tile_nseg segments of tile_rows rows.
+  int sweep_seg = 64, sweep_nstrips = 0;
+  int tile_cols = 0, tile_base = 0, tile_extra = 0, tile_rows = 0, tile_nseg = 0;
+  int want_rows = 0;             // tile height where segments would leave warps idle
+  int resident = 1;              // warps of the kernel the device holds
   double *d_cta = nullptr;       // per-CTA partials written by the sweep kernel
   size_t cta_bytes = 0;
   int plan_gen = 0;              // bumped when the tiling or the record array changes
@@ -51,7 +57,6 @@ struct lb_handle {
   int mon_cap = 0;
   // Multi-step launches (lb_step with nsteps >= 2 while not monitoring):
   // per-tile completion counters and dependency lists of the current tiling.
-  int persist_cap = 0;           // resident CTAs of that kernel (0: not queried, < 0: unavailable)
   unsigned *d_done = nullptr;
   int *d_dep = nullptr;          // CSR: ntiles + 1 offsets, then indices
   unsigned *d_ticket = nullptr;  // ticket counter of a launch
@@ -297,7 +302,11 @@ cudaError_t current_f32(lb_handle *h, const float **out) {
   return lbk::launch_widen(h->store, h->f[h->cur], h->wide, h->plane, h->ref_ax, h->ref_dg, h->st);
 }
 
-lbk::SweepArgs sweep_args(const lb_handle *h, float *fout) {
+// Whether the handle's lattice takes the tau = 1 form of the sweep.
+bool tau1(const lb_handle *h) { return (float)(1.0 - 1.0 / h->p.tau) == 0.0f; }
+
+// Arguments of a step that reads buffer `in` and writes the other one.
+lbk::SweepArgs sweep_args(const lb_handle *h, int in) {
   const lb_params &p = h->p;
   lbk::SweepArgs A;
   A.nx = p.nx;
@@ -306,38 +315,59 @@ lbk::SweepArgs sweep_args(const lb_handle *h, float *fout) {
   A.pitch = h->pitch;
   A.plane = h->plane;
   A.off = h->off;
-  A.seg_h = h->sweep_seg;
-  A.nseg = h->sweep_nseg;
-  A.nstrips = h->sweep_nstrips;
-  A.base_w = h->sweep_base;
-  A.extra = h->sweep_extra;
+  A.seg_h = h->tile_rows;
+  A.nseg = h->tile_nseg;
+  A.nstrips = h->tile_cols;
+  A.base_w = h->tile_base;
+  A.extra = h->tile_extra;
   const double T0 = 1.0 / 3.0;
-  A.T = (float)p.T;
-  A.a = (float)p.a;
-  A.b = (float)p.b;
-  A.kappa = (float)p.kappa;
-  A.omega = (float)(1.0 / p.tau);
-  A.one_minus_omega = (float)(1.0 - 1.0 / p.tau);
-  A.g = (float)(1.0 - 1.0 / (2.0 * p.tau));
-  A.th = (float)(T0 - p.T);
-  A.A0 = (float)p.A0;
+  auto two = [](float v) { return make_float2(v, v); };
+  lbk::SweepConsts &c = A.k;
+  const float omega = (float)(1.0 / p.tau);
+  const double k = (p.T - T0) / (2.0 * T0 * T0);  // rest factors A_i = 1 + k (c.c - 2 T0)
+  const float A_ax = (float)(1.0 + k * (1.0 - 2.0 * T0)), A_diag = (float)(1.0 + k * (2.0 - 2.0 * T0));
+  c.T = two((float)p.T);
+  c.nb = two(-(float)p.b);
+  c.one = two(1.0f);
+  c.a = two((float)p.a);
+  c.kappa = two((float)p.kappa);
+  c.A0 = two((float)p.A0);
+  c.N = two((float)p.N);
+  c.M = two((float)((1.0 - 2.0 * p.N) / 4.0));
+  c.Q = two((float)p.Q);
+  c.R = two((float)((1.0 - p.Q) / 2.0));
+  c.m4QR = two(-(float)(4.0 * (p.Q + (1.0 - p.Q) / 2.0)));
+  c.half = two(0.5f);
+  c.two = two(2.0f);
+  c.th = two((float)(T0 - p.T));
+  c.g = two((float)(1.0 - 1.0 / (2.0 * p.tau)));
+  c.om = two(omega);
+  c.om1 = two((float)(1.0 - 1.0 / p.tau));
+  c.Aax = two(A_ax * (1.f / 9.f));
+  c.Adg = two(A_diag * (1.f / 36.f));
+  c.m6 = two(-1.f / 6.f);
+  c.m24 = two(-1.f / 24.f);
+  c.e8 = two(0.125f);
+  c.q4 = two(0.25f);
+  c.mq4 = two(-0.25f);
+  c.third = two(1.f / 3.f);
+  c.mthird = two(-1.f / 3.f);
+  c.twelfth = two(1.f / 12.f);
+  c.mtwelfth = two(-1.f / 12.f);
+  c.r_sum = two(4.f * (h->ref_ax + h->ref_dg));
+  c.mwr_ax = two(-(omega * h->ref_ax));
+  c.mwr_dg = two(-(omega * h->ref_dg));
   A.u_bot = (float)p.u_bot;
   A.u_top = (float)p.u_top;
-  A.N = (float)p.N;
-  A.M = (float)((1.0 - 2.0 * p.N) / 4.0);
-  A.Q = (float)p.Q;
-  A.R = (float)((1.0 - p.Q) / 2.0);
-  A.four_QR = (float)(4.0 * (p.Q + (1.0 - p.Q) / 2.0));
-  const double k = (p.T - T0) / (2.0 * T0 * T0);
-  A.A_rest = (float)(1.0 + k * (0.0 - 2.0 * T0));
-  A.A_ax = (float)(1.0 + k * (1.0 - 2.0 * T0));
-  A.A_diag = (float)(1.0 + k * (2.0 - 2.0 * T0));
   A.nmax = p.b > 0.0 ? (float)(1.0 / p.b) : 3.0e38f;
   A.ref_ax = h->ref_ax;
   A.ref_dg = h->ref_dg;
   A.sinx = (const float *)h->sinx;
-  A.fout = fout;
-  A.fdev = dev16(h) ? (void *)((char *)fout + (size_t)h->plane * sizeof(float)) : nullptr;
+  auto planes16 = [&](void *f) { return dev16(h) ? (void *)((char *)f + (size_t)h->plane * sizeof(float)) : nullptr; };
+  A.fin = (const float *)h->f[in];
+  A.fdin = planes16(h->f[in]);
+  A.fout = (float *)h->f[in ^ 1];
+  A.fdev = planes16(h->f[in ^ 1]);
   A.partials = h->d_cta;
   A.records = 1;
   A.err = h->d_err;
@@ -348,19 +378,35 @@ lbk::SweepArgs sweep_args(const lb_handle *h, float *fout) {
   return A;
 }
 
-// Segment height of a sweep handle; the per-CTA record array must already
+// Tiling of a sweep handle: nstrips strips by segments of seg_h rows.  Strips
+// wider than a tile can be become the fewest columns of tiles; segments that
+// would leave warps idle are cut to the height that fills the device (in a
+// batch, where the lattices share it: always).  The record array must already
 // be large enough (see ensure_records).
-void set_segments(lb_handle *h, int seg_h) {
-  h->sweep_seg = std::max(1, std::min(seg_h, h->p.ny));
-  h->sweep_nseg = (h->p.ny + h->sweep_seg - 1) / h->sweep_seg;
+void set_tiles(lb_handle *h, int nstrips, int seg_h) {
+  const int ny = h->p.ny;
+  h->sweep_nstrips = nstrips;
+  h->sweep_seg = std::max(1, std::min(seg_h, ny));
+  h->tile_cols = lbk::sweep_tile_cols(h->store, h->p.nx, nstrips);
+  lbk::sweep_strips(h->store, h->p.nx, h->tile_cols, &h->tile_base, &h->tile_extra);
+  int rows = h->sweep_seg;
+  if (rows > h->want_rows && (h->in_batch || (long long)h->tile_cols * ((ny + rows - 1) / rows) < h->resident)) {
+    // cut into equal parts of a multiple of 4 rows, no higher than the segments
+    const int parts = (ny + h->want_rows - 1) / h->want_rows, even = (ny + parts - 1) / parts;
+    rows = std::min(rows, even < 4 ? even : (even + 3) / 4 * 4);
+  }
+  h->tile_rows = rows;
+  h->tile_nseg = (ny + rows - 1) / rows;
   h->cta_valid = false;
   h->total_valid = false;
   h->plan_gen++;
 }
 
-// Grow the per-CTA record array to hold `nseg` segments of records.
-cudaError_t ensure_records(lb_handle *h, int nseg) {
-  const size_t need = 4 * sizeof(double) * (size_t)h->sweep_nstrips * nseg;
+int ntiles(const lb_handle *h) { return h->tile_cols * h->tile_nseg; }
+
+// Grow the per-tile record array to hold the current tiling's records.
+cudaError_t ensure_records(lb_handle *h) {
+  const size_t need = 4 * sizeof(double) * (size_t)ntiles(h);
   if (need <= h->cta_bytes) return cudaSuccess;
   double *p = nullptr;
   cudaError_t e = cudaStreamSynchronize(h->st);
@@ -375,14 +421,23 @@ cudaError_t ensure_records(lb_handle *h, int nseg) {
   return cudaSuccess;
 }
 
+// set_tiles and ensure_records; on failure the old tiling stays.
+cudaError_t change_tiles(lb_handle *h, int nstrips, int seg_h) {
+  const int strips0 = h->sweep_nstrips, seg0 = h->sweep_seg;
+  set_tiles(h, nstrips, seg_h);
+  const cudaError_t e = ensure_records(h);
+  if (e != cudaSuccess) set_tiles(h, strips0, seg0);
+  return e;
+}
+
 // Dependency lists and counters of the multi-step kernel for the current
 // tiling (rebuilt when the tiling changes; counters then restart at 0).
 cudaError_t ensure_deps(lb_handle *h) {
   if (h->deps_gen == h->plan_gen) return cudaSuccess;
   std::vector<int> ofs, idx;
-  lbk::sweep_deps(h->store, h->p.nx, h->p.ny, h->p.walls, h->sweep_nstrips, h->sweep_base, h->sweep_extra,
-                  h->sweep_seg, ofs, idx);
-  const int ntiles = h->sweep_nstrips * h->sweep_nseg;
+  lbk::sweep_deps(h->store, h->p.nx, h->p.ny, h->p.walls, h->tile_cols, h->tile_base, h->tile_extra, h->tile_rows,
+                  lbk::kSweepWindow, ofs, idx);
+  const int ntiles = h->tile_cols * h->tile_nseg;
   std::vector<int> csr(ofs);
   csr.insert(csr.end(), idx.begin(), idx.end());
   cudaError_t e = cudaStreamSynchronize(h->st);  // no launch may still use the old lists
@@ -402,6 +457,15 @@ cudaError_t ensure_deps(lb_handle *h) {
   h->epoch = 0;
   h->deps_gen = h->plan_gen;
   return cudaSuccess;
+}
+
+// Warps of the sweep kernel the current device holds at once.
+int resident_warps(int store, bool form_tau1) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    sms = 1;  // (lb_create reports the missing device)
+  return std::max(sms, 1) * lbk::sweep_warps_per_sm(store, form_tau1);
 }
 
 constexpr int kMonSlots = 64;  // steps per multi-step launch while monitoring
@@ -424,20 +488,10 @@ cudaError_t ensure_mon_slots(lb_handle *h, int ntiles) {
 }
 
 // nsteps >= 2 steps of a strip-sweep handle in multi-step launches.
-// Returns LB_OK, an error code, or 1 when that kernel cannot run here (the
-// caller then launches one kernel per step).
 int multi_steps(lb_handle *h, int64_t nsteps) {
-  if (h->persist_cap == 0) {
-    int cap = 0;
-    const cudaError_t e = lbk::persist_capacity(h->store, h->sweep_smem, &cap);
-    if (e != cudaSuccess) cudaGetLastError();
-    h->persist_cap = (e == cudaSuccess && cap > 0) ? cap : -1;
-  }
-  if (h->persist_cap < 0) return 1;
   LB_CUDA(h, ensure_deps(h));
   const int ntiles = h->deps_ntiles;
-  const lbk::SweepArgs A = sweep_args(h, nullptr);
-  const int grid = std::min(ntiles, h->persist_cap);
+  const lbk::SweepArgs A = sweep_args(h, h->cur);
   lbk::MultiOut Q{};
   for (int b = 0; b < 2; ++b) {
     Q.fout[b] = (float *)h->f[b ^ 1];  // a step reading buffer b writes buffer b ^ 1
@@ -463,7 +517,7 @@ int multi_steps(lb_handle *h, int64_t nsteps) {
   for (int64_t done = 0; done < nsteps;) {
     const int chunk = (int)std::min<int64_t>(nsteps - done, per_launch);
     Q.mon_step0 = h->step + 1;  // step number of the first step's result
-    lbk::PersistArgs P{};
+    lbk::MultiArgs P{};
     P.nitems = ntiles;
     P.nsteps = chunk;
     P.kpar0 = h->cur;
@@ -473,7 +527,7 @@ int multi_steps(lb_handle *h, int64_t nsteps) {
     P.dep_idx = h->d_dep + ntiles + 1;
     P.next = h->d_ticket;
     LB_CUDA(h, cudaMemsetAsync(h->d_ticket, 0, sizeof(unsigned), h->st));
-    const cudaError_t e = lbk::launch_sweep_multi(h->store, h->tmap, A, P, Q, grid, h->sweep_smem, h->st);
+    const cudaError_t e = lbk::launch_sweep_multi(h->store, tau1(h), h->tmap, A, P, Q, h->sweep_smem, h->st);
     if (e != cudaSuccess) return cuda_fail(h, e, "lb_step: multi-step sweep kernel");
     h->cur ^= chunk & 1;
     h->step += chunk;
@@ -532,8 +586,11 @@ int lb_create(const lb_params *p, lb_handle **out) {
     h->pitch = ((p->nx + 8 + 31) / 32) * 32;
     h->plane = (long long)h->pitch * (p->ny + 8);
     h->off = 4LL * h->pitch + 4;
-    lbk::sweep_plan(h->store, p->nx, p->ny, &h->sweep_nstrips, &h->sweep_base, &h->sweep_extra, &h->sweep_seg,
-                    &h->sweep_nseg);
+    int nstrips = 0, seg = 0;
+    lbk::sweep_plan(h->store, p->nx, p->ny, &nstrips, &seg);
+    h->resident = resident_warps(h->store, tau1(h));
+    h->want_rows = lbk::sweep_seg_rule(lbk::sweep_tile_cols(h->store, p->nx, nstrips), p->ny, h->resident);
+    set_tiles(h, nstrips, seg);
   } else {
     h->pitch = p->nx;
     h->plane = (long long)h->S;
@@ -548,9 +605,9 @@ int lb_create(const lb_params *p, lb_handle **out) {
   if (e == cudaSuccess) e = cudaMalloc((void **)&h->d_err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(h->d_err, 0, sizeof(int));
   if (e == cudaSuccess && h->sweep) {
-    h->cta_bytes = 4 * sizeof(double) * (size_t)h->sweep_nstrips * h->sweep_nseg;
+    h->cta_bytes = 4 * sizeof(double) * (size_t)ntiles(h);
     e = cudaMalloc((void **)&h->d_cta, h->cta_bytes);
-    if (e == cudaSuccess) e = lbk::sweep_prepare(h->store, &h->sweep_smem);
+    if (e == cudaSuccess) e = lbk::sweep_prepare(h->store, tau1(h), &h->sweep_smem);
     for (int b = 0; b < 2 && e == cudaSuccess; b++)
       e = lbk::sweep_make_maps(h->store, h->f[b], h->pitch, p->ny, h->plane, &h->tmap[b][0], &h->tmap[b][1]);
   }
@@ -651,14 +708,11 @@ int lb_step(lb_handle *h, int64_t nsteps) {
     }
   } else if (h->sweep) {
     // Two steps or more: multi-step launches.
-    if (nsteps >= 2) {
-      const int rc = multi_steps(h, nsteps);
-      if (rc != 1) return rc;
-    }
+    if (nsteps >= 2) return multi_steps(h, nsteps);
     // Per-CTA mass/momentum records only on the last step: lb_reduce reads
     // only the current state's.
     for (int64_t k = 0; k < nsteps; k++) {
-      lbk::SweepArgs A = sweep_args(h, (float *)h->f[h->cur ^ 1]);
+      lbk::SweepArgs A = sweep_args(h, h->cur);
       // records on the last step, or on every step while monitoring
       A.records = (k == nsteps - 1 || h->mon_cap > 0) ? 1 : 0;
       if (A.records) {  // the last CTA also leaves the global sums in d_out
@@ -670,7 +724,7 @@ int lb_step(lb_handle *h, int64_t nsteps) {
         A.monitor = h->mon_ring + 6 * (s % h->mon_cap);
         A.mon_step = (double)s;
       }
-      cudaError_t e = lbk::launch_sweep(h->store, h->tmap[h->cur][0], h->tmap[h->cur][1], A, h->sweep_smem, h->st);
+      cudaError_t e = lbk::launch_sweep(h->store, tau1(h), h->tmap[h->cur][0], h->tmap[h->cur][1], A, h->sweep_smem, h->st);
       if (e != cudaSuccess) return cuda_fail(h, e, "lb_step: sweep kernel");
       h->cur ^= 1;
       h->step++;
@@ -739,7 +793,7 @@ static int enqueue_reduce(lb_handle *h) {
   if (h->sweep && h->cta_valid) {
     // The last sweep step left one record per CTA (site sums in FP32,
     // totals in FP64): only the final pass remains.
-    reduce_cta<<<1, RED_THREADS, 0, h->st>>>(h->d_cta, h->sweep_nstrips * h->sweep_nseg, h->d_out, h->d_err);
+    reduce_cta<<<1, RED_THREADS, 0, h->st>>>(h->d_cta, ntiles(h), h->d_out, h->d_err);
   } else {
     LB_CUDA(h, cudaMemsetAsync(h->d_flag, 0, sizeof(int), h->st));
     if (fp64(h))
@@ -802,7 +856,7 @@ int lb_monitor(lb_handle *h, double *host_ring, int32_t capacity) {
   if (!dev) return fail(h, LB_ERR_ARG, "lb_monitor: the ring is not page-locked memory the device can address");
   // the per-step record slots of the current tiling now, not at the first
   // monitored step (a later, finer tiling grows them at its launch)
-  LB_CUDA(h, ensure_mon_slots(h, h->sweep_nstrips * h->sweep_nseg));
+  LB_CUDA(h, ensure_mon_slots(h, ntiles(h)));
   h->mon_ring = static_cast<double *>(dev);
   h->mon_cap = capacity;
   return LB_OK;
@@ -882,41 +936,23 @@ int lb_autotune(lb_handle *h, int steps, int32_t *seg_h) {
     if (seg_h) *seg_h = 0;
     return LB_OK;  // the tile kernel has no tiling choice
   }
-  // Candidate segment heights (rows per CTA): fewer rows give more CTAs per
-  // SM and more warm-up rows; the best trade depends on the lattice and on
-  // the storage's occupancy.
-  const int cand[] = {24, 32, 40, 48, 52, 56, 64, 72, 80, 96, 128, 192, 256};
+  // Candidate segment heights: lower tiles fill the device better, higher ones
+  // repeat fewer warm-up rows; the best trade depends on the lattice and on
+  // the storage's occupancy.  Candidates that give the same tiles are timed
+  // once.
+  const int cand[] = {24, 28, 32, 36, 40, 44, 48, 56, 64, 80, 96, 128};
   const int ny = h->p.ny;
-  int max_nseg = h->sweep_nseg;
-  for (int c : cand) max_nseg = std::max(max_nseg, (ny + std::min(c, ny) - 1) / std::min(c, ny));
-  // Strip counts: the fewest strips, and up to three more while the strips
-  // stay at least 64 columns wide.  More, narrower strips cost more halo
-  // columns but change how the tiles of the last step fill the GPU (the
-  // tail of a multi-step launch); the timing decides.
-  const int s_min = lbk::sweep_min_strips(h->store, h->p.nx);
-  std::vector<int> strips{s_min};
-  for (int sc = s_min + 1; sc <= s_min + 3; ++sc) {
-    int bw = 0, ex = 0;
-    lbk::sweep_strips(h->store, h->p.nx, sc, &bw, &ex);
-    if (bw >= 64) strips.push_back(sc);
-  }
-  const int strips0 = h->sweep_nstrips, base0 = h->sweep_base, extra0 = h->sweep_extra;
-  // Per-CTA records sized for the most strips and the smallest segments
-  // (kept afterwards).
-  h->sweep_nstrips = strips.back();
-  cudaError_t er = ensure_records(h, max_nseg);
-  h->sweep_nstrips = strips0;
-  LB_CUDA(h, er);
+  const int strips = lbk::sweep_min_strips(h->store, h->p.nx);
+  const int strips0 = h->sweep_nstrips, seg0 = h->sweep_seg;
   h->cta_valid = false;
   h->total_valid = false;
 
   const size_t buf_bytes = lbk::sweep_buffer_bytes(h->store, h->plane);
   const int cur0 = h->cur;
   const int64_t step0 = h->step;
-  const int seg0 = h->sweep_seg;
   void *save = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  int best = seg0, best_strips = strips0, rc = LB_OK;
+  int best = seg0, rc = LB_OK;
   float best_ms = 3.0e38f;
   cudaError_t e = cudaMalloc(&save, buf_bytes);
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
@@ -924,11 +960,10 @@ int lb_autotune(lb_handle *h, int steps, int32_t *seg_h) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(save, h->f[cur0], buf_bytes, cudaMemcpyDeviceToDevice, h->st);
   // One timing of `steps` steps (after a 2-step warm-up) of a tiling, from
   // the saved state, which is restored afterwards; < 0 on failure.
-  auto time_tiling = [&](int sc, int sh) -> float {
-    h->sweep_nstrips = sc;
-    lbk::sweep_strips(h->store, h->p.nx, sc, &h->sweep_base, &h->sweep_extra);
-    set_segments(h, sh);
+  auto time_tiling = [&](int sh) -> float {
     float ms = -1.f;
+    e = change_tiles(h, strips, sh);
+    if (e != cudaSuccess) return ms;
     rc = lb_step(h, 2);  // warm-up
     if (rc == LB_OK) e = cudaEventRecord(e0, h->st);
     if (rc == LB_OK && e == cudaSuccess) rc = lb_step(h, steps);
@@ -944,45 +979,36 @@ int lb_autotune(lb_handle *h, int steps, int32_t *seg_h) {
   // differ by less than their run-to-run spread).
   struct Timed {
     float ms;
-    int sc, sh;
+    int sh, rows;
   };
   std::vector<Timed> timed;
-  for (int sc : strips) {
-    int last = -1;
-    for (int c : cand) {
-      if (e != cudaSuccess || rc != LB_OK) break;
-      const int sh = std::min(c, ny);
-      if (sh == last) continue;
-      last = sh;
-      const float ms = time_tiling(sc, sh);
-      if (ms >= 0.f) timed.push_back({ms, sc, sh});
-    }
+  for (int c : cand) {
+    if (e != cudaSuccess || rc != LB_OK) break;
+    const int sh = std::min(c, ny);
+    set_tiles(h, strips, sh);
+    bool seen = false;
+    for (const Timed &t : timed) seen = seen || t.rows == h->tile_rows;
+    if (seen) continue;
+    const float ms = time_tiling(sh);
+    if (ms >= 0.f) timed.push_back({ms, sh, h->tile_rows});
   }
   std::sort(timed.begin(), timed.end(), [](const Timed &a, const Timed &b) { return a.ms < b.ms; });
   if (timed.size() > 3) timed.resize(3);
   for (int rep = 0; rep < 2; ++rep)
     for (Timed &t : timed) {
       if (e != cudaSuccess || rc != LB_OK) break;
-      const float ms = time_tiling(t.sc, t.sh);
+      const float ms = time_tiling(t.sh);
       if (ms >= 0.f) t.ms = std::min(t.ms, ms);
     }
   for (const Timed &t : timed)
     if (t.ms < best_ms) {
       best_ms = t.ms;
       best = t.sh;
-      best_strips = t.sc;
     }
   h->cur = cur0;
   h->step = step0;
   const bool tuned = rc == LB_OK && e == cudaSuccess;
-  h->sweep_nstrips = tuned ? best_strips : strips0;
-  if (tuned)
-    lbk::sweep_strips(h->store, h->p.nx, h->sweep_nstrips, &h->sweep_base, &h->sweep_extra);
-  else {
-    h->sweep_base = base0;
-    h->sweep_extra = extra0;
-  }
-  set_segments(h, tuned ? best : seg0);
+  set_tiles(h, tuned ? strips : strips0, tuned ? best : seg0);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
   cudaFree(save);
   if (e0) cudaEventDestroy(e0);
@@ -1005,7 +1031,7 @@ int lb_sweep_dependencies(int32_t precision, int32_t nx, int32_t ny, int32_t wal
   int base = 0, extra = 0;
   lbk::sweep_strips(store, nx, nstrips, &base, &extra);
   std::vector<int> o, d;
-  lbk::sweep_deps(store, nx, ny, walls, nstrips, base, extra, std::min((int)seg_h, (int)ny), o, d);
+  lbk::sweep_deps(store, nx, ny, walls, nstrips, base, extra, std::min((int)seg_h, (int)ny), 128, o, d);
   *count = (int64_t)d.size();
   if (cap < *count) return LB_ERR_ARG;
   for (size_t i = 0; i < o.size(); ++i) ofs[i] = o[i];
@@ -1027,26 +1053,15 @@ int lb_set_tiling(lb_handle *h, int32_t nstrips, int32_t seg_h) {
   const int qn = h->store == lbk::kStoreF32 ? 4 : 8;
   if (nstrips < s_min || nstrips > h->p.nx / (2 * qn) || seg_h < 1)
     return fail(h, LB_ERR_ARG, "lb_set_tiling: strip count or segment height out of range");
-  const int sh = std::min((int)seg_h, h->p.ny);
-  const int old = h->sweep_nstrips;
-  h->sweep_nstrips = nstrips;
-  const cudaError_t e = ensure_records(h, (h->p.ny + sh - 1) / sh);
-  if (e != cudaSuccess) {
-    h->sweep_nstrips = old;
-    return cuda_fail(h, e, "lb_set_tiling");
-  }
-  lbk::sweep_strips(h->store, h->p.nx, nstrips, &h->sweep_base, &h->sweep_extra);
-  set_segments(h, sh);
-  return LB_OK;
+  const cudaError_t e = change_tiles(h, nstrips, seg_h);
+  return e == cudaSuccess ? LB_OK : cuda_fail(h, e, "lb_set_tiling");
 }
 
 int lb_set_seg_h(lb_handle *h, int32_t seg_h) {
   if (!h) return LB_ERR_ARG;
   if (seg_h < 1) return fail(h, LB_ERR_ARG, "lb_set_seg_h: seg_h must be >= 1");
   if (!h->sweep) return LB_OK;
-  const int sh = std::min((int)seg_h, h->p.ny);
-  LB_CUDA(h, ensure_records(h, (h->p.ny + sh - 1) / sh));
-  set_segments(h, sh);
+  LB_CUDA(h, change_tiles(h, h->sweep_nstrips, seg_h));
   return LB_OK;
 }
 
@@ -1094,8 +1109,9 @@ const char *lb_last_error(const lb_handle *h) {
 struct lb_batch {
   std::vector<lb_handle *> hs;
   cudaStream_t st = nullptr;
-  cudaStream_t cap = nullptr;  // private stream for graph capture
   int store = 0;
+  bool tau1 = true;  // every instance has relaxation time 1
+  lbk::SweepConsts consts;  // those of the scheme, the same for every instance
   size_t smem = 0;
   lbk::BatchItem *d_items = nullptr;
   lbk::SweepArgs *d_args = nullptr;
@@ -1105,10 +1121,8 @@ struct lb_batch {
   std::vector<int> gen;   // plan_gen of each instance when the list was built
   int kpar = 0;           // parity of the next batch step
   bool dirty = true;      // device work list out of date
-  cudaGraphExec_t graph = nullptr;  // two consecutive steps, kpar 0 then 1
   // Multi-step launches (lb_batch_step with nsteps >= 2): per-item
   // completion counters and dependency lists, rebuilt with the work list.
-  int persist_cap = 0;              // resident CTAs of that kernel (0: not queried, < 0: unavailable)
   unsigned *d_done = nullptr;
   int *d_dep = nullptr;             // CSR: nitems + 1 offsets, then indices
   int done_cap = 0, dep_cap = 0;
@@ -1146,20 +1160,20 @@ int batch_rebuild(lb_batch *b) {
     b->par0[i] = h->cur;
     b->gen[i] = h->plan_gen;
     for (int p = 0; p < 2; p++) {
-      args[2 * i + p] = sweep_args(h, (float *)h->f[p ^ 1]);
+      args[2 * i + p] = sweep_args(h, p);
       maps[4 * i + 2 * p + 0] = h->tmap[p][0];
       maps[4 * i + 2 * p + 1] = h->tmap[p][1];
     }
-    for (int sg = 0; sg < h->sweep_nseg; sg++)
-      for (int sp = 0; sp < h->sweep_nstrips; sp++)
-        items.push_back({i, sp, sg, sg * h->sweep_nstrips + sp, h->cur});
+    for (int sg = 0; sg < h->tile_nseg; sg++)
+      for (int sp = 0; sp < h->tile_cols; sp++)
+        items.push_back({i, sp, sg, sg * h->tile_cols + sp, h->cur});
   }
   // Longest CTAs first (rows of the segment plus the 7-row warm-up), so the
   // block scheduler fills the tail with the short ones.
   auto rows = [&](const lbk::BatchItem &it) {
     const lb_handle *h = b->hs[it.inst];
-    const int ya = it.seg * h->sweep_seg;
-    return std::min(h->p.ny, ya + h->sweep_seg) - ya;
+    const int ya = it.seg * h->tile_rows;
+    return std::min(h->p.ny, ya + h->tile_rows) - ya;
   };
   std::stable_sort(items.begin(), items.end(),
                    [&](const lbk::BatchItem &x, const lbk::BatchItem &y) { return rows(x) > rows(y); });
@@ -1176,19 +1190,19 @@ int batch_rebuild(lb_batch *b) {
   std::vector<int> csr(1, 0), dep_idx;
   {
     std::vector<std::vector<int>> item_of(n);
-    for (int i = 0; i < n; i++) item_of[i].assign((size_t)b->hs[i]->sweep_nstrips * b->hs[i]->sweep_nseg, -1);
+    for (int i = 0; i < n; i++) item_of[i].assign((size_t)ntiles(b->hs[i]), -1);
     for (int j = 0; j < (int)items.size(); j++) {
       const lbk::BatchItem &it = items[j];
-      item_of[it.inst][(size_t)it.seg * b->hs[it.inst]->sweep_nstrips + it.strip] = j;
+      item_of[it.inst][(size_t)it.seg * b->hs[it.inst]->tile_cols + it.strip] = j;
     }
     std::vector<std::vector<int>> ofs(n), idx(n);
     for (int i = 0; i < n; i++) {
       const lb_handle *h = b->hs[i];
-      lbk::sweep_deps(h->store, h->p.nx, h->p.ny, h->p.walls, h->sweep_nstrips, h->sweep_base, h->sweep_extra,
-                      h->sweep_seg, ofs[i], idx[i]);
+      lbk::sweep_deps(h->store, h->p.nx, h->p.ny, h->p.walls, h->tile_cols, h->tile_base, h->tile_extra, h->tile_rows,
+                      lbk::kSweepWindow, ofs[i], idx[i]);
     }
     for (const lbk::BatchItem &it : items) {
-      const size_t tile = (size_t)it.seg * b->hs[it.inst]->sweep_nstrips + it.strip;
+      const size_t tile = (size_t)it.seg * b->hs[it.inst]->tile_cols + it.strip;
       for (int d = ofs[it.inst][tile]; d < ofs[it.inst][tile + 1]; d++) dep_idx.push_back(item_of[it.inst][idx[it.inst][d]]);
       csr.push_back((int)dep_idx.size());
     }
@@ -1216,34 +1230,9 @@ int batch_rebuild(lb_batch *b) {
   LB_BCUDA(b, cudaMemcpyAsync(b->d_maps, maps.data(), maps.size() * sizeof(CUtensorMap),
                               cudaMemcpyHostToDevice, b->st));
   LB_BCUDA(b, cudaStreamSynchronize(b->st));  // host arrays go out of scope
-  if (b->graph) {
-    cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
-  }
+  b->consts = args[0].k;
   b->kpar = 0;
   b->dirty = false;
-  return LB_OK;
-}
-
-// Two consecutive batch steps (kpar 0, then 1) as one CUDA graph.
-int batch_graph(lb_batch *b) {
-  if (b->graph) return LB_OK;
-  cudaGraph_t g = nullptr;
-  LB_BCUDA(b, cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-  cudaError_t e1 = lbk::launch_sweep_batch(b->store, b->d_items, b->nitems, b->d_args, b->d_maps, 0, 0, b->smem, b->cap);
-  cudaError_t e2 = lbk::launch_sweep_batch(b->store, b->d_items, b->nitems, b->d_args, b->d_maps, 1, 1, b->smem, b->cap);
-  cudaError_t e3 = cudaStreamEndCapture(b->cap, &g);
-  if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
-    if (g) cudaGraphDestroy(g);
-    cudaGetLastError();
-    return bfail(b, LB_ERR_CUDA, "lb_batch_step: graph capture failed");
-  }
-  cudaError_t e = cudaGraphInstantiate(&b->graph, g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) {
-    b->graph = nullptr;
-    return bfail(b, LB_ERR_CUDA, std::string("lb_batch_step: graph instantiation: ") + cudaGetErrorString(e));
-  }
   return LB_OK;
 }
 
@@ -1285,12 +1274,22 @@ int lb_batch_create(const lb_params *ps, int32_t count, lb_batch **out) {
       return bfail(nullptr, rc, m);
     }
     h->in_batch = true;
+    b->tau1 = b->tau1 && tau1(h);
     b->hs.push_back(h);
   }
-  cudaError_t e = lbk::sweep_prepare(b->store, &b->smem);
+  // One tile height for the ensemble: the lattices share the device's warps.
+  double cols = 0.0;
+  int tall = 1;
+  for (const lb_handle *h : b->hs) tall = std::max(tall, (int)h->p.ny);
+  for (const lb_handle *h : b->hs) cols += (double)h->tile_cols * h->p.ny / tall;
+  const int want = lbk::sweep_seg_rule(cols, tall, resident_warps(b->store, b->tau1));
+  for (lb_handle *h : b->hs) {
+    h->want_rows = std::min(want, (int)h->p.ny);
+    set_tiles(h, h->sweep_nstrips, h->sweep_seg);
+  }
+  cudaError_t e = lbk::sweep_prepare(b->store, b->tau1, &b->smem);
   if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_args, 2 * (size_t)count * sizeof(lbk::SweepArgs));
   if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_maps, 4 * (size_t)count * sizeof(CUtensorMap));
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
     std::string m = std::string("lb_batch_create: ") + cudaGetErrorString(e);
     lb_batch_destroy(b);
@@ -1315,19 +1314,12 @@ int lb_batch_step(lb_batch *b, int64_t nsteps) {
     int rc = batch_rebuild(b);
     if (rc != LB_OK) return rc;
   }
-  if (nsteps >= 2 && b->persist_cap == 0) {
-    int cap = 0;
-    const cudaError_t e = lbk::persist_capacity(b->store, b->smem, &cap);
-    if (e != cudaSuccess) cudaGetLastError();
-    b->persist_cap = (e == cudaSuccess && cap > 0) ? cap : -1;
-  }
-  if (nsteps >= 2 && b->persist_cap > 0) {
-    // Every step in multi-step launches (chunks of at most 2^16 steps).
-    const int grid = std::min(b->nitems, b->persist_cap);
+  if (nsteps >= 2) {
+    // Every step in multi-step launches.
     if (!b->d_ticket) LB_BCUDA(b, cudaMalloc((void **)&b->d_ticket, sizeof(unsigned)));
     for (int64_t done = 0; done < nsteps;) {
       const int chunk = (int)std::min<int64_t>(nsteps - done, std::max<int64_t>(1, (1LL << 30) / b->nitems));
-      lbk::PersistArgs P{};
+      lbk::MultiArgs P{};
       P.nitems = b->nitems;
       P.nsteps = chunk;
       P.kpar0 = b->kpar;
@@ -1337,8 +1329,7 @@ int lb_batch_step(lb_batch *b, int64_t nsteps) {
       P.dep_idx = b->d_dep + b->nitems + 1;
       P.next = b->d_ticket;
       LB_BCUDA(b, cudaMemsetAsync(b->d_ticket, 0, sizeof(unsigned), b->st));
-      LB_BCUDA(b, lbk::launch_sweep_batch_persist(b->store, b->d_items, b->d_args, b->d_maps, P, grid, b->smem,
-                                                  b->st));
+      LB_BCUDA(b, lbk::launch_sweep_batch_multi(b->store, b->tau1, b->d_items, b->d_args, b->consts, b->d_maps, P, b->smem, b->st));
       b->kpar = (b->kpar + chunk) & 1;
       b->epoch += (unsigned)chunk;
       done += chunk;
@@ -1351,22 +1342,10 @@ int lb_batch_step(lb_batch *b, int64_t nsteps) {
     }
     return LB_OK;
   }
-  int64_t k = 0;
-  if (b->kpar == 1) {  // one plain step to reach kpar 0
-    LB_BCUDA(b, lbk::launch_sweep_batch(b->store, b->d_items, b->nitems, b->d_args, b->d_maps, 1, 1, b->smem, b->st));
-    b->kpar = 0;
-    k = 1;
-  }
-  if (nsteps - k >= 2) {
-    int rc = batch_graph(b);
-    if (rc != LB_OK) return rc;
-    for (; k + 2 <= nsteps; k += 2) LB_BCUDA(b, cudaGraphLaunch(b->graph, b->st));
-  }
-  if (k < nsteps) {
-    LB_BCUDA(b, lbk::launch_sweep_batch(b->store, b->d_items, b->nitems, b->d_args, b->d_maps, 0, 1, b->smem, b->st));
-    b->kpar = 1;
-    k++;
-  }
+  // a single step: one plain launch
+  LB_BCUDA(b, lbk::launch_sweep_batch(b->store, b->tau1, b->d_items, b->nitems, b->d_args, b->consts, b->d_maps, b->kpar, 1,
+                                      b->smem, b->st));
+  b->kpar ^= 1;
   for (lb_handle *h : b->hs) {
     h->cur ^= (int)(nsteps & 1);
     h->step += nsteps;
@@ -1382,14 +1361,9 @@ int lb_batch_autotune(lb_batch *b, int steps, int32_t *seg_h) {
   const int n = (int)b->hs.size();
   for (lb_handle *h : b->hs)
     if (!h->initialised) return bfail(b, LB_ERR_STATE, "lb_batch_autotune: an instance is not initialised");
-  const int cand[] = {24, 32, 40, 48, 56, 64, 80, 96, 128};
+  const int cand[] = {16, 24, 32, 40, 48, 56, 64};
   // Lattice classes by height: short, medium, tall.
   auto cls = [](int ny) { return ny <= 96 ? 0 : (ny <= 160 ? 1 : 2); };
-  for (lb_handle *h : b->hs) {
-    int mx = h->sweep_nseg;
-    for (int c : cand) mx = std::max(mx, (h->p.ny + std::min(c, h->p.ny) - 1) / std::min(c, h->p.ny));
-    LB_BCUDA(b, ensure_records(h, mx));
-  }
   // Save every state; each trial starts from it.
   std::vector<void *> save(n, nullptr);
   std::vector<int> cur0(n), seg0(n);
@@ -1436,7 +1410,9 @@ int lb_batch_autotune(lb_batch *b, int steps, int32_t *seg_h) {
   float best_ms = 3.0e38f;
   for (int c : cand) {
     if (e != cudaSuccess || rc != LB_OK) break;
-    for (lb_handle *h : b->hs) set_segments(h, c);
+    for (lb_handle *h : b->hs)
+      if (e == cudaSuccess) e = change_tiles(h, h->sweep_nstrips, c);
+    if (e != cudaSuccess) break;
     float ms = 0.f;
     rc = trial(&ms);
     if (rc == LB_OK && e == cudaSuccess && ms < best_ms) {
@@ -1452,7 +1428,9 @@ int lb_batch_autotune(lb_batch *b, int steps, int32_t *seg_h) {
     for (int c : cand) {
       if (e != cudaSuccess || rc != LB_OK) break;
       if (c == best_cls[k]) continue;
-      for (lb_handle *h : b->hs) set_segments(h, cls(h->p.ny) == k ? c : best_cls[cls(h->p.ny)]);
+      for (lb_handle *h : b->hs)
+        if (e == cudaSuccess) e = change_tiles(h, h->sweep_nstrips, cls(h->p.ny) == k ? c : best_cls[cls(h->p.ny)]);
+      if (e != cudaSuccess) break;
       float ms = 0.f;
       rc = trial(&ms);
       if (rc == LB_OK && e == cudaSuccess && ms < best_ms) {
@@ -1463,7 +1441,7 @@ int lb_batch_autotune(lb_batch *b, int steps, int32_t *seg_h) {
   }
   for (int i = 0; i < n; i++) {
     lb_handle *h = b->hs[i];
-    set_segments(h, (rc == LB_OK && e == cudaSuccess) ? best_cls[cls(h->p.ny)] : seg0[i]);
+    set_tiles(h, h->sweep_nstrips, (rc == LB_OK && e == cudaSuccess) ? best_cls[cls(h->p.ny)] : seg0[i]);
     if (seg_h) seg_h[i] = h->sweep_seg;
   }
   if (e == cudaSuccess) e = restore();
@@ -1480,7 +1458,6 @@ int lb_batch_autotune(lb_batch *b, int steps, int32_t *seg_h) {
 int lb_batch_destroy(lb_batch *b) {
   if (!b) return LB_OK;
   if (b->st || !b->hs.empty()) cudaStreamSynchronize(b->st);
-  if (b->graph) cudaGraphExecDestroy(b->graph);
   for (lb_handle *h : b->hs) lb_destroy(h);
   cudaFree(b->d_items);
   cudaFree(b->d_args);
@@ -1488,7 +1465,6 @@ int lb_batch_destroy(lb_batch *b) {
   cudaFree(b->d_done);
   cudaFree(b->d_dep);
   cudaFree(b->d_ticket);
-  if (b->cap) cudaStreamDestroy(b->cap);
   delete b;
   return LB_OK;
 }

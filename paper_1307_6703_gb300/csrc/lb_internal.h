@@ -17,17 +17,37 @@ namespace lbk {
 // storage: the rest population as one float plane at fout, the deviations
 // d_i = f_i - r_i (i = 1..8) as eight 16-bit planes at fdev (same pitch,
 // plane and offset, counted in 16-bit elements).
+//
+// Constants of the packed FP32 arithmetic, each twice (one per half of a
+// pair): a pair instruction reads them as one 64-bit operand, and no
+// instruction is spent on building the pair.
+struct SweepConsts {
+  // of the lattice
+  float2 T, nb /* -b */, a, kappa, A0;
+  float2 N, M, Q, R, m4QR /* -4 (Q + R) */;
+  float2 th, g, om /* omega */, om1 /* 1 - omega */;
+  float2 Aax /* A_ax / 9 */, Adg /* A_diag / 36 */;
+  float2 r_sum;           // 16-bit storage: sum of the moving links' references
+  float2 mwr_ax, mwr_dg;  // -omega r_ax, -omega r_dg
+  // of the scheme
+  float2 one, half, two, m6 /* -1/6 */, m24 /* -1/24 */, e8 /* 1/8 */, q4 /* 1/4 */, mq4;
+  float2 third, mthird, twelfth, mtwelfth;
+};
+constexpr int kLatticeConsts = 19;  // the first of them, those of the lattice
 struct SweepArgs {
   int nx, ny, walls;
   int pitch;
   long long plane, off;
+  // tiles: nseg segments of seg_h rows by nstrips columns of tiles, base_w
+  // wide (the first `extra` wider by the column quantum)
   int seg_h, nseg, nstrips, base_w, extra;
-  float T, a, b, kappa, omega, one_minus_omega, g, th, A0, u_bot, u_top;
-  float N, M, Q, R, four_QR;
-  float A_rest, A_ax, A_diag;  // rest factors 1 + (T - T0)(c.c - 2 T0) / (2 T0^2)
+  SweepConsts k;
+  float u_bot, u_top;
   float nmax;                  // 1/b (upper bound of a valid density)
   float ref_ax, ref_dg;        // reference populations r_i of the 16-bit format
   const float *sinx;
+  const float *fin;            // the input state and its deviation planes
+  const void *fdin;
   float *fout;
   void *fdev;
   double *partials;            // 4 doubles per CTA: mass, J_x, J_y, bad-site flag
@@ -51,12 +71,22 @@ constexpr int kStoreF32 = 1, kStoreBF16 = 2, kStoreFP16 = 3;
 // Whether the sweep kernel of storage `store` can run an nx x ny lattice
 // (column quantum of its TMA boxes, ghost bands, 32-bit plane offsets).
 bool sweep_supported(int store, int nx, int ny);
-cudaError_t sweep_prepare(int store, size_t *smem_bytes);
-// Strips (widths base_w or base_w + quantum, the first `extra` wider; the
-// quantum is 4 columns for FP32 storage and 8 for 16-bit storage) and row
-// segments of the sweep kernel for an nx x ny lattice.
-void sweep_plan(int store, int nx, int ny, int *nstrips, int *base_w, int *extra, int *seg_h, int *nseg);
-// Widths of nstrips strips (>= sweep_min_strips) over nx columns: base_w or
+// (tau1 here and below: the form for relaxation time exactly 1, whose collision
+// reads no populations; every lattice of the launch must have it)
+cudaError_t sweep_prepare(int store, bool tau1, size_t *smem_bytes);
+// Default tiling of the sweep kernel for an nx x ny lattice: the fewest strips
+// and segments of 64 rows.
+void sweep_plan(int store, int nx, int ny, int *nstrips, int *seg_h);
+// Columns of tiles of a tiling with nstrips strips: one per strip, or, where a
+// strip is wider than a tile can be, the fewest that cover the lattice.
+int sweep_tile_cols(int store, int nx, int nstrips);
+// Segment height that gives about as many tiles in all as `resident` warps
+// want, for lattices of `cols` tile columns over ny rows (cols may sum over
+// several lattices).
+int sweep_seg_rule(double cols, int ny, int resident);
+// Warps of the sweep kernel one SM holds (shared memory and registers).
+int sweep_warps_per_sm(int store, bool tau1);
+// Widths of nstrips strips (>= sweep_min_strips, the fewest a tiling may name) over nx columns: base_w or
 // base_w + quantum, the first `extra` wider.
 void sweep_strips(int store, int nx, int nstrips, int *base_w, int *extra);
 int sweep_min_strips(int store, int nx);
@@ -68,12 +98,15 @@ cudaError_t sweep_make_maps(int store, void *base, int pitch, int ny, long long 
                             CUtensorMap *m1);
 // Bytes of one padded state buffer of the given storage.
 size_t sweep_buffer_bytes(int store, long long plane);
-cudaError_t launch_sweep(int store, const CUtensorMap &m0, const CUtensorMap &m1, const SweepArgs &A,
+cudaError_t launch_sweep(int store, bool tau1, const CUtensorMap &m0, const CUtensorMap &m1, const SweepArgs &A,
                          size_t smem, cudaStream_t st);
 
 // Dependency lists of the tiles (CSR): tile a waits for the tiles
-// idx[ofs[a] .. ofs[a+1]) before each step.
-void sweep_deps(int store, int nx, int ny, int walls, int nstrips, int base_w, int extra, int seg_h,
+// idx[ofs[a] .. ofs[a+1]) before each step.  Tile = column + ncol * segment;
+// `window` is the number of columns a tile is taken to read from its origin
+// - 4 (kSweepWindow: what the kernel reads).
+constexpr int kSweepWindow = 64;
+void sweep_deps(int store, int nx, int ny, int walls, int ncol, int base_w, int extra, int seg_h, int window,
                 std::vector<int> &ofs, std::vector<int> &idx);
 
 // One CTA of the batched sweep: instance `inst`, its strip and segment, the
@@ -85,13 +118,14 @@ struct BatchItem {
 // Batched step over a work list.  args: 2 per instance (input buffer 0, 1);
 // maps: 4 per instance ([input buffer][map], map 1 = deviation planes of
 // 16-bit storage or a copy of map 0), 64-byte aligned device memory.
-cudaError_t launch_sweep_batch(int store, const BatchItem *items, int nitems, const SweepArgs *args,
+// (k: the consts of the scheme)
+cudaError_t launch_sweep_batch(int store, bool tau1, const BatchItem *items, int nitems, const SweepArgs *args, const SweepConsts &k,
                                const CUtensorMap *maps, int kpar, int records, size_t smem, cudaStream_t st);
-// Multi-step batched sweep (one cooperative launch, many steps, per-item
-// completion counters instead of a grid-wide barrier between steps).
+// Multi-step sweeps (one launch, many steps, per-item completion counters
+// instead of a grid-wide barrier between steps).
 // Item i of a step whose batch parity is kpar reads the input buffer
 // items[i].par0 ^ kpar of its lattice; kpar = (kpar0 + k) & 1 at step k.
-struct PersistArgs {
+struct MultiArgs {
   int nitems;
   int nsteps;
   int kpar0;
@@ -122,18 +156,14 @@ struct MultiOut {
   int mon_cap;
   long long mon_step0;
 };
-// One lattice, P.nsteps steps in one cooperative launch (P.kpar0 = the
+// One lattice, P.nsteps steps in one launch (P.kpar0 = the
 // input buffer of the first step; items are the tiles in index order).
-cudaError_t launch_sweep_multi(int store, const CUtensorMap (&maps)[2][2], const SweepArgs &A, const PersistArgs &P,
-                               const MultiOut &Q, int grid, size_t smem, cudaStream_t st);
-// Resident CTAs of the multi-step batched kernel on this device (its grid
-// may not exceed this: the dependency waits need every CTA resident).
-cudaError_t persist_capacity(int store, size_t smem, int *blocks);
-// P.nsteps batch steps in one cooperative launch of `grid` CTAs; the mass /
-// momentum records of the last step go to each instance's record array.
-cudaError_t launch_sweep_batch_persist(int store, const BatchItem *items, const SweepArgs *args,
-                                       const CUtensorMap *maps, const PersistArgs &P, int grid, size_t smem,
-                                       cudaStream_t st);
+cudaError_t launch_sweep_multi(int store, bool tau1, const CUtensorMap (&maps)[2][2], const SweepArgs &A, const MultiArgs &P,
+                               const MultiOut &Q, size_t smem, cudaStream_t st);
+// P.nsteps batch steps in one launch; the mass / momentum records of the last
+// step go to each instance's record array.
+cudaError_t launch_sweep_batch_multi(int store, bool tau1, const BatchItem *items, const SweepArgs *args, const SweepConsts &k,
+                                     const CUtensorMap *maps, const MultiArgs &P, size_t smem, cudaStream_t st);
 // Copy the periodic images into the ghost band of `nplanes` planes of
 // `elem_bytes`-byte elements (4 or 2).
 cudaError_t launch_ghost_fill(void *f, int elem_bytes, int nplanes, int nx, int ny, int pitch, long long plane,
