@@ -106,8 +106,7 @@ typedef struct lb_handle lb_handle;
 
 /* Create a solver for the problem *p and allocate its device state (two
  * population buffers of 9*nx*ny elements -- 16-bit storage: one float and
- * eight 16-bit planes -- plus small work buffers; 16-bit storage adds one
- * float copy of the nine planes for moments, reductions and init).
+ * eight 16-bit planes -- plus small work buffers).
  * *out receives the handle.  Errors: LB_ERR_ARG (bad sizes, tau <= 1/2,
  * b*n range, precision), LB_ERR_CUDA, LB_ERR_OOM.                          */
 int lb_create(const lb_params *p, lb_handle **out);

@@ -22,6 +22,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 UNITS = {
     "lb_api.cu": [],
     "lb_f32.cu": [],
+    "lb_init.cu": [],
     "lb_f64.cu": ["--fmad=false"],
     "lb_noalloc.cu": [],
     "lb_sweep.cu": [],

@@ -8,6 +8,9 @@
 #include <string>
 #include <vector>
 
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
 #include "lb.h"
 #include "lb_device.cuh"
 #include "lb_internal.h"
@@ -29,7 +32,6 @@ struct lb_handle {
   int store = 0;                 // its storage format (lbk::kStoreF32, kStoreBF16, kStoreFP16)
   CUtensorMap tmap[2][2];        // TMA descriptors of the two state buffers
   float ref_ax = 0.f, ref_dg = 0.f;  // reference populations of 16-bit storage
-  float *wide = nullptr;         // 16-bit storage: nine float planes (moments, reductions, init)
   size_t sweep_smem = 0;
   // The tiling as lb_set_tiling names it, and the tiles the kernel runs on
   // (set_tiles): tile_cols columns of tiles, base_w wide (the first `extra`
@@ -162,12 +164,32 @@ StepArgs<real_t> make_args(const lb_handle *h) {
 
 constexpr int RED_THREADS = 256;
 
+// The populations of a site (element e of a plane) in FP64.
+template <typename real_t>
+struct LoadPlanes {
+  const real_t *f;
+  long long plane;
+  __device__ double operator()(int i, long long e) const { return (double)f[i * plane + e]; }
+};
+// 16-bit storage: f_0 as stored, f_i = r_i + d_i rounded to FP32.
+template <typename H>
+struct LoadDev {
+  const float *f0;
+  const H *d;
+  long long plane;
+  float ref_ax, ref_dg;
+  __device__ double operator()(int i, long long e) const {
+    if (i == 0) return (double)f0[e];
+    return (double)((i <= 4 ? ref_ax : ref_dg) + (float)d[(i - 1) * plane + e]);
+  }
+};
+
 // Pass 1: each block sums mass and momentum of its grid-stride share of the
 // sites in FP64 (fixed order) and flags non-finite or out-of-range sites.
-template <typename real_t>
+template <class Load>
 __global__ void __launch_bounds__(RED_THREADS)
-reduce_pass1(const real_t *__restrict__ f, int nx, size_t S, int pitch, long long plane,
-             long long off, double nmax, double *__restrict__ partials, int *__restrict__ flag) {
+reduce_pass1(const Load load, int nx, size_t S, int pitch, long long off, double nmax, double *__restrict__ partials,
+             int *__restrict__ flag) {
   __shared__ double sm[3][RED_THREADS];
   double m = 0.0, jx = 0.0, jy = 0.0;
   int bad = 0;
@@ -176,7 +198,7 @@ reduce_pass1(const real_t *__restrict__ f, int nx, size_t S, int pitch, long lon
     const long long e = off + (long long)(s / (size_t)nx) * pitch + (long long)(s % (size_t)nx);
     double v[9];
 #pragma unroll
-    for (int i = 0; i < 9; i++) v[i] = (double)f[i * plane + e];
+    for (int i = 0; i < 9; i++) v[i] = load(i, e);
     double ms = 0.0;
 #pragma unroll
     for (int i = 0; i < 9; i++) ms += v[i];
@@ -289,17 +311,6 @@ char *plane_ptr(const lb_handle *h, int b, int q, size_t *esize) {
   }
   *esize = 2;
   return base + (size_t)h->plane * sizeof(float) + ((size_t)(q - 1) * h->plane + h->off) * 2;
-}
-
-// The nine float planes of the current state: the state buffer itself for
-// FP32, else the widened copy.
-cudaError_t current_f32(lb_handle *h, const float **out) {
-  if (!dev16(h)) {
-    *out = (const float *)h->f[h->cur];
-    return cudaSuccess;
-  }
-  *out = h->wide;
-  return lbk::launch_widen(h->store, h->f[h->cur], h->wide, h->plane, h->ref_ax, h->ref_dg, h->st);
 }
 
 // Whether the handle's lattice takes the tau = 1 form of the sweep.
@@ -611,8 +622,6 @@ int lb_create(const lb_params *p, lb_handle **out) {
     for (int b = 0; b < 2 && e == cudaSuccess; b++)
       e = lbk::sweep_make_maps(h->store, h->f[b], h->pitch, p->ny, h->plane, &h->tmap[b][0], &h->tmap[b][1]);
   }
-  if (e == cudaSuccess && dev16(h)) e = cudaMalloc((void **)&h->wide, 9 * (size_t)h->plane * sizeof(float));
-  if (e == cudaSuccess && dev16(h)) e = cudaMemset(h->wide, 0, 9 * (size_t)h->plane * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&h->sinx, (size_t)p->nx * h->elem);
   h->red_blocks = (int)std::min<size_t>((h->S + RED_THREADS - 1) / RED_THREADS, 1024);
   if (e == cudaSuccess) e = cudaMalloc((void **)&h->d_partials, 3 * (size_t)h->red_blocks * sizeof(double));
@@ -668,24 +677,18 @@ int lb_init(lb_handle *h, int mode, uint64_t seed, double rho_mean, double noise
     }
   }
   h->cur = 0;
-  // 16-bit storage: the float equilibrium goes through the storage format.
-  float *f32 = dev16(h) ? h->wide : (float *)h->f[0];
-  cudaError_t e = fp64(h)
-                      ? lbk::launch_init((double *)h->f[0], h->p.nx, h->p.ny, h->pitch, h->plane,
-                                         h->off, mode, seed, rho_mean, noise_amp, dr, du, dv,
-                                         h->p.T, h->st)
-                      : lbk::launch_init(f32, h->p.nx, h->p.ny, h->pitch, h->plane,
-                                         h->off, mode, seed, rho_mean, noise_amp, dr, du, dv,
-                                         h->p.T, h->st);
+  cudaError_t e;
+  if (fp64(h)) {
+    e = lbk::launch_init((double *)h->f[0], h->p.nx, h->p.ny, h->pitch, h->plane, h->off, mode, seed, rho_mean,
+                         noise_amp, dr, du, dv, h->p.T, h->st);
+  } else {
+    const int images = !h->sweep ? 0 : (h->p.walls ? 1 : 2);
+    e = lbk::launch_init_f32(h->store, h->f[0],
+                             {h->p.nx, h->p.ny, h->pitch, h->plane, h->off, images, seed, rho_mean, noise_amp, h->p.T,
+                              dr, du, dv, h->ref_ax, h->ref_dg},
+                             h->st);
+  }
   if (e != cudaSuccess) return cuda_fail(h, e, "lb_init: init kernel");
-  if (h->sweep) {
-    e = lbk::launch_ghost_fill(f32, 4, 9, h->p.nx, h->p.ny, h->pitch, h->plane, h->off, h->p.walls, h->st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "lb_init: ghost fill");
-  }
-  if (dev16(h)) {
-    e = lbk::launch_narrow(h->store, h->wide, h->f[0], h->plane, h->ref_ax, h->ref_dg, h->st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "lb_init: 16-bit store");
-  }
   h->cta_valid = false;
   h->total_valid = false;
   if (mode == 1) LB_CUDA(h, cudaStreamSynchronize(h->st));
@@ -769,10 +772,21 @@ int lb_moments(lb_handle *h, void *rho, void *ux, void *uy, int dtype, int on_de
   cudaError_t e;
   if (fp64(h)) {
     e = lbk::launch_moments((const double *)h->f[h->cur], make_args<double>(h), dn, du, dv, dtype, h->st);
+  } else if (h->sweep) {
+    lbk::SweepArgs A = sweep_args(h, h->cur);
+    if (!on_device && !(staged[0] || staged[1] || staged[2])) {
+      // Written over the host link: tiles of 32 columns, so that a warp writes
+      // whole 128-byte lines (4096 x 1024 in 285 us; 332 with tiles of 56).
+      A.nstrips = (h->p.nx + 31) / 32;
+      lbk::sweep_strips(h->store, h->p.nx, A.nstrips, &A.base_w, &A.extra);
+    }
+    // tiles that fill the device with this lattice alone (a batch cuts its
+    // lattices into higher ones: 30 us for one of them, against 6)
+    A.seg_h = lbk::sweep_seg_rule(A.nstrips, h->p.ny, h->resident);
+    A.nseg = (h->p.ny + A.seg_h - 1) / A.seg_h;
+    e = lbk::launch_sweep_moments(h->store, h->tmap[h->cur][0], h->tmap[h->cur][1], A, dn, du, dv, dtype, h->st);
   } else {
-    const float *f32 = nullptr;
-    e = current_f32(h, &f32);
-    if (e == cudaSuccess) e = lbk::launch_moments(f32, make_args<float>(h), dn, du, dv, dtype, h->st);
+    e = lbk::launch_moments((const float *)h->f[h->cur], make_args<float>(h), dn, du, dv, dtype, h->st);
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "lb_moments: kernel");
   if (!on_device) {
@@ -796,16 +810,18 @@ static int enqueue_reduce(lb_handle *h) {
     reduce_cta<<<1, RED_THREADS, 0, h->st>>>(h->d_cta, ntiles(h), h->d_out, h->d_err);
   } else {
     LB_CUDA(h, cudaMemsetAsync(h->d_flag, 0, sizeof(int), h->st));
-    if (fp64(h))
-      reduce_pass1<double><<<h->red_blocks, RED_THREADS, 0, h->st>>>(
-          (const double *)h->f[h->cur], h->p.nx, h->S, h->pitch, h->plane, h->off, nmax,
-          h->d_partials, h->d_flag);
-    else {
-      const float *f32 = nullptr;
-      LB_CUDA(h, current_f32(h, &f32));
-      reduce_pass1<float><<<h->red_blocks, RED_THREADS, 0, h->st>>>(
-          f32, h->p.nx, h->S, h->pitch, h->plane, h->off, nmax, h->d_partials, h->d_flag);
-    }
+    const void *f = h->f[h->cur];
+    auto pass1 = [&](auto load) {
+      reduce_pass1<<<h->red_blocks, RED_THREADS, 0, h->st>>>(load, h->p.nx, h->S, h->pitch, h->off, nmax, h->d_partials,
+                                                             h->d_flag);
+    };
+    const float *f0 = (const float *)f;
+    const void *d = f0 + h->plane;
+    if (fp64(h)) pass1(LoadPlanes<double>{(const double *)f, h->plane});
+    else if (h->p.precision == LB_FP32) pass1(LoadPlanes<float>{f0, h->plane});
+    else if (h->p.precision == LB_BF16DEV)
+      pass1(LoadDev<__nv_bfloat16>{f0, (const __nv_bfloat16 *)d, h->plane, h->ref_ax, h->ref_dg});
+    else pass1(LoadDev<__half>{f0, (const __half *)d, h->plane, h->ref_ax, h->ref_dg});
     LB_CUDA(h, cudaGetLastError());
     reduce_pass2<<<1, RED_THREADS, 0, h->st>>>(h->d_partials, h->red_blocks, h->d_out, h->d_flag, h->d_err);
   }
@@ -1085,7 +1101,6 @@ int lb_destroy(lb_handle *h) {
   cudaFree(h->d_arrive);
   cudaFree(h->d_cta);
   cudaFree(h->d_err);
-  cudaFree(h->wide);
   cudaFree(h->d_done);
   cudaFree(h->d_dep);
   cudaFree(h->d_ticket);

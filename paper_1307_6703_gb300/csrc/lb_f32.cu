@@ -28,13 +28,6 @@ cudaError_t launch_moments(const float *fin, const StepArgs<float> &A, void *n, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_init(float *f, int nx, int ny, int pitch, long long plane, long long off, int mode, uint64_t seed, double rho_mean,
-                        double amp, const double *rho0, const double *ux0, const double *uy0,
-                        double T, cudaStream_t st) {
-  init_kernel<float><<<init_grid(nx, ny), 256, 0, st>>>(f, nx, ny, pitch, plane, off, mode, seed, rho_mean, amp, rho0, ux0, uy0, T);
-  return cudaGetLastError();
-}
-
 // Copy the periodic images into the ghost band of nplanes padded planes.
 // Only band elements are visited (blockIdx.y is the plane): first the
 // 4 + 4 ghost columns of rows -4 .. ny+3 (with walls rows 0 .. ny-1 only:

@@ -101,6 +101,11 @@ size_t sweep_buffer_bytes(int store, long long plane);
 cudaError_t launch_sweep(int store, bool tau1, const CUtensorMap &m0, const CUtensorMap &m1, const SweepArgs &A,
                          size_t smem, cudaStream_t st);
 
+// Density and velocity u* of the state A.fin describes (maps m0, m1) into
+// compact arrays n, ux, uy (each may be null; dtype 0 = double, 1 = float).
+cudaError_t launch_sweep_moments(int store, const CUtensorMap &m0, const CUtensorMap &m1, const SweepArgs &A, void *n,
+                                 void *ux, void *uy, int dtype, cudaStream_t st);
+
 // Dependency lists of the tiles (CSR): tile a waits for the tiles
 // idx[ofs[a] .. ofs[a+1]) before each step.  Tile = column + ncol * segment;
 // `window` is the number of columns a tile is taken to read from its origin
@@ -168,14 +173,6 @@ cudaError_t launch_sweep_batch_multi(int store, bool tau1, const BatchItem *item
 // `elem_bytes`-byte elements (4 or 2).
 cudaError_t launch_ghost_fill(void *f, int elem_bytes, int nplanes, int nx, int ny, int pitch, long long plane,
                               long long off, int walls, cudaStream_t st);
-// 16-bit storage <-> nine float planes (same padded layout, every element
-// of the planes, ghost bands included).  narrow: d_i = f_i - r_i rounded to
-// nearest even, rest plane = n - sum_{i>=1} (r_i + d_i).
-cudaError_t launch_widen(int store, const void *buf, float *wide, long long plane, float ref_ax, float ref_dg,
-                         cudaStream_t st);
-cudaError_t launch_narrow(int store, const float *wide, void *buf, long long plane, float ref_ax, float ref_dg,
-                          cudaStream_t st);
-
 template <typename real_t>
 struct StepArgs;
 
@@ -193,8 +190,17 @@ cudaError_t launch_moments(const float *fin, const StepArgs<float> &A, void *n, 
 cudaError_t launch_init(double *f, int nx, int ny, int pitch, long long plane, long long off, int mode, uint64_t seed, double rho_mean,
                         double amp, const double *rho0, const double *ux0, const double *uy0,
                         double T, cudaStream_t st);
-cudaError_t launch_init(float *f, int nx, int ny, int pitch, long long plane, long long off, int mode, uint64_t seed, double rho_mean,
-                        double amp, const double *rho0, const double *ux0, const double *uy0,
-                        double T, cudaStream_t st);
+// The same for FP32 and 16-bit lattices (lb_init.cu): the state buffer buf of
+// storage `store` in one pass, its ghost band included.
+struct InitState {
+  int nx, ny, pitch;
+  long long plane, off;
+  int images;  // periodic images to write: 0 none (compact planes), 1 along x (walls), 2 along x and y
+  uint64_t seed;
+  double rho_mean, amp, T;
+  const double *n0, *ux, *uy;  // density and velocity fields; n0 null: noise
+  float ref_ax, ref_dg;
+};
+cudaError_t launch_init_f32(int store, void *buf, const InitState &I, cudaStream_t st);
 
 }  // namespace lbk

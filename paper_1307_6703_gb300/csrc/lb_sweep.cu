@@ -186,9 +186,7 @@ struct StoreDev {
     const unsigned *w = words(r, q);
     return make_float2(hi(w[0]), lo(w[1]));
   }
-  // element form (format conversion kernels)
-  __device__ static float dec(H v);
-  __device__ static H enc(float v);
+  __device__ static float dec(H v);  // one element
 };
 template <>
 __device__ __forceinline__ float StoreDev<__nv_bfloat16>::lo(unsigned w) { return __uint_as_float(w << 16); }
@@ -201,8 +199,6 @@ __device__ __forceinline__ unsigned StoreDev<__nv_bfloat16>::enc2(float2 v) {
 }
 template <>
 __device__ __forceinline__ float StoreDev<__nv_bfloat16>::dec(__nv_bfloat16 v) { return __bfloat162float(v); }
-template <>
-__device__ __forceinline__ __nv_bfloat16 StoreDev<__nv_bfloat16>::enc(float v) { return __float2bfloat16_rn(v); }
 template <>
 __device__ __forceinline__ float StoreDev<__half>::lo(unsigned w) {
   return __low2float(*reinterpret_cast<const __half2 *>(&w));
@@ -218,8 +214,6 @@ __device__ __forceinline__ unsigned StoreDev<__half>::enc2(float2 v) {
 }
 template <>
 __device__ __forceinline__ float StoreDev<__half>::dec(__half v) { return __half2float(v); }
-template <>
-__device__ __forceinline__ __half StoreDev<__half>::enc(float v) { return __float2half_rn(v); }
 
 using StoreBF16 = StoreDev<__nv_bfloat16>;
 using StoreFP16 = StoreDev<__half>;
@@ -584,6 +578,30 @@ struct WaitGrid {
   }
 };
 
+// Where a moments launch writes: compact [ny][nx] arrays (null: not wanted)
+// of T; a lane's two columns in one store where the arrays are aligned for it.
+struct NoMoments {
+  static constexpr bool kOn = false;
+};
+template <class T>
+struct Moments {
+  static constexpr bool kOn = true;
+  T *n, *ux, *uy;
+  int pairs;
+  __device__ __forceinline__ void put(T *p, size_t s, float2 v) const {
+    if (p == nullptr) return;
+    if (pairs) {
+      struct alignas(2 * sizeof(T)) Two {
+        T a, b;
+      };
+      *reinterpret_cast<Two *>(p + s) = Two{(T)v.x, (T)v.y};
+    } else {
+      p[s] = (T)v.x;
+      p[s + 1] = (T)v.y;
+    }
+  }
+};
+
 // Origin and width of tile column i: base_w columns, the first `extra`
 // columns of tiles one quantum wider.
 template <class St>
@@ -599,10 +617,11 @@ __device__ __forceinline__ void tile_columns(const SweepArgs &A, int i, int &x0,
 // (the warp then stopped and drained the copies still in flight).
 // kMulti: called once per tile by the multi-step kernel, which does not
 // hand its SM slots to a dependent grid early.
-template <class St, bool kTau1, bool kMulti = false, class Wait = WaitGrid, class Done = NoDone>
+template <class St, bool kTau1, bool kMulti = false, class Wait = WaitGrid, class Done = NoDone, class Mom = NoMoments>
 __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtensorMap *tdev, const SweepArgs &A, const SweepConsts &K,
                                            const StepIO &O, const int strip, const int seg, double *rec,
-                                           const bool records, const Wait &wait = Wait{}, const Done &done = Done{}) {
+                                           const bool records, const Wait &wait = Wait{}, const Done &done = Done{},
+                                           const Mom &mom = Mom{}) {
   using Row = typename St::Row;
   using Smem = SmemOf<St, kTau1>;
   using V = V2;
@@ -774,6 +793,24 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
         JxC[j] = V::fma(K.half, Fx, sx);
         JyC[j] = V::fma(K.half, Fy, sy);
       }
+    }
+    if constexpr (Mom::kOn) {
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int y = a - 2 + j;
+        if (!actD || y < ya || y >= yb) continue;
+        const float2 n = j ? N1.c : N0.c;
+        const size_t s = (size_t)y * nx + x;
+        mom.put(mom.n, s, n);
+        if (mom.ux != nullptr) mom.put(mom.ux, s, make_float2(__fdiv_rn(JxC[j].x, n.x), __fdiv_rn(JxC[j].y, n.y)));
+        if (mom.uy != nullptr) mom.put(mom.uy, s, make_float2(__fdiv_rn(JyC[j].x, n.x), __fdiv_rn(JyC[j].y, n.y)));
+      }
+      n3 = N1.c;
+      N0 = N2; N1 = N3;
+      sx2 = sxA[0]; sy2 = syA[0]; sx1 = sxA[1]; sy1 = syA[1];
+      P0 = P2; P1 = P3; L0 = L2; L1 = L3;
+      s0 = s1;
+      return;
     }
     const float2 dJ2 = xdiff(spread(JxC[0])), dJ1 = xdiff(spread(JxC[1]));
     const Nbr Jy2 = spread(JyC[0]), Jy1 = spread(JyC[1]);
@@ -1043,6 +1080,16 @@ __device__ __forceinline__ SweepConsts lattice_consts(const SweepConsts &own, co
   return k;
 }
 
+// Density and velocity of a state: the same sweep, stages A to C only.  Reads
+// the populations once (36 or 20 bytes a site) and writes the three fields.
+template <class St, class T>
+__global__ void __launch_bounds__(kThreads, Form<St, true>::kMinBlocks)
+sweep_moments_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tdev,
+                     const __grid_constant__ SweepArgs A, const Moments<T> M) {
+  const StepIO O{A.fin, A.fdin, nullptr, nullptr, nullptr, 0u, nullptr, nullptr, nullptr, 0.0};
+  (void)sweep_body<St, true>(&tin, &tdev, A, A.k, O, blockIdx.x, blockIdx.y, nullptr, false, WaitGrid{}, NoDone{}, M);
+}
+
 // Batched step: CTA b works on items[b] (instance, strip, segment) of a
 // work list over many independent lattices.  Arguments and tensor maps of
 // each instance sit in device memory for both buffer parities; an instance
@@ -1200,40 +1247,6 @@ sweep_multi_kernel(const __grid_constant__ CUtensorMap tin0, const __grid_consta
   }
 }
 
-// 16-bit storage -> nine float planes: f_0 as stored, f_i = r_i + d_i.
-template <class St, typename H>
-__global__ void widen_kernel(const float *__restrict__ f0, const H *__restrict__ d, float *__restrict__ out,
-                             long long plane, float ref_ax, float ref_dg) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < plane;
-       e += (long long)gridDim.x * blockDim.x) {
-    out[e] = f0[e];
-#pragma unroll
-    for (int q = 1; q < 9; ++q) out[q * plane + e] = (q <= 4 ? ref_ax : ref_dg) + St::dec(d[(q - 1) * plane + e]);
-  }
-}
-
-// Nine float planes -> 16-bit storage (the rounding of the step kernel's
-// store, with n the float sum of the nine values).
-template <class St, typename H>
-__global__ void narrow_kernel(const float *__restrict__ in, float *__restrict__ f0, H *__restrict__ d,
-                              long long plane, float ref_ax, float ref_dg) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < plane;
-       e += (long long)gridDim.x * blockDim.x) {
-    float f[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) f[q] = in[q * plane + e];
-    const float n = (((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]))) + f[8];
-#pragma unroll
-    for (int q = 1; q < 9; ++q) {
-      const float r = q <= 4 ? ref_ax : ref_dg;
-      const H c = St::enc(f[q] - r);
-      d[(q - 1) * plane + e] = c;
-      f[q] = r + St::dec(c);
-    }
-    f0[e] = n - (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
-  }
-}
-
 namespace {
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point.
@@ -1335,7 +1348,17 @@ cudaError_t launch_multi_one(const CUtensorMap (&m)[2][2], const SweepArgs &A, c
   return cudaLaunchKernelEx(&cfg, sweep_multi_kernel<St, kTau1>, m[0][0], m[0][1], m[1][0], m[1][1], A, P, Q);
 }
 
-unsigned elementwise_blocks(long long n) { return (unsigned)std::min<long long>((n + 255) / 256, 4096); }
+template <class St, class T>
+cudaError_t launch_moments_one(const CUtensorMap &m0, const CUtensorMap &m1, const SweepArgs &A, void *n, void *ux,
+                               void *uy, cudaStream_t st) {
+  const int smem = (int)sizeof(SmemOf<St, true>);
+  cudaError_t e = cudaFuncSetAttribute(sweep_moments_kernel<St, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const uintptr_t all = (uintptr_t)n | (uintptr_t)ux | (uintptr_t)uy;  // (nx is a multiple of 4: rows keep the alignment)
+  const Moments<T> M{(T *)n, (T *)ux, (T *)uy, all % (2 * sizeof(T)) == 0};
+  sweep_moments_kernel<St, T><<<dim3((unsigned)A.nstrips, (unsigned)A.nseg), kThreads, smem, st>>>(m0, m1, A, M);
+  return cudaGetLastError();
+}
 
 }  // namespace
 
@@ -1413,6 +1436,22 @@ cudaError_t sweep_prepare(int store, bool tau1, size_t *smem_bytes) {
 cudaError_t launch_sweep(int store, bool tau1, const CUtensorMap &m0, const CUtensorMap &m1, const SweepArgs &A,
                          size_t smem, cudaStream_t st) {
   LB_SWEEP_FORM(store, tau1, launch_one, m0, m1, A, smem, st);
+}
+
+cudaError_t launch_sweep_moments(int store, const CUtensorMap &m0, const CUtensorMap &m1, const SweepArgs &A, void *n,
+                                 void *ux, void *uy, int dtype, cudaStream_t st) {
+  switch (store) {
+    case kStoreF32:
+      return dtype == 0 ? launch_moments_one<StoreF32, double>(m0, m1, A, n, ux, uy, st)
+                        : launch_moments_one<StoreF32, float>(m0, m1, A, n, ux, uy, st);
+    case kStoreBF16:
+      return dtype == 0 ? launch_moments_one<StoreBF16, double>(m0, m1, A, n, ux, uy, st)
+                        : launch_moments_one<StoreBF16, float>(m0, m1, A, n, ux, uy, st);
+    case kStoreFP16:
+      return dtype == 0 ? launch_moments_one<StoreFP16, double>(m0, m1, A, n, ux, uy, st)
+                        : launch_moments_one<StoreFP16, float>(m0, m1, A, n, ux, uy, st);
+  }
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_sweep_batch(int store, bool tau1, const BatchItem *items, int nitems, const SweepArgs *args,
@@ -1495,34 +1534,6 @@ void sweep_deps(int store, int nx, int ny, int walls, int ncol, int base_w, int 
           if (v.how & c.how) idx.push_back(c.i + ncol * v.i);
       ofs[(size_t)s + (size_t)ncol * g + 1] = (int)idx.size();
     }
-}
-
-cudaError_t launch_widen(int store, const void *buf, float *wide, long long plane, float ref_ax, float ref_dg,
-                         cudaStream_t st) {
-  const float *f0 = static_cast<const float *>(buf);
-  const void *d = static_cast<const char *>(buf) + (size_t)plane * sizeof(float);
-  const unsigned blocks = elementwise_blocks(plane);
-  if (store == kStoreBF16)
-    widen_kernel<StoreBF16><<<blocks, 256, 0, st>>>(f0, (const __nv_bfloat16 *)d, wide, plane, ref_ax, ref_dg);
-  else if (store == kStoreFP16)
-    widen_kernel<StoreFP16><<<blocks, 256, 0, st>>>(f0, (const __half *)d, wide, plane, ref_ax, ref_dg);
-  else
-    return cudaErrorInvalidValue;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_narrow(int store, const float *wide, void *buf, long long plane, float ref_ax, float ref_dg,
-                          cudaStream_t st) {
-  float *f0 = static_cast<float *>(buf);
-  void *d = static_cast<char *>(buf) + (size_t)plane * sizeof(float);
-  const unsigned blocks = elementwise_blocks(plane);
-  if (store == kStoreBF16)
-    narrow_kernel<StoreBF16><<<blocks, 256, 0, st>>>(wide, f0, (__nv_bfloat16 *)d, plane, ref_ax, ref_dg);
-  else if (store == kStoreFP16)
-    narrow_kernel<StoreFP16><<<blocks, 256, 0, st>>>(wide, f0, (__half *)d, plane, ref_ax, ref_dg);
-  else
-    return cudaErrorInvalidValue;
-  return cudaGetLastError();
 }
 
 }  // namespace lbk
