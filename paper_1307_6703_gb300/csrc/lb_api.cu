@@ -38,6 +38,7 @@ struct lb_handle {
   // one quantum wider), by tile_nseg segments of tile_rows rows.
   int sweep_seg = 64, sweep_nstrips = 0;
   int tile_cols = 0, tile_base = 0, tile_extra = 0, tile_rows = 0, tile_nseg = 0;
+  int tile_ty = 0;               // tile kernel: rows of its tiles
   int want_rows = 0;             // tile height where segments would leave warps idle
   int resident = 1;              // warps of the kernel the device holds
   double *d_cta = nullptr;       // per-CTA partials written by the sweep kernel
@@ -157,6 +158,7 @@ StepArgs<real_t> make_args(const lb_handle *h) {
   A.R = (real_t)R;
   A.four_QR = (real_t)(4.0 * (p.Q + R));
   A.sinx = (const real_t *)h->sinx;
+  A.ty = h->tile_ty;
   return A;
 }
 
@@ -470,14 +472,17 @@ cudaError_t ensure_deps(lb_handle *h) {
   return cudaSuccess;
 }
 
-// Warps of the sweep kernel the current device holds at once.
-int resident_warps(int store, bool form_tau1) {
+// SMs of the current device.
+int device_sms() {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     sms = 1;  // (lb_create reports the missing device)
-  return std::max(sms, 1) * lbk::sweep_warps_per_sm(store, form_tau1);
+  return std::max(sms, 1);
 }
+
+// Warps of the sweep kernel the current device holds at once.
+int resident_warps(int store, bool form_tau1) { return device_sms() * lbk::sweep_warps_per_sm(store, form_tau1); }
 
 constexpr int kMonSlots = 64;  // steps per multi-step launch while monitoring
 
@@ -606,6 +611,7 @@ int lb_create(const lb_params *p, lb_handle **out) {
     h->pitch = p->nx;
     h->plane = (long long)h->S;
     h->off = 0;
+    h->tile_ty = lbk::tile_height(p->nx, p->ny, device_sms());
   }
   const size_t buf_bytes = h->sweep ? lbk::sweep_buffer_bytes(h->store, h->plane) : 9 * (size_t)h->plane * h->elem;
   cudaError_t e = cudaGetDevice(&h->device);

@@ -43,52 +43,78 @@ struct StepArgs {
   real_t A0, u_bot, u_top;
   real_t N, M, Q, R, four_QR /* 4 (Q + R) */;
   const real_t *sinx;   // sin(2 pi x / lambda), device, [nx]
+  int ty;               // tile height of the launch (tile_height)
 };
 
 // ------------------------------------------------------------ site physics
 
-// Eq. (eqfunc) with general T0.
-template <typename real_t>
-__device__ __forceinline__ void feq9(real_t n, real_t ux, real_t uy, real_t T, real_t *fe) {
-  constexpr real_t T0 = Consts<real_t>::T0;
-  const real_t uu = ux * ux + uy * uy;
-#pragma unroll
-  for (int i = 0; i < 9; i++) {
-    const real_t cu = real_t(cx(i)) * ux + real_t(cy(i)) * uy;
-    const real_t cc = real_t(cx(i) * cx(i) + cy(i) * cy(i));
-    const real_t t1 = cu / T0;
-    const real_t t2 = (cu * cu - T0 * uu) / (real_t(2.0) * T0 * T0);
-    const real_t t3 = (T - T0) * (cc - real_t(2.0) * T0) / (real_t(2.0) * T0 * T0);
-    fe[i] = Consts<real_t>::w(i) * n * (((real_t(1.0) + t1) + t2) + t3);
-  }
+// x / c for a constant c whose reciprocal z = RN(1/c) is at hand: the quotient
+// x z with one correction by its exact remainder (Markstein, IBM J. Res. Dev.
+// 34 (1990) 111; Brisebarre, Muller & Raina, IEEE Trans. Comput. 53 (2004)
+// 1069).  Three operations instead of a division's ten, and the same value: the
+// result can differ from the rounded quotient only where x/c lies within 2^-52
+// units of the last place of a midpoint, and for the two divisors used here
+// (T0 and 2 T0^2 in FP64) every such x gives the rounded quotient too (the few
+// candidates solve a congruence modulo 2^53).  Zero, infinite and NaN x and
+// results below the normal range aside.
+__device__ __forceinline__ double div_const(double x, double c, double z) {
+  const double q = __dmul_rn(x, z);
+  return __fma_rn(__fma_rn(-c, q, x), z, q);
+}
+__device__ __forceinline__ float div_const(float x, float c, float z) {
+  const float q = __fmul_rn(x, z);
+  return __fmaf_rn(__fmaf_rn(-c, q, x), z, q);
 }
 
-// Eqs. (forceterm, coeff), A = 0.
+// Eq. (eqfunc) with general T0.  Opposite links share their terms (c.u changes
+// sign, nothing else); iso[c.c] = (T - T0)(c.c - 2 T0) / (2 T0^2).
+template <typename real_t>
+__device__ __forceinline__ void isotropic3(real_t T, real_t *iso) {
+  constexpr real_t T0 = Consts<real_t>::T0;
+#pragma unroll
+  for (int c = 0; c < 3; c++) iso[c] = (T - T0) * (real_t(c) - real_t(2.0) * T0) / (real_t(2.0) * T0 * T0);
+}
+template <typename real_t>
+__device__ __forceinline__ void feq9(real_t n, real_t ux, real_t uy, const real_t *iso, real_t *fe) {
+  constexpr real_t T0 = Consts<real_t>::T0, zT0 = real_t(1.0) / T0;
+  constexpr real_t c2 = real_t(2.0) * T0 * T0, zc2 = real_t(1.0) / c2;
+  const real_t Tuu = T0 * (ux * ux + uy * uy);
+  const real_t wn[3] = {Consts<real_t>::w(0) * n, Consts<real_t>::w(1) * n, Consts<real_t>::w(5) * n};
+  fe[0] = wn[0] * ((real_t(1.0) + div_const(-Tuu, c2, zc2)) + iso[0]);
+  auto pair = [&](int i, int j, int c, real_t cu) {
+    const real_t t1 = div_const(cu, T0, zT0), t2 = div_const(cu * cu - Tuu, c2, zc2);
+    fe[i] = wn[c] * (((real_t(1.0) + t1) + t2) + iso[c]);
+    fe[j] = wn[c] * (((real_t(1.0) - t1) + t2) + iso[c]);
+  };
+  pair(1, 3, 1, ux);
+  pair(2, 4, 1, uy);
+  pair(5, 7, 2, ux + uy);
+  pair(6, 8, 2, uy - ux);
+}
+
+// Eqs. (forceterm, coeff), A = 0; C is symmetric.
 template <typename real_t>
 __device__ __forceinline__ void forcing9(real_t g, real_t th, real_t ux, real_t uy, real_t Fx,
                                          real_t Fy, real_t dnx, real_t dny, real_t divJ,
                                          real_t *Fi) {
-  constexpr real_t T0 = Consts<real_t>::T0;
-  const real_t u[2] = {ux, uy}, F[2] = {Fx, Fy}, dn[2] = {dnx, dny};
-  real_t B[2], C[2][2];
-#pragma unroll
-  for (int a = 0; a < 2; a++) {
-    B[a] = g * F[a];
-#pragma unroll
-    for (int b = 0; b < 2; b++) {
-      const real_t delta = (a == b) ? real_t(1.0) : real_t(0.0);
-      C[a][b] = g * ((u[a] * F[b] + F[a] * u[b]) + th * ((u[a] * dn[b] + u[b] * dn[a]) + delta * divJ));
-    }
-  }
-  const real_t trC = C[0][0] + C[1][1];
-#pragma unroll
-  for (int i = 0; i < 9; i++) {
-    const real_t c0 = real_t(cx(i)), c1 = real_t(cy(i));
-    const real_t cB = c0 * B[0] + c1 * B[1];
-    const real_t Ccc = ((C[0][0] * c0 * c0 + C[0][1] * c0 * c1) + C[1][0] * c1 * c0) + C[1][1] * c1 * c1;
-    const real_t A = real_t(0.0);
-    Fi[i] = Consts<real_t>::w(i) * ((A + cB / T0) + (Ccc - T0 * trC) / (real_t(2.0) * T0 * T0));
-  }
+  constexpr real_t T0 = Consts<real_t>::T0, zT0 = real_t(1.0) / T0;
+  constexpr real_t c2 = real_t(2.0) * T0 * T0, zc2 = real_t(1.0) / c2;
+  const real_t Bx = g * Fx, By = g * Fy;
+  const real_t uFx = ux * Fx, uFy = uy * Fy, ux_n = ux * dnx, uy_n = uy * dny;
+  const real_t Cxx = g * ((uFx + uFx) + th * ((ux_n + ux_n) + divJ));
+  const real_t Cyy = g * ((uFy + uFy) + th * ((uy_n + uy_n) + divJ));
+  const real_t Cxy = g * ((ux * Fy + Fx * uy) + th * (ux * dny + uy * dnx));
+  const real_t TtrC = T0 * (Cxx + Cyy);
+  Fi[0] = Consts<real_t>::w(0) * div_const(-TtrC, c2, zc2);
+  auto pair = [&](int i, int j, real_t cB, real_t Ccc) {
+    const real_t b = div_const(cB, T0, zT0), e = div_const(Ccc - TtrC, c2, zc2);
+    Fi[i] = Consts<real_t>::w(i) * (b + e);
+    Fi[j] = Consts<real_t>::w(j) * (e - b);
+  };
+  pair(1, 3, Bx, Cxx);
+  pair(2, 4, By, Cyy);
+  pair(5, 7, Bx + By, ((Cxx + Cxy) + Cxy) + Cyy);
+  pair(6, 8, By - Bx, ((Cxx - Cxy) - Cxy) + Cyy);
 }
 
 // p^i - p^w, Eqs. (eqstate, force2).
@@ -200,14 +226,39 @@ __device__ __forceinline__ int ghost_row(int y, int ny, int walls) {
 
 // ------------------------------------------------ the tile kernel (one step)
 //
-// One CTA owns a TX x TY tile of sites.  Shared memory holds the density on
+// One CTA owns a TX x A.ty tile of sites (A.ty <= TY).  Shared memory holds the density on
 // the tile plus a 3-site ring, p^i - p^w and lap n on a 2-site ring, and the
 // force and n u* on a 1-site ring; populations are pulled straight from the
 // previous state (L1/L2 serve the halo re-reads).
 //
 // MODE 0: full step, writes fout.  MODE 1: moments only (n, u*) into mom.
 
-constexpr int TX = 32, TY = 8, TTHREADS = TX * TY;
+// In FP64 the kernel is bound by the FP64 pipe (two operations a clock and SM),
+// so every operation counts: divisions by constants in three operations,
+// opposite links and the symmetric C evaluated once, and tiles of 32 x 16 sites,
+// whose rings repeat 1.6 (n), 1.4 (P, L) and 1.2 (F, J) times the tile's sites
+// (32 x 8: 2.1, 1.7, 1.3).
+constexpr int TX = 32, TY = 16, TTHREADS = 256;
+
+// Tile height of an nx x ny lattice on `sms` SMs: the operations of a tile (its
+// rings included) times the tiles the busiest SM gets, least.  512 x 256 on
+// 152 SMs: 14 rows, 304 tiles, two on every SM (16 rows: 256 tiles, two on most
+// SMs and one on the others).
+inline int tile_height(int nx, int ny, int sms) {
+  int best = TY;
+  double least = 1e300;
+  for (int ty = TY; ty >= 4; ty--) {
+    const long long tiles = (long long)((nx + TX - 1) / TX) * ((ny + ty - 1) / ty);
+    const double ops = 8.0 * (TX + 6) * (ty + 6) + 45.0 * (TX + 4) * (ty + 4) + 50.0 * (TX + 2) * (ty + 2) + 250.0 * TX * ty;
+    const double cost = ops * (double)((tiles + sms - 1) / sms);
+    if (cost < least) {
+      least = cost;
+      best = ty;
+    }
+  }
+  return best;
+}
+
 constexpr int NXR3 = TX + 6, NYR3 = TY + 6;
 constexpr int NXR2 = TX + 4, NYR2 = TY + 4;
 constexpr int NXR1 = TX + 2, NYR1 = TY + 2;
@@ -223,12 +274,12 @@ tile_step_kernel(const real_t *__restrict__ fin, real_t *__restrict__ fout,
   __shared__ real_t s_Jx[NYR1 * NXR1], s_Jy[NYR1 * NXR1];
 
   const int tid = threadIdx.x;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+  const int ty = A.ty, x0 = blockIdx.x * TX, y0 = blockIdx.y * ty;
   const int nx = A.nx, ny = A.ny;
   const bool walls = A.walls != 0;
 
   // 1. density on tile + 3 (ghost rows: reflection or periodic image).
-  for (int k = tid; k < NYR3 * NXR3; k += TTHREADS) {
+  for (int k = tid; k < (ty + 6) * NXR3; k += TTHREADS) {
     const int lx = k % NXR3, ly = k / NXR3;
     const int gx = wrapi(x0 + lx - 3, nx);
     const int gy = ghost_row(y0 + ly - 3, ny, A.walls);
@@ -237,7 +288,7 @@ tile_step_kernel(const real_t *__restrict__ fin, real_t *__restrict__ fout,
   __syncthreads();
 
   // 2. P = p^i - p^w and L = lap n on tile + 2.
-  for (int k = tid; k < NYR2 * NXR2; k += TTHREADS) {
+  for (int k = tid; k < (ty + 4) * NXR2; k += TTHREADS) {
     const int lx = k % NXR2 + 1, ly = k / NXR2 + 1;  // centre in s_n coords
     real_t p[9];
 #pragma unroll
@@ -248,7 +299,7 @@ tile_step_kernel(const real_t *__restrict__ fin, real_t *__restrict__ fout,
   __syncthreads();
 
   // 3. F and n u* on tile + 1 (real rows; ghost rows by reflection below).
-  for (int k = tid; k < NYR1 * NXR1; k += TTHREADS) {
+  for (int k = tid; k < (ty + 2) * NXR1; k += TTHREADS) {
     const int lx = k % NXR1 + 1, ly = k / NXR1 + 1;  // centre in s_P coords
     const int gy_raw = y0 + ly - 2;
     if (walls && (gy_raw < 0 || gy_raw > ny - 1)) continue;
@@ -279,13 +330,13 @@ tile_step_kernel(const real_t *__restrict__ fin, real_t *__restrict__ fout,
   }
   __syncthreads();
   if (walls) {
-    for (int k = tid; k < NYR1 * NXR1; k += TTHREADS) {
+    for (int k = tid; k < (ty + 2) * NXR1; k += TTHREADS) {
       const int lx = k % NXR1, ly = k / NXR1;
       const int gy = y0 + ly - 1;
       int src = -1;
       if (gy < 0) src = 2 * (0 - y0 + 1) - ly;                  // row -gy
       if (gy > ny - 1) src = 2 * ((ny - 1) - y0 + 1) - ly;      // mirror
-      if (src >= 0 && src < NYR1) {
+      if (src >= 0 && src < ty + 2) {
         s_Jx[k] = s_Jx[src * NXR1 + lx];
         s_Jy[k] = -s_Jy[src * NXR1 + lx];
       }
@@ -294,10 +345,12 @@ tile_step_kernel(const real_t *__restrict__ fin, real_t *__restrict__ fout,
   }
 
   // 4. interior: gradients, u*, equilibrium, forcing, collision.
-  {
-    const int lx = tid % TX, ly = tid / TX;
+  real_t iso[3];
+  isotropic3(A.T, iso);
+  for (int k = tid; k < TX * ty; k += TTHREADS) {
+    const int lx = k % TX, ly = k / TX;
     const int gx = x0 + lx, gy = y0 + ly;
-    if (gx >= nx || gy >= ny) return;
+    if (gx >= nx || gy >= ny) continue;
     const int c1 = (ly + 1) * NXR1 + lx + 1;   // in ring-1 arrays
     const real_t n = s_n[(ly + 3) * NXR3 + lx + 3];
     const real_t Jx = s_Jx[c1], Jy = s_Jy[c1];
@@ -308,30 +361,30 @@ tile_step_kernel(const real_t *__restrict__ fin, real_t *__restrict__ fout,
       if (mom_ux) mom_ux[s] = (mom_t)ux;
       if (mom_uy) mom_uy[s] = (mom_t)uy;
     } else {
-    real_t p[9], dnx, dny, dJx, dJy, tmp;
+      real_t p[9], dnx, dny, dJx, dJy, tmp;
 #pragma unroll
-    for (int i = 0; i < 9; i++) p[i] = s_n[(ly + 3 + cy(i)) * NXR3 + lx + 3 + cx(i)];
-    grad9(A, p, dnx, dny);
+      for (int i = 0; i < 9; i++) p[i] = s_n[(ly + 3 + cy(i)) * NXR3 + lx + 3 + cx(i)];
+      grad9(A, p, dnx, dny);
 #pragma unroll
-    for (int i = 0; i < 9; i++) p[i] = s_Jx[(ly + 1 + cy(i)) * NXR1 + lx + 1 + cx(i)];
-    grad9(A, p, dJx, tmp);
+      for (int i = 0; i < 9; i++) p[i] = s_Jx[(ly + 1 + cy(i)) * NXR1 + lx + 1 + cx(i)];
+      grad9(A, p, dJx, tmp);
 #pragma unroll
-    for (int i = 0; i < 9; i++) p[i] = s_Jy[(ly + 1 + cy(i)) * NXR1 + lx + 1 + cx(i)];
-    grad9(A, p, tmp, dJy);
-    const real_t divJ = dJx + dJy;
-    real_t f[9], g[9];
-    pull9(fin, A, gx, gy, f, g);
-    const real_t Fx = s_Fx[c1], Fy = s_Fy[c1];
-    if (walls && (gy == 0 || gy == ny - 1)) {
-      const bool top = (gy != 0);
-      wall_fill(top, top ? A.u_top : A.u_bot, Fx, Fy, n, f);
-    }
-    real_t fe[9], Fi[9];
-    feq9(n, ux, uy, A.T, fe);
-    forcing9(A.g, A.th, ux, uy, Fx, Fy, dnx, dny, divJ, Fi);
-    const size_t s = (size_t)(A.off + (long long)gy * A.pitch + gx);
+      for (int i = 0; i < 9; i++) p[i] = s_Jy[(ly + 1 + cy(i)) * NXR1 + lx + 1 + cx(i)];
+      grad9(A, p, tmp, dJy);
+      const real_t divJ = dJx + dJy;
+      real_t f[9], g[9];
+      pull9(fin, A, gx, gy, f, g);
+      const real_t Fx = s_Fx[c1], Fy = s_Fy[c1];
+      if (walls && (gy == 0 || gy == ny - 1)) {
+        const bool top = (gy != 0);
+        wall_fill(top, top ? A.u_top : A.u_bot, Fx, Fy, n, f);
+      }
+      real_t fe[9], Fi[9];
+      feq9(n, ux, uy, iso, fe);
+      forcing9(A.g, A.th, ux, uy, Fx, Fy, dnx, dny, divJ, Fi);
+      const size_t s = (size_t)(A.off + (long long)gy * A.pitch + gx);
 #pragma unroll
-    for (int i = 0; i < 9; i++) fout[i * A.plane + s] = (f[i] - A.omega * (f[i] - fe[i])) + Fi[i];
+      for (int i = 0; i < 9; i++) fout[i * A.plane + s] = (f[i] - A.omega * (f[i] - fe[i])) + Fi[i];
     }
   }
 }
@@ -346,27 +399,21 @@ __device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t k) {
   return z ^ (z >> 31);
 }
 
-// f*_i = f_i^eq(n0, u0) evaluated in FP64, stored as real_t.  Threads run
-// along x, blocks stride over rows (blockIdx.y); site s = y * nx + x is the
-// noise counter and the index into the host fields.  With zero velocity
-// (noise, or a density field alone) t1 = +-0 and t2 = +0 in feq9, so
-// f^eq_i = (w_i n) (1 + t3_i) with the same roundings: the three isotropic
-// factors 1 + t3 (rest, axes, diagonals) are evaluated once per thread by
-// the same expression and each site costs two FP64 products per link
-// class instead of feq9's divisions.
+// FP64 lattices: f*_i = f_i^eq(n0, u0).  Threads run along x, blocks stride
+// over rows (blockIdx.y); site s = y * nx + x is the noise counter and the
+// index into the fields.  With zero velocity (noise, or a density field alone)
+// t1 = +-0 and t2 = +0 in feq9, so f^eq_i = (w_i n) (1 + t3_i) with the same
+// roundings.
 template <typename real_t>
 __global__ void init_kernel(real_t *__restrict__ f, int nx, int ny, int pitch, long long plane,
                             long long off, int mode, uint64_t seed, double rho_mean, double amp,
                             const double *__restrict__ rho0, const double *__restrict__ ux0,
                             const double *__restrict__ uy0, double T) {
-  constexpr double T0 = Consts<double>::T0;
   const bool at_rest = mode == 0 || (ux0 == nullptr && uy0 == nullptr);
-  double iso[3];
+  double t3[3], iso[3];
+  isotropic3(T, t3);
 #pragma unroll
-  for (int c = 0; c < 3; c++) {
-    const double t3 = (T - T0) * (double(c) - 2.0 * T0) / (2.0 * T0 * T0);
-    iso[c] = 1.0 + t3;
-  }
+  for (int c = 0; c < 3; c++) iso[c] = 1.0 + t3[c];
   for (int y = blockIdx.y; y < ny; y += gridDim.y) {
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nx; x += gridDim.x * blockDim.x) {
       const size_t s = (size_t)y * nx + x;
@@ -384,7 +431,7 @@ __global__ void init_kernel(real_t *__restrict__ f, int nx, int ny, int pitch, l
 #pragma unroll
         for (int i = 0; i < 9; i++) fe[i] = Consts<double>::w(i) * n0 * iso[cx(i) * cx(i) + cy(i) * cy(i)];
       } else {
-        feq9<double>(n0, u, v, T, fe);
+        feq9<double>(n0, u, v, t3, fe);
       }
       const long long e = off + (long long)y * pitch + x;
 #pragma unroll

@@ -6,12 +6,13 @@
 
 namespace lbk {
 
-static dim3 tile_grid(int nx, int ny) {
-  return dim3((unsigned)((nx + TX - 1) / TX), (unsigned)((ny + TY - 1) / TY));
+template <typename real_t>
+static dim3 tile_grid(const StepArgs<real_t> &A) {
+  return dim3((unsigned)((A.nx + TX - 1) / TX), (unsigned)((A.ny + A.ty - 1) / A.ty));
 }
 
 cudaError_t launch_step(const double *fin, double *fout, const StepArgs<double> &A, cudaStream_t st) {
-  tile_step_kernel<double, 0, double><<<tile_grid(A.nx, A.ny), TTHREADS, 0, st>>>(
+  tile_step_kernel<double, 0, double><<<tile_grid(A), TTHREADS, 0, st>>>(
       fin, fout, nullptr, nullptr, nullptr, A);
   return cudaGetLastError();
 }
@@ -19,10 +20,10 @@ cudaError_t launch_step(const double *fin, double *fout, const StepArgs<double> 
 cudaError_t launch_moments(const double *fin, const StepArgs<double> &A, void *n, void *ux,
                            void *uy, int dtype, cudaStream_t st) {
   if (dtype == 0)
-    tile_step_kernel<double, 1, double><<<tile_grid(A.nx, A.ny), TTHREADS, 0, st>>>(
+    tile_step_kernel<double, 1, double><<<tile_grid(A), TTHREADS, 0, st>>>(
         fin, nullptr, (double *)n, (double *)ux, (double *)uy, A);
   else
-    tile_step_kernel<double, 1, float><<<tile_grid(A.nx, A.ny), TTHREADS, 0, st>>>(
+    tile_step_kernel<double, 1, float><<<tile_grid(A), TTHREADS, 0, st>>>(
         fin, nullptr, (float *)n, (float *)ux, (float *)uy, A);
   return cudaGetLastError();
 }

@@ -70,3 +70,19 @@ def test_batch_takes_the_form_of_all_its_lattices(taus):
     for v, w, n in zip(b, ws, n0):
         assert rel_err(v.get_state(), oracle_for(w).init_fields(n).step(STEPS).f) <= TOL
     b.close()
+
+
+@pytest.mark.parametrize("walls", [True, False], ids=["walls", "periodic"])
+@pytest.mark.parametrize("nx,ny", [(31, 3), (33, 4), (32, 15), (64, 16), (65, 17), (97, 61)])
+def test_fp64_tiles_give_the_oracle_bit_for_bit(nx, ny, walls):
+    """The FP64 tile kernel (32 columns by 4 to 16 rows, chosen by the lattice):
+    one column or row below, at and above a tile, with velocities given."""
+    from paper_1307_6703_gb300 import LB_FP64
+    w = _w(nx, ny, walls, 2.0)
+    rng = np.random.default_rng(nx + ny)
+    f = [_n0(nx, ny), 0.05 * rng.uniform(-1, 1, (ny, nx)), 0.05 * rng.uniform(-1, 1, (ny, nx))]
+    s = solver_for(w, LB_FP64).init_fields(*f).step(3)
+    ref = oracle_for(w).init_fields(*f).step(3)
+    assert np.array_equal(s.get_state(), ref.f)
+    for g, r in zip(s.moments(), ref.moments()):
+        assert np.array_equal(g, r)
