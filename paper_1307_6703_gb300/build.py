@@ -27,6 +27,7 @@ UNITS = {
     "lb_noalloc.cu": [],
     "lb_sweep.cu": [],
     "fno.cu": [],
+    "fno_fused.cu": [],
     "gemm_tc.cu": [],
 }
 

@@ -28,6 +28,8 @@
 #include <cuda_runtime.h>
 
 #include "fno.h"
+#include "fno_fused.h"
+#include "fno_math.cuh"
 #include "gemm_tc.h"
 
 namespace {
@@ -62,10 +64,8 @@ Offsets make_offsets(const fno_config &c) {
 
 // ------------------------------------------------------------------ helpers
 
-__device__ __forceinline__ float gelu(float z) { return z * normcdff(z); }
-__device__ __forceinline__ float gelu_grad(float z) {
-  return normcdff(z) + z * (0.3989422804014327f * expf(-0.5f * z * z));
-}
+using fno::gelu;
+using fno::gelu_grad;
 
 // Kept y-mode number of mode index k (0..my-1): 0..my/2-1, then -my/2..-1.
 __device__ __forceinline__ int ymode(int k, int my) { return k < my / 2 ? k : k - my; }
@@ -191,7 +191,7 @@ ydft_kernel(const float *__restrict__ A, const float2 *__restrict__ Ty, int ny, 
 
 // Inverse y-transform (and the adjoint of the y-transform, which has the
 // same form): X[bc][y][kx] = sum_ky Y[bc][ky][kx] e^{+i theta}, written as
-// (real, imaginary) rows with a BF16 copy.  One block per line set;
+// (real, imaginary) rows (X null: not wanted) with a BF16 copy.  One block per line set;
 // dynamic shared memory (2 my mx + 2 my kYChunk) floats.
 __global__ void __launch_bounds__(kThreads)
 iy_kernel(const float *__restrict__ Y, const float2 *__restrict__ Ty, int ny, int mx, int my, float *__restrict__ X,
@@ -219,8 +219,10 @@ iy_kernel(const float *__restrict__ Y, const float2 *__restrict__ Ty, int ny, in
         gi += yr * tw.y + yi * tw.x;
       }
       const long long g = ((long long)bc * ny + y0 + y) * 2 * mx;
-      X[g + kx] = gr;
-      X[g + mx + kx] = gi;
+      if (X) {
+        X[g + kx] = gr;
+        X[g + mx + kx] = gi;
+      }
       Xb[g + kx] = __float2bfloat16_rn(gr);
       Xb[g + mx + kx] = __float2bfloat16_rn(gi);
     }
@@ -471,24 +473,27 @@ outer_pass1_kernel(const float *__restrict__ a, const float *__restrict__ o2, in
 // Pass 1 of the channel sums when S % 4 == 0: block (ch, b * nsplit + j)
 // sums float4s j * 256 + t, (j + nsplit) * 256 + t, ... of field b's channel
 // ch, two at a time into two FP32 partials (then a fixed-order warp and
-// block tree, FP64 across warps); part[ch][b * nsplit + j].
+// block tree, FP64 across warps); part[ch][b * nsplit + j].  kQuads: a holds
+// the float4s' sums already (as the fused kernels leave them), same order.
+template <bool kQuads>
 __global__ void __launch_bounds__(kThreads)
 reduce_pass1_v4_kernel(const float *__restrict__ a, int C, long long S, int nsplit, double *__restrict__ part) {
   __shared__ double ws[kThreads / 32];
   const int ch = blockIdx.x, b = blockIdx.y / nsplit, j = blockIdx.y % nsplit;
-  const float4 *p = reinterpret_cast<const float4 *>(a + ((long long)b * C + ch) * S);
-  const long long S4 = S / 4, step = (long long)nsplit * blockDim.x;
+  const long long S4 = S / 4, step = (long long)nsplit * blockDim.x, row = (long long)b * C + ch;
+  auto sum4 = [&](long long i) {
+    if constexpr (kQuads) return a[row * S4 + i];
+    const float4 u = reinterpret_cast<const float4 *>(a + row * S)[i];
+    return (u.x + u.y) + (u.z + u.w);
+  };
   float acc0 = 0.f, acc1 = 0.f;
   long long i = (long long)j * blockDim.x + threadIdx.x;
   for (; i + step < S4; i += 2 * step) {
-    const float4 u = p[i], v = p[i + step];
-    acc0 += (u.x + u.y) + (u.z + u.w);
-    acc1 += (v.x + v.y) + (v.z + v.w);
+    const float u = sum4(i), v = sum4(i + step);
+    acc0 += u;
+    acc1 += v;
   }
-  if (i < S4) {
-    const float4 u = p[i];
-    acc0 += (u.x + u.y) + (u.z + u.w);
-  }
+  if (i < S4) acc0 += sum4(i);
   float acc = acc0 + acc1;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -749,6 +754,9 @@ struct fno_handle {
   // site-major BF16 copies ([b][site][channel]) for the products that
   // contract over channels; transposed BF16 weights (W_l^T per layer, Q1^T)
   __nv_bfloat16 *VbT[kMaxLayers + 1] = {}, *dZT = nullptr, *dhpT = nullptr, *wTb = nullptr;
+  bool fused = false;       // layers and projection as fused kernels (fno_fused.cu)
+  double *fpart = nullptr;  // their per-tile sums
+  float *quads = nullptr;   // sums over groups of four sites
   int *gerr = nullptr;  // set by a tensor-core product whose bounded wait gave up
   float2 *Ty = nullptr;
   int tab_nx = 0, tab_ny = 0;
@@ -814,12 +822,22 @@ void site_major(fno_handle *h, const __nv_bfloat16 *in, int B, int rows, long lo
     transpose_bf16_kernel<<<grid, 256, 0, h->st>>>(in, rows, S, out);
 }
 
+// Shares of a field in pass 1 of the channel sums: about 2048 blocks in all.
+int reduce_splits(int B, int C) { return std::max(1, std::min(kReduceBlocks, (2048 + C * B - 1) / (C * B))); }
+
+// The channel sums from the float4s' sums quads[b][ch][S / 4].
+void quad_reduce(fno_handle *h, const float *quads, int B, int C, long long S, float *out) {
+  const int nsplit = reduce_splits(B, C);
+  reduce_pass1_v4_kernel<true><<<dim3(C, B * nsplit), kThreads, 0, h->st>>>(quads, C, S, nsplit, h->rpart);
+  reduce_pass2_kernel<<<(C + 7) / 8, kThreads, 0, h->st>>>(h->rpart, C, B * nsplit, out);
+}
+
 // out[ch] = sum over (b, s) of a[b, ch, s] for the C channels of a.
 void chan_reduce(fno_handle *h, const float *a, int B, int C, long long S, float *out) {
   if (S % 4 == 0 && B * kReduceBlocks <= h->rpart_fields) {
     // float4 loads; about 2048 blocks, at most 32 shares of a field
-    const int nsplit = std::max(1, std::min(kReduceBlocks, (2048 + C * B - 1) / (C * B)));
-    reduce_pass1_v4_kernel<<<dim3(C, B * nsplit), kThreads, 0, h->st>>>(a, C, S, nsplit, h->rpart);
+    const int nsplit = reduce_splits(B, C);
+    reduce_pass1_v4_kernel<false><<<dim3(C, B * nsplit), kThreads, 0, h->st>>>(a, C, S, nsplit, h->rpart);
     reduce_pass2_kernel<<<(C + 7) / 8, kThreads, 0, h->st>>>(h->rpart, C, B * nsplit, out);
     return;
   }
@@ -846,7 +864,7 @@ cudaError_t alloc(T **p, long long n) {
 void free_workspace(fno_handle *h) {
   void *ps[] = {h->x0, h->A, h->G, h->Gb, h->hp, h->out, h->dout, h->dhp, h->dhpb, h->dV, h->dZ, h->dZb, h->dG,
                 h->dA, h->dAb, h->dY, h->dS, h->partial, h->loss, h->Fx, h->Fxi, h->Fxb, h->Fxib, h->rpart, h->wpart, h->Ty,
-                h->FxTb, h->FxiTb, h->dZT, h->dhpT, h->wTb, h->gerr};
+                h->FxTb, h->FxiTb, h->dZT, h->dhpT, h->wTb, h->gerr, h->fpart, h->quads};
   for (void *p : ps) cudaFree(p);
   for (int l = 0; l <= kMaxLayers; l++) {
     cudaFree(h->V[l]);
@@ -874,12 +892,18 @@ cudaError_t alloc_workspace(fno_handle *h) {
   h->cap_modes = B * c.width * (long long)c.modes_x * c.modes_y * 2;
   cudaError_t e = alloc(&h->x0, B * kFeatures * S);
   for (int l = 0; l <= c.layers && e == cudaSuccess; l++) {
-    e = alloc(&h->V[l], h->cap_bcs);
+    if (!h->fused) e = alloc(&h->V[l], h->cap_bcs);
     if (e == cudaSuccess) e = alloc(&h->Vb[l], h->cap_bcs);
     if (e == cudaSuccess && c.gemm_bf16) e = alloc(&h->VbT[l], h->cap_bcs);
   }
   if (e == cudaSuccess && c.gemm_bf16) e = alloc(&h->dZT, h->cap_bcs);
-  if (e == cudaSuccess && c.gemm_bf16) e = alloc(&h->dhpT, h->cap_bhs);
+  if (e == cudaSuccess && c.gemm_bf16 && !h->fused) e = alloc(&h->dhpT, h->cap_bhs);
+  if (e == cudaSuccess && h->fused) {
+    const fno::Shape s{c.batch_max, c.nx_max, c.ny_max, c.hidden, c.outputs, 2 * c.modes_x};
+    const int nval = fno::project_back_sums(s);
+    e = alloc(&h->fpart, fno::fused_tiles(s) * nval + fno::finish_scratch(nval));
+    if (e == cudaSuccess) e = alloc(&h->quads, h->cap_bcs / 4 + 1);
+  }
   if (e == cudaSuccess) e = alloc(&h->wTb, (long long)c.layers * c.width * c.width + (long long)c.width * c.hidden);
   if (e == cudaSuccess) e = alloc(&h->gerr, 1);
   if (e == cudaSuccess) e = cudaMemset(h->gerr, 0, sizeof(int));
@@ -888,18 +912,18 @@ cudaError_t alloc_workspace(fno_handle *h) {
     if (e == cudaSuccess) e = alloc(&h->Sh[l], h->cap_modes);
   }
   if (e == cudaSuccess) e = alloc(&h->A, h->cap_line);
-  if (e == cudaSuccess) e = alloc(&h->G, h->cap_line);
+  if (e == cudaSuccess && !h->fused) e = alloc(&h->G, h->cap_line);
   if (e == cudaSuccess) e = alloc(&h->Gb, h->cap_line);
-  if (e == cudaSuccess) e = alloc(&h->hp, h->cap_bhs);
+  if (e == cudaSuccess && !h->fused) e = alloc(&h->hp, h->cap_bhs);
   if (e == cudaSuccess) e = alloc(&h->out, h->cap_bs);
-  if (e == cudaSuccess) e = alloc(&h->dout, h->cap_bs);
-  if (e == cudaSuccess) e = alloc(&h->dhp, h->cap_bhs);
+  if (e == cudaSuccess && !h->fused) e = alloc(&h->dout, h->cap_bs);
+  if (e == cudaSuccess && !h->fused) e = alloc(&h->dhp, h->cap_bhs);
   if (e == cudaSuccess) e = alloc(&h->dhpb, h->cap_bhs);
   if (e == cudaSuccess) e = alloc(&h->dV, h->cap_bcs);
-  if (e == cudaSuccess) e = alloc(&h->dZ, h->cap_bcs);
+  if (e == cudaSuccess && !h->fused) e = alloc(&h->dZ, h->cap_bcs);
   if (e == cudaSuccess) e = alloc(&h->dZb, h->cap_bcs);
   if (e == cudaSuccess) e = alloc(&h->dG, h->cap_line);
-  if (e == cudaSuccess) e = alloc(&h->dA, h->cap_line);
+  if (e == cudaSuccess && !h->fused) e = alloc(&h->dA, h->cap_line);
   if (e == cudaSuccess) e = alloc(&h->dAb, h->cap_line);
   if (e == cudaSuccess) e = alloc(&h->dY, h->cap_modes);
   if (e == cudaSuccess) e = alloc(&h->dS, h->cap_modes);
@@ -919,6 +943,91 @@ cudaError_t alloc_workspace(fno_handle *h) {
   if (e == cudaSuccess) e = alloc(&h->FxiTb, (long long)c.nx_max * 2 * c.modes_x);
   if (e == cudaSuccess) e = alloc(&h->Ty, (long long)c.ny_max * c.modes_y);
   return e;
+}
+
+// The loss and the products' error flag, when the caller wants the loss.
+int read_loss(fno_handle *h, double *loss) {
+  if (!loss) return LB_OK;
+  int gerr = 0;
+  FNO_CUDA(h, cudaMemcpyAsync(loss, h->loss, sizeof(double), cudaMemcpyDeviceToHost, h->st));
+  FNO_CUDA(h, cudaMemcpyAsync(&gerr, h->gerr, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+  FNO_CUDA(h, cudaStreamSynchronize(h->st));
+  if (gerr) return ffail(h, LB_ERR_TIMEOUT, "fno_backward: a tensor-core product's bounded wait gave up");
+  return LB_OK;
+}
+
+// Forward pass on the fused kernels: per layer the x-transform, the spectral
+// path and one kernel for everything per site.
+int forward_fused(fno_handle *h, int B, int nx, int ny, const float *params_dev, float *out) {
+  const fno_config &c = h->c;
+  const int L = c.layers, mx = c.modes_x, my = c.modes_y, R = B * c.width * ny;
+  const fno::Shape sh{B, nx, ny, c.hidden, c.outputs, 2 * mx};
+  const float *P = h->prm;
+  cudaStream_t st = h->st;
+  FNO_CUDA(h, fno::lift(sh, params_dev, P + h->o.P, P + h->o.p, h->x0, h->Vb[0], h->VbT[0], st));
+  for (int l = 0; l < L; l++) {
+    FNO_GEMM(h, tcg(h, h->Vb[l], nx, 0, h->FxTb, nx, 0, h->A, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 1, 0.f));
+    ydft_kernel<<<B * c.width, kThreads, ydft_smem(mx, my), st>>>(h->A, h->Ty, ny, mx, my, h->Sh[l]);
+    mix_kernel<<<my * mx, kThreads, mix_smem(B, c.width, false), st>>>(h->Sh[l], P + h->o.Rr[l], P + h->o.Ri[l], B,
+                                                                         c.width, my * mx, h->dY);
+    iy_kernel<<<B * c.width, kThreads, iy_smem(mx, my), st>>>(h->dY, h->Ty, ny, mx, my, nullptr, h->Gb);
+    FNO_CUDA(h, cudaGetLastError());
+    FNO_GEMM(h, fno::layer_forward(sh, h->VbT[l], h->prmb + h->o.W[l], P + h->o.w[l], h->Gb, h->FxiTb, l == L - 1,
+                                   h->Z[l], h->Vb[l + 1], h->VbT[l + 1], h->gerr, st));
+  }
+  FNO_GEMM(h, fno::project_forward(sh, h->VbT[L], h->prmb + h->o.Q1, P + h->o.q1, P + h->o.Q2, P + h->o.q2, h->out, out,
+                                   h->gerr, st));
+  h->B = B;
+  h->nx = nx;
+  h->ny = ny;
+  h->have_forward = true;
+  return LB_OK;
+}
+
+// Backward pass on the fused kernels.
+int backward_fused(fno_handle *h, const float *target, double *loss) {
+  const fno_config &c = h->c;
+  const int B = h->B, nx = h->nx, ny = h->ny, C = c.width, H = c.hidden, L = c.layers, O = c.outputs;
+  const int mx = c.modes_x, my = c.modes_y, R = B * C * ny, parts = B * kWSplit;
+  const long long S = (long long)nx * ny, CS = C * S, HS = H * S;
+  const fno::Shape sh{B, nx, ny, H, O, 2 * mx};
+  const long long tiles = fno::fused_tiles(sh);
+  const float *P = h->prm;
+  const Offsets &o = h->o;
+  float *g = h->grd;
+  cudaStream_t st = h->st;
+  FNO_GEMM(h, fno::project_backward(sh, h->VbT[L], h->prmb + o.Q1, P + o.q1, P + o.Q2, h->wTb + (size_t)L * C * C,
+                                    h->out, target, h->dhpb, h->dZb, h->dZT, h->quads, h->fpart, h->gerr, st));
+  const int nval = fno::project_back_sums(sh);
+  FNO_CUDA(h, fno::finish_sums(h->fpart, tiles, nval, {{g + o.q1, H}, {g + o.Q2, O * H}, {g + o.q2, O}}, h->loss,
+                               (double)B * O * S, h->fpart + tiles * nval, st));
+  // dQ1 = sum_b dhp[b] v_L[b]^T
+  FNO_GEMM(h, tcg(h, h->dhpb, (int)S, HS, h->Vb[L], (int)S, CS, h->wpart, C, 1, (long long)H * C, H, C, (int)S, B,
+                  kWSplit, 0.f));
+  sum_fields_kernel<<<(H * C + 31) / 32, kThreads, 0, st>>>(h->wpart, parts, H * C, g + o.Q1);
+  for (int l = L - 1; l >= 0; l--) {
+    // dw = sum dz, dW = sum_b dz[b] v[b]^T
+    quad_reduce(h, h->quads, B, C, S, g + o.w[l]);
+    FNO_GEMM(h, tcg(h, h->dZb, (int)S, CS, h->Vb[l], (int)S, CS, h->wpart, C, 1, (long long)C * C, C, C, (int)S, B,
+                    kWSplit, 0.f));
+    sum_fields_kernel<<<(C * C + 31) / 32, kThreads, 0, st>>>(h->wpart, parts, C * C, g + o.W[l]);
+    // spectral path: dG = dz Fxi^T, the adjoints of the mixing and of the y-transforms
+    FNO_GEMM(h, tcg(h, h->dZb, nx, 0, h->Fxib, nx, 0, h->dG, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 1, 0.f));
+    ydft_kernel<<<B * C, kThreads, ydft_smem(mx, my), st>>>(h->dG, h->Ty, ny, mx, my, h->dY);
+    mix_back_kernel<<<my * mx, kThreads, mix_smem(B, C, true), st>>>(h->dY, h->Sh[l], P + o.Rr[l], P + o.Ri[l], B, C,
+                                                                       my * mx, h->dS, g + o.Rr[l], g + o.Ri[l]);
+    iy_kernel<<<B * C, kThreads, iy_smem(mx, my), st>>>(h->dS, h->Ty, ny, mx, my, nullptr, h->dAb);
+    FNO_CUDA(h, cudaGetLastError());
+    // everything per site: dv, through the activation below (in place: a tile
+    // reads and writes its own sites)
+    FNO_GEMM(h, fno::layer_backward(sh, h->dZT, h->wTb + (size_t)l * C * C, h->dAb, h->Fxb, l > 0 ? h->Z[l - 1] : nullptr,
+                                    h->dZb, h->dZT, h->quads, h->dV, h->gerr, st));
+  }
+  // lift: dp = sum dv0, dP[o, c] = sum dv0[b, o, s] x0[b, c, s]
+  chan_reduce(h, h->dV, B, C, S, g + o.p);
+  outer_reduce<8, kFeatures, false>(h, h->dV, h->x0, B, C, kFeatures, S, g + o.P);
+  FNO_CUDA(h, cudaGetLastError());
+  return read_loss(h, loss);
 }
 
 }  // namespace
@@ -944,6 +1053,7 @@ int fno_create(const fno_config *cfg, fno_handle **out) {
   h->c = c;
   h->st = (cudaStream_t)c.stream;
   h->o = make_offsets(c);
+  h->fused = c.gemm_bf16 && fno::fused_supported(c.width, c.hidden, c.modes_x);
   const long long np = (long long)h->o.total;
   cudaError_t e = alloc(&h->prm, np);
   if (e == cudaSuccess) e = alloc(&h->grd, np);
@@ -1011,6 +1121,7 @@ int fno_forward(fno_handle *h, int32_t B, int32_t nx, int32_t ny, const float *p
     h->tab_ny = ny;
   }
   const float *P = h->prm;
+  if (h->fused) return forward_fused(h, B, nx, ny, params_dev, out);
   features_kernel<<<blocks_for((long long)B * S), kThreads, 0, st>>>(params_dev, B, nx, ny, h->x0);
   lift_kernel<<<grid2(S, B * C), kThreads, 0, st>>>(h->x0, P + h->o.P, P + h->o.p, C, S, h->V[0], h->Vb[0]);
   FNO_CUDA(h, cudaGetLastError());
@@ -1073,6 +1184,7 @@ int fno_backward(fno_handle *h, const float *target, double *loss) {
   const float *P = h->prm;
   const Offsets &o = h->o;
   float *g = h->grd;
+  if (h->fused) return backward_fused(h, target, loss);
   const unsigned lb = blocks_for(BS);
   loss_kernel<<<lb, kThreads, 0, st>>>(h->out, target, BS, h->dout, h->partial);
   finish_loss_kernel<<<1, kThreads, 0, st>>>(h->partial, (int)lb, BS, h->loss);
@@ -1138,14 +1250,7 @@ int fno_backward(fno_handle *h, const float *target, double *loss) {
   chan_reduce(h, h->dV, B, C, S, g + o.p);
   outer_reduce<8, kFeatures, false>(h, h->dV, h->x0, B, C, kFeatures, S, g + o.P);
   FNO_CUDA(h, cudaGetLastError());
-  if (loss) {
-    int gerr = 0;
-    FNO_CUDA(h, cudaMemcpyAsync(loss, h->loss, sizeof(double), cudaMemcpyDeviceToHost, st));
-    FNO_CUDA(h, cudaMemcpyAsync(&gerr, h->gerr, sizeof(int), cudaMemcpyDeviceToHost, st));
-    FNO_CUDA(h, cudaStreamSynchronize(st));
-    if (gerr) return ffail(h, LB_ERR_TIMEOUT, "fno_backward: a tensor-core product's bounded wait gave up");
-  }
-  return LB_OK;
+  return read_loss(h, loss);
 }
 
 int fno_fields(fno_handle *h, const float *out, int32_t batch, int32_t nx, int32_t ny, const double *scales,

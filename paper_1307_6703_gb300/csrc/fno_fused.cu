@@ -1,0 +1,615 @@
+// fno_fused.cu -- forward and backward of the network's layers and projection
+// (include/fno.h) as fused tensor-core kernels, for the width the warm start
+// uses (32 channels, 32 or 64 hidden).
+//
+// A tile is 128 sites of one lattice row: the rows of an MMA.  Per site the
+// layer is two products with K <= 64 -- the channel mixing (the site-major
+// BF16 copy of v against W) and the inverse x-transform (the table FxiT[x][j]
+// against the 2 modes_x transformed values of each channel at this y) -- so one
+// CTA brings all four operand tiles by TMA (128-byte swizzle, zero fill where
+// K < 64), one thread issues the MMAs into two accumulators in tensor memory,
+// and each of the four warps then holds 32 sites by all 32 channels in
+// registers: bias, activation, and every copy the next products need (BF16
+// channel-major and site-major), with no pass over memory of its own.  The
+// backward kernels do the same with the transposed operands, multiply by
+// gelu', and add the tile's channel sums (weight gradients of the biases, the
+// lift and the projection) with a shuffle tree in FP32, FP64 across warps and
+// tiles.
+//
+// The separate kernels this replaces moved every FP32 activation through memory
+// four to six times (z written by one product, read and written by the next,
+// then by the bias and activation, then transposed: 570 MB a layer for 8 fields
+// of 512 x 128 against 170 here).  The sums of a product are grouped as before
+// (each product in its own accumulator, then added, then the bias), so a
+// layer's values are the same bits.  Bound by the activations (normcdff) and
+// by memory about equally.  Measured: training step of 16 fields of 256 x 64
+// 1.61 -> STEP16 ms, of 8 fields of 512 x 128 2.75 -> STEP8 ms; forward pass of
+// a 2048 x 512 field 1.83 -> FWD ms.
+#include "fno_fused.h"
+
+#include <algorithm>
+
+#include "fno_math.cuh"
+#include "gemm_tc.h"
+#include "tc_device.cuh"
+
+namespace fno {
+
+namespace {
+
+constexpr int kThreads = 128;
+constexpr int C = kWidth;
+
+// Operand tiles and the two accumulators of a layer kernel.
+struct __align__(1024) LayerSmem {
+  __nv_bfloat16 a1[tc::kBM * tc::kBK], a2[tc::kBM * tc::kBK];
+  __nv_bfloat16 b1[C * tc::kBK], b2[C * tc::kBK];
+  unsigned long long full, done;
+  uint32_t tmem;
+};
+constexpr uint32_t kLayerTx = 2 * (tc::kBM + C) * tc::kBK * 2;
+
+// Tensor memory of a CTA: `cols` columns (a power of two >= 32), and the
+// barriers' initialisation; all threads.
+__device__ __forceinline__ uint32_t setup(uint32_t *slot, uint32_t cols, unsigned long long *bars, int nbars) {
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < nbars; ++i) tc::mbar_init(tc::smem_u32(bars + i));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (threadIdx.x < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(slot)), "r"(cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  return *slot;
+}
+__device__ __forceinline__ void release_tmem(uint32_t tmem, uint32_t cols) {
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
+  }
+}
+
+// The MMAs a thread issued are complete (every thread calls it); false after a
+// bounded wait that gave up.
+__device__ __forceinline__ bool wait_done(unsigned long long *bar, int *err) {
+  const bool ok = tc::mbar_try(tc::smem_u32(bar), 0u);
+  if (!ok && (threadIdx.x & 31) == 0) atomicOr(err, 1);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  return ok;
+}
+
+// Sums of v[i] over the warp's lanes; lane i returns that of v[i] (31 shuffles:
+// each stage halves the values a lane still carries).
+__device__ __forceinline__ float warp_sums(float (&v)[32]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const float send = up ? v[i] : v[i + o], keep = up ? v[i + o] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  return v[0];
+}
+
+// Sums over groups of four sites (the lanes 4g .. 4g+3), ((x0 + x1) + (x2 + x3))
+// as a float4 sum of a row takes them: lane 4g + r returns channels 16 (r & 1) +
+// 8 (r >> 1) .. + 7 of group g in q.
+__device__ __forceinline__ void quad_sums(const float (&v)[32], float (&q)[8]) {
+  const int lane = threadIdx.x & 31;
+  float h[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const float send = lane & 1 ? v[i] : v[i + 16], keep = lane & 1 ? v[i + 16] : v[i];
+    h[i] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float send = lane & 2 ? h[i] : h[i + 8], keep = lane & 2 ? h[i + 8] : h[i];
+    q[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+  }
+}
+// The quad sums of a warp's 32 sites into quads[c][s / 4] (lanes of valid
+// sites; rows are whole groups of four).
+__device__ __forceinline__ void put_quads(const float (&v)[32], bool valid, float *quads, long long S4, long long s) {
+  float q[8];
+  quad_sums(v, q);
+  if (!valid) return;
+  const int lane = threadIdx.x & 31, c0 = 16 * (lane & 1) + 8 * ((lane >> 1) & 1);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) quads[(c0 + i) * S4 + (s >> 2)] = q[i];
+}
+
+// A site's 32 channels as BF16: channel-major (32 sites of a channel are
+// consecutive) and, 64 bytes a site, site-major.
+__device__ __forceinline__ void put_bf16(const float (&v)[32], bool valid, __nv_bfloat16 *cm, long long S,
+                                         __nv_bfloat16 *sm) {
+  if (!valid) return;
+  __align__(16) __nv_bfloat16 h[32];
+#pragma unroll
+  for (int o = 0; o < 32; ++o) {
+    h[o] = __float2bfloat16_rn(v[o]);
+    cm[o * S] = h[o];
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) reinterpret_cast<uint4 *>(sm)[q] = reinterpret_cast<const uint4 *>(h)[q];
+}
+
+// x, as a value of its own to the compiler: gelu and gelu' of the same z are
+// then contracted as they are in the kernels that evaluate one of them (a
+// shared normcdff result changes the last bit of gelu').
+__device__ __forceinline__ float opaque(float x) {
+  asm volatile("" : "+f"(x));
+  return x;
+}
+
+enum Mode { kForward, kForwardLast, kBackward, kBackwardFirst };
+
+struct LayerArgs {
+  int nx, ny, K2;
+  const float *w;               // forward: bias
+  float *z;                     // forward: z (out)
+  const float *zprev;           // backward: z of the layer below
+  __nv_bfloat16 *cm, *sm;       // results
+  float *quads;                 // backward: sums of dz over groups of four sites
+  float *dv;                    // backward, first layer: dv
+  int *err;
+};
+
+// One tile (x0 .. x0+127 of row y, field b) through both products.
+template <int kMode>
+__global__ void __launch_bounds__(kThreads, 4)
+layer_kernel(const __grid_constant__ CUtensorMap ma1, const __grid_constant__ CUtensorMap mb1,
+             const __grid_constant__ CUtensorMap ma2, const __grid_constant__ CUtensorMap mb2, const LayerArgs p) {
+  extern __shared__ unsigned char raw[];
+  LayerSmem &S = *reinterpret_cast<LayerSmem *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int xt = blockIdx.x * tc::kBM, y = blockIdx.y, b = blockIdx.z;
+  const uint32_t tmem = setup(&S.tmem, 64, &S.full, 2);
+  bool ok = true;
+  if (t == 0) {
+    const uint32_t bar = tc::smem_u32(&S.full);
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(kLayerTx) : "memory");
+    tc::tma_load_3d(&ma1, tc::smem_u32(S.a1), bar, 0, xt, b * p.ny + y);
+    tc::tma_load_3d(&mb1, tc::smem_u32(S.b1), bar, 0, 0, 0);
+    tc::tma_load_3d(&ma2, tc::smem_u32(S.a2), bar, 0, xt, 0);
+    tc::tma_load_3d(&mb2, tc::smem_u32(S.b2), bar, 0, b * C, y);
+    ok = tc::mbar_try(bar, 0u);
+    if (ok) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      constexpr uint32_t idesc = tc::idesc_bf16<C>();
+      tc::mma_tile(tmem, tc::smem_u32(S.a1), tc::smem_u32(S.b1), C / 16, idesc);
+      tc::mma_tile(tmem + C, tc::smem_u32(S.a2), tc::smem_u32(S.b2), p.K2 / 16, idesc);
+    } else {  // (the copies in flight land before the CTA leaves: waited for once more)
+      atomicOr(p.err, 1);
+      (void)tc::mbar_try(bar, 0u);
+    }
+    tc::mma_commit(tc::smem_u32(&S.done));
+  }
+  __syncthreads();
+  (void)wait_done(&S.done, p.err);
+
+  const int x = xt + warp * 32 + lane;
+  const bool valid = x < p.nx;
+  const long long sites = (long long)p.nx * p.ny, s = (long long)y * p.nx + x;
+  const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);
+  float v[32], u[32];
+  tc::tmem_load32(lanes, v);        // the channel mixing
+  tc::tmem_load32(lanes + C, u);    // the transform
+  if constexpr (kMode == kForward || kMode == kForwardLast) {
+    float *z = p.z + (long long)b * C * sites + s;
+#pragma unroll
+    for (int o = 0; o < C; ++o) {
+      const float zz = (u[o] + v[o]) + p.w[o];
+      if (valid) z[o * sites] = zz;
+      v[o] = kMode == kForward ? gelu(zz) : zz;
+    }
+    put_bf16(v, valid, p.cm + (long long)b * C * sites + s, sites, p.sm + ((long long)b * sites + s) * C);
+  } else if constexpr (kMode == kBackward) {
+    const float *z = p.zprev + (long long)b * C * sites + s;
+#pragma unroll
+    for (int o = 0; o < C; ++o) u[o] = (v[o] + u[o]) * gelu_grad(valid ? z[o * sites] : 0.f);
+    put_bf16(u, valid, p.cm + (long long)b * C * sites + s, sites, p.sm + ((long long)b * sites + s) * C);
+    put_quads(u, valid, p.quads + (long long)b * C * (sites / 4), sites / 4, s);
+  } else {
+    float *dv = p.dv + (long long)b * C * sites + s;
+#pragma unroll
+    for (int o = 0; o < C; ++o)
+      if (valid) dv[o * sites] = v[o] + u[o];
+  }
+  release_tmem(tmem, 64);
+}
+
+// Features of a site (include/fno.h).
+__device__ __forceinline__ void features(const float *prm, int b, int x, int y, int ny, float *f) {
+  const float uw = prm[4 * b], a0 = prm[4 * b + 1], lam = prm[4 * b + 2], tr = prm[4 * b + 3];
+  float sn, cs;
+  sincospif(2.0f * (float)x / lam, &sn, &cs);
+  const float yy = 2.0f * (float)y / (float)(ny - 1) - 1.0f;
+  f[0] = (a0 / 1e-3f) * sn;
+  f[1] = (a0 / 1e-3f) * cs;
+  f[2] = (uw / 0.05f) * yy;
+  f[3] = (tr - 0.94f) / 0.02f;
+  f[4] = yy;
+}
+
+__global__ void __launch_bounds__(kThreads)
+lift_kernel(int nx, int ny, const float *__restrict__ prm, const float *__restrict__ P, const float *__restrict__ pb,
+            float *__restrict__ x0, __nv_bfloat16 *__restrict__ cm, __nv_bfloat16 *__restrict__ sm) {
+  __shared__ float Ps[C * kFeat], ps[C];
+  for (int i = threadIdx.x; i < C * kFeat; i += kThreads) Ps[i] = P[i];
+  if (threadIdx.x < C) ps[threadIdx.x] = pb[threadIdx.x];
+  __syncthreads();
+  const int x = blockIdx.x * kThreads + threadIdx.x, y = blockIdx.y, b = blockIdx.z;
+  if (x >= nx) return;
+  const long long sites = (long long)nx * ny, s = (long long)y * nx + x;
+  float f[kFeat], v[32];
+  features(prm, b, x, y, ny, f);
+#pragma unroll
+  for (int c = 0; c < kFeat; ++c) x0[((long long)b * kFeat + c) * sites + s] = f[c];
+#pragma unroll
+  for (int o = 0; o < C; ++o) {
+    float acc = ps[o];
+#pragma unroll
+    for (int c = 0; c < kFeat; ++c) acc += Ps[o * kFeat + c] * f[c];
+    v[o] = acc;
+  }
+  put_bf16(v, true, cm + (long long)b * C * sites + s, sites, sm + ((long long)b * sites + s) * C);
+}
+
+// ---------------------------------------------------------- the projection
+
+constexpr int kMaxO = 4;
+
+template <int H>
+struct __align__(1024) ProjSmem {
+  __nv_bfloat16 a[tc::kBM * tc::kBK];   // v tile (K = C); then dhp tile (K = H)
+  __nv_bfloat16 b1[H * tc::kBK];        // Q1 [h][c]
+  __nv_bfloat16 b2[C * tc::kBK];        // Q1^T [c][h] (backward)
+  float q1[H], Q2[kMaxO * H], q2[kMaxO];
+  double red[4][H * (1 + kMaxO) + kMaxO + 1];
+  unsigned long long full, done, done2;
+  uint32_t tmem;
+};
+
+struct ProjArgs {
+  int nx, ny, O;
+  const float *q1, *Q2, *q2;
+  float *out, *out_user;        // forward
+  const float *o_in, *target;   // backward
+  float scale;                  // 2 / (elements of out)
+  __nv_bfloat16 *dhp, *cm, *sm;
+  float *quads;
+  double *part;
+  int *err;
+};
+
+template <int H, bool kBack>
+__global__ void __launch_bounds__(kThreads, 4)
+project_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb1,
+               const __grid_constant__ CUtensorMap mb2, const ProjArgs p) {
+  extern __shared__ unsigned char raw[];
+  using Sm = ProjSmem<H>;
+  Sm &S = *reinterpret_cast<Sm *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int xt = blockIdx.x * tc::kBM, y = blockIdx.y, b = blockIdx.z;
+  constexpr uint32_t kCols = kBack ? 128 : H;  // accumulators: H, then C (a power of two in all)
+  for (int i = t; i < H; i += kThreads) S.q1[i] = p.q1[i];
+  for (int i = t; i < p.O * H; i += kThreads) S.Q2[i] = p.Q2[i];
+  if (!kBack && t < p.O) S.q2[t] = p.q2[t];
+  const uint32_t tmem = setup(&S.tmem, kCols, &S.full, 3);
+  if (t == 0) {
+    const uint32_t bar = tc::smem_u32(&S.full);
+    const uint32_t tx = (uint32_t)(tc::kBM + H + (kBack ? C : 0)) * tc::kBK * 2;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(tx) : "memory");
+    tc::tma_load_3d(&ma, tc::smem_u32(S.a), bar, 0, xt, b * p.ny + y);
+    tc::tma_load_3d(&mb1, tc::smem_u32(S.b1), bar, 0, 0, 0);
+    if (kBack) tc::tma_load_3d(&mb2, tc::smem_u32(S.b2), bar, 0, 0, 0);
+    if (tc::mbar_try(bar, 0u)) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      tc::mma_tile(tmem, tc::smem_u32(S.a), tc::smem_u32(S.b1), C / 16, tc::idesc_bf16<H>());
+    } else {
+      atomicOr(p.err, 1);
+      (void)tc::mbar_try(bar, 0u);
+    }
+    tc::mma_commit(tc::smem_u32(&S.done));
+  }
+  __syncthreads();
+  (void)wait_done(&S.done, p.err);
+
+  const int r = warp * 32 + lane, x = xt + r;
+  const bool valid = x < p.nx;
+  const long long sites = (long long)p.nx * p.ny, s = (long long)y * p.nx + x;
+  const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);
+  if constexpr (!kBack) {
+    float acc[kMaxO];
+#pragma unroll
+    for (int j = 0; j < kMaxO; ++j) acc[j] = j < p.O ? S.q2[j] : 0.f;
+#pragma unroll 1
+    for (int h0 = 0; h0 < H; h0 += 32) {
+      float v[32];
+      tc::tmem_load32(lanes + h0, v);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const float a = gelu(v[i] + S.q1[h0 + i]);
+#pragma unroll
+        for (int j = 0; j < kMaxO; ++j)
+          if (j < p.O) acc[j] += S.Q2[j * H + h0 + i] * a;
+      }
+    }
+    if (valid) {
+      for (int j = 0; j < p.O; ++j) {
+        const long long e = ((long long)b * p.O + j) * sites + s;
+        p.out[e] = acc[j];
+        if (p.out_user) p.out_user[e] = acc[j];
+      }
+    }
+  } else {
+    // d loss / d out of this site, and the loss
+    float dout[kMaxO];
+    double loss = 0.0;
+#pragma unroll
+    for (int j = 0; j < kMaxO; ++j) {
+      dout[j] = 0.f;
+      if (j < p.O && valid) {
+        const long long e = ((long long)b * p.O + j) * sites + s;
+        const float d = p.o_in[e] - p.target[e];
+        dout[j] = p.scale * d;
+        loss += (double)d * (double)d;
+      }
+    }
+    unsigned char *arow = reinterpret_cast<unsigned char *>(S.a) + r * 128;  // this site's row of the dhp tile
+#pragma unroll 1
+    for (int h0 = 0; h0 < H; h0 += 32) {
+      float a[32], d[32];
+      tc::tmem_load32(lanes + h0, a);
+      __nv_bfloat16 *dh = p.dhp + ((long long)b * H + h0) * sites + s;
+      __align__(16) __nv_bfloat16 hb[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const float z = a[i] + S.q1[h0 + i];
+        float q = 0.f;
+#pragma unroll
+        for (int j = 0; j < kMaxO; ++j)
+          if (j < p.O) q += S.Q2[j * H + h0 + i] * dout[j];
+        d[i] = q * gelu_grad(z);
+        a[i] = gelu(opaque(z));
+        hb[i] = __float2bfloat16_rn(d[i]);
+        if (valid) dh[i * sites] = hb[i];
+      }
+      // 16-byte chunk c of row r sits at chunk c ^ (r & 7) (128-byte swizzle)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<uint4 *>(arow + (((h0 / 8 + q) ^ (r & 7)) << 4)) = reinterpret_cast<const uint4 *>(hb)[q];
+      S.red[warp][h0 + lane] = (double)warp_sums(d);
+      for (int j = 0; j < p.O; ++j) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) d[i] = dout[j] * a[i];
+        S.red[warp][H + j * H + h0 + lane] = (double)warp_sums(d);
+      }
+    }
+    // dv = Q1^T dhp: the tile just written against Q1^T
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (t == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      tc::mma_tile(tmem + H, tc::smem_u32(S.a), tc::smem_u32(S.b2), H / 16, tc::idesc_bf16<C>());
+      tc::mma_commit(tc::smem_u32(&S.done2));
+    }
+    __syncwarp();
+    (void)wait_done(&S.done2, p.err);
+    float v[32];
+    tc::tmem_load32(lanes + H, v);
+    put_bf16(v, valid, p.cm + (long long)b * C * sites + s, sites, p.sm + ((long long)b * sites + s) * C);
+    put_quads(v, valid, p.quads + (long long)b * C * (sites / 4), sites / 4, s);
+    const int base = H * (1 + p.O), n = base + p.O + 1;
+    double tail[kMaxO + 1];
+#pragma unroll
+    for (int j = 0; j < kMaxO; ++j) tail[j] = (double)dout[j];
+    tail[kMaxO] = loss;
+#pragma unroll
+    for (int j = 0; j <= kMaxO; ++j)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) tail[j] += __shfl_down_sync(0xffffffffu, tail[j], o);
+    if (lane == 0) {
+      for (int j = 0; j < p.O; ++j) S.red[warp][base + j] = j == 0 ? tail[0] : (j == 1 ? tail[1] : (j == 2 ? tail[2] : tail[3]));
+      S.red[warp][base + p.O] = tail[kMaxO];
+    }
+    __syncthreads();
+    double *part = p.part + (((long long)b * gridDim.y + y) * gridDim.x + blockIdx.x) * n;
+    for (int i = t; i < n; i += kThreads) part[i] = ((S.red[0][i] + S.red[1][i]) + S.red[2][i]) + S.red[3][i];
+  }
+  release_tmem(tmem, kCols);
+}
+
+// ------------------------------------------------------------- tile sums
+
+constexpr int kSumWarps = 8, kSumSplits = 16;
+
+// Block (k, q) adds values 32k .. 32k+31 over tiles q, q + 16, ...: warp w every
+// eighth of them, four loads in flight; then the warps' sums in order, into
+// split q of part2.
+__global__ void __launch_bounds__(32 * kSumWarps)
+tile_sums_kernel(const double *__restrict__ part, long long tiles, int nval, double *__restrict__ part2) {
+  __shared__ double ws[kSumWarps][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+  double acc = 0.0;
+  if (i < nval) {
+    constexpr long long step = kSumWarps * kSumSplits;
+    long long k = blockIdx.y + (long long)w * kSumSplits;
+    for (; k + 3 * step < tiles; k += 4 * step) {
+      double v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[q] = part[(k + q * step) * nval + i];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc += v[q];
+    }
+    for (; k < tiles; k += step) acc += part[k * nval + i];
+  }
+  ws[w][lane] = acc;
+  __syncthreads();
+  if (w == 0 && i < nval) {
+    double r = ws[0][lane];
+    for (int q = 1; q < kSumWarps; ++q) r += ws[q][lane];
+    part2[blockIdx.y * nval + i] = r;
+  }
+}
+
+// The splits' sums, in order, into up to three ranges of outputs and the loss.
+__global__ void finish_kernel(const double *__restrict__ part2, int nval, SumOut o0, SumOut o1, SumOut o2,
+                              double *__restrict__ loss, double count) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nval) return;
+  double r = part2[i];
+  for (int q = 1; q < kSumSplits; ++q) r += part2[q * nval + i];
+  int e = i;
+  const SumOut o[3] = {o0, o1, o2};
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (e >= 0 && e < o[q].n) o[q].out[e] = (float)r;
+    e -= o[q].n;
+  }
+  if (e == 0) *loss = r / count;
+}
+
+dim3 tile_grid(const Shape &s) { return dim3((unsigned)((s.nx + tc::kBM - 1) / tc::kBM), (unsigned)s.ny, (unsigned)s.B); }
+
+template <class K>
+cudaError_t allow_smem(K kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+struct LayerMaps {
+  CUtensorMap a1, b1, a2, b2;
+};
+
+cudaError_t layer_maps(const Shape &s, const __nv_bfloat16 *a1, const __nv_bfloat16 *b1, const __nv_bfloat16 *a2,
+                       const __nv_bfloat16 *b2, LayerMaps *m) {
+  cudaError_t e = tc::operand_map(a1, C, s.nx, C, (long long)s.nx * C, s.B * s.ny, tc::kBM, &m->a1);
+  if (e == cudaSuccess) e = tc::operand_map(b1, C, C, C, 0, 1, C, &m->b1);
+  if (e == cudaSuccess) e = tc::operand_map(a2, s.K2, s.nx, s.K2, 0, 1, tc::kBM, &m->a2);
+  // rows: the channels of all fields at one y
+  if (e == cudaSuccess) e = tc::operand_map(b2, s.K2, s.B * C, s.ny * s.K2, s.K2, s.ny, C, &m->b2);
+  return e;
+}
+
+template <int kMode>
+cudaError_t launch_layer(const Shape &s, const LayerMaps &m, const LayerArgs &p, cudaStream_t st) {
+  const size_t smem = sizeof(LayerSmem) + 1024;
+  const cudaError_t e = allow_smem(layer_kernel<kMode>, smem);
+  if (e != cudaSuccess) return e;
+  layer_kernel<kMode><<<tile_grid(s), kThreads, smem, st>>>(m.a1, m.b1, m.a2, m.b2, p);
+  return cudaGetLastError();
+}
+
+template <int H, bool kBack>
+cudaError_t launch_project(const Shape &s, const __nv_bfloat16 *v_sm, const __nv_bfloat16 *Q1, const __nv_bfloat16 *Q1T,
+                           const ProjArgs &p, cudaStream_t st) {
+  CUtensorMap ma, mb1, mb2;
+  cudaError_t e = tc::operand_map(v_sm, C, s.nx, C, (long long)s.nx * C, s.B * s.ny, tc::kBM, &ma);
+  if (e == cudaSuccess) e = tc::operand_map(Q1, C, H, C, 0, 1, H, &mb1);
+  mb2 = mb1;
+  if (e == cudaSuccess && kBack) e = tc::operand_map(Q1T, H, C, H, 0, 1, C, &mb2);
+  const size_t smem = sizeof(ProjSmem<H>) + 1024;
+  if (e == cudaSuccess) e = allow_smem(project_kernel<H, kBack>, smem);
+  if (e != cudaSuccess) return e;
+  project_kernel<H, kBack><<<tile_grid(s), kThreads, smem, st>>>(ma, mb1, mb2, p);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+// The sizes the tiles are laid out for; other networks take the separate
+// products and pointwise kernels of fno.cu.
+bool fused_supported(int width, int hidden, int modes_x) {
+  return width == C && (hidden == 32 || hidden == 64) && modes_x % 8 == 0 && 2 * modes_x <= tc::kBK;
+}
+
+long long fused_tiles(const Shape &s) { return (long long)((s.nx + tc::kBM - 1) / tc::kBM) * s.ny * s.B; }
+
+cudaError_t lift(const Shape &s, const float *prm, const float *P, const float *pb, float *x0, __nv_bfloat16 *cm,
+                 __nv_bfloat16 *sm, cudaStream_t st) {
+  lift_kernel<<<tile_grid(s), kThreads, 0, st>>>(s.nx, s.ny, prm, P, pb, x0, cm, sm);
+  return cudaGetLastError();
+}
+
+cudaError_t layer_forward(const Shape &s, const __nv_bfloat16 *v_sm, const __nv_bfloat16 *W, const float *w,
+                          const __nv_bfloat16 *G, const __nv_bfloat16 *FxiT, bool last, float *z, __nv_bfloat16 *cm,
+                          __nv_bfloat16 *sm, int *err, cudaStream_t st) {
+  LayerMaps m;
+  const cudaError_t e = layer_maps(s, v_sm, W, FxiT, G, &m);
+  if (e != cudaSuccess) return e;
+  const LayerArgs p{s.nx, s.ny, s.K2, w, z, nullptr, cm, sm, nullptr, nullptr, err};
+  return last ? launch_layer<kForwardLast>(s, m, p, st) : launch_layer<kForward>(s, m, p, st);
+}
+
+cudaError_t project_forward(const Shape &s, const __nv_bfloat16 *v_sm, const __nv_bfloat16 *Q1, const float *q1,
+                            const float *Q2, const float *q2, float *out, float *out_user, int *err, cudaStream_t st) {
+  ProjArgs p{};
+  p.nx = s.nx;
+  p.ny = s.ny;
+  p.O = s.O;
+  p.q1 = q1;
+  p.Q2 = Q2;
+  p.q2 = q2;
+  p.out = out;
+  p.out_user = out_user;
+  p.err = err;
+  return s.H == 64 ? launch_project<64, false>(s, v_sm, Q1, nullptr, p, st)
+                   : launch_project<32, false>(s, v_sm, Q1, nullptr, p, st);
+}
+
+int project_back_sums(const Shape &s) { return s.H * (1 + s.O) + s.O + 1; }
+
+cudaError_t project_backward(const Shape &s, const __nv_bfloat16 *v_sm, const __nv_bfloat16 *Q1, const float *q1,
+                             const float *Q2, const __nv_bfloat16 *Q1T, const float *out, const float *target,
+                             __nv_bfloat16 *dhp, __nv_bfloat16 *dz_cm, __nv_bfloat16 *dz_sm, float *quads, double *part,
+                             int *err, cudaStream_t st) {
+  ProjArgs p{};
+  p.nx = s.nx;
+  p.ny = s.ny;
+  p.O = s.O;
+  p.q1 = q1;
+  p.Q2 = Q2;
+  p.o_in = out;
+  p.target = target;
+  p.scale = 2.0f / (float)((long long)s.B * s.O * s.nx * s.ny);
+  p.dhp = dhp;
+  p.cm = dz_cm;
+  p.sm = dz_sm;
+  p.quads = quads;
+  p.part = part;
+  p.err = err;
+  return s.H == 64 ? launch_project<64, true>(s, v_sm, Q1, Q1T, p, st)
+                   : launch_project<32, true>(s, v_sm, Q1, Q1T, p, st);
+}
+
+cudaError_t layer_backward(const Shape &s, const __nv_bfloat16 *dz_sm, const __nv_bfloat16 *WT, const __nv_bfloat16 *dA,
+                           const __nv_bfloat16 *Fx, const float *zprev, __nv_bfloat16 *cm, __nv_bfloat16 *sm,
+                           float *quads, float *dv, int *err, cudaStream_t st) {
+  LayerMaps m;
+  const cudaError_t e = layer_maps(s, dz_sm, WT, Fx, dA, &m);
+  if (e != cudaSuccess) return e;
+  const LayerArgs p{s.nx, s.ny, s.K2, nullptr, nullptr, zprev, cm, sm, quads, dv, err};
+  return zprev ? launch_layer<kBackward>(s, m, p, st) : launch_layer<kBackwardFirst>(s, m, p, st);
+}
+
+cudaError_t finish_sums(const double *part, long long tiles, int nval, const SumOut (&o)[3], double *loss, double count,
+                        double *part2, cudaStream_t st) {
+  tile_sums_kernel<<<dim3((nval + 31) / 32, kSumSplits), 32 * kSumWarps, 0, st>>>(part, tiles, nval, part2);
+  finish_kernel<<<(nval + 127) / 128, 128, 0, st>>>(part2, nval, o[0], o[1], o[2], loss, count);
+  return cudaGetLastError();
+}
+
+long long finish_scratch(int nval) { return (long long)kSumSplits * nval; }
+
+}  // namespace fno

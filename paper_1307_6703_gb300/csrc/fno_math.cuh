@@ -1,0 +1,15 @@
+// fno_math.cuh -- the network's activation, shared by its kernels.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace fno {
+
+// gelu(z) = z Phi(z), Phi the standard normal distribution function.
+__device__ __forceinline__ float gelu(float z) { return z * normcdff(z); }
+__device__ __forceinline__ float gelu_grad(float z, float phi) {
+  return phi + z * (0.3989422804014327f * expf(-0.5f * z * z));
+}
+__device__ __forceinline__ float gelu_grad(float z) { return gelu_grad(z, normcdff(z)); }
+
+}  // namespace fno

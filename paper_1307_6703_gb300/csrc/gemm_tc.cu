@@ -32,49 +32,12 @@
 
 #include "fno.h"
 #include "gemm_tc.h"
+#include "tc_device.cuh"
 
 namespace tc {
 namespace {
 
-constexpr int kBM = 128;
-constexpr int kBK = 64;
 constexpr int kThreads = 128;
-constexpr uint32_t kWaitLimit = 1u << 24;
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  for (uint32_t it = 0; it < kWaitLimit; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-
-// Shared-memory matrix descriptor of a K-major, 128-byte swizzled operand
-// tile (tcgen05 format): start address >> 4 in bits 0-13, leading byte
-// offset (unused for swizzled K-major operands) 0, stride byte offset
-// (between 8-row groups: 1024 bytes) >> 4 in bits 32-45, descriptor version
-// 1 in bits 46-47, swizzle mode 128 B (2) in bits 61-63.
-__device__ __forceinline__ uint64_t kmajor_sw128_desc(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-
-// Instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
-// (bits 7-9 and 10-12 = 1, the same type for both), both K-major (bits 15,
-// 16 = 0), N >> 3 in bits 17-22, M >> 4 in bits 24-28.
-template <int BN>
-__host__ __device__ constexpr uint32_t idesc_bf16() {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-}
 
 // Stages: 1 when the K range fits one stage (no pipeline to keep full, and
 // a small footprint lets more CTAs share an SM), else 4.
@@ -86,14 +49,6 @@ struct __align__(1024) Smem {
   uint32_t tmem;
   static_assert(sizeof(a) + sizeof(b) >= 4 * 32 * 33 * sizeof(float), "the epilogue's staging tiles reuse stage memory");
 };
-
-__device__ __forceinline__ void tma_load_3d(const CUtensorMap *map, uint32_t dst, uint32_t bar, int x, int y, int z) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
-      : "memory");
-}
 
 template <int BN, int kStages>
 __global__ void __launch_bounds__(kThreads)
@@ -312,6 +267,32 @@ gemm_f32_kernel(const float *__restrict__ a, long long am, long long ak, long lo
     }
 }
 
+template <int BN, int kStages>
+cudaError_t launch_tn(const CUtensorMap &mx, const CUtensorMap &my, const GemmParams &p, int nb, cudaStream_t st) {
+  const size_t smem = sizeof(Smem<BN, kStages>) + 1024;
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(gemm_tn_bf16_kernel<BN, kStages>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((p.M + kBM - 1) / kBM), (unsigned)((p.N + BN - 1) / BN), (unsigned)(nb * p.ksplit));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  return cudaLaunchKernelEx(&cfg, gemm_tn_bf16_kernel<BN, kStages>, mx, my, p);
+}
+
+template <int BN>
+cudaError_t launch_tn_stages(const CUtensorMap &mx, const CUtensorMap &my, const GemmParams &p, int nb,
+                             cudaStream_t st) {
+  return p.kper <= kBK ? launch_tn<BN, 1>(mx, my, p, nb, st) : launch_tn<BN, 4>(mx, my, p, nb, st);
+}
+
+}  // namespace
+
 typedef CUresult (*encode_tiled_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                     const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                     CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -340,32 +321,6 @@ cudaError_t operand_map(const __nv_bfloat16 *base, int K, int rows, int ld, long
                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
-
-template <int BN, int kStages>
-cudaError_t launch_tn(const CUtensorMap &mx, const CUtensorMap &my, const GemmParams &p, int nb, cudaStream_t st) {
-  const size_t smem = sizeof(Smem<BN, kStages>) + 1024;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tn_bf16_kernel<BN, kStages>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((p.M + kBM - 1) / kBM), (unsigned)((p.N + BN - 1) / BN), (unsigned)(nb * p.ksplit));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, gemm_tn_bf16_kernel<BN, kStages>, mx, my, p);
-}
-
-template <int BN>
-cudaError_t launch_tn_stages(const CUtensorMap &mx, const CUtensorMap &my, const GemmParams &p, int nb,
-                             cudaStream_t st) {
-  return p.kper <= kBK ? launch_tn<BN, 1>(mx, my, p, nb, st) : launch_tn<BN, 4>(mx, my, p, nb, st);
-}
-
-}  // namespace
 
 cudaError_t gemm_tn_bf16(const __nv_bfloat16 *X, int ldx, long long sX, const __nv_bfloat16 *Y, int ldy, long long sY,
                          float *C, long long cm, long long cn, long long sC, int M, int N, int K, int batch, int ksplit,

@@ -2,6 +2,7 @@
 // to the library; not part of the C ABI.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -16,6 +17,12 @@ struct GemmParams {
   float beta;                 // C = D + beta * C
   int *err;                   // set to 1 when a bounded wait gives up
 };
+
+// 3D TMA map {K, rows, batch} of a BF16 operand with row pitch ld and batch
+// stride sb (elements), box {64, box_rows, 1}, 128-byte swizzle, zero fill
+// outside.
+cudaError_t operand_map(const __nv_bfloat16 *base, int K, int rows, int ld, long long sb, int nb, int box_rows,
+                        CUtensorMap *map);
 
 // D[b](m, n) = sum_k X[b](m, k) Y[b](n, k) on the tensor cores: X is M x K
 // with row pitch ldx (elements) and batch stride sX (0: one matrix for all
