@@ -40,14 +40,15 @@ namespace {
 constexpr int kThreads = 128;
 constexpr int C = kWidth;
 
-// Operand tiles and the two accumulators of a layer kernel.
+// Operand tiles of a layer kernel; kK: K columns of a tile (32 where 2 modes_x
+// allows, with 64-byte swizzle rows: half the shared memory, twice the CTAs).
+template <int kK>
 struct __align__(1024) LayerSmem {
-  __nv_bfloat16 a1[tc::kBM * tc::kBK], a2[tc::kBM * tc::kBK];
-  __nv_bfloat16 b1[C * tc::kBK], b2[C * tc::kBK];
+  __nv_bfloat16 a1[tc::kBM * kK], a2[tc::kBM * kK];
+  __nv_bfloat16 b1[C * kK], b2[C * kK];
   unsigned long long full, done;
   uint32_t tmem;
 };
-constexpr uint32_t kLayerTx = 2 * (tc::kBM + C) * tc::kBK * 2;
 
 // Tensor memory of a CTA: `cols` columns (a power of two >= 32), and the
 // barriers' initialisation; all threads.
@@ -84,63 +85,60 @@ __device__ __forceinline__ bool wait_done(unsigned long long *bar, int *err) {
   return ok;
 }
 
-// Sums of v[i] over the warp's lanes; lane i returns that of v[i] (31 shuffles:
-// each stage halves the values a lane still carries).
-__device__ __forceinline__ float warp_sums(float (&v)[32]) {
+// Sums of v[0..7] over the warp's lanes: lane l returns that of v[l >> 2] (the
+// first three stages halve the values a lane still carries).
+__device__ __forceinline__ float warp_sums(const float (&v)[8]) {
   const int lane = threadIdx.x & 31;
+  float h[8];
 #pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) {
-    const bool up = lane & o;
+  for (int i = 0; i < 8; ++i) h[i] = v[i];
+#pragma unroll
+  for (int o = 4; o >= 1; o >>= 1) {
+    const bool up = lane & (4 * o);
 #pragma unroll
     for (int i = 0; i < o; ++i) {
-      const float send = up ? v[i] : v[i + o], keep = up ? v[i + o] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      const float send = up ? h[i] : h[i + o], keep = up ? h[i + o] : h[i];
+      h[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * o);
     }
   }
-  return v[0];
+  h[0] += __shfl_xor_sync(0xffffffffu, h[0], 2);
+  return h[0] + __shfl_xor_sync(0xffffffffu, h[0], 1);
 }
 
-// Sums over groups of four sites (the lanes 4g .. 4g+3), ((x0 + x1) + (x2 + x3))
-// as a float4 sum of a row takes them: lane 4g + r returns channels 16 (r & 1) +
-// 8 (r >> 1) .. + 7 of group g in q.
-__device__ __forceinline__ void quad_sums(const float (&v)[32], float (&q)[8]) {
+// Sums of eight channels over groups of four sites (the lanes 4g .. 4g+3),
+// ((x0 + x1) + (x2 + x3)) as a float4 sum of a row takes them, into quads[c][s / 4]
+// (lanes of valid sites; rows are whole groups of four).
+__device__ __forceinline__ void put_quads(const float (&v)[8], bool valid, float *quads, long long S4, long long s) {
   const int lane = threadIdx.x & 31;
-  float h[16];
+  float h[4], q[2];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const float send = lane & 1 ? v[i] : v[i + 16], keep = lane & 1 ? v[i + 16] : v[i];
+  for (int i = 0; i < 4; ++i) {
+    const float send = lane & 1 ? v[i] : v[i + 4], keep = lane & 1 ? v[i + 4] : v[i];
     h[i] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
   }
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float send = lane & 2 ? h[i] : h[i + 8], keep = lane & 2 ? h[i + 8] : h[i];
+  for (int i = 0; i < 2; ++i) {
+    const float send = lane & 2 ? h[i] : h[i + 2], keep = lane & 2 ? h[i + 2] : h[i];
     q[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
   }
-}
-// The quad sums of a warp's 32 sites into quads[c][s / 4] (lanes of valid
-// sites; rows are whole groups of four).
-__device__ __forceinline__ void put_quads(const float (&v)[32], bool valid, float *quads, long long S4, long long s) {
-  float q[8];
-  quad_sums(v, q);
   if (!valid) return;
-  const int lane = threadIdx.x & 31, c0 = 16 * (lane & 1) + 8 * ((lane >> 1) & 1);
+  const int c0 = 4 * (lane & 1) + 2 * ((lane >> 1) & 1);
 #pragma unroll
-  for (int i = 0; i < 8; ++i) quads[(c0 + i) * S4 + (s >> 2)] = q[i];
+  for (int i = 0; i < 2; ++i) quads[(c0 + i) * S4 + (s >> 2)] = q[i];
 }
 
-// A site's 32 channels as BF16: channel-major (32 sites of a channel are
-// consecutive) and, 64 bytes a site, site-major.
-__device__ __forceinline__ void put_bf16(const float (&v)[32], bool valid, __nv_bfloat16 *cm, long long S,
+// Eight channels of a site as BF16: channel-major (32 sites of a channel are
+// consecutive) and 16 bytes of the site's row of the site-major copy.
+__device__ __forceinline__ void put_bf16(const float (&v)[8], bool valid, __nv_bfloat16 *cm, long long S,
                                          __nv_bfloat16 *sm) {
   if (!valid) return;
-  __align__(16) __nv_bfloat16 h[32];
+  __align__(16) __nv_bfloat16 h[8];
 #pragma unroll
-  for (int o = 0; o < 32; ++o) {
+  for (int o = 0; o < 8; ++o) {
     h[o] = __float2bfloat16_rn(v[o]);
     cm[o * S] = h[o];
   }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) reinterpret_cast<uint4 *>(sm)[q] = reinterpret_cast<const uint4 *>(h)[q];
+  *reinterpret_cast<uint4 *>(sm) = *reinterpret_cast<const uint4 *>(h);
 }
 
 // x, as a value of its own to the compiler: gelu and gelu' of the same z are
@@ -164,30 +162,32 @@ struct LayerArgs {
   int *err;
 };
 
-// One tile (x0 .. x0+127 of row y, field b) through both products.
-template <int kMode>
-__global__ void __launch_bounds__(kThreads, 4)
+// One tile (x0 .. x0+127 of row y, field b) through both products.  The
+// epilogue takes eight channels at a time (unrolled over all 32 its code did
+// not fit the instruction cache: 1.05 of 6.7 stall cycles an instruction).
+template <int kMode, int kK>
+__global__ void __launch_bounds__(kThreads, kK == 32 ? 8 : 5)
 layer_kernel(const __grid_constant__ CUtensorMap ma1, const __grid_constant__ CUtensorMap mb1,
              const __grid_constant__ CUtensorMap ma2, const __grid_constant__ CUtensorMap mb2, const LayerArgs p) {
   extern __shared__ unsigned char raw[];
-  LayerSmem &S = *reinterpret_cast<LayerSmem *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+  using Sm = LayerSmem<kK>;
+  Sm &S = *reinterpret_cast<Sm *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int xt = blockIdx.x * tc::kBM, y = blockIdx.y, b = blockIdx.z;
   const uint32_t tmem = setup(&S.tmem, 64, &S.full, 2);
-  bool ok = true;
   if (t == 0) {
     const uint32_t bar = tc::smem_u32(&S.full);
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(kLayerTx) : "memory");
+    constexpr uint32_t tx = 2 * (tc::kBM + C) * kK * 2;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(tx) : "memory");
     tc::tma_load_3d(&ma1, tc::smem_u32(S.a1), bar, 0, xt, b * p.ny + y);
     tc::tma_load_3d(&mb1, tc::smem_u32(S.b1), bar, 0, 0, 0);
     tc::tma_load_3d(&ma2, tc::smem_u32(S.a2), bar, 0, xt, 0);
     tc::tma_load_3d(&mb2, tc::smem_u32(S.b2), bar, 0, b * C, y);
-    ok = tc::mbar_try(bar, 0u);
-    if (ok) {
+    if (tc::mbar_try(bar, 0u)) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       constexpr uint32_t idesc = tc::idesc_bf16<C>();
-      tc::mma_tile(tmem, tc::smem_u32(S.a1), tc::smem_u32(S.b1), C / 16, idesc);
-      tc::mma_tile(tmem + C, tc::smem_u32(S.a2), tc::smem_u32(S.b2), p.K2 / 16, idesc);
+      tc::mma_tile<2 * kK>(tmem, tc::smem_u32(S.a1), tc::smem_u32(S.b1), C / 16, idesc);
+      tc::mma_tile<2 * kK>(tmem + C, tc::smem_u32(S.a2), tc::smem_u32(S.b2), p.K2 / 16, idesc);
     } else {  // (the copies in flight land before the CTA leaves: waited for once more)
       atomicOr(p.err, 1);
       (void)tc::mbar_try(bar, 0u);
@@ -200,30 +200,36 @@ layer_kernel(const __grid_constant__ CUtensorMap ma1, const __grid_constant__ CU
   const int x = xt + warp * 32 + lane;
   const bool valid = x < p.nx;
   const long long sites = (long long)p.nx * p.ny, s = (long long)y * p.nx + x;
+  const long long row = (long long)b * C * sites + s;
   const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);
-  float v[32], u[32];
-  tc::tmem_load32(lanes, v);        // the channel mixing
-  tc::tmem_load32(lanes + C, u);    // the transform
-  if constexpr (kMode == kForward || kMode == kForwardLast) {
-    float *z = p.z + (long long)b * C * sites + s;
+#pragma unroll 1
+  for (int c0 = 0; c0 < C; c0 += 8) {
+    float v[8], u[8];
+    tc::tmem_load8(lanes + c0, v);      // the channel mixing
+    tc::tmem_load8(lanes + C + c0, u);  // the transform
+    const long long e = row + c0 * sites;
+    __nv_bfloat16 *cm = p.cm + e, *sm = p.sm + ((long long)b * sites + s) * C + c0;
+    if constexpr (kMode == kForward || kMode == kForwardLast) {
 #pragma unroll
-    for (int o = 0; o < C; ++o) {
-      const float zz = (u[o] + v[o]) + p.w[o];
-      if (valid) z[o * sites] = zz;
-      v[o] = kMode == kForward ? gelu(zz) : zz;
+      for (int o = 0; o < 8; ++o) {
+        const float zz = (u[o] + v[o]) + p.w[c0 + o];
+        if (valid) p.z[e + o * sites] = zz;
+        v[o] = kMode == kForward ? gelu(zz) : zz;
+      }
+      put_bf16(v, valid, cm, sites, sm);
+    } else if constexpr (kMode == kBackward) {
+      float z[8];
+#pragma unroll
+      for (int o = 0; o < 8; ++o) z[o] = valid ? p.zprev[e + o * sites] : 0.f;
+#pragma unroll
+      for (int o = 0; o < 8; ++o) u[o] = (v[o] + u[o]) * gelu_grad(z[o]);
+      put_bf16(u, valid, cm, sites, sm);
+      put_quads(u, valid, p.quads + ((long long)b * C + c0) * (sites / 4), sites / 4, s);
+    } else {
+#pragma unroll
+      for (int o = 0; o < 8; ++o)
+        if (valid) p.dv[e + o * sites] = v[o] + u[o];
     }
-    put_bf16(v, valid, p.cm + (long long)b * C * sites + s, sites, p.sm + ((long long)b * sites + s) * C);
-  } else if constexpr (kMode == kBackward) {
-    const float *z = p.zprev + (long long)b * C * sites + s;
-#pragma unroll
-    for (int o = 0; o < C; ++o) u[o] = (v[o] + u[o]) * gelu_grad(valid ? z[o * sites] : 0.f);
-    put_bf16(u, valid, p.cm + (long long)b * C * sites + s, sites, p.sm + ((long long)b * sites + s) * C);
-    put_quads(u, valid, p.quads + (long long)b * C * (sites / 4), sites / 4, s);
-  } else {
-    float *dv = p.dv + (long long)b * C * sites + s;
-#pragma unroll
-    for (int o = 0; o < C; ++o)
-      if (valid) dv[o * sites] = v[o] + u[o];
   }
   release_tmem(tmem, 64);
 }
@@ -251,18 +257,22 @@ lift_kernel(int nx, int ny, const float *__restrict__ prm, const float *__restri
   const int x = blockIdx.x * kThreads + threadIdx.x, y = blockIdx.y, b = blockIdx.z;
   if (x >= nx) return;
   const long long sites = (long long)nx * ny, s = (long long)y * nx + x;
-  float f[kFeat], v[32];
+  float f[kFeat];
   features(prm, b, x, y, ny, f);
 #pragma unroll
   for (int c = 0; c < kFeat; ++c) x0[((long long)b * kFeat + c) * sites + s] = f[c];
 #pragma unroll
-  for (int o = 0; o < C; ++o) {
-    float acc = ps[o];
+  for (int c0 = 0; c0 < C; c0 += 8) {
+    float v[8];
 #pragma unroll
-    for (int c = 0; c < kFeat; ++c) acc += Ps[o * kFeat + c] * f[c];
-    v[o] = acc;
+    for (int o = 0; o < 8; ++o) {
+      float acc = ps[c0 + o];
+#pragma unroll
+      for (int c = 0; c < kFeat; ++c) acc += Ps[(c0 + o) * kFeat + c] * f[c];
+      v[o] = acc;
+    }
+    put_bf16(v, true, cm + ((long long)b * C + c0) * sites + s, sites, sm + ((long long)b * sites + s) * C + c0);
   }
-  put_bf16(v, true, cm + (long long)b * C * sites + s, sites, sm + ((long long)b * sites + s) * C);
 }
 
 // ---------------------------------------------------------- the projection
@@ -293,7 +303,7 @@ struct ProjArgs {
 };
 
 template <int H, bool kBack>
-__global__ void __launch_bounds__(kThreads, 4)
+__global__ void __launch_bounds__(kThreads, kBack ? 4 : 5)
 project_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb1,
                const __grid_constant__ CUtensorMap mb2, const ProjArgs p) {
   extern __shared__ unsigned char raw[];
@@ -315,7 +325,7 @@ project_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ C
     if (kBack) tc::tma_load_3d(&mb2, tc::smem_u32(S.b2), bar, 0, 0, 0);
     if (tc::mbar_try(bar, 0u)) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      tc::mma_tile(tmem, tc::smem_u32(S.a), tc::smem_u32(S.b1), C / 16, tc::idesc_bf16<H>());
+      tc::mma_tile<128>(tmem, tc::smem_u32(S.a), tc::smem_u32(S.b1), C / 16, tc::idesc_bf16<H>());
     } else {
       atomicOr(p.err, 1);
       (void)tc::mbar_try(bar, 0u);
@@ -334,11 +344,11 @@ project_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ C
 #pragma unroll
     for (int j = 0; j < kMaxO; ++j) acc[j] = j < p.O ? S.q2[j] : 0.f;
 #pragma unroll 1
-    for (int h0 = 0; h0 < H; h0 += 32) {
-      float v[32];
-      tc::tmem_load32(lanes + h0, v);
+    for (int h0 = 0; h0 < H; h0 += 8) {
+      float v[8];
+      tc::tmem_load8(lanes + h0, v);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
+      for (int i = 0; i < 8; ++i) {
         const float a = gelu(v[i] + S.q1[h0 + i]);
 #pragma unroll
         for (int j = 0; j < kMaxO; ++j)
@@ -368,13 +378,13 @@ project_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ C
     }
     unsigned char *arow = reinterpret_cast<unsigned char *>(S.a) + r * 128;  // this site's row of the dhp tile
 #pragma unroll 1
-    for (int h0 = 0; h0 < H; h0 += 32) {
-      float a[32], d[32];
-      tc::tmem_load32(lanes + h0, a);
+    for (int h0 = 0; h0 < H; h0 += 8) {
+      float a[8], d[8];
+      tc::tmem_load8(lanes + h0, a);
       __nv_bfloat16 *dh = p.dhp + ((long long)b * H + h0) * sites + s;
-      __align__(16) __nv_bfloat16 hb[32];
+      __align__(16) __nv_bfloat16 hb[8];
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
+      for (int i = 0; i < 8; ++i) {
         const float z = a[i] + S.q1[h0 + i];
         float q = 0.f;
 #pragma unroll
@@ -386,14 +396,16 @@ project_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ C
         if (valid) dh[i * sites] = hb[i];
       }
       // 16-byte chunk c of row r sits at chunk c ^ (r & 7) (128-byte swizzle)
+      *reinterpret_cast<uint4 *>(arow + (((h0 / 8) ^ (r & 7)) << 4)) = *reinterpret_cast<const uint4 *>(hb);
+      const float ds = warp_sums(d);
+      if ((lane & 3) == 0) S.red[warp][h0 + (lane >> 2)] = (double)ds;
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        *reinterpret_cast<uint4 *>(arow + (((h0 / 8 + q) ^ (r & 7)) << 4)) = reinterpret_cast<const uint4 *>(hb)[q];
-      S.red[warp][h0 + lane] = (double)warp_sums(d);
-      for (int j = 0; j < p.O; ++j) {
+      for (int j = 0; j < kMaxO; ++j) {
+        if (j >= p.O) break;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) d[i] = dout[j] * a[i];
-        S.red[warp][H + j * H + h0 + lane] = (double)warp_sums(d);
+        for (int i = 0; i < 8; ++i) d[i] = dout[j] * a[i];
+        const float as = warp_sums(d);
+        if ((lane & 3) == 0) S.red[warp][H + j * H + h0 + (lane >> 2)] = (double)as;
       }
     }
     // dv = Q1^T dhp: the tile just written against Q1^T
@@ -402,15 +414,18 @@ project_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ C
     __syncthreads();
     if (t == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      tc::mma_tile(tmem + H, tc::smem_u32(S.a), tc::smem_u32(S.b2), H / 16, tc::idesc_bf16<C>());
+      tc::mma_tile<128>(tmem + H, tc::smem_u32(S.a), tc::smem_u32(S.b2), H / 16, tc::idesc_bf16<C>());
       tc::mma_commit(tc::smem_u32(&S.done2));
     }
     __syncwarp();
     (void)wait_done(&S.done2, p.err);
-    float v[32];
-    tc::tmem_load32(lanes + H, v);
-    put_bf16(v, valid, p.cm + (long long)b * C * sites + s, sites, p.sm + ((long long)b * sites + s) * C);
-    put_quads(v, valid, p.quads + (long long)b * C * (sites / 4), sites / 4, s);
+#pragma unroll 1
+    for (int c0 = 0; c0 < C; c0 += 8) {
+      float v[8];
+      tc::tmem_load8(lanes + H + c0, v);
+      put_bf16(v, valid, p.cm + ((long long)b * C + c0) * sites + s, sites, p.sm + ((long long)b * sites + s) * C + c0);
+      put_quads(v, valid, p.quads + ((long long)b * C + c0) * (sites / 4), sites / 4, s);
+    }
     const int base = H * (1 + p.O), n = base + p.O + 1;
     double tail[kMaxO + 1];
 #pragma unroll
@@ -494,21 +509,26 @@ struct LayerMaps {
 
 cudaError_t layer_maps(const Shape &s, const __nv_bfloat16 *a1, const __nv_bfloat16 *b1, const __nv_bfloat16 *a2,
                        const __nv_bfloat16 *b2, LayerMaps *m) {
-  cudaError_t e = tc::operand_map(a1, C, s.nx, C, (long long)s.nx * C, s.B * s.ny, tc::kBM, &m->a1);
-  if (e == cudaSuccess) e = tc::operand_map(b1, C, C, C, 0, 1, C, &m->b1);
-  if (e == cudaSuccess) e = tc::operand_map(a2, s.K2, s.nx, s.K2, 0, 1, tc::kBM, &m->a2);
+  const int kk = s.K2 <= 32 ? 32 : 64;
+  cudaError_t e = tc::operand_map(a1, C, s.nx, C, (long long)s.nx * C, s.B * s.ny, tc::kBM, &m->a1, kk);
+  if (e == cudaSuccess) e = tc::operand_map(b1, C, C, C, 0, 1, C, &m->b1, kk);
+  if (e == cudaSuccess) e = tc::operand_map(a2, s.K2, s.nx, s.K2, 0, 1, tc::kBM, &m->a2, kk);
   // rows: the channels of all fields at one y
-  if (e == cudaSuccess) e = tc::operand_map(b2, s.K2, s.B * C, s.ny * s.K2, s.K2, s.ny, C, &m->b2);
+  if (e == cudaSuccess) e = tc::operand_map(b2, s.K2, s.B * C, s.ny * s.K2, s.K2, s.ny, C, &m->b2, kk);
   return e;
 }
 
+template <int kMode, int kK>
+cudaError_t launch_layer_k(const Shape &s, const LayerMaps &m, const LayerArgs &p, cudaStream_t st) {
+  const size_t smem = sizeof(LayerSmem<kK>) + 1024;
+  const cudaError_t e = allow_smem(layer_kernel<kMode, kK>, smem);
+  if (e != cudaSuccess) return e;
+  layer_kernel<kMode, kK><<<tile_grid(s), kThreads, smem, st>>>(m.a1, m.b1, m.a2, m.b2, p);
+  return cudaGetLastError();
+}
 template <int kMode>
 cudaError_t launch_layer(const Shape &s, const LayerMaps &m, const LayerArgs &p, cudaStream_t st) {
-  const size_t smem = sizeof(LayerSmem) + 1024;
-  const cudaError_t e = allow_smem(layer_kernel<kMode>, smem);
-  if (e != cudaSuccess) return e;
-  layer_kernel<kMode><<<tile_grid(s), kThreads, smem, st>>>(m.a1, m.b1, m.a2, m.b2, p);
-  return cudaGetLastError();
+  return s.K2 <= 32 ? launch_layer_k<kMode, 32>(s, m, p, st) : launch_layer_k<kMode, 64>(s, m, p, st);
 }
 
 template <int H, bool kBack>

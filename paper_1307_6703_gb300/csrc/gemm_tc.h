@@ -19,10 +19,10 @@ struct GemmParams {
 };
 
 // 3D TMA map {K, rows, batch} of a BF16 operand with row pitch ld and batch
-// stride sb (elements), box {64, box_rows, 1}, 128-byte swizzle, zero fill
-// outside.
+// stride sb (elements), box {kbox, box_rows, 1}, zero fill outside; kbox 64:
+// 128-byte swizzle, 32: 64-byte.
 cudaError_t operand_map(const __nv_bfloat16 *base, int K, int rows, int ld, long long sb, int nb, int box_rows,
-                        CUtensorMap *map);
+                        CUtensorMap *map, int kbox = 64);
 
 // D[b](m, n) = sum_k X[b](m, k) Y[b](n, k) on the tensor cores: X is M x K
 // with row pitch ldx (elements) and batch stride sX (0: one matrix for all

@@ -42,6 +42,11 @@ __device__ __forceinline__ uint64_t kmajor_sw128_desc(uint32_t saddr) {
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 
+// The same for 64-byte rows (K = 32): 64-byte swizzle (4), eight rows 512 bytes.
+__device__ __forceinline__ uint64_t kmajor_sw64_desc(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
+}
+
 // Instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
 // (bits 7-9 and 10-12 = 1, the same type for both), both K-major (bits 15,
 // 16 = 0), N >> 3 in bits 17-22, M >> 4 in bits 24-28.
@@ -63,10 +68,14 @@ __device__ __forceinline__ void mbar_init(uint32_t bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
 }
 
-// D (+)= A B^T on `nk` K = 16 steps of two K-major tiles (one thread issues).
+// D = A B^T on `nk` K = 16 steps of two K-major tiles with rows of kRow bytes
+// (one thread issues).
+template <int kRow>
 __device__ __forceinline__ void mma_tile(uint32_t tmem, uint32_t a, uint32_t b, int nk, uint32_t idesc) {
+  static_assert(kRow == 128 || kRow == 64, "swizzle rows");
   for (int j = 0; j < nk; ++j) {  // K = 16 per MMA: 32 bytes along the swizzle row
-    const uint64_t ad = kmajor_sw128_desc(a + 32 * j), bd = kmajor_sw128_desc(b + 32 * j);
+    const uint64_t ad = kRow == 128 ? kmajor_sw128_desc(a + 32 * j) : kmajor_sw64_desc(a + 32 * j);
+    const uint64_t bd = kRow == 128 ? kmajor_sw128_desc(b + 32 * j) : kmajor_sw64_desc(b + 32 * j);
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
@@ -78,21 +87,16 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// 32 accumulator columns of this warp's 32 rows: lane = row.
-__device__ __forceinline__ void tmem_load32(uint32_t taddr, float *v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
+// Eight accumulator columns of this warp's 32 rows: lane = row.
+__device__ __forceinline__ void tmem_load8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 }  // namespace tc
