@@ -132,44 +132,61 @@ __global__ void lift_kernel(const float *__restrict__ x0, const float *__restric
   }
 }
 
+constexpr int kYChunk = 64;  // rows of a chunk of ydft_kernel and iy_kernel
+
 // Spectral kernels.  Rows of the x-transformed lines hold the mx kept
 // modes as (real parts, then imaginary parts): X[bc][y][j], j < mx real and
 // j >= mx imaginary part of mode j - mx; mode sets are [bc][ky][kx][2].
 // Ty[ky][y] = (cos theta, sin theta) with theta = 2 pi ky' y / ny.  Rows are
 // processed in chunks of kYChunk staged in shared memory with the chunk's
 // twiddles; sums run over y in order.
-constexpr int kYChunk = 64;
 
-// y-transform: S[bc][ky][kx] = sum_y (X_r + i X_i)[y][kx] e^{-i theta}.
-// One block per line set bc; dynamic shared memory (kYChunk (2 mx + 2 my))
-// floats.
+// y-transform: S[bc][ky][kx] = sum_y (X_r + i X_i)[y][kx] e^{-i theta}, one
+// thread per (ky, kx) (two where there are more than kThreads), its sum over y
+// in order.  Block (bc, g) takes gx of the kx, from g gx: all of them where the
+// line sets fill the GPU, four where they are few (the 32 of a 2048 x 512
+// field: 25 us with one block each, 13 us).  Rows in chunks of kYChunk; dynamic
+// shared memory kYChunk (2 gx + 2 my) floats.
 __global__ void __launch_bounds__(kThreads)
-ydft_kernel(const float *__restrict__ A, const float2 *__restrict__ Ty, int ny, int mx, int my,
+ydft_kernel(const float *__restrict__ A, const float2 *__restrict__ Ty, int ny, int mx, int my, int gx,
             float *__restrict__ Sh) {
   extern __shared__ float ysm[];
-  float *xs = ysm;                                              // [kYChunk][2 mx]
-  float2 *ts = reinterpret_cast<float2 *>(ysm + kYChunk * 2 * mx);  // [my][kYChunk]
-  const int bc = blockIdx.x, t = threadIdx.x, M = my * mx;
+  float *xs = ysm;                                                  // [kYChunk][2 gx]
+  float2 *ts = reinterpret_cast<float2 *>(ysm + kYChunk * 2 * gx);  // [my][kYChunk]
+  const int bc = blockIdx.x, k0 = blockIdx.y * gx, nk = min(gx, mx - k0), t = threadIdx.x, M = my * gx;
   const float *a = A + (long long)bc * ny * 2 * mx;
   float sr[2] = {0.f, 0.f}, si[2] = {0.f, 0.f};  // outputs t and t + kThreads
   for (int y0 = 0; y0 < ny; y0 += kYChunk) {
     const int yc = min(kYChunk, ny - y0);
     __syncthreads();
-    for (int e = t; e < yc * 2 * mx; e += kThreads) xs[e] = a[(long long)y0 * 2 * mx + e];
-    for (int e = t; e < my * yc; e += kThreads) {
-      const int k = e / yc, y = e - k * yc;
-      ts[k * kYChunk + y] = Ty[k * ny + y0 + y];
+    if (gx == mx && mx % 2 == 0) {  // whole rows: one contiguous block
+      const float4 *src = reinterpret_cast<const float4 *>(a + (long long)y0 * 2 * mx);
+      for (int e = t; e < yc * mx / 2; e += kThreads) reinterpret_cast<float4 *>(xs)[e] = src[e];
+    } else {
+      for (int e = t; e < yc * gx; e += kThreads) {
+        const int y = e / gx, k = e - y * gx;
+        const float *p = a + (long long)(y0 + y) * 2 * mx + k0 + k;
+        xs[y * 2 * gx + k] = k < nk ? p[0] : 0.f;
+        xs[y * 2 * gx + gx + k] = k < nk ? p[mx] : 0.f;
+      }
+    }
+    for (int e = t; e < my * kYChunk; e += kThreads) {
+      const int k = e / kYChunk, y = e % kYChunk;
+      if (y < yc) ts[e] = Ty[k * ny + y0 + y];
     }
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int o = t + q * kThreads;
       if (o < M) {
-        const int k = o / mx, kx = o - k * mx;
+        const int k = o / gx, kx = o - k * gx;
+        const float *x = xs + kx;
+        const float2 *w = ts + k * kYChunk;
         float r = sr[q], im = si[q];
+#pragma unroll 8
         for (int y = 0; y < yc; y++) {
-          const float2 tw = ts[k * kYChunk + y];
-          const float ar = xs[y * 2 * mx + kx], ai = xs[y * 2 * mx + mx + kx];
+          const float2 tw = w[y];
+          const float ar = x[y * 2 * gx], ai = x[y * 2 * gx + gx];
           r += ar * tw.x + ai * tw.y;
           im += ai * tw.x - ar * tw.y;
         }
@@ -182,50 +199,47 @@ ydft_kernel(const float *__restrict__ A, const float2 *__restrict__ Ty, int ny, 
   for (int q = 0; q < 2; ++q) {
     const int o = t + q * kThreads;
     if (o < M) {
-      float *d = Sh + ((long long)bc * M + o) * 2;
-      d[0] = sr[q];
-      d[1] = si[q];
+      const int k = o / gx, kx = o - k * gx;
+      if (kx < nk)
+        *reinterpret_cast<float2 *>(Sh + (((long long)bc * my + k) * mx + k0 + kx) * 2) = make_float2(sr[q], si[q]);
     }
   }
 }
 
 // Inverse y-transform (and the adjoint of the y-transform, which has the
 // same form): X[bc][y][kx] = sum_ky Y[bc][ky][kx] e^{+i theta}, written as
-// (real, imaginary) rows (X null: not wanted) with a BF16 copy.  One block per line set;
-// dynamic shared memory (2 my mx + 2 my kYChunk) floats.
+// (real, imaginary) rows (X null: not wanted) with a BF16 copy.  Block (bc, c)
+// takes rows kYChunk c ...; dynamic shared memory (2 my mx + 2 my kYChunk)
+// floats.
 __global__ void __launch_bounds__(kThreads)
 iy_kernel(const float *__restrict__ Y, const float2 *__restrict__ Ty, int ny, int mx, int my, float *__restrict__ X,
           __nv_bfloat16 *__restrict__ Xb) {
   extern __shared__ float ysm[];
   float *ys = ysm;                                              // [my][mx][2]
   float2 *ts = reinterpret_cast<float2 *>(ysm + 2 * my * mx);   // [my][kYChunk]
-  const int bc = blockIdx.x, t = threadIdx.x;
+  const int bc = blockIdx.x, y0 = blockIdx.y * kYChunk, yc = min(kYChunk, ny - y0), t = threadIdx.x;
   for (int e = t; e < 2 * my * mx; e += kThreads) ys[e] = Y[(long long)bc * 2 * my * mx + e];
-  for (int y0 = 0; y0 < ny; y0 += kYChunk) {
-    const int yc = min(kYChunk, ny - y0);
-    __syncthreads();
-    for (int e = t; e < my * yc; e += kThreads) {
-      const int k = e / yc, y = e - k * yc;
-      ts[k * kYChunk + y] = Ty[k * ny + y0 + y];
+  for (int e = t; e < my * yc; e += kThreads) {
+    const int k = e / yc, y = e - k * yc;
+    ts[k * kYChunk + y] = Ty[k * ny + y0 + y];
+  }
+  __syncthreads();
+  for (int e = t; e < yc * mx; e += kThreads) {
+    const int y = e / mx, kx = e - y * mx;
+    float gr = 0.f, gi = 0.f;
+    for (int k = 0; k < my; k++) {
+      const float2 tw = ts[k * kYChunk + y];
+      const float yr = ys[(k * mx + kx) * 2], yi = ys[(k * mx + kx) * 2 + 1];
+      gr += yr * tw.x - yi * tw.y;
+      gi += yr * tw.y + yi * tw.x;
     }
-    __syncthreads();
-    for (int e = t; e < yc * mx; e += kThreads) {
-      const int y = e / mx, kx = e - y * mx;
-      float gr = 0.f, gi = 0.f;
-      for (int k = 0; k < my; k++) {
-        const float2 tw = ts[k * kYChunk + y];
-        const float yr = ys[(k * mx + kx) * 2], yi = ys[(k * mx + kx) * 2 + 1];
-        gr += yr * tw.x - yi * tw.y;
-        gi += yr * tw.y + yi * tw.x;
-      }
-      const long long g = ((long long)bc * ny + y0 + y) * 2 * mx;
-      if (X) {
-        X[g + kx] = gr;
-        X[g + mx + kx] = gi;
-      }
-      Xb[g + kx] = __float2bfloat16_rn(gr);
-      Xb[g + mx + kx] = __float2bfloat16_rn(gi);
+    const long long g = ((long long)bc * ny + y0 + y) * 2 * mx;
+    if (X) {
+      X[g + kx] = gr;
+      X[g + mx + kx] = gi;
     }
+    Xb[g + kx] = __float2bfloat16_rn(gr);
+    Xb[g + mx + kx] = __float2bfloat16_rn(gi);
   }
 }
 
@@ -323,6 +337,14 @@ __global__ void finish_loss_kernel(const double *__restrict__ partial, int n, lo
   if (threadIdx.x == 0) *loss = r / (double)total;
 }
 
+// (double)x by integer arithmetic: the conversion instruction shares the FP64
+// pipe, which bounds the two kernels below.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+  if (e - 1u >= 254u) return (double)x;  // zero, subnormal, infinite, NaN
+  return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b >> 3) & 0xfffffu)), (int)(b << 29));
+}
+
 // Initial fields of the solver from the network output (fno_fields):
 // per field b, block j: FP64 sum of the density d = 1 + s0 o0 over the
 // block's sites (grid-strided, then the fixed-order block tree).
@@ -332,30 +354,35 @@ __global__ void field_mass_kernel(const float *__restrict__ out, int outputs, lo
   const float *o = out + (size_t)blockIdx.y * outputs * S;
   double acc = 0.0;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < S; e += (long long)gridDim.x * blockDim.x)
-    acc += __dadd_rn(__dmul_rn(s0, (double)o[e]), 1.0);
+    acc += __dadd_rn(__dmul_rn(s0, widen(o[e])), 1.0);
   const double r = block_sum(acc, sm);
   if (threadIdx.x == 0) part[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = r;
 }
 
-// fields[b] = (d + (rho_mean - mean d), s1 o1, s2 o2); the mean from the
-// nblk block sums of field b in a fixed order.
+// Both bound by the FP64 adds and the stores: one wide grid after the shift is
+// known (38 us for a 2048 x 512 field where every block first summed the
+// partial masses again, 19 + 4 us here).
+
+// The density shift of field b, rho_mean - mean d, from its nblk <= kThreads
+// block sums by a fixed tree, in the place of the first of them.
+__global__ void shift_kernel(double *__restrict__ part, int nblk, long long S, double rho_mean) {
+  __shared__ double sm[kThreads];
+  double *p = part + (size_t)blockIdx.x * nblk;
+  const double m = block_sum((int)threadIdx.x < nblk ? p[threadIdx.x] : 0.0, sm);
+  if (threadIdx.x == 0) p[0] = rho_mean - m / (double)S;
+}
+
+// fields[b] = (d + shift, s1 o1, s2 o2).
 __global__ void fields_kernel(const float *__restrict__ out, int outputs, long long S, double s0, double s1,
-                              double s2, double rho_mean, const double *__restrict__ part, int nblk,
-                              double *__restrict__ fields) {
-  __shared__ double shift;
+                              double s2, const double *__restrict__ part, int nblk, double *__restrict__ fields) {
   const int b = blockIdx.y;
-  if (threadIdx.x == 0) {
-    double m = 0.0;
-    for (int j = 0; j < nblk; ++j) m += part[(size_t)b * nblk + j];
-    shift = rho_mean - m / (double)S;
-  }
-  __syncthreads();
+  const double shift = part[(size_t)b * nblk];
   const float *o = out + (size_t)b * outputs * S;
   double *f = fields + (size_t)b * 3 * S;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < S; e += (long long)gridDim.x * blockDim.x) {
-    f[e] = __dadd_rn(__dadd_rn(__dmul_rn(s0, (double)o[e]), 1.0), shift);
-    f[S + e] = __dmul_rn(s1, (double)o[S + e]);
-    f[2 * S + e] = __dmul_rn(s2, (double)o[2 * S + e]);
+    f[e] = __dadd_rn(__dadd_rn(__dmul_rn(s0, widen(o[e])), 1.0), shift);
+    f[S + e] = __dmul_rn(s1, widen(o[S + e]));
+    f[2 * S + e] = __dmul_rn(s2, widen(o[2 * S + e]));
   }
 }
 
@@ -420,6 +447,7 @@ template <int NA, int NB, bool kGelu>
 __global__ void __launch_bounds__(kThreads)
 outer_pass1_kernel(const float *__restrict__ a, const float *__restrict__ o2, int B, int Ca, int Cb, long long S,
                    double *__restrict__ part) {
+  constexpr int kFly = kGelu ? 1 : 4;
   __shared__ double sm[kThreads / 32][NA * NB];
   const int ntb = (Cb + NB - 1) / NB;
   const int ca0 = (blockIdx.y / ntb) * NA, cb0 = (blockIdx.y % ntb) * NB;
@@ -432,23 +460,32 @@ outer_pass1_kernel(const float *__restrict__ a, const float *__restrict__ o2, in
   const long long lo = blockIdx.x * per, hi = min(n, lo + per);
   long long e = lo + threadIdx.x;
   long long b = e / S, s = e - b * S;  // then advanced without dividing
-  for (; e < hi; e += blockDim.x, s += blockDim.x) {
-    while (s >= S) {
-      s -= S;
-      b++;
+  while (e < hi) {  // sites in order, the loads of four in flight
+    float av[kFly][NA], bv[kFly][NB];
+#pragma unroll
+    for (int q = 0; q < kFly; q++) {
+      while (s >= S) {
+        s -= S;
+        b++;
+      }
+      const bool in = e + q * (long long)blockDim.x < hi;
+#pragma unroll
+      for (int i = 0; i < NA; i++) av[q][i] = in && ca0 + i < Ca ? a[(b * Ca + ca0 + i) * S + s] : 0.f;
+#pragma unroll
+      for (int j = 0; j < NB; j++) bv[q][j] = in && cb0 + j < Cb ? o2[(b * Cb + cb0 + j) * S + s] : 0.f;
+      s += blockDim.x;
     }
-    float av[NA], bv[NB];
 #pragma unroll
-    for (int i = 0; i < NA; i++) av[i] = ca0 + i < Ca ? a[(b * Ca + ca0 + i) * S + s] : 0.f;
+    for (int q = 0; q < kFly; q++) {
+      if (e >= hi) break;
 #pragma unroll
-    for (int j = 0; j < NB; j++) {
-      const float v = cb0 + j < Cb ? o2[(b * Cb + cb0 + j) * S + s] : 0.f;
-      bv[j] = kGelu ? gelu(v) : v;
+      for (int j = 0; j < NB; j++) {
+        const float v = kGelu ? gelu(bv[q][j]) : bv[q][j];
+#pragma unroll
+        for (int i = 0; i < NA; i++) acc[i][j] = fmaf(av[q][i], v, acc[i][j]);
+      }
+      e += blockDim.x;
     }
-#pragma unroll
-    for (int i = 0; i < NA; i++)
-#pragma unroll
-      for (int j = 0; j < NB; j++) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
   }
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
@@ -810,9 +847,18 @@ cudaError_t sg(fno_handle *h, const float *A, long long am, long long ak, long l
 
 // Site-major copy of a [B][rows][S] BF16 activation: out[b][s][row].
 // Dynamic shared memory of the spectral kernels (bytes).
-size_t ydft_smem(int mx, int my) { return (size_t)kYChunk * (2 * mx + 2 * my) * sizeof(float); }
+// kx of a block of ydft_kernel.
+int ydft_group(int lines, int mx) { return lines >= 128 ? mx : std::min(mx, 4); }
+size_t ydft_smem(int gx, int my) { return (size_t)kYChunk * (2 * gx + 2 * my) * sizeof(float); }
 size_t iy_smem(int mx, int my) { return (size_t)(2 * my * mx + 2 * my * kYChunk) * sizeof(float); }
+dim3 iy_grid(int lines, int ny) { return dim3((unsigned)lines, (unsigned)((ny + kYChunk - 1) / kYChunk)); }
 size_t mix_smem(int B, int C, bool back) { return (size_t)((back ? 4 : 2) * B * C + 2 * C * C) * sizeof(float); }
+
+void ydft(fno_handle *h, const float *A, int lines, int ny, float *Sh) {
+  const int mx = h->c.modes_x, my = h->c.modes_y, gx = ydft_group(lines, mx);
+  ydft_kernel<<<dim3((unsigned)lines, (unsigned)((mx + gx - 1) / gx)), kThreads, ydft_smem(gx, my), h->st>>>(
+      A, h->Ty, ny, mx, my, gx, Sh);
+}
 
 void site_major(fno_handle *h, const __nv_bfloat16 *in, int B, int rows, long long S, __nv_bfloat16 *out) {
   const dim3 grid((unsigned)((rows + 31) / 32), (unsigned)((S + 63) / 64), (unsigned)B);
@@ -967,10 +1013,10 @@ int forward_fused(fno_handle *h, int B, int nx, int ny, const float *params_dev,
   FNO_CUDA(h, fno::lift(sh, params_dev, P + h->o.P, P + h->o.p, h->x0, h->Vb[0], h->VbT[0], st));
   for (int l = 0; l < L; l++) {
     FNO_GEMM(h, tcg(h, h->Vb[l], nx, 0, h->FxTb, nx, 0, h->A, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 1, 0.f));
-    ydft_kernel<<<B * c.width, kThreads, ydft_smem(mx, my), st>>>(h->A, h->Ty, ny, mx, my, h->Sh[l]);
+    ydft(h, h->A, B * c.width, ny, h->Sh[l]);
     mix_kernel<<<my * mx, kThreads, mix_smem(B, c.width, false), st>>>(h->Sh[l], P + h->o.Rr[l], P + h->o.Ri[l], B,
                                                                          c.width, my * mx, h->dY);
-    iy_kernel<<<B * c.width, kThreads, iy_smem(mx, my), st>>>(h->dY, h->Ty, ny, mx, my, nullptr, h->Gb);
+    iy_kernel<<<iy_grid(B * c.width, ny), kThreads, iy_smem(mx, my), st>>>(h->dY, h->Ty, ny, mx, my, nullptr, h->Gb);
     FNO_CUDA(h, cudaGetLastError());
     FNO_GEMM(h, fno::layer_forward(sh, h->VbT[l], h->prmb + h->o.W[l], P + h->o.w[l], h->Gb, h->FxiTb, l == L - 1,
                                    h->Z[l], h->Vb[l + 1], h->VbT[l + 1], h->gerr, st));
@@ -1013,10 +1059,10 @@ int backward_fused(fno_handle *h, const float *target, double *loss) {
     sum_fields_kernel<<<(C * C + 31) / 32, kThreads, 0, st>>>(h->wpart, parts, C * C, g + o.W[l]);
     // spectral path: dG = dz Fxi^T, the adjoints of the mixing and of the y-transforms
     FNO_GEMM(h, tcg(h, h->dZb, nx, 0, h->Fxib, nx, 0, h->dG, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 1, 0.f));
-    ydft_kernel<<<B * C, kThreads, ydft_smem(mx, my), st>>>(h->dG, h->Ty, ny, mx, my, h->dY);
+    ydft(h, h->dG, B * C, ny, h->dY);
     mix_back_kernel<<<my * mx, kThreads, mix_smem(B, C, true), st>>>(h->dY, h->Sh[l], P + o.Rr[l], P + o.Ri[l], B, C,
                                                                        my * mx, h->dS, g + o.Rr[l], g + o.Ri[l]);
-    iy_kernel<<<B * C, kThreads, iy_smem(mx, my), st>>>(h->dS, h->Ty, ny, mx, my, nullptr, h->dAb);
+    iy_kernel<<<iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st>>>(h->dS, h->Ty, ny, mx, my, nullptr, h->dAb);
     FNO_CUDA(h, cudaGetLastError());
     // everything per site: dv, through the activation below (in place: a tile
     // reads and writes its own sites)
@@ -1041,9 +1087,8 @@ int fno_create(const fno_config *cfg, fno_handle **out) {
   if (c.width < 1 || c.hidden < 1 || c.layers < 1 || c.layers > kMaxLayers || c.modes_x < 1 || c.modes_y < 2 ||
       c.modes_y % 2 != 0 || c.batch_max < 1 || c.nx_max < 2 || c.ny_max < 2 || 2 * c.modes_x > c.nx_max ||
       c.modes_y > c.ny_max || c.outputs < 1 || c.outputs > kMaxOutputs ||
-      c.modes_x * c.modes_y > 2 * kThreads ||  // ydft_kernel: two modes per thread
-      std::max(ydft_smem(c.modes_x, c.modes_y), std::max(iy_smem(c.modes_x, c.modes_y),
-                                                            mix_smem(c.batch_max, c.width, true))) > 48 * 1024)
+      c.modes_x * c.modes_y > 2 * kThreads || c.modes_x + c.modes_y > 96 ||
+      std::max(iy_smem(c.modes_x, c.modes_y), mix_smem(c.batch_max, c.width, true)) > 48 * 1024)
     return ffail(nullptr, LB_ERR_ARG, "fno_create: bad sizes");
   if (c.gemm_bf16 && (c.width % 8 || c.hidden % 8 || (2 * c.modes_x) % 8))
     return ffail(nullptr, LB_ERR_ARG, "fno_create: BF16 tensor-core products need width, hidden and 2 modes_x "
@@ -1135,10 +1180,10 @@ int fno_forward(fno_handle *h, int32_t B, int32_t nx, int32_t ny, const float *p
     else
       FNO_GEMM(h, sg(h, h->V[l], nx, 1, 0, h->Fx, 2 * mx, 1, 0, h->A, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 0.f));
     // y-transform, per-mode mixing (into the dY scratch), inverse y-transform
-    ydft_kernel<<<B * C, kThreads, ydft_smem(mx, my), st>>>(h->A, h->Ty, ny, mx, my, h->Sh[l]);
+    ydft(h, h->A, B * C, ny, h->Sh[l]);
     mix_kernel<<<my * mx, kThreads, mix_smem(B, C, false), st>>>(h->Sh[l], P + h->o.Rr[l], P + h->o.Ri[l], B, C,
                                                                    my * mx, h->dY);
-    iy_kernel<<<B * C, kThreads, iy_smem(mx, my), st>>>(h->dY, h->Ty, ny, mx, my, h->G, h->Gb);
+    iy_kernel<<<iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st>>>(h->dY, h->Ty, ny, mx, my, h->G, h->Gb);
     FNO_CUDA(h, cudaGetLastError());
     // inverse x-transform into z: Z[R, nx] = G[R, 2mx] Fxi[2mx, nx]
     if (bf)
@@ -1231,10 +1276,10 @@ int fno_backward(fno_handle *h, const float *target, double *loss) {
       FNO_GEMM(h, sg(h, h->dZ, nx, 1, 0, h->Fxi, 1, nx, 0, h->dG, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 0.f));
     // adjoints: of the inverse y-transform (a y-transform), of the mixing
     // (with the weights' gradient), of the y-transform (an inverse one)
-    ydft_kernel<<<B * C, kThreads, ydft_smem(mx, my), st>>>(h->dG, h->Ty, ny, mx, my, h->dY);
+    ydft(h, h->dG, B * C, ny, h->dY);
     mix_back_kernel<<<my * mx, kThreads, mix_smem(B, C, true), st>>>(h->dY, h->Sh[l], P + o.Rr[l], P + o.Ri[l], B, C,
                                                                        my * mx, h->dS, g + o.Rr[l], g + o.Ri[l]);
-    iy_kernel<<<B * C, kThreads, iy_smem(mx, my), st>>>(h->dS, h->Ty, ny, mx, my, h->dA, h->dAb);
+    iy_kernel<<<iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st>>>(h->dS, h->Ty, ny, mx, my, h->dA, h->dAb);
     FNO_CUDA(h, cudaGetLastError());
     // dv = W^T dz (pointwise path) + dA Fx^T (spectral path)
     if (bf) {
@@ -1264,8 +1309,10 @@ int fno_fields(fno_handle *h, const float *out, int32_t batch, int32_t nx, int32
   // same stream orders their uses)
   const int nblk = (int)std::max<long long>(1, std::min<long long>({256, 8192 / batch, (S + kThreads - 1) / kThreads}));
   field_mass_kernel<<<dim3(nblk, batch), kThreads, 0, h->st>>>(out, h->c.outputs, S, scales[0], h->partial);
-  fields_kernel<<<dim3(nblk, batch), kThreads, 0, h->st>>>(out, h->c.outputs, S, scales[0], scales[1], scales[2],
-                                                           rho_mean, h->partial, nblk, fields);
+  shift_kernel<<<batch, kThreads, 0, h->st>>>(h->partial, nblk, S, rho_mean);
+  const unsigned fblk = (unsigned)std::min<long long>((S + kThreads - 1) / kThreads, std::max(1, 8192 / batch));
+  fields_kernel<<<dim3(fblk, batch), kThreads, 0, h->st>>>(out, h->c.outputs, S, scales[0], scales[1], scales[2],
+                                                           h->partial, nblk, fields);
   FNO_CUDA(h, cudaGetLastError());
   return LB_OK;
 }

@@ -23,8 +23,8 @@
 // (each product in its own accumulator, then added, then the bias), so a
 // layer's values are the same bits.  Bound by the activations (normcdff) and
 // by memory about equally.  Measured: training step of 16 fields of 256 x 64
-// 1.61 -> STEP16 ms, of 8 fields of 512 x 128 2.75 -> STEP8 ms; forward pass of
-// a 2048 x 512 field 1.83 -> FWD ms.
+// 1.61 -> 1.07 ms, of 8 fields of 512 x 128 2.74 -> 1.65 ms; warm start of a
+// 2048 x 512 lattice (forward pass, fields, initial state) 2.36 -> 0.90 ms.
 #include "fno_fused.h"
 
 #include <algorithm>
@@ -142,8 +142,9 @@ __device__ __forceinline__ void put_bf16(const float (&v)[8], bool valid, __nv_b
 }
 
 // x, as a value of its own to the compiler: gelu and gelu' of the same z are
-// then contracted as they are in the kernels that evaluate one of them (a
-// shared normcdff result changes the last bit of gelu').
+// then contracted as they are in the kernels that evaluate one of them (with a
+// shared normcdff result, or Phi recovered from gelu', the last bit of gelu'
+// changes, and with it BF16 roundings of the whole backward pass).
 __device__ __forceinline__ float opaque(float x) {
   asm volatile("" : "+f"(x));
   return x;

@@ -7,9 +7,8 @@ namespace fno {
 
 // gelu(z) = z Phi(z), Phi the standard normal distribution function.
 __device__ __forceinline__ float gelu(float z) { return z * normcdff(z); }
-__device__ __forceinline__ float gelu_grad(float z, float phi) {
-  return phi + z * (0.3989422804014327f * expf(-0.5f * z * z));
+__device__ __forceinline__ float gelu_grad(float z) {
+  return normcdff(z) + z * (0.3989422804014327f * expf(-0.5f * z * z));
 }
-__device__ __forceinline__ float gelu_grad(float z) { return gelu_grad(z, normcdff(z)); }
 
 }  // namespace fno
