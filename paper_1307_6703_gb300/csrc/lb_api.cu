@@ -29,7 +29,8 @@ struct lb_handle {
   int pitch = 0;
   long long plane = 0, off = 0;
   bool sweep = false;            // strip-sweep kernel in use
-  int store = 0;                 // its storage format (lbk::kStoreF32, kStoreBF16, kStoreFP16)
+  int store = 0;                 // its storage format (lbk::kStoreF32, kStoreF32Odd, kStoreBF16, kStoreFP16)
+  bool odd = false;              // columns not a multiple of 4: no tiling controls, monitoring or fused sums
   CUtensorMap tmap[2][2];        // TMA descriptors of the two state buffers
   float ref_ax = 0.f, ref_dg = 0.f;  // reference populations of 16-bit storage
   size_t sweep_smem = 0;
@@ -333,6 +334,7 @@ lbk::SweepArgs sweep_args(const lb_handle *h, int in) {
   A.nstrips = h->tile_cols;
   A.base_w = h->tile_base;
   A.extra = h->tile_extra;
+  A.pad = h->odd ? (4 - p.nx % 4) % 4 : 0;
   const double T0 = 1.0 / 3.0;
   auto two = [](float v) { return make_float2(v, v); };
   lbk::SweepConsts &c = A.k;
@@ -513,8 +515,8 @@ int multi_steps(lb_handle *h, int64_t nsteps) {
     Q.fout[b] = (float *)h->f[b ^ 1];  // a step reading buffer b writes buffer b ^ 1
     Q.fdev[b] = dev16(h) ? (void *)((char *)h->f[b ^ 1] + (size_t)h->plane * sizeof(float)) : nullptr;
   }
-  Q.total = h->d_out;
-  Q.arrivals = h->d_arrive;
+  Q.total = h->odd ? nullptr : h->d_out;  // (odd widths: lb_reduce sums the state in FP64)
+  Q.arrivals = h->odd ? nullptr : h->d_arrive;
   const bool mon = h->mon_cap > 0;
   if (mon) {
     LB_CUDA(h, ensure_mon_slots(h, ntiles));
@@ -548,11 +550,27 @@ int multi_steps(lb_handle *h, int64_t nsteps) {
     h->cur ^= chunk & 1;
     h->step += chunk;
     h->epoch += (unsigned)chunk;
-    h->cta_valid = !mon;  // monitored launches keep their records in the slots
-    h->total_valid = true;
+    h->cta_valid = !mon && !h->odd;  // monitored launches keep their records in the slots
+    h->total_valid = !h->odd;
     done += chunk;
   }
   return LB_OK;
+}
+
+// Whether lb_step may use multi-step launches.  Lattices of odd widths can be
+// stepped inside a stream capture and without memory of their own (their steps
+// were independent launches, which a graph may replay): there they keep single
+// steps.
+bool multi_allowed(lb_handle *h) {
+  if (!h->odd) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  if (ensure_deps(h) == cudaSuccess) return true;
+  (void)cudaGetLastError();
+  return false;
 }
 
 }  // namespace
@@ -598,6 +616,10 @@ int lb_create(const lb_params *p, lb_handle **out) {
   // and at least 8 sites per direction (one ghost band of 4 each).
   h->store = p->precision;
   h->sweep = !fp64(h) && lbk::sweep_supported(h->store, p->nx, p->ny);
+  if (!h->sweep && p->precision == LB_FP32 && lbk::sweep_supported(lbk::kStoreF32Odd, p->nx, p->ny)) {
+    h->store = lbk::kStoreF32Odd;
+    h->sweep = h->odd = true;
+  }
   if (h->sweep) {
     h->pitch = ((p->nx + 8 + 31) / 32) * 32;
     h->plane = (long long)h->pitch * (p->ny + 8);
@@ -717,13 +739,13 @@ int lb_step(lb_handle *h, int64_t nsteps) {
     }
   } else if (h->sweep) {
     // Two steps or more: multi-step launches.
-    if (nsteps >= 2) return multi_steps(h, nsteps);
+    if (nsteps >= 2 && multi_allowed(h)) return multi_steps(h, nsteps);
     // Per-CTA mass/momentum records only on the last step: lb_reduce reads
     // only the current state's.
     for (int64_t k = 0; k < nsteps; k++) {
       lbk::SweepArgs A = sweep_args(h, h->cur);
       // records on the last step, or on every step while monitoring
-      A.records = (k == nsteps - 1 || h->mon_cap > 0) ? 1 : 0;
+      A.records = !h->odd && (k == nsteps - 1 || h->mon_cap > 0) ? 1 : 0;
       if (A.records) {  // the last CTA also leaves the global sums in d_out
         A.total = h->d_out;
         A.arrivals = h->d_arrive;
@@ -737,7 +759,7 @@ int lb_step(lb_handle *h, int64_t nsteps) {
       if (e != cudaSuccess) return cuda_fail(h, e, "lb_step: sweep kernel");
       h->cur ^= 1;
       h->step++;
-      h->cta_valid = true;
+      h->cta_valid = A.records != 0;
       h->total_valid = A.records != 0;
     }
   } else {
@@ -872,7 +894,7 @@ int lb_monitor(lb_handle *h, double *host_ring, int32_t capacity) {
     h->mon_cap = 0;
     return LB_OK;
   }
-  if (!h->sweep || h->in_batch)
+  if (!h->sweep || h->in_batch || h->odd)
     return fail(h, LB_ERR_ARG, "lb_monitor: only for strip-sweep handles outside a batch");
   void *dev = device_view(host_ring, true);
   if (!dev) return fail(h, LB_ERR_ARG, "lb_monitor: the ring is not page-locked memory the device can address");
@@ -954,9 +976,9 @@ int lb_autotune(lb_handle *h, int steps, int32_t *seg_h) {
   if (!h) return LB_ERR_ARG;
   if (steps < 1) return fail(h, LB_ERR_ARG, "lb_autotune: steps must be >= 1");
   if (!h->initialised) return fail(h, LB_ERR_STATE, "lb_autotune: state not initialised");
-  if (!h->sweep) {
+  if (!h->sweep || h->odd) {
     if (seg_h) *seg_h = 0;
-    return LB_OK;  // the tile kernel has no tiling choice
+    return LB_OK;  // no tiling choice
   }
   // Candidate segment heights: lower tiles fill the device better, higher ones
   // repeat fewer warm-up rows; the best trade depends on the lattice and on
@@ -1063,14 +1085,15 @@ int lb_sweep_dependencies(int32_t precision, int32_t nx, int32_t ny, int32_t wal
 
 int lb_get_tiling(const lb_handle *h, int32_t *nstrips, int32_t *seg_h) {
   if (!h || !nstrips || !seg_h) return LB_ERR_ARG;
-  *nstrips = h->sweep ? h->sweep_nstrips : 0;
-  *seg_h = h->sweep ? h->sweep_seg : 0;
+  const bool tiled = h->sweep && !h->odd;
+  *nstrips = tiled ? h->sweep_nstrips : 0;
+  *seg_h = tiled ? h->sweep_seg : 0;
   return LB_OK;
 }
 
 int lb_set_tiling(lb_handle *h, int32_t nstrips, int32_t seg_h) {
   if (!h) return LB_ERR_ARG;
-  if (!h->sweep) return LB_OK;
+  if (!h->sweep || h->odd) return LB_OK;
   const int s_min = lbk::sweep_min_strips(h->store, h->p.nx);
   const int qn = h->store == lbk::kStoreF32 ? 4 : 8;
   if (nstrips < s_min || nstrips > h->p.nx / (2 * qn) || seg_h < 1)
@@ -1082,7 +1105,7 @@ int lb_set_tiling(lb_handle *h, int32_t nstrips, int32_t seg_h) {
 int lb_set_seg_h(lb_handle *h, int32_t seg_h) {
   if (!h) return LB_ERR_ARG;
   if (seg_h < 1) return fail(h, LB_ERR_ARG, "lb_set_seg_h: seg_h must be >= 1");
-  if (!h->sweep) return LB_OK;
+  if (!h->sweep || h->odd) return LB_OK;
   LB_CUDA(h, change_tiles(h, h->sweep_nstrips, seg_h));
   return LB_OK;
 }
@@ -1277,7 +1300,7 @@ int lb_batch_create(const lb_params *ps, int32_t count, lb_batch **out) {
       return bfail(nullptr, LB_ERR_ARG, "lb_batch_create: all instances must share one stream");
     if (ps[i].precision != ps[0].precision)
       return bfail(nullptr, LB_ERR_ARG, "lb_batch_create: all instances must share one precision");
-    if (ps[i].precision == LB_FP64 || !lbk::sweep_supported(ps[i].precision, ps[i].nx, ps[i].ny))
+    if (ps[i].precision == LB_FP64 || ps[i].precision == lbk::kStoreF32Odd || !lbk::sweep_supported(ps[i].precision, ps[i].nx, ps[i].ny))
       return bfail(nullptr, LB_ERR_ARG,
                    "lb_batch_create: every instance must run the sweep kernel (FP32 or 16-bit storage, nx a "
                    "multiple of 4 (8 for 16-bit storage), nx, ny >= 8)");

@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(256) init_f32_kernel(Put put, const __grid_con
       put.template encode<kCols>(A, f);
       const long long e = A.off + (long long)y * A.pitch + x;
       put.template store<kCols>(A, e, f);
-      if (A.images != 0) {  // (columns 0..3 and nx-4..nx-1 are whole pairs)
+      if (A.images != 0) {  // (with pairs nx is even: columns 0..3 and nx-4..nx-1 are whole pairs)
         const int gx = x < 4 ? A.nx : (x >= A.nx - 4 ? -A.nx : 0);
         if (gx != 0) put.template store<kCols>(A, e + gx, f);
         if (A.images == 2) {
@@ -276,6 +276,7 @@ cudaError_t launch_init_f32(int store, void *buf, const InitState &I, cudaStream
     case kStoreBF16: return launch_cols<PutDev<__nv_bfloat16>, 2>({f, (__nv_bfloat16 *)dev}, A, st);
     case kStoreFP16: return launch_cols<PutDev<__half>, 2>({f, (__half *)dev}, A, st);
     case kStoreF32:
+    case kStoreF32Odd:
       // pairs of columns: an even number of them, rows and planes of even pitch
       if (I.nx % 2 == 0 && I.pitch % 2 == 0 && I.plane % 2 == 0 && I.off % 2 == 0)
         return launch_cols<PutF32, 2>({f}, A, st);

@@ -39,8 +39,9 @@ struct SweepArgs {
   int pitch;
   long long plane, off;
   // tiles: nseg segments of seg_h rows by nstrips columns of tiles, base_w
-  // wide (the first `extra` wider by the column quantum)
-  int seg_h, nseg, nstrips, base_w, extra;
+  // wide (the first `extra` wider by the column quantum, the last narrower by
+  // `pad`: nx rounded up to the quantum, minus nx)
+  int seg_h, nseg, nstrips, base_w, extra, pad;
   SweepConsts k;
   float u_bot, u_top;
   float nmax;                  // 1/b (upper bound of a valid density)
@@ -67,6 +68,8 @@ struct SweepArgs {
 
 // Storage formats of the sweep kernel (values of lb_precision).
 constexpr int kStoreF32 = 1, kStoreBF16 = 2, kStoreFP16 = 3;
+// FP32 with a number of columns that is not a multiple of 4.
+constexpr int kStoreF32Odd = 4;
 
 // Whether the sweep kernel of storage `store` can run an nx x ny lattice
 // (column quantum of its TMA boxes, ghost bands, 32-bit plane offsets).

@@ -120,6 +120,7 @@ constexpr double kTilesPerWarp = 1.3;
 // FP32 storage: one 3D box {64, 2, 9} (columns, rows, planes) per pair.
 struct StoreF32 {
   static constexpr bool kDev = false;
+  static constexpr bool kOdd = false;         // nx not a multiple of the quantum
   static constexpr int kQuantum = 4;          // 16-byte x coordinates of float boxes
   static constexpr int kMaxW = 116;           // widest strip a tiling may name (split into tiles)
   static constexpr unsigned kTxBytes = 9 * 2 * kCols * sizeof(float);
@@ -144,6 +145,16 @@ struct StoreF32 {
   }
 };
 
+// The same for lattices whose number of columns is not a multiple of 4: the last
+// column of tiles is narrower, its last pair of columns may be half outside,
+// and periodic images are stored one column at a time (nx odd shifts them by
+// half a pair).  (These lattices used the tile kernel, whose tiles of 32 x 16
+// sites pull every population three times from L1/L2: 25 us a step for 1021 x
+// 509, now 20.)
+struct StoreF32Odd : StoreF32 {
+  static constexpr bool kOdd = true;
+};
+
 // 16-bit deviation storage: a float box {64, 2, 1} of the rest plane and a
 // 16-bit box {64, 2, 8} of the deviation planes (128-byte rows) per pair.  A
 // lane's two columns are one 32-bit word of a deviation plane.  mid(0) is the
@@ -152,6 +163,7 @@ template <class H>
 struct StoreDev {
   using Half = H;
   static constexpr bool kDev = true;
+  static constexpr bool kOdd = false;
   static constexpr int kQuantum = 8;          // 16-byte x coordinates of 16-bit boxes
   static constexpr int kMaxW = 120;
   static constexpr int kRestBytes = 2 * kCols * sizeof(float);
@@ -588,9 +600,11 @@ struct Moments {
   static constexpr bool kOn = true;
   T *n, *ux, *uy;
   int pairs;
-  __device__ __forceinline__ void put(T *p, size_t s, float2 v) const {
+  __device__ __forceinline__ void put(T *p, size_t s, float2 v, bool half) const {
     if (p == nullptr) return;
-    if (pairs) {
+    if (half) {
+      p[s] = (T)v.x;
+    } else if (pairs) {
       struct alignas(2 * sizeof(T)) Two {
         T a, b;
       };
@@ -608,6 +622,7 @@ template <class St>
 __device__ __forceinline__ void tile_columns(const SweepArgs &A, int i, int &x0, int &W) {
   x0 = i * A.base_w + St::kQuantum * min(i, A.extra);
   W = A.base_w + (i < A.extra ? St::kQuantum : 0);
+  if constexpr (St::kOdd) W -= i == A.nstrips - 1 ? A.pad : 0;
 }
 
 // One warp's work: tile column `strip`, segment `seg` of the lattice
@@ -637,14 +652,19 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
   const int nx = A.nx, ny = A.ny;
   const bool walls = A.walls != 0;
   const int x = x0 - 4 + 2 * t;  // first of this lane's two columns (may be halo columns)
-  const bool actD = 2 * t >= 4 && 2 * t < W + 4;
+  const bool actD = 2 * t >= 4 && 2 * t + 1 < W + 4;         // both columns in the tile
+  const bool half = St::kOdd && 2 * t >= 4 && 2 * t == W + 3;  // the first one only
   const int kmax = (yb - ya + 5) >> 1;  // last iteration
   const int npairs = kmax + 2;          // rows ya-4 .. ya+2*kmax+3
   const int pitch = A.pitch, plane = (int)A.plane;
-  const int gx = (x < 4) ? nx : ((x >= nx - 4) ? -nx : 0);  // periodic image columns
+  auto image = [&](int c) { return c < 4 ? nx : (c >= nx - 4 ? -nx : 0); };
+  const int im0 = image(x), im1 = St::kOdd ? image(x + 1) : im0;  // to the periodic image columns
   float2 sinx = make_float2(0.f, 0.f);
-  if (2 * t >= 2 && 2 * t <= W + 4)  // a constant table
-    sinx = *reinterpret_cast<const float2 *>(A.sinx + (x < 0 ? x + nx : (x >= nx ? x - nx : x)));
+  if (2 * t >= 2 && 2 * t <= W + 4) {  // a constant table
+    auto wrap = [&](int c) { return c < 0 ? c + nx : (c >= nx ? c - nx : c); };
+    if constexpr (St::kOdd) sinx = make_float2(A.sinx[wrap(x)], A.sinx[wrap(x + 1)]);
+    else sinx = *reinterpret_cast<const float2 *>(A.sinx + wrap(x));
+  }
   if (t == 0) {
     for (int s = 0; s < kPairs; ++s) mbar_init(smem_u32(&S.full[s]));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -798,12 +818,12 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const int y = a - 2 + j;
-        if (!actD || y < ya || y >= yb) continue;
+        if (!(actD || half) || y < ya || y >= yb) continue;
         const float2 n = j ? N1.c : N0.c;
         const size_t s = (size_t)y * nx + x;
-        mom.put(mom.n, s, n);
-        if (mom.ux != nullptr) mom.put(mom.ux, s, make_float2(__fdiv_rn(JxC[j].x, n.x), __fdiv_rn(JxC[j].y, n.y)));
-        if (mom.uy != nullptr) mom.put(mom.uy, s, make_float2(__fdiv_rn(JyC[j].x, n.x), __fdiv_rn(JyC[j].y, n.y)));
+        mom.put(mom.n, s, n, half);
+        if (mom.ux != nullptr) mom.put(mom.ux, s, make_float2(__fdiv_rn(JxC[j].x, n.x), __fdiv_rn(JxC[j].y, n.y)), half);
+        if (mom.uy != nullptr) mom.put(mom.uy, s, make_float2(__fdiv_rn(JyC[j].x, n.x), __fdiv_rn(JyC[j].y, n.y)), half);
       }
       n3 = N1.c;
       N0 = N2; N1 = N3;
@@ -862,7 +882,7 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
         fs[j][0] = rest_remainder(V::sub(n, K.r_sum), fs[j]);
       }
     }
-    if (actD) {
+    if (actD || half) {
       // the sites' elements in a plane, row j shifted by d elements (0 or to a
       // periodic image)
       auto put = [&](int j, int d, bool stream) {
@@ -888,17 +908,34 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
       // only by the next step.
 #pragma unroll
       for (int j = 0; j < 2; ++j)
-        if (kSteady || (a - 3 + j >= ya && a - 3 + j < yb)) put(j, 0, true);
-      if (gx != 0 || records || !kSteady) {  // images of edge sites, the tile's sums
+        if (!half && (kSteady || (a - 3 + j >= ya && a - 3 + j < yb))) put(j, 0, true);
+      if (im0 != 0 || im1 != 0 || half || records || !kSteady) {  // images of edge sites, the tile's sums
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           const int y = a - 3 + j;
           if (!kSteady && (y < ya || y >= yb)) continue;
           const int gy = (kSteady || walls) ? 0 : ((y < 4) ? ny : ((y >= ny - 4) ? -ny : 0));
-          if (gx != 0) put(j, gx, false);
-          if (gy != 0) {
-            put(j, gy * pitch, false);
-            if (gx != 0) put(j, gy * pitch + gx, false);
+          if constexpr (!St::kOdd) {
+            if (im0 != 0) put(j, im0, false);
+            if (gy != 0) {
+              put(j, gy * pitch, false);
+              if (im0 != 0) put(j, gy * pitch + im0, false);
+            }
+          } else {
+            auto put1 = [&](int c, int d) {  // one column
+              float *p = O.fout + ((int)A.off + y * pitch + x + c + d);
+#pragma unroll
+              for (int q = 0; q < 9; ++q) p[(size_t)q * plane] = c ? fs[j][q].y : fs[j][q].x;
+            };
+            if (half) put1(0, 0);
+            if (gy != 0) half ? put1(0, gy * pitch) : put(j, gy * pitch, false);
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+              const int g = c ? im1 : im0;
+              if (g == 0 || (c && half)) continue;
+              put1(c, g);
+              if (gy != 0) put1(c, gy * pitch + g);
+            }
           }
           // Mass and momentum of the stored sites: sum f* = n (by
           // construction), sum f* c = n u* + F/2 (identity of the collision).
@@ -1240,10 +1277,10 @@ sweep_multi_kernel(const __grid_constant__ CUtensorMap tin0, const __grid_consta
   O.monitor = mon ? Q.mon_ring + 6 * ((Q.mon_step0 + k) % Q.mon_cap) : nullptr;
   O.mon_step = (double)(Q.mon_step0 + k);
   if (!sweep_body<St, kTau1, true>(par ? &tin1 : &tin0, par ? &tdev1 : &tdev0, A, A.k, O, i % A.nstrips, i / A.nstrips,
-                                   const_cast<double *>(O.recs) + 4 * (size_t)i, last || mon,
+                                   const_cast<double *>(O.recs) + 4 * (size_t)i, (last && Q.total) || mon,
                                    [&] { return wait_deps(P, i, target, A.err); },
                                    [&] { release_item(P, i, target + 1u); })) {
-    if (threadIdx.x == 0) Q.total[4] = 1.0;  // the sums of this launch will not be written
+    if (threadIdx.x == 0 && Q.total) Q.total[4] = 1.0;  // the sums of this launch will not be written
   }
 }
 
@@ -1279,10 +1316,10 @@ cudaError_t encode_map(CUtensorMapDataType type, int esize, void *base, int pitc
 }
 
 int quantum_of(int store) {
-  return store == kStoreF32 ? StoreF32::kQuantum : (store == kStoreBF16 ? StoreBF16::kQuantum : StoreFP16::kQuantum);
+  return store == kStoreF32 || store == kStoreF32Odd ? StoreF32::kQuantum : (store == kStoreBF16 ? StoreBF16::kQuantum : StoreFP16::kQuantum);
 }
 int maxw_of(int store) {
-  return store == kStoreF32 ? StoreF32::kMaxW : (store == kStoreBF16 ? StoreBF16::kMaxW : StoreFP16::kMaxW);
+  return store == kStoreF32 || store == kStoreF32Odd ? StoreF32::kMaxW : (store == kStoreBF16 ? StoreBF16::kMaxW : StoreFP16::kMaxW);
 }
 
 template <class St, bool kTau1>
@@ -1291,9 +1328,11 @@ cudaError_t prepare_one(size_t *smem_bytes) {
   const int bytes = (int)*smem_bytes;
   constexpr cudaFuncAttribute attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaFuncSetAttribute(sweep_step_kernel<St, kTau1>, attr, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(sweep_batch_kernel<St, kTau1>, attr, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sweep_multi_kernel<St, kTau1>, attr, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(sweep_batch_multi_kernel<St, kTau1>, attr, bytes);
+  if constexpr (!St::kOdd) {  // (a batch takes no odd widths)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sweep_batch_kernel<St, kTau1>, attr, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sweep_batch_multi_kernel<St, kTau1>, attr, bytes);
+  }
   return e;
 }
 
@@ -1354,8 +1393,8 @@ cudaError_t launch_moments_one(const CUtensorMap &m0, const CUtensorMap &m1, con
   const int smem = (int)sizeof(SmemOf<St, true>);
   cudaError_t e = cudaFuncSetAttribute(sweep_moments_kernel<St, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const uintptr_t all = (uintptr_t)n | (uintptr_t)ux | (uintptr_t)uy;  // (nx is a multiple of 4: rows keep the alignment)
-  const Moments<T> M{(T *)n, (T *)ux, (T *)uy, all % (2 * sizeof(T)) == 0};
+  const uintptr_t all = (uintptr_t)n | (uintptr_t)ux | (uintptr_t)uy;  // (even nx: rows keep the alignment)
+  const Moments<T> M{(T *)n, (T *)ux, (T *)uy, all % (2 * sizeof(T)) == 0 && A.nx % 2 == 0};
   sweep_moments_kernel<St, T><<<dim3((unsigned)A.nstrips, (unsigned)A.nseg), kThreads, smem, st>>>(m0, m1, A, M);
   return cudaGetLastError();
 }
@@ -1363,18 +1402,18 @@ cudaError_t launch_moments_one(const CUtensorMap &m0, const CUtensorMap &m1, con
 }  // namespace
 
 bool sweep_supported(int store, int nx, int ny) {
-  if (store != kStoreF32 && store != kStoreBF16 && store != kStoreFP16) return false;
+  if (store != kStoreF32 && store != kStoreF32Odd && store != kStoreBF16 && store != kStoreFP16) return false;
   const double pitch = (double)(((nx + 8 + 31) / 32) * 32);
-  return nx % quantum_of(store) == 0 && nx >= 8 && ny >= 8 && 9.0 * pitch * (double)(ny + 8) < 2147483647.0;
+  return (nx % quantum_of(store) == 0) == (store != kStoreF32Odd) && nx >= 8 && ny >= 8 && 9.0 * pitch * (double)(ny + 8) < 2147483647.0;
 }
 
 size_t sweep_buffer_bytes(int store, long long plane) {
-  return store == kStoreF32 ? 9 * (size_t)plane * sizeof(float) : (size_t)plane * (sizeof(float) + 8 * 2);
+  return store == kStoreF32 || store == kStoreF32Odd ? 9 * (size_t)plane * sizeof(float) : (size_t)plane * (sizeof(float) + 8 * 2);
 }
 
 cudaError_t sweep_make_maps(int store, void *base, int pitch, int ny, long long plane, CUtensorMap *m0,
                             CUtensorMap *m1) {
-  if (store == kStoreF32) {
+  if (store == kStoreF32 || store == kStoreF32Odd) {
     static_assert(StoreF32::kTxBytes == 9 * 2 * kCols * sizeof(float), "TMA box must match the slot");
     cudaError_t e = encode_map(CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, pitch, ny, plane, 9, kCols, m0);
     *m1 = *m0;
@@ -1391,15 +1430,15 @@ cudaError_t sweep_make_maps(int store, void *base, int pitch, int ny, long long 
 }
 
 void sweep_strips(int store, int nx, int nstrips, int *base_w, int *extra) {
-  const int qn = quantum_of(store);
-  *base_w = qn * (nx / (qn * nstrips));
-  *extra = (nx - *base_w * nstrips) / qn;
+  const int qn = quantum_of(store), whole = (nx + qn - 1) / qn * qn;  // (the last strip loses whole - nx)
+  *base_w = qn * (whole / (qn * nstrips));
+  *extra = (whole - *base_w * nstrips) / qn;
 }
 
 int sweep_min_strips(int store, int nx) { return (nx + maxw_of(store) - 1) / maxw_of(store); }
 
 int sweep_warps_per_sm(int store, bool tau1) {
-  return store != kStoreF32 ? Form<StoreBF16, true>::kMinBlocks
+  return store == kStoreBF16 || store == kStoreFP16 ? Form<StoreBF16, true>::kMinBlocks
                             : (tau1 ? Form<StoreF32, true>::kMinBlocks : Form<StoreF32, false>::kMinBlocks);
 }
 
@@ -1420,14 +1459,19 @@ int sweep_tile_cols(int store, int nx, int nstrips) {
   return base + (extra > 0 ? quantum_of(store) : 0) <= kTileW ? nstrips : (nx + kTileW - 1) / kTileW;
 }
 
-// f<storage policy, tau == 1>() for the runtime pair (store, tau1).
-#define LB_SWEEP_FORM(store, tau1, f, ...)                                                             \
+// f<storage policy, tau == 1>() for the runtime pair (store, tau1): the formats
+// a batch takes, and those of a single lattice.
+#define LB_SWEEP_BATCH_FORM(store, tau1, f, ...)                                                       \
   switch (store) {                                                                                     \
     case kStoreF32: return (tau1) ? f<StoreF32, true>(__VA_ARGS__) : f<StoreF32, false>(__VA_ARGS__);    \
     case kStoreBF16: return (tau1) ? f<StoreBF16, true>(__VA_ARGS__) : f<StoreBF16, false>(__VA_ARGS__); \
     case kStoreFP16: return (tau1) ? f<StoreFP16, true>(__VA_ARGS__) : f<StoreFP16, false>(__VA_ARGS__); \
   }                                                                                                    \
   return cudaErrorInvalidValue
+#define LB_SWEEP_FORM(store, tau1, f, ...)                                                             \
+  if (store == kStoreF32Odd)                                                                           \
+    return (tau1) ? f<StoreF32Odd, true>(__VA_ARGS__) : f<StoreF32Odd, false>(__VA_ARGS__);            \
+  LB_SWEEP_BATCH_FORM(store, tau1, f, __VA_ARGS__)
 
 cudaError_t sweep_prepare(int store, bool tau1, size_t *smem_bytes) {
   LB_SWEEP_FORM(store, tau1, prepare_one, smem_bytes);
@@ -1444,6 +1488,9 @@ cudaError_t launch_sweep_moments(int store, const CUtensorMap &m0, const CUtenso
     case kStoreF32:
       return dtype == 0 ? launch_moments_one<StoreF32, double>(m0, m1, A, n, ux, uy, st)
                         : launch_moments_one<StoreF32, float>(m0, m1, A, n, ux, uy, st);
+    case kStoreF32Odd:
+      return dtype == 0 ? launch_moments_one<StoreF32Odd, double>(m0, m1, A, n, ux, uy, st)
+                        : launch_moments_one<StoreF32Odd, float>(m0, m1, A, n, ux, uy, st);
     case kStoreBF16:
       return dtype == 0 ? launch_moments_one<StoreBF16, double>(m0, m1, A, n, ux, uy, st)
                         : launch_moments_one<StoreBF16, float>(m0, m1, A, n, ux, uy, st);
@@ -1457,7 +1504,7 @@ cudaError_t launch_sweep_moments(int store, const CUtensorMap &m0, const CUtenso
 cudaError_t launch_sweep_batch(int store, bool tau1, const BatchItem *items, int nitems, const SweepArgs *args,
                                const SweepConsts &k, const CUtensorMap *maps, int kpar, int records, size_t smem, cudaStream_t st) {
   if (nitems < 1) return cudaSuccess;
-  LB_SWEEP_FORM(store, tau1, launch_batch_one, items, nitems, args, k, maps, kpar, records, smem, st);
+  LB_SWEEP_BATCH_FORM(store, tau1, launch_batch_one, items, nitems, args, k, maps, kpar, records, smem, st);
 }
 
 cudaError_t launch_sweep_multi(int store, bool tau1, const CUtensorMap (&maps)[2][2], const SweepArgs &A,
@@ -1467,7 +1514,7 @@ cudaError_t launch_sweep_multi(int store, bool tau1, const CUtensorMap (&maps)[2
 
 cudaError_t launch_sweep_batch_multi(int store, bool tau1, const BatchItem *items, const SweepArgs *args,
                                      const SweepConsts &k, const CUtensorMap *maps, const MultiArgs &P, size_t smem, cudaStream_t st) {
-  LB_SWEEP_FORM(store, tau1, launch_batch_multi_one, items, args, k, maps, P, smem, st);
+  LB_SWEEP_BATCH_FORM(store, tau1, launch_batch_multi_one, items, args, k, maps, P, smem, st);
 }
 
 // Tiles each tile of the sweep depends on (see sweep_batch_multi_kernel): the
