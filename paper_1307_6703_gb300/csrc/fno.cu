@@ -799,6 +799,10 @@ struct fno_handle {
   int tab_nx = 0, tab_ny = 0;
   int B = 0, nx = 0, ny = 0;  // shape of the last forward pass
   bool have_forward = false;
+  // The fused backward pass's weight gradients run on a stream of their own,
+  // forked from and joined to `st` within the call.
+  cudaStream_t side = nullptr;
+  cudaEvent_t ev_dz = nullptr, ev_sums = nullptr, ev_dw[2] = {};
   std::string err;
 };
 
@@ -834,8 +838,9 @@ constexpr int kWSplit = 8;
 // gemm_tc.h for the argument layout.
 cudaError_t tcg(fno_handle *h, const __nv_bfloat16 *X, int ldx, long long sX, const __nv_bfloat16 *Y, int ldy,
                 long long sY, float *C, long long cm, long long cn, long long sC, int M, int N, int K, int batch,
-                int ksplit, float beta) {
-  return tc::gemm_tn_bf16(X, ldx, sX, Y, ldy, sY, C, cm, cn, sC, M, N, K, batch, ksplit, beta, h->gerr, h->st);
+                int ksplit, float beta, bool side = false) {
+  return tc::gemm_tn_bf16(X, ldx, sX, Y, ldy, sY, C, cm, cn, sC, M, N, K, batch, ksplit, beta, h->gerr,
+                          side ? h->side : h->st);
 }
 
 // SIMT product (FP32 mode): C(m, n) = sum_k A(m, k) B(k, n), general strides.
@@ -872,10 +877,10 @@ void site_major(fno_handle *h, const __nv_bfloat16 *in, int B, int rows, long lo
 int reduce_splits(int B, int C) { return std::max(1, std::min(kReduceBlocks, (2048 + C * B - 1) / (C * B))); }
 
 // The channel sums from the float4s' sums quads[b][ch][S / 4].
-void quad_reduce(fno_handle *h, const float *quads, int B, int C, long long S, float *out) {
+void quad_reduce(fno_handle *h, const float *quads, int B, int C, long long S, float *out, cudaStream_t st) {
   const int nsplit = reduce_splits(B, C);
-  reduce_pass1_v4_kernel<true><<<dim3(C, B * nsplit), kThreads, 0, h->st>>>(quads, C, S, nsplit, h->rpart);
-  reduce_pass2_kernel<<<(C + 7) / 8, kThreads, 0, h->st>>>(h->rpart, C, B * nsplit, out);
+  reduce_pass1_v4_kernel<true><<<dim3(C, B * nsplit), kThreads, 0, st>>>(quads, C, S, nsplit, h->rpart);
+  reduce_pass2_kernel<<<(C + 7) / 8, kThreads, 0, st>>>(h->rpart, C, B * nsplit, out);
 }
 
 // out[ch] = sum over (b, s) of a[b, ch, s] for the C channels of a.
@@ -1030,6 +1035,32 @@ int forward_fused(fno_handle *h, int B, int nx, int ny, const float *params_dev,
   return LB_OK;
 }
 
+// Makes the handle's stream wait for its side stream, at the latest when the
+// call returns: nothing is left running beside `st`.
+struct SideJoin {
+  fno_handle *h;
+  bool forked = false;
+  cudaError_t fork() {
+    forked = true;
+    const cudaError_t e = cudaEventRecord(h->ev_dz, h->st);
+    return e == cudaSuccess ? cudaStreamWaitEvent(h->side, h->ev_dz, 0) : e;
+  }
+  cudaError_t now() {
+    forked = false;
+    const cudaError_t e = cudaEventRecord(h->ev_dz, h->side);
+    return e == cudaSuccess ? cudaStreamWaitEvent(h->st, h->ev_dz, 0) : e;
+  }
+  ~SideJoin() {
+    if (forked) (void)now();
+  }
+};
+
+// The weight gradients are products of 32 x 32 with K = all sites: few CTAs,
+// each one chain of dependent MMAs whose order fixes the result (60 us for 8
+// fields of 512 x 128, no unit of the SM above 18 %).  They run beside the
+// spectral path and the layer below: a training step of 8 fields of 512 x 128
+// 1650 -> 1414 us, of 16 fields of 256 x 64 1066 -> 963 us.
+//
 // Backward pass on the fused kernels.
 int backward_fused(fno_handle *h, const float *target, double *loss) {
   const fno_config &c = h->c;
@@ -1042,33 +1073,48 @@ int backward_fused(fno_handle *h, const float *target, double *loss) {
   const Offsets &o = h->o;
   float *g = h->grd;
   cudaStream_t st = h->st;
+  // dz of layer l, channel-major: two buffers in turn, so that dW of a layer may
+  // still read its own while the layer below is done.  The second one is dV,
+  // written when the first layer is, after dW of the second.
+  __nv_bfloat16 *const dz[2] = {h->dZb, reinterpret_cast<__nv_bfloat16 *>(h->dV)};
+  SideJoin join{h};
   FNO_GEMM(h, fno::project_backward(sh, h->VbT[L], h->prmb + o.Q1, P + o.q1, P + o.Q2, h->wTb + (size_t)L * C * C,
-                                    h->out, target, h->dhpb, h->dZb, h->dZT, h->quads, h->fpart, h->gerr, st));
+                                    h->out, target, h->dhpb, dz[(L - 1) & 1], h->dZT, h->quads, h->fpart, h->gerr, st));
   const int nval = fno::project_back_sums(sh);
   FNO_CUDA(h, fno::finish_sums(h->fpart, tiles, nval, {{g + o.q1, H}, {g + o.Q2, O * H}, {g + o.q2, O}}, h->loss,
                                (double)B * O * S, h->fpart + tiles * nval, st));
-  // dQ1 = sum_b dhp[b] v_L[b]^T
-  FNO_GEMM(h, tcg(h, h->dhpb, (int)S, HS, h->Vb[L], (int)S, CS, h->wpart, C, 1, (long long)H * C, H, C, (int)S, B,
-                  kWSplit, 0.f));
-  sum_fields_kernel<<<(H * C + 31) / 32, kThreads, 0, st>>>(h->wpart, parts, H * C, g + o.Q1);
   for (int l = L - 1; l >= 0; l--) {
-    // dw = sum dz, dW = sum_b dz[b] v[b]^T
-    quad_reduce(h, h->quads, B, C, S, g + o.w[l]);
-    FNO_GEMM(h, tcg(h, h->dZb, (int)S, CS, h->Vb[l], (int)S, CS, h->wpart, C, 1, (long long)C * C, C, C, (int)S, B,
-                    kWSplit, 0.f));
-    sum_fields_kernel<<<(C * C + 31) / 32, kThreads, 0, st>>>(h->wpart, parts, C * C, g + o.W[l]);
+    const __nv_bfloat16 *dzl = dz[l & 1];
+    // on the side: dw = sum dz, dW = sum_b dz[b] v[b]^T (and of the projection
+    // dQ1 = sum_b dhp[b] v_L[b]^T)
+    FNO_CUDA(h, join.fork());
+    quad_reduce(h, h->quads, B, C, S, g + o.w[l], h->side);
+    FNO_CUDA(h, cudaEventRecord(h->ev_sums, h->side));
+    FNO_GEMM(h, tcg(h, dzl, (int)S, CS, h->Vb[l], (int)S, CS, h->wpart, C, 1, (long long)C * C, C, C, (int)S, B,
+                    kWSplit, 0.f, true));
+    sum_fields_kernel<<<(C * C + 31) / 32, kThreads, 0, h->side>>>(h->wpart, parts, C * C, g + o.W[l]);
+    FNO_CUDA(h, cudaEventRecord(h->ev_dw[l & 1], h->side));
+    if (l == L - 1) {
+      FNO_GEMM(h, tcg(h, h->dhpb, (int)S, HS, h->Vb[L], (int)S, CS, h->wpart, C, 1, (long long)H * C, H, C, (int)S, B,
+                      kWSplit, 0.f, true));
+      sum_fields_kernel<<<(H * C + 31) / 32, kThreads, 0, h->side>>>(h->wpart, parts, H * C, g + o.Q1);
+    }
     // spectral path: dG = dz Fxi^T, the adjoints of the mixing and of the y-transforms
-    FNO_GEMM(h, tcg(h, h->dZb, nx, 0, h->Fxib, nx, 0, h->dG, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 1, 0.f));
+    FNO_GEMM(h, tcg(h, dzl, nx, 0, h->Fxib, nx, 0, h->dG, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 1, 0.f));
     ydft(h, h->dG, B * C, ny, h->dY);
     mix_back_kernel<<<my * mx, kThreads, mix_smem(B, C, true), st>>>(h->dY, h->Sh[l], P + o.Rr[l], P + o.Ri[l], B, C,
                                                                        my * mx, h->dS, g + o.Rr[l], g + o.Ri[l]);
     iy_kernel<<<iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st>>>(h->dS, h->Ty, ny, mx, my, nullptr, h->dAb);
     FNO_CUDA(h, cudaGetLastError());
-    // everything per site: dv, through the activation below (in place: a tile
-    // reads and writes its own sites)
+    // everything per site: dv, through the activation below (the site-major
+    // copy in place: a tile reads and writes its own sites), when the channel
+    // sums are read and dW of the layer above no longer reads the other buffer
+    FNO_CUDA(h, cudaStreamWaitEvent(st, h->ev_sums, 0));
+    if (l + 1 < L) FNO_CUDA(h, cudaStreamWaitEvent(st, h->ev_dw[(l + 1) & 1], 0));
     FNO_GEMM(h, fno::layer_backward(sh, h->dZT, h->wTb + (size_t)l * C * C, h->dAb, h->Fxb, l > 0 ? h->Z[l - 1] : nullptr,
-                                    h->dZb, h->dZT, h->quads, h->dV, h->gerr, st));
+                                    dz[(l + 1) & 1], h->dZT, h->quads, h->dV, h->gerr, st));
   }
+  FNO_CUDA(h, join.now());
   // lift: dp = sum dv0, dP[o, c] = sum dv0[b, o, s] x0[b, c, s]
   chan_reduce(h, h->dV, B, C, S, g + o.p);
   outer_reduce<8, kFeatures, false>(h, h->dV, h->x0, B, C, kFeatures, S, g + o.P);
@@ -1111,6 +1157,11 @@ int fno_create(const fno_config *cfg, fno_handle **out) {
   if (e == cudaSuccess) e = cudaMemset(h->m2, 0, np * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(h->prmb, 0, np * sizeof(__nv_bfloat16));
   if (e == cudaSuccess) e = alloc_workspace(h);
+  if (h->fused) {
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);
+    for (cudaEvent_t *v : {&h->ev_dz, &h->ev_sums, &h->ev_dw[0], &h->ev_dw[1]})
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(v, cudaEventDisableTiming);
+  }
   if (e != cudaSuccess) {
     std::string m = std::string("fno_create: ") + cudaGetErrorString(e);
     fno_destroy(h);
@@ -1332,6 +1383,9 @@ int fno_adam(fno_handle *h, float lr, float beta1, float beta2, float eps, int32
 int fno_destroy(fno_handle *h) {
   if (!h) return LB_OK;
   cudaStreamSynchronize(h->st);
+  if (h->side) cudaStreamDestroy(h->side);
+  for (cudaEvent_t v : {h->ev_dz, h->ev_sums, h->ev_dw[0], h->ev_dw[1]})
+    if (v) cudaEventDestroy(v);
   free_workspace(h);
   cudaFree(h->prm);
   cudaFree(h->grd);

@@ -23,7 +23,8 @@
 // (each product in its own accumulator, then added, then the bias), so a
 // layer's values are the same bits.  Bound by the activations (normcdff) and
 // by memory about equally.  Measured: training step of 16 fields of 256 x 64
-// 1.61 -> 1.07 ms, of 8 fields of 512 x 128 2.74 -> 1.65 ms; warm start of a
+// 1.61 -> 1.07 ms, of 8 fields of 512 x 128 2.74 -> 1.65 ms (0.96 and 1.41 with
+// the weight gradients beside them); warm start of a
 // 2048 x 512 lattice (forward pass, fields, initial state) 2.36 -> 0.90 ms.
 #include "fno_fused.h"
 
