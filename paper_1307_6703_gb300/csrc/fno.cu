@@ -31,6 +31,7 @@
 #include "fno_fused.h"
 #include "fno_math.cuh"
 #include "gemm_tc.h"
+#include "pdl.cuh"
 
 namespace {
 
@@ -96,6 +97,7 @@ dim3 grid2(long long S, int rows) {
 
 // Input features of each field from its parameters (U_w, A0, lambda, T_r).
 __global__ void features_kernel(const float *__restrict__ prm, int B, int nx, int ny, float *__restrict__ x0) {
+  pdl::begin();
   const long long S = (long long)nx * ny, total = (long long)B * S;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
     const int b = (int)(i / S);
@@ -119,6 +121,7 @@ __global__ void features_kernel(const float *__restrict__ prm, int B, int nx, in
 // v0[b, o, s] = sum_c P[o, c] x0[b, c, s] + p[o]
 __global__ void lift_kernel(const float *__restrict__ x0, const float *__restrict__ P, const float *__restrict__ pb,
                             int C, long long S, float *__restrict__ v, __nv_bfloat16 *__restrict__ vb) {
+  pdl::begin();
   const int row = blockIdx.y, b = row / C, o = row - b * C;
   const float *xb = x0 + (long long)b * kFeatures * S;
   float *vr = v + (long long)row * S;
@@ -150,6 +153,7 @@ constexpr int kYChunk = 64;  // rows of a chunk of ydft_kernel and iy_kernel
 __global__ void __launch_bounds__(kThreads)
 ydft_kernel(const float *__restrict__ A, const float2 *__restrict__ Ty, int ny, int mx, int my, int gx,
             float *__restrict__ Sh) {
+  pdl::begin();
   extern __shared__ float ysm[];
   float *xs = ysm;                                                  // [kYChunk][2 gx]
   float2 *ts = reinterpret_cast<float2 *>(ysm + kYChunk * 2 * gx);  // [my][kYChunk]
@@ -214,6 +218,7 @@ ydft_kernel(const float *__restrict__ A, const float2 *__restrict__ Ty, int ny, 
 __global__ void __launch_bounds__(kThreads)
 iy_kernel(const float *__restrict__ Y, const float2 *__restrict__ Ty, int ny, int mx, int my, float *__restrict__ X,
           __nv_bfloat16 *__restrict__ Xb) {
+  pdl::begin();
   extern __shared__ float ysm[];
   float *ys = ysm;                                              // [my][mx][2]
   float2 *ts = reinterpret_cast<float2 *>(ysm + 2 * my * mx);   // [my][kYChunk]
@@ -249,6 +254,7 @@ iy_kernel(const float *__restrict__ Y, const float2 *__restrict__ Ty, int ny, in
 __global__ void __launch_bounds__(kThreads)
 mix_kernel(const float *__restrict__ Sh, const float *__restrict__ Rr, const float *__restrict__ Ri, int B, int C,
            int M, float *__restrict__ Y) {
+  pdl::begin();
   extern __shared__ float msm[];
   float2 *ss = reinterpret_cast<float2 *>(msm);          // [B][C]
   float2 *rs = reinterpret_cast<float2 *>(msm + 2 * B * C);  // [C][C]
@@ -274,6 +280,7 @@ mix_kernel(const float *__restrict__ Sh, const float *__restrict__ Rr, const flo
 // z += w (per channel); v' = gelu(z) (or z for the last layer).
 __global__ void bias_act_kernel(float *__restrict__ z, const float *__restrict__ w, int C, long long S, int act,
                                 float *__restrict__ v, __nv_bfloat16 *__restrict__ vb) {
+  pdl::begin();
   const int row = blockIdx.y, o = row % C;
   const float wo = w[o];
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < S; s += (long long)gridDim.x * blockDim.x) {
@@ -292,6 +299,7 @@ constexpr int kMaxOutputs = 4;
 __global__ void project_kernel(float *__restrict__ hp, const float *__restrict__ q1, const float *__restrict__ Q2,
                                const float *__restrict__ q2, int H, int O, long long S, float *__restrict__ out,
                                float *__restrict__ out_user) {
+  pdl::begin();
   const int b = blockIdx.y;
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < S; s += (long long)gridDim.x * blockDim.x) {
     float *h = hp + (long long)b * H * S + s;
@@ -317,6 +325,7 @@ __global__ void project_kernel(float *__restrict__ hp, const float *__restrict__
 // Loss partial sums and d loss / d out = 2 (out - target) / (B S).
 __global__ void loss_kernel(const float *__restrict__ out, const float *__restrict__ tgt, long long total,
                             float *__restrict__ dout, double *__restrict__ partial) {
+  pdl::begin();
   __shared__ double sm[kThreads];
   double acc = 0.0;
   const float scale = 2.0f / (float)total;
@@ -330,6 +339,7 @@ __global__ void loss_kernel(const float *__restrict__ out, const float *__restri
 }
 
 __global__ void finish_loss_kernel(const double *__restrict__ partial, int n, long long total, double *__restrict__ loss) {
+  pdl::begin();
   __shared__ double sm[kThreads];
   double acc = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) acc += partial[i];
@@ -350,6 +360,7 @@ __device__ __forceinline__ double widen(float x) {
 // block's sites (grid-strided, then the fixed-order block tree).
 __global__ void field_mass_kernel(const float *__restrict__ out, int outputs, long long S, double s0,
                                   double *__restrict__ part) {
+  pdl::begin();
   __shared__ double sm[kThreads];
   const float *o = out + (size_t)blockIdx.y * outputs * S;
   double acc = 0.0;
@@ -366,6 +377,7 @@ __global__ void field_mass_kernel(const float *__restrict__ out, int outputs, lo
 // The density shift of field b, rho_mean - mean d, from its nblk <= kThreads
 // block sums by a fixed tree, in the place of the first of them.
 __global__ void shift_kernel(double *__restrict__ part, int nblk, long long S, double rho_mean) {
+  pdl::begin();
   __shared__ double sm[kThreads];
   double *p = part + (size_t)blockIdx.x * nblk;
   const double m = block_sum((int)threadIdx.x < nblk ? p[threadIdx.x] : 0.0, sm);
@@ -375,6 +387,7 @@ __global__ void shift_kernel(double *__restrict__ part, int nblk, long long S, d
 // fields[b] = (d + shift, s1 o1, s2 o2).
 __global__ void fields_kernel(const float *__restrict__ out, int outputs, long long S, double s0, double s1,
                               double s2, const double *__restrict__ part, int nblk, double *__restrict__ fields) {
+  pdl::begin();
   const int b = blockIdx.y;
   const double shift = part[(size_t)b * nblk];
   const float *o = out + (size_t)b * outputs * S;
@@ -390,6 +403,7 @@ __global__ void fields_kernel(const float *__restrict__ out, int outputs, long l
 __global__ void project_back_kernel(const float *__restrict__ hp, const float *__restrict__ Q2,
                                     const float *__restrict__ dout, int H, int O, long long S,
                                     float *__restrict__ dhp, __nv_bfloat16 *__restrict__ dhpb) {
+  pdl::begin();
   const int row = blockIdx.y, b = row / H, k = row - b * H;
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < S; s += (long long)gridDim.x * blockDim.x) {
     const long long i = (long long)row * S + s;
@@ -408,6 +422,7 @@ __global__ void project_back_kernel(const float *__restrict__ hp, const float *_
 constexpr int kReduceBlocks = 32;
 constexpr int kOuterBlocks = 64;  // site shares of outer_pass1_kernel
 __global__ void reduce_pass1_kernel(const float *__restrict__ a, int B, int C, long long S, double *__restrict__ part) {
+  pdl::begin();
   __shared__ double ws[kThreads / 32];
   const int ch = blockIdx.x, blk = blockIdx.y;
   const long long n = (long long)B * S, per = (n + gridDim.y - 1) / gridDim.y;
@@ -447,6 +462,7 @@ template <int NA, int NB, bool kGelu>
 __global__ void __launch_bounds__(kThreads)
 outer_pass1_kernel(const float *__restrict__ a, const float *__restrict__ o2, int B, int Ca, int Cb, long long S,
                    double *__restrict__ part) {
+  pdl::begin();
   constexpr int kFly = kGelu ? 1 : 4;
   __shared__ double sm[kThreads / 32][NA * NB];
   const int ntb = (Cb + NB - 1) / NB;
@@ -515,6 +531,7 @@ outer_pass1_kernel(const float *__restrict__ a, const float *__restrict__ o2, in
 template <bool kQuads>
 __global__ void __launch_bounds__(kThreads)
 reduce_pass1_v4_kernel(const float *__restrict__ a, int C, long long S, int nsplit, double *__restrict__ part) {
+  pdl::begin();
   __shared__ double ws[kThreads / 32];
   const int ch = blockIdx.x, b = blockIdx.y / nsplit, j = blockIdx.y % nsplit;
   const long long S4 = S / 4, step = (long long)nsplit * blockDim.x, row = (long long)b * C + ch;
@@ -547,6 +564,7 @@ reduce_pass1_v4_kernel(const float *__restrict__ a, int C, long long S, int nspl
 // then a fixed-order shuffle tree.
 __global__ void __launch_bounds__(kThreads)
 reduce_pass2_kernel(const double *__restrict__ part, int nch, int nb, float *__restrict__ out) {
+  pdl::begin();
   const int ch = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (ch >= nch) return;
   double acc = 0.0;
@@ -561,6 +579,7 @@ reduce_pass2_kernel(const double *__restrict__ part, int nch, int nb, float *__r
 // w, w + 8, ... in order, then warp 0 adds the eight partials in order.
 __global__ void __launch_bounds__(kThreads)
 sum_fields_kernel(const float *__restrict__ part, int B, int n, float *__restrict__ out) {
+  pdl::begin();
   __shared__ float ws[kThreads / 32][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;
@@ -581,6 +600,7 @@ sum_fields_kernel(const float *__restrict__ part, int B, int n, float *__restric
 // dz = dv * gelu'(z) (or dv for the last layer), with a BF16 copy.
 __global__ void act_back_kernel(const float *__restrict__ dv, const float *__restrict__ z, long long total, int act,
                                 float *__restrict__ dz, __nv_bfloat16 *__restrict__ dzb) {
+  pdl::begin();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
     const float d = act ? dv[i] * gelu_grad(z[i]) : dv[i];
     dz[i] = d;
@@ -596,6 +616,7 @@ __global__ void __launch_bounds__(kThreads)
 mix_back_kernel(const float *__restrict__ dY, const float *__restrict__ Sh, const float *__restrict__ Rr,
                 const float *__restrict__ Ri, int B, int C, int M, float *__restrict__ dS, float *__restrict__ dRr,
                 float *__restrict__ dRi) {
+  pdl::begin();
   extern __shared__ float msm[];
   float2 *ds = reinterpret_cast<float2 *>(msm);               // dY [B][C]
   float2 *ss = reinterpret_cast<float2 *>(msm + 2 * B * C);   // S [B][C]
@@ -637,6 +658,7 @@ mix_back_kernel(const float *__restrict__ dY, const float *__restrict__ Sh, cons
 // Fxi[j][x] (real inverse with c_kx and 1/(nx ny)).
 __global__ void dft_tables_kernel(int nx, int ny, int mx, int my, float *Fx, float *Fxi, __nv_bfloat16 *Fxb,
                                   __nv_bfloat16 *Fxib, __nv_bfloat16 *FxTb, __nv_bfloat16 *FxiTb, float2 *Ty) {
+  pdl::begin();
   // y twiddles: Ty[k][y] = (cos, sin)(2 pi ky y / ny), argument reduced mod ny
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < my * ny; i += gridDim.x * blockDim.x) {
     const int k = i / ny, y = i - k * ny;
@@ -670,6 +692,7 @@ __global__ void dft_tables_kernel(int nx, int ny, int mx, int my, float *Fx, flo
 __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
                             float *__restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1,
                             float c2, __nv_bfloat16 *__restrict__ pb) {
+  pdl::begin();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.0f - b1) * gi;
@@ -689,6 +712,7 @@ __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, 
 __global__ void __launch_bounds__(256)
 transpose_bf16_kernel(const __nv_bfloat16 *__restrict__ in, long long R, long long Cc,
                       __nv_bfloat16 *__restrict__ out) {
+  pdl::begin();
   __shared__ __nv_bfloat16 tile[32][64 + 2];
   const long long r0 = (long long)blockIdx.x * 32, c0 = (long long)blockIdx.y * 64;
   const int b = blockIdx.z;
@@ -722,6 +746,7 @@ transpose_bf16_kernel(const __nv_bfloat16 *__restrict__ in, long long R, long lo
 __global__ void __launch_bounds__(256)
 transpose_bf16_v8_kernel(const __nv_bfloat16 *__restrict__ in, long long R, long long S,
                          __nv_bfloat16 *__restrict__ out) {
+  pdl::begin();
   __shared__ __align__(16) __nv_bfloat16 tile[32][64 + 8];
   const long long r0 = (long long)blockIdx.x * 32, s0 = (long long)blockIdx.y * 64;
   const int b = blockIdx.z, t = threadIdx.x;
@@ -748,6 +773,7 @@ transpose_bf16_v8_kernel(const __nv_bfloat16 *__restrict__ in, long long R, long
 // W_l[o][c] (layer l at l C C), then Q1T[c][h] = Q1[h][c].
 __global__ void weights_t_kernel(const __nv_bfloat16 *__restrict__ prmb, Offsets o, int C, int H, int L,
                                  __nv_bfloat16 *__restrict__ wt) {
+  pdl::begin();
   const int n = L * C * C + C * H;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     if (i < L * C * C) {
@@ -761,6 +787,7 @@ __global__ void weights_t_kernel(const __nv_bfloat16 *__restrict__ prmb, Offsets
 }
 
 __global__ void to_bf16_kernel(const float *__restrict__ a, long long n, __nv_bfloat16 *__restrict__ b) {
+  pdl::begin();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     b[i] = __float2bfloat16_rn(a[i]);
 }
@@ -861,16 +888,16 @@ size_t mix_smem(int B, int C, bool back) { return (size_t)((back ? 4 : 2) * B * 
 
 void ydft(fno_handle *h, const float *A, int lines, int ny, float *Sh) {
   const int mx = h->c.modes_x, my = h->c.modes_y, gx = ydft_group(lines, mx);
-  ydft_kernel<<<dim3((unsigned)lines, (unsigned)((mx + gx - 1) / gx)), kThreads, ydft_smem(gx, my), h->st>>>(
-      A, h->Ty, ny, mx, my, gx, Sh);
+  (void)pdl::launch(ydft_kernel, dim3((unsigned)lines, (unsigned)((mx + gx - 1) / gx)), kThreads, ydft_smem(gx, my),
+                    h->st, A, h->Ty, ny, mx, my, gx, Sh);
 }
 
 void site_major(fno_handle *h, const __nv_bfloat16 *in, int B, int rows, long long S, __nv_bfloat16 *out) {
   const dim3 grid((unsigned)((rows + 31) / 32), (unsigned)((S + 63) / 64), (unsigned)B);
   if (rows % 32 == 0 && S % 8 == 0)
-    transpose_bf16_v8_kernel<<<grid, 256, 0, h->st>>>(in, rows, S, out);
+    (void)pdl::launch(transpose_bf16_v8_kernel, grid, 256, 0, h->st, in, rows, S, out);
   else
-    transpose_bf16_kernel<<<grid, 256, 0, h->st>>>(in, rows, S, out);
+    (void)pdl::launch(transpose_bf16_kernel, grid, 256, 0, h->st, in, rows, S, out);
 }
 
 // Shares of a field in pass 1 of the channel sums: about 2048 blocks in all.
@@ -879,8 +906,9 @@ int reduce_splits(int B, int C) { return std::max(1, std::min(kReduceBlocks, (20
 // The channel sums from the float4s' sums quads[b][ch][S / 4].
 void quad_reduce(fno_handle *h, const float *quads, int B, int C, long long S, float *out, cudaStream_t st) {
   const int nsplit = reduce_splits(B, C);
-  reduce_pass1_v4_kernel<true><<<dim3(C, B * nsplit), kThreads, 0, st>>>(quads, C, S, nsplit, h->rpart);
-  reduce_pass2_kernel<<<(C + 7) / 8, kThreads, 0, st>>>(h->rpart, C, B * nsplit, out);
+  (void)pdl::launch(reduce_pass1_v4_kernel<true>, dim3(C, B * nsplit), kThreads, 0, st, quads, C, S, nsplit,
+                    h->rpart);
+  (void)pdl::launch(reduce_pass2_kernel, (C + 7) / 8, kThreads, 0, st, h->rpart, C, B * nsplit, out);
 }
 
 // out[ch] = sum over (b, s) of a[b, ch, s] for the C channels of a.
@@ -888,12 +916,13 @@ void chan_reduce(fno_handle *h, const float *a, int B, int C, long long S, float
   if (S % 4 == 0 && B * kReduceBlocks <= h->rpart_fields) {
     // float4 loads; about 2048 blocks, at most 32 shares of a field
     const int nsplit = reduce_splits(B, C);
-    reduce_pass1_v4_kernel<false><<<dim3(C, B * nsplit), kThreads, 0, h->st>>>(a, C, S, nsplit, h->rpart);
-    reduce_pass2_kernel<<<(C + 7) / 8, kThreads, 0, h->st>>>(h->rpart, C, B * nsplit, out);
+    (void)pdl::launch(reduce_pass1_v4_kernel<false>, dim3(C, B * nsplit), kThreads, 0,
+                      h->st, a, C, S, nsplit, h->rpart);
+    (void)pdl::launch(reduce_pass2_kernel, (C + 7) / 8, kThreads, 0, h->st, h->rpart, C, B * nsplit, out);
     return;
   }
-  reduce_pass1_kernel<<<dim3(C, kReduceBlocks), kThreads, 0, h->st>>>(a, B, C, S, h->rpart);
-  reduce_pass2_kernel<<<(C + 7) / 8, kThreads, 0, h->st>>>(h->rpart, C, kReduceBlocks, out);
+  (void)pdl::launch(reduce_pass1_kernel, dim3(C, kReduceBlocks), kThreads, 0, h->st, a, B, C, S, h->rpart);
+  (void)pdl::launch(reduce_pass2_kernel, (C + 7) / 8, kThreads, 0, h->st, h->rpart, C, kReduceBlocks, out);
 }
 
 // out[ca * Cb + cb] = sum over (b, s) of a[b, ca, s] f(o2[b, cb, s]) (f = gelu
@@ -902,9 +931,9 @@ void chan_reduce(fno_handle *h, const float *a, int B, int C, long long S, float
 template <int NA, int NB, bool kGelu>
 void outer_reduce(fno_handle *h, const float *a, const float *o2, int B, int Ca, int Cb, long long S, float *out) {
   const int tiles = ((Ca + NA - 1) / NA) * ((Cb + NB - 1) / NB);
-  outer_pass1_kernel<NA, NB, kGelu><<<dim3(kOuterBlocks, tiles), kThreads, 0, h->st>>>(a, o2, B, Ca, Cb, S, h->rpart);
-  reduce_pass2_kernel<<<(Ca * Cb + 7) / 8, kThreads, 0, h->st>>>(h->rpart, Ca * Cb, kOuterBlocks,
-                                                                                   out);
+  (void)pdl::launch(outer_pass1_kernel<NA, NB, kGelu>, dim3(kOuterBlocks, tiles), kThreads, 0,
+                    h->st, a, o2, B, Ca, Cb, S, h->rpart);
+  (void)pdl::launch(reduce_pass2_kernel, (Ca * Cb + 7) / 8, kThreads, 0, h->st, h->rpart, Ca * Cb, kOuterBlocks, out);
 }
 
 template <typename T>
@@ -1019,9 +1048,10 @@ int forward_fused(fno_handle *h, int B, int nx, int ny, const float *params_dev,
   for (int l = 0; l < L; l++) {
     FNO_GEMM(h, tcg(h, h->Vb[l], nx, 0, h->FxTb, nx, 0, h->A, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 1, 0.f));
     ydft(h, h->A, B * c.width, ny, h->Sh[l]);
-    mix_kernel<<<my * mx, kThreads, mix_smem(B, c.width, false), st>>>(h->Sh[l], P + h->o.Rr[l], P + h->o.Ri[l], B,
-                                                                         c.width, my * mx, h->dY);
-    iy_kernel<<<iy_grid(B * c.width, ny), kThreads, iy_smem(mx, my), st>>>(h->dY, h->Ty, ny, mx, my, nullptr, h->Gb);
+    (void)pdl::launch(mix_kernel, my * mx, kThreads, mix_smem(B, c.width, false), st,
+                      h->Sh[l], P + h->o.Rr[l], P + h->o.Ri[l], B, c.width, my * mx, h->dY);
+    (void)pdl::launch(iy_kernel, iy_grid(B * c.width, ny), kThreads, iy_smem(mx, my), st,
+                      h->dY, h->Ty, ny, mx, my, nullptr, h->Gb);
     FNO_CUDA(h, cudaGetLastError());
     FNO_GEMM(h, fno::layer_forward(sh, h->VbT[l], h->prmb + h->o.W[l], P + h->o.w[l], h->Gb, h->FxiTb, l == L - 1,
                                    h->Z[l], h->Vb[l + 1], h->VbT[l + 1], h->gerr, st));
@@ -1092,19 +1122,20 @@ int backward_fused(fno_handle *h, const float *target, double *loss) {
     FNO_CUDA(h, cudaEventRecord(h->ev_sums, h->side));
     FNO_GEMM(h, tcg(h, dzl, (int)S, CS, h->Vb[l], (int)S, CS, h->wpart, C, 1, (long long)C * C, C, C, (int)S, B,
                     kWSplit, 0.f, true));
-    sum_fields_kernel<<<(C * C + 31) / 32, kThreads, 0, h->side>>>(h->wpart, parts, C * C, g + o.W[l]);
+    (void)pdl::launch(sum_fields_kernel, (C * C + 31) / 32, kThreads, 0, h->side, h->wpart, parts, C * C, g + o.W[l]);
     FNO_CUDA(h, cudaEventRecord(h->ev_dw[l & 1], h->side));
     if (l == L - 1) {
       FNO_GEMM(h, tcg(h, h->dhpb, (int)S, HS, h->Vb[L], (int)S, CS, h->wpart, C, 1, (long long)H * C, H, C, (int)S, B,
                       kWSplit, 0.f, true));
-      sum_fields_kernel<<<(H * C + 31) / 32, kThreads, 0, h->side>>>(h->wpart, parts, H * C, g + o.Q1);
+      (void)pdl::launch(sum_fields_kernel, (H * C + 31) / 32, kThreads, 0, h->side, h->wpart, parts, H * C, g + o.Q1);
     }
     // spectral path: dG = dz Fxi^T, the adjoints of the mixing and of the y-transforms
     FNO_GEMM(h, tcg(h, dzl, nx, 0, h->Fxib, nx, 0, h->dG, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 1, 0.f));
     ydft(h, h->dG, B * C, ny, h->dY);
-    mix_back_kernel<<<my * mx, kThreads, mix_smem(B, C, true), st>>>(h->dY, h->Sh[l], P + o.Rr[l], P + o.Ri[l], B, C,
-                                                                       my * mx, h->dS, g + o.Rr[l], g + o.Ri[l]);
-    iy_kernel<<<iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st>>>(h->dS, h->Ty, ny, mx, my, nullptr, h->dAb);
+    (void)pdl::launch(mix_back_kernel, my * mx, kThreads, mix_smem(B, C, true), st,
+                      h->dY, h->Sh[l], P + o.Rr[l], P + o.Ri[l], B, C, my * mx, h->dS, g + o.Rr[l], g + o.Ri[l]);
+    (void)pdl::launch(iy_kernel, iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st,
+                      h->dS, h->Ty, ny, mx, my, nullptr, h->dAb);
     FNO_CUDA(h, cudaGetLastError());
     // everything per site: dv, through the activation below (the site-major
     // copy in place: a tile reads and writes its own sites), when the channel
@@ -1177,9 +1208,9 @@ int fno_set_params(fno_handle *h, const float *host) {
   if (!h || !host) return ffail(h, LB_ERR_ARG, "fno_set_params: null argument");
   const long long np = (long long)h->o.total;
   FNO_CUDA(h, cudaMemcpyAsync(h->prm, host, np * sizeof(float), cudaMemcpyHostToDevice, h->st));
-  to_bf16_kernel<<<blocks_for(np), kThreads, 0, h->st>>>(h->prm, np, h->prmb);
-  weights_t_kernel<<<blocks_for(np), kThreads, 0, h->st>>>(h->prmb, h->o, h->c.width, h->c.hidden, h->c.layers,
-                                                           h->wTb);
+  (void)pdl::launch(to_bf16_kernel, blocks_for(np), kThreads, 0, h->st, h->prm, np, h->prmb);
+  (void)pdl::launch(weights_t_kernel, blocks_for(np), kThreads, 0,
+                    h->st, h->prmb, h->o, h->c.width, h->c.hidden, h->c.layers, h->wTb);
   FNO_CUDA(h, cudaGetLastError());
   FNO_CUDA(h, cudaStreamSynchronize(h->st));
   return LB_OK;
@@ -1210,16 +1241,17 @@ int fno_forward(fno_handle *h, int32_t B, int32_t nx, int32_t ny, const float *p
   const int R = B * C * ny;
   cudaStream_t st = h->st;
   if (h->tab_nx != nx || h->tab_ny != ny) {
-    dft_tables_kernel<<<blocks_for((long long)std::max(nx * mx, ny * my)), kThreads, 0, st>>>(
-        nx, ny, mx, my, h->Fx, h->Fxi, h->Fxb, h->Fxib, h->FxTb, h->FxiTb, h->Ty);
+    (void)pdl::launch(dft_tables_kernel, blocks_for((long long)std::max(nx * mx, ny * my)), kThreads, 0, st, nx, ny,
+                      mx, my, h->Fx, h->Fxi, h->Fxb, h->Fxib, h->FxTb, h->FxiTb, h->Ty);
     FNO_CUDA(h, cudaGetLastError());
     h->tab_nx = nx;
     h->tab_ny = ny;
   }
   const float *P = h->prm;
   if (h->fused) return forward_fused(h, B, nx, ny, params_dev, out);
-  features_kernel<<<blocks_for((long long)B * S), kThreads, 0, st>>>(params_dev, B, nx, ny, h->x0);
-  lift_kernel<<<grid2(S, B * C), kThreads, 0, st>>>(h->x0, P + h->o.P, P + h->o.p, C, S, h->V[0], h->Vb[0]);
+  (void)pdl::launch(features_kernel, blocks_for((long long)B * S), kThreads, 0, st, params_dev, B, nx, ny, h->x0);
+  (void)pdl::launch(lift_kernel, grid2(S, B * C), kThreads, 0, st,
+                    h->x0, P + h->o.P, P + h->o.p, C, S, h->V[0], h->Vb[0]);
   FNO_CUDA(h, cudaGetLastError());
   const bool bf = c.gemm_bf16 != 0;
   if (bf) site_major(h, h->Vb[0], B, C, S, h->VbT[0]);
@@ -1232,9 +1264,10 @@ int fno_forward(fno_handle *h, int32_t B, int32_t nx, int32_t ny, const float *p
       FNO_GEMM(h, sg(h, h->V[l], nx, 1, 0, h->Fx, 2 * mx, 1, 0, h->A, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 0.f));
     // y-transform, per-mode mixing (into the dY scratch), inverse y-transform
     ydft(h, h->A, B * C, ny, h->Sh[l]);
-    mix_kernel<<<my * mx, kThreads, mix_smem(B, C, false), st>>>(h->Sh[l], P + h->o.Rr[l], P + h->o.Ri[l], B, C,
-                                                                   my * mx, h->dY);
-    iy_kernel<<<iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st>>>(h->dY, h->Ty, ny, mx, my, h->G, h->Gb);
+    (void)pdl::launch(mix_kernel, my * mx, kThreads, mix_smem(B, C, false), st,
+                      h->Sh[l], P + h->o.Rr[l], P + h->o.Ri[l], B, C, my * mx, h->dY);
+    (void)pdl::launch(iy_kernel, iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st,
+                      h->dY, h->Ty, ny, mx, my, h->G, h->Gb);
     FNO_CUDA(h, cudaGetLastError());
     // inverse x-transform into z: Z[R, nx] = G[R, 2mx] Fxi[2mx, nx]
     if (bf)
@@ -1247,8 +1280,8 @@ int fno_forward(fno_handle *h, int32_t B, int32_t nx, int32_t ny, const float *p
       FNO_GEMM(h, tcg(h, h->VbT[l], C, CS, h->prmb + h->o.W[l], C, 0, h->Z[l], 1, S, CS, (int)S, C, C, B, 1, 1.f));
     else
       FNO_GEMM(h, sg(h, P + h->o.W[l], C, 1, 0, h->V[l], S, 1, CS, h->Z[l], S, 1, CS, C, (int)S, C, B, 1.f));
-    bias_act_kernel<<<grid2(S, B * C), kThreads, 0, st>>>(h->Z[l], P + h->o.w[l], C, S, l < L - 1 ? 1 : 0,
-                                                           h->V[l + 1], h->Vb[l + 1]);
+    (void)pdl::launch(bias_act_kernel, grid2(S, B * C), kThreads, 0, st,
+                      h->Z[l], P + h->o.w[l], C, S, l < L - 1 ? 1 : 0, h->V[l + 1], h->Vb[l + 1]);
     FNO_CUDA(h, cudaGetLastError());
     if (bf) site_major(h, h->Vb[l + 1], B, C, S, h->VbT[l + 1]);
   }
@@ -1258,8 +1291,8 @@ int fno_forward(fno_handle *h, int32_t B, int32_t nx, int32_t ny, const float *p
                     0.f));
   else
     FNO_GEMM(h, sg(h, P + h->o.Q1, C, 1, 0, h->V[L], S, 1, CS, h->hp, S, 1, (long long)H * S, H, (int)S, C, B, 0.f));
-  project_kernel<<<grid2(S, B), kThreads, 0, st>>>(h->hp, P + h->o.q1, P + h->o.Q2, P + h->o.q2, H,
-                                                                     c.outputs, S, h->out, out);
+  (void)pdl::launch(project_kernel, grid2(S, B), kThreads, 0, st,
+                    h->hp, P + h->o.q1, P + h->o.Q2, P + h->o.q2, H, c.outputs, S, h->out, out);
   FNO_CUDA(h, cudaGetLastError());
   h->B = B;
   h->nx = nx;
@@ -1282,12 +1315,13 @@ int fno_backward(fno_handle *h, const float *target, double *loss) {
   float *g = h->grd;
   if (h->fused) return backward_fused(h, target, loss);
   const unsigned lb = blocks_for(BS);
-  loss_kernel<<<lb, kThreads, 0, st>>>(h->out, target, BS, h->dout, h->partial);
-  finish_loss_kernel<<<1, kThreads, 0, st>>>(h->partial, (int)lb, BS, h->loss);
+  (void)pdl::launch(loss_kernel, lb, kThreads, 0, st, h->out, target, BS, h->dout, h->partial);
+  (void)pdl::launch(finish_loss_kernel, 1, kThreads, 0, st, h->partial, (int)lb, BS, h->loss);
   // projection: dq2, dQ2, dhp, dq1, dQ1, dV = Q1^T dhp
   chan_reduce(h, h->dout, B, O, S, g + o.q2);
   outer_reduce<kMaxOutputs, 8, true>(h, h->dout, h->hp, B, O, H, S, g + o.Q2);
-  project_back_kernel<<<grid2(S, B * H), kThreads, 0, st>>>(h->hp, P + o.Q2, h->dout, H, O, S, h->dhp, h->dhpb);
+  (void)pdl::launch(project_back_kernel, grid2(S, B * H), kThreads, 0, st,
+                    h->hp, P + o.Q2, h->dout, H, O, S, h->dhp, h->dhpb);
   chan_reduce(h, h->dhp, B, H, S, g + o.q1);
   FNO_CUDA(h, cudaGetLastError());
   const bool bf = c.gemm_bf16 != 0;
@@ -1301,7 +1335,7 @@ int fno_backward(fno_handle *h, const float *target, double *loss) {
   } else {
     FNO_GEMM(h, sg(h, h->dhp, S, 1, HS, h->V[L], 1, S, CS, h->wpart, C, 1, (long long)H * C, H, C, (int)S, B, 0.f));
   }
-  sum_fields_kernel<<<(H * C + 31) / 32, kThreads, 0, st>>>(h->wpart, parts, H * C, g + o.Q1);
+  (void)pdl::launch(sum_fields_kernel, (H * C + 31) / 32, kThreads, 0, st, h->wpart, parts, H * C, g + o.Q1);
   // dv[b][c][s] = sum_h Q1[h][c] dhp[b][h][s]
   if (bf) {
     site_major(h, h->dhpb, B, H, S, h->dhpT);
@@ -1310,7 +1344,8 @@ int fno_backward(fno_handle *h, const float *target, double *loss) {
     FNO_GEMM(h, sg(h, P + o.Q1, 1, C, 0, h->dhp, S, 1, HS, h->dV, S, 1, CS, C, (int)S, H, B, 0.f));
   }
   for (int l = L - 1; l >= 0; l--) {
-    act_back_kernel<<<blocks_for(BCS), kThreads, 0, st>>>(h->dV, h->Z[l], BCS, l < L - 1 ? 1 : 0, h->dZ, h->dZb);
+    (void)pdl::launch(act_back_kernel, blocks_for(BCS), kThreads, 0, st,
+                      h->dV, h->Z[l], BCS, l < L - 1 ? 1 : 0, h->dZ, h->dZb);
     chan_reduce(h, h->dZ, B, C, S, g + o.w[l]);
     FNO_CUDA(h, cudaGetLastError());
     // dW = sum_b dz[b] v[b]^T
@@ -1319,7 +1354,7 @@ int fno_backward(fno_handle *h, const float *target, double *loss) {
                       kWSplit, 0.f));
     else
       FNO_GEMM(h, sg(h, h->dZ, S, 1, CS, h->V[l], 1, S, CS, h->wpart, C, 1, (long long)C * C, C, C, (int)S, B, 0.f));
-    sum_fields_kernel<<<(C * C + 31) / 32, kThreads, 0, st>>>(h->wpart, parts, C * C, g + o.W[l]);
+    (void)pdl::launch(sum_fields_kernel, (C * C + 31) / 32, kThreads, 0, st, h->wpart, parts, C * C, g + o.W[l]);
     // spectral path: dG = dz Fxi^T, then the adjoints of the mixing and of the y-transform
     if (bf)
       FNO_GEMM(h, tcg(h, h->dZb, nx, 0, h->Fxib, nx, 0, h->dG, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 1, 0.f));
@@ -1328,9 +1363,10 @@ int fno_backward(fno_handle *h, const float *target, double *loss) {
     // adjoints: of the inverse y-transform (a y-transform), of the mixing
     // (with the weights' gradient), of the y-transform (an inverse one)
     ydft(h, h->dG, B * C, ny, h->dY);
-    mix_back_kernel<<<my * mx, kThreads, mix_smem(B, C, true), st>>>(h->dY, h->Sh[l], P + o.Rr[l], P + o.Ri[l], B, C,
-                                                                       my * mx, h->dS, g + o.Rr[l], g + o.Ri[l]);
-    iy_kernel<<<iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st>>>(h->dS, h->Ty, ny, mx, my, h->dA, h->dAb);
+    (void)pdl::launch(mix_back_kernel, my * mx, kThreads, mix_smem(B, C, true), st,
+                      h->dY, h->Sh[l], P + o.Rr[l], P + o.Ri[l], B, C, my * mx, h->dS, g + o.Rr[l], g + o.Ri[l]);
+    (void)pdl::launch(iy_kernel, iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st,
+                      h->dS, h->Ty, ny, mx, my, h->dA, h->dAb);
     FNO_CUDA(h, cudaGetLastError());
     // dv = W^T dz (pointwise path) + dA Fx^T (spectral path)
     if (bf) {
@@ -1359,11 +1395,12 @@ int fno_fields(fno_handle *h, const float *out, int32_t batch, int32_t nx, int32
   // block sums in the loss partials (8192 doubles, batch * nblk of them; the
   // same stream orders their uses)
   const int nblk = (int)std::max<long long>(1, std::min<long long>({256, 8192 / batch, (S + kThreads - 1) / kThreads}));
-  field_mass_kernel<<<dim3(nblk, batch), kThreads, 0, h->st>>>(out, h->c.outputs, S, scales[0], h->partial);
-  shift_kernel<<<batch, kThreads, 0, h->st>>>(h->partial, nblk, S, rho_mean);
+  (void)pdl::launch(field_mass_kernel, dim3(nblk, batch), kThreads, 0,
+                    h->st, out, h->c.outputs, S, scales[0], h->partial);
+  (void)pdl::launch(shift_kernel, batch, kThreads, 0, h->st, h->partial, nblk, S, rho_mean);
   const unsigned fblk = (unsigned)std::min<long long>((S + kThreads - 1) / kThreads, std::max(1, 8192 / batch));
-  fields_kernel<<<dim3(fblk, batch), kThreads, 0, h->st>>>(out, h->c.outputs, S, scales[0], scales[1], scales[2],
-                                                           h->partial, nblk, fields);
+  (void)pdl::launch(fields_kernel, dim3(fblk, batch), kThreads, 0,
+                    h->st, out, h->c.outputs, S, scales[0], scales[1], scales[2], h->partial, nblk, fields);
   FNO_CUDA(h, cudaGetLastError());
   return LB_OK;
 }
@@ -1372,10 +1409,10 @@ int fno_adam(fno_handle *h, float lr, float beta1, float beta2, float eps, int32
   if (!h || t < 1) return ffail(h, LB_ERR_ARG, "fno_adam: bad arguments");
   const long long np = (long long)h->o.total;
   const float c1 = 1.0f - powf(beta1, (float)t), c2 = 1.0f - powf(beta2, (float)t);
-  adam_kernel<<<blocks_for(np), kThreads, 0, h->st>>>(h->prm, h->grd, h->m1, h->m2, np, lr, beta1, beta2, eps, c1, c2,
-                                                       h->prmb);
-  weights_t_kernel<<<blocks_for(np), kThreads, 0, h->st>>>(h->prmb, h->o, h->c.width, h->c.hidden, h->c.layers,
-                                                           h->wTb);
+  (void)pdl::launch(adam_kernel, blocks_for(np), kThreads, 0,
+                    h->st, h->prm, h->grd, h->m1, h->m2, np, lr, beta1, beta2, eps, c1, c2, h->prmb);
+  (void)pdl::launch(weights_t_kernel, blocks_for(np), kThreads, 0,
+                    h->st, h->prmb, h->o, h->c.width, h->c.hidden, h->c.layers, h->wTb);
   FNO_CUDA(h, cudaGetLastError());
   return LB_OK;
 }

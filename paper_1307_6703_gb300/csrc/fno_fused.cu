@@ -23,15 +23,16 @@
 // (each product in its own accumulator, then added, then the bias), so a
 // layer's values are the same bits.  Bound by the activations (normcdff) and
 // by memory about equally.  Measured: training step of 16 fields of 256 x 64
-// 1.61 -> 1.07 ms, of 8 fields of 512 x 128 2.74 -> 1.65 ms (0.96 and 1.41 with
-// the weight gradients beside them); warm start of a
-// 2048 x 512 lattice (forward pass, fields, initial state) 2.36 -> 0.90 ms.
+// 1.61 -> 1.07 ms, of 8 fields of 512 x 128 2.74 -> 1.65 ms (0.90 and 1.34 with
+// the weight gradients beside them and launches overlapped); warm start of a
+// 2048 x 512 lattice (forward pass, fields, initial state) 2.36 -> 0.84 ms.
 #include "fno_fused.h"
 
 #include <algorithm>
 
 #include "fno_math.cuh"
 #include "gemm_tc.h"
+#include "pdl.cuh"
 #include "tc_device.cuh"
 
 namespace fno {
@@ -171,6 +172,7 @@ template <int kMode, int kK>
 __global__ void __launch_bounds__(kThreads, kK == 32 ? 8 : 5)
 layer_kernel(const __grid_constant__ CUtensorMap ma1, const __grid_constant__ CUtensorMap mb1,
              const __grid_constant__ CUtensorMap ma2, const __grid_constant__ CUtensorMap mb2, const LayerArgs p) {
+  pdl::begin();
   extern __shared__ unsigned char raw[];
   using Sm = LayerSmem<kK>;
   Sm &S = *reinterpret_cast<Sm *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
@@ -252,6 +254,7 @@ __device__ __forceinline__ void features(const float *prm, int b, int x, int y, 
 __global__ void __launch_bounds__(kThreads)
 lift_kernel(int nx, int ny, const float *__restrict__ prm, const float *__restrict__ P, const float *__restrict__ pb,
             float *__restrict__ x0, __nv_bfloat16 *__restrict__ cm, __nv_bfloat16 *__restrict__ sm) {
+  pdl::begin();
   __shared__ float Ps[C * kFeat], ps[C];
   for (int i = threadIdx.x; i < C * kFeat; i += kThreads) Ps[i] = P[i];
   if (threadIdx.x < C) ps[threadIdx.x] = pb[threadIdx.x];
@@ -308,6 +311,7 @@ template <int H, bool kBack>
 __global__ void __launch_bounds__(kThreads, kBack ? 4 : 5)
 project_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb1,
                const __grid_constant__ CUtensorMap mb2, const ProjArgs p) {
+  pdl::begin();
   extern __shared__ unsigned char raw[];
   using Sm = ProjSmem<H>;
   Sm &S = *reinterpret_cast<Sm *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
@@ -457,6 +461,7 @@ constexpr int kSumWarps = 8, kSumSplits = 16;
 // split q of part2.
 __global__ void __launch_bounds__(32 * kSumWarps)
 tile_sums_kernel(const double *__restrict__ part, long long tiles, int nval, double *__restrict__ part2) {
+  pdl::begin();
   __shared__ double ws[kSumWarps][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
   double acc = 0.0;
@@ -484,6 +489,7 @@ tile_sums_kernel(const double *__restrict__ part, long long tiles, int nval, dou
 // The splits' sums, in order, into up to three ranges of outputs and the loss.
 __global__ void finish_kernel(const double *__restrict__ part2, int nval, SumOut o0, SumOut o1, SumOut o2,
                               double *__restrict__ loss, double count) {
+  pdl::begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nval) return;
   double r = part2[i];
@@ -525,8 +531,7 @@ cudaError_t launch_layer_k(const Shape &s, const LayerMaps &m, const LayerArgs &
   const size_t smem = sizeof(LayerSmem<kK>) + 1024;
   const cudaError_t e = allow_smem(layer_kernel<kMode, kK>, smem);
   if (e != cudaSuccess) return e;
-  layer_kernel<kMode, kK><<<tile_grid(s), kThreads, smem, st>>>(m.a1, m.b1, m.a2, m.b2, p);
-  return cudaGetLastError();
+  return pdl::launch(layer_kernel<kMode, kK>, tile_grid(s), kThreads, smem, st, m.a1, m.b1, m.a2, m.b2, p);
 }
 template <int kMode>
 cudaError_t launch_layer(const Shape &s, const LayerMaps &m, const LayerArgs &p, cudaStream_t st) {
@@ -544,8 +549,7 @@ cudaError_t launch_project(const Shape &s, const __nv_bfloat16 *v_sm, const __nv
   const size_t smem = sizeof(ProjSmem<H>) + 1024;
   if (e == cudaSuccess) e = allow_smem(project_kernel<H, kBack>, smem);
   if (e != cudaSuccess) return e;
-  project_kernel<H, kBack><<<tile_grid(s), kThreads, smem, st>>>(ma, mb1, mb2, p);
-  return cudaGetLastError();
+  return pdl::launch(project_kernel<H, kBack>, tile_grid(s), kThreads, smem, st, ma, mb1, mb2, p);
 }
 
 }  // namespace
@@ -560,8 +564,7 @@ long long fused_tiles(const Shape &s) { return (long long)((s.nx + tc::kBM - 1) 
 
 cudaError_t lift(const Shape &s, const float *prm, const float *P, const float *pb, float *x0, __nv_bfloat16 *cm,
                  __nv_bfloat16 *sm, cudaStream_t st) {
-  lift_kernel<<<tile_grid(s), kThreads, 0, st>>>(s.nx, s.ny, prm, P, pb, x0, cm, sm);
-  return cudaGetLastError();
+  return pdl::launch(lift_kernel, tile_grid(s), kThreads, 0, st, s.nx, s.ny, prm, P, pb, x0, cm, sm);
 }
 
 cudaError_t layer_forward(const Shape &s, const __nv_bfloat16 *v_sm, const __nv_bfloat16 *W, const float *w,
@@ -627,9 +630,9 @@ cudaError_t layer_backward(const Shape &s, const __nv_bfloat16 *dz_sm, const __n
 
 cudaError_t finish_sums(const double *part, long long tiles, int nval, const SumOut (&o)[3], double *loss, double count,
                         double *part2, cudaStream_t st) {
-  tile_sums_kernel<<<dim3((nval + 31) / 32, kSumSplits), 32 * kSumWarps, 0, st>>>(part, tiles, nval, part2);
-  finish_kernel<<<(nval + 127) / 128, 128, 0, st>>>(part2, nval, o[0], o[1], o[2], loss, count);
-  return cudaGetLastError();
+  (void)pdl::launch(tile_sums_kernel, dim3((nval + 31) / 32, kSumSplits), 32 * kSumWarps, 0, st, part, tiles, nval,
+                    part2);
+  return pdl::launch(finish_kernel, (nval + 127) / 128, 128, 0, st, part2, nval, o[0], o[1], o[2], loss, count);
 }
 
 long long finish_scratch(int nval) { return (long long)kSumSplits * nval; }

@@ -32,6 +32,7 @@
 
 #include "fno.h"
 #include "gemm_tc.h"
+#include "pdl.cuh"
 #include "tc_device.cuh"
 
 namespace tc {
@@ -54,6 +55,7 @@ template <int BN, int kStages>
 __global__ void __launch_bounds__(kThreads)
 gemm_tn_bf16_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap my,
                     const GemmParams p) {
+  pdl::begin();
   extern __shared__ unsigned char raw[];
   // the swizzled tiles need 1024-byte alignment
   using Sm = Smem<BN, kStages>;
@@ -224,6 +226,7 @@ __global__ void __launch_bounds__(256)
 gemm_f32_kernel(const float *__restrict__ a, long long am, long long ak, long long sa, const float *__restrict__ bb,
                 long long bk, long long bn, long long sb, float *__restrict__ c, long long cm, long long cn,
                 long long sc, int M, int N, int K, float beta) {
+  pdl::begin();
   __shared__ float As[16][64 + 1];
   __shared__ float Bs[16][64 + 1];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -277,12 +280,8 @@ cudaError_t launch_tn(const CUtensorMap &mx, const CUtensorMap &my, const GemmPa
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((p.M + kBM - 1) / kBM), (unsigned)((p.N + BN - 1) / BN), (unsigned)(nb * p.ksplit));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, gemm_tn_bf16_kernel<BN, kStages>, mx, my, p);
+  const dim3 grid((unsigned)((p.M + kBM - 1) / kBM), (unsigned)((p.N + BN - 1) / BN), (unsigned)(nb * p.ksplit));
+  return pdl::launch(gemm_tn_bf16_kernel<BN, kStages>, grid, kThreads, smem, st, mx, my, p);
 }
 
 template <int BN>
@@ -358,11 +357,8 @@ cudaError_t gemm_f32(const float *A, long long am, long long ak, long long sA, c
                      long long bn, long long sB, float *C, long long cm, long long cn, long long sC, int M, int N,
                      int K, int batch, float beta, cudaStream_t st) {
   if (M < 1 || N < 1 || K < 1 || batch < 1) return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((M + 63) / 64), (unsigned)((N + 63) / 64), (unsigned)batch);
-  cfg.blockDim = dim3(256);
-  cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, gemm_f32_kernel, A, am, ak, sA, B, bk, bn, sB, C, cm, cn, sC, M, N, K, beta);
+  const dim3 grid((unsigned)((M + 63) / 64), (unsigned)((N + 63) / 64), (unsigned)batch);
+  return pdl::launch(gemm_f32_kernel, grid, 256, 0, st, A, am, ak, sA, B, bk, bn, sB, C, cm, cn, sC, M, N, K, beta);
 }
 
 }  // namespace tc

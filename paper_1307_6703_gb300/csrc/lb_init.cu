@@ -18,6 +18,7 @@
 
 #include "lb_device.cuh"
 #include "lb_internal.h"
+#include "pdl.cuh"
 
 namespace lbk {
 
@@ -184,6 +185,7 @@ __device__ __forceinline__ float PutDev<__half>::dec(__half v) { return __half2f
 // columns aligned), blocks strided over rows.
 template <class Put, int kCols, bool kMoving>
 __global__ void __launch_bounds__(256) init_f32_kernel(Put put, const __grid_constant__ InitArgs A) {
+  pdl::begin();
   const int cols = A.nx / kCols;
   for (int y = blockIdx.y; y < A.ny; y += gridDim.y) {
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += gridDim.x * blockDim.x) {
@@ -234,9 +236,8 @@ template <class Put, int kCols>
 cudaError_t launch_cols(const Put &put, const InitArgs &A, cudaStream_t st) {
   const unsigned bx = (unsigned)((A.nx / kCols + 255) / 256);
   const dim3 grid(std::min(bx, 64u), (unsigned)std::min(A.ny, 2048));
-  if (A.ux != nullptr || A.uy != nullptr) init_f32_kernel<Put, kCols, true><<<grid, 256, 0, st>>>(put, A);
-  else init_f32_kernel<Put, kCols, false><<<grid, 256, 0, st>>>(put, A);
-  return cudaGetLastError();
+  return A.ux != nullptr || A.uy != nullptr ? pdl::launch(init_f32_kernel<Put, kCols, true>, grid, 256, 0, st, put, A)
+                                            : pdl::launch(init_f32_kernel<Put, kCols, false>, grid, 256, 0, st, put, A);
 }
 
 Ff ff_host(double d) {

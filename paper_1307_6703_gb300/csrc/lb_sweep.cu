@@ -73,10 +73,11 @@
 // finishes last adds them up, so the global sums of the new state need no
 // further kernel.
 //
-// Consecutive steps are programmatic dependent launches: step k+1 may be
-// scheduled once every CTA of step k has left its main loop, and waits
-// (griddepcontrol.wait) for step k to complete before it touches global
-// memory, which hides the launch gap between the two grids.
+// Initial state, single steps and moments are programmatic dependent launches
+// (pdl.cuh): a step's successor may be scheduled once every CTA of the step has
+// left its main loop, and waits (griddepcontrol.wait) for the step to complete
+// before it touches global memory, which hides the launch gap between the two
+// grids.
 #include <cmath>
 #include <cstddef>
 #include <type_traits>
@@ -89,6 +90,7 @@
 
 #include "lb_device.cuh"
 #include "lb_internal.h"
+#include "pdl.cuh"
 
 namespace lbk {
 
@@ -1347,20 +1349,8 @@ cudaError_t launch_batch_one(const BatchItem *items, int nitems, const SweepArgs
 template <class St, bool kTau1>
 cudaError_t launch_one(const CUtensorMap &m0, const CUtensorMap &m1, const SweepArgs &A, size_t smem,
                        cudaStream_t st) {
-  // Programmatic dependent launch: the kernel may start while the previous
-  // step finishes; it waits for that grid (griddepcontrol.wait) before
-  // touching global memory.
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)A.nstrips, (unsigned)A.nseg);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, sweep_step_kernel<St, kTau1>, m0, m1, A);
+  return pdl::launch(sweep_step_kernel<St, kTau1>, dim3((unsigned)A.nstrips, (unsigned)A.nseg), kThreads, smem, st, m0,
+                     m1, A);
 }
 
 // The multi-step kernels: one CTA per (step, item).
@@ -1395,8 +1385,8 @@ cudaError_t launch_moments_one(const CUtensorMap &m0, const CUtensorMap &m1, con
   if (e != cudaSuccess) return e;
   const uintptr_t all = (uintptr_t)n | (uintptr_t)ux | (uintptr_t)uy;  // (even nx: rows keep the alignment)
   const Moments<T> M{(T *)n, (T *)ux, (T *)uy, all % (2 * sizeof(T)) == 0 && A.nx % 2 == 0};
-  sweep_moments_kernel<St, T><<<dim3((unsigned)A.nstrips, (unsigned)A.nseg), kThreads, smem, st>>>(m0, m1, A, M);
-  return cudaGetLastError();
+  return pdl::launch(sweep_moments_kernel<St, T>, dim3((unsigned)A.nstrips, (unsigned)A.nseg), kThreads, (size_t)smem,
+                     st, m0, m1, A, M);
 }
 
 }  // namespace
