@@ -470,7 +470,7 @@ def run_batch(args):
     # one persistent launch (its chunks hold 2^30 / items steps, over a
     # million for this ensemble's few hundred items)
     launches = 1
-    kernel = "lbk::sweep_batch_kernel" if args.steps == 1 else "lbk::sweep_batch_persist_kernel"
+    kernel = "lbk::sweep_batch_kernel" if args.steps == 1 else "lbk::sweep_batch_multi_kernel"
     achieved = b_alg * sites * (args.steps // launches) / (t_ms * 1e-3 / launches) / 1e9
     traffic, traffic_basis = (profiled_traffic("batch:" + args.precision, args.steps // launches)
                               if args.steps > 1 else (None, "single-step launches are not profiled"))

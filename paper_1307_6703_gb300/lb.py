@@ -218,7 +218,7 @@ def lb_autotune(h, steps: int = 20) -> int:
 
 
 def lb_set_seg_h(h, seg_h: int) -> None:
-    """Fix the sweep kernel's segment height (rows per CTA) without tuning."""
+    """Fix the sweep kernel's segment height (rows) without tuning."""
     _check(load_library().lb_set_seg_h(h, seg_h), h)
 
 
