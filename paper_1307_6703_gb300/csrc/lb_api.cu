@@ -544,6 +544,7 @@ int multi_steps(lb_handle *h, int64_t nsteps) {
     P.dep_ofs = h->d_dep;
     P.dep_idx = h->d_dep + ntiles + 1;
     P.next = h->d_ticket;
+    P.poll_ns = lbk::sweep_poll_ns(ntiles, h->resident);
     LB_CUDA(h, cudaMemsetAsync(h->d_ticket, 0, sizeof(unsigned), h->st));
     const cudaError_t e = lbk::launch_sweep_multi(h->store, tau1(h), h->tmap, A, P, Q, h->sweep_smem, h->st);
     if (e != cudaSuccess) return cuda_fail(h, e, "lb_step: multi-step sweep kernel");
@@ -1372,6 +1373,7 @@ int lb_batch_step(lb_batch *b, int64_t nsteps) {
       P.dep_ofs = b->d_dep;
       P.dep_idx = b->d_dep + b->nitems + 1;
       P.next = b->d_ticket;
+      P.poll_ns = lbk::sweep_poll_ns(b->nitems, resident_warps(b->store, b->tau1));
       LB_BCUDA(b, cudaMemsetAsync(b->d_ticket, 0, sizeof(unsigned), b->st));
       LB_BCUDA(b, lbk::launch_sweep_batch_multi(b->store, b->tau1, b->d_items, b->d_args, b->consts, b->d_maps, P, b->smem, b->st));
       b->kpar = (b->kpar + chunk) & 1;

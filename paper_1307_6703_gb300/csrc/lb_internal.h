@@ -87,6 +87,9 @@ int sweep_tile_cols(int store, int nx, int nstrips);
 // want, for lattices of `cols` tile columns over ny rows (cols may sum over
 // several lattices).
 int sweep_seg_rule(double cols, int ny, int resident);
+// Sleep (ns) between two looks at a dependency in a launch of nitems tiles a
+// step on a device that holds `resident` warps.
+unsigned sweep_poll_ns(int nitems, int resident);
 // Warps of the sweep kernel one SM holds (shared memory and registers).
 int sweep_warps_per_sm(int store, bool tau1);
 // Widths of nstrips strips (>= sweep_min_strips, the fewest a tiling may name) over nx columns: base_w or
@@ -142,6 +145,7 @@ struct MultiArgs {
   const int *dep_ofs;   // item i depends on dep_idx[dep_ofs[i] .. dep_ofs[i+1])
   const int *dep_idx;
   unsigned *next;       // ticket counter, zero at launch
+  unsigned poll_ns;     // sleep between two looks at a counter (sweep_poll_ns)
 };
 // Outputs of the single-lattice multi-step kernel: the step that reads
 // buffer b writes fout[b] (and fdev[b], the deviation planes of 16-bit

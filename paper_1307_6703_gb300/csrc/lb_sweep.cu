@@ -40,7 +40,7 @@
 // 16-bit storage, the issue rate and the latency of 12 warps an SM.  Measured
 // per step of 4096 x 1024, tau = 1, 20 steps a launch: FP32 58.7 -> 51.9 us
 // (5,820 GB/s; 49.3 us in 200-step launches), bf16 59.4 -> 49.2 us; 512 x 256
-// FP32, 100 steps: 35.8 -> 9.7 us.
+// FP32, 100 steps: 35.8 -> 8.8 us.
 //
 // Walls: rows -1 and ny of n, P, L and n u* are the mirror images of rows 1
 // and ny-2 (even reflection; y part of n u* odd): the stages of a wall row
@@ -1200,7 +1200,7 @@ __device__ __forceinline__ bool wait_deps(const MultiArgs &P, int i, unsigned ta
     const unsigned *f = P.done + P.dep_idx[d];
     while ((int)(ld_acquire_gpu(f) - target) < 0 && n < kWaitLimit) {
       n = (n & 1023u) == 1023u && __ldcg(err) != 0 ? kWaitLimit : n + 1;
-      __nanosleep(64);
+      __nanosleep(P.poll_ns);
     }
   }
   __syncwarp();
@@ -1437,6 +1437,16 @@ int sweep_seg_rule(double cols, int ny, int resident) {
   const int h = rows < 3.0 ? 2 : std::min(kSegMax, 4 * std::max(1, (int)(rows / 4.0 + 0.5)));
   return std::min(ny, h);
 }
+
+// Where the device holds more warps than three quarters of a step's tiles need,
+// the others wait for most of a step, and their looks at the counters (a lane
+// per dependency, some 20 of them) slow the tiles that run: 256 ns between
+// them.  Measured per step against 64 ns: FP32 64 x 32 8.5 -> 7.45 us, 256 x 128
+// 11.6 -> 9.7, 512 x 256 (0.70 of the warps) 9.6 -> 8.7; batches of 4 of 64 x 32
+// and of 128 x 64 (9.4) 6.2 and 6.9.  Nearer to one tile a
+// warp the waits are short and end late with 256 ns: 768 x 256 (0.98) 9.5 us at
+// 64, 10.2 at 256; from 1024 x 256 on there is no difference.
+unsigned sweep_poll_ns(int nitems, int resident) { return 4ll * nitems <= 3ll * resident ? 256u : 64u; }
 
 void sweep_plan(int store, int nx, int ny, int *nstrips, int *seg_h) {
   *nstrips = sweep_min_strips(store, nx);
