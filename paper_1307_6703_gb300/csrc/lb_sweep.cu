@@ -1442,10 +1442,10 @@ int sweep_seg_rule(double cols, int ny, int resident) {
 // the others wait for most of a step, and their looks at the counters (a lane
 // per dependency, some 20 of them) slow the tiles that run: 256 ns between
 // them.  Measured per step against 64 ns: FP32 64 x 32 8.5 -> 7.45 us, 256 x 128
-// 11.6 -> 9.7, 512 x 256 (0.70 of the warps) 9.6 -> 8.7; batches of 4 of 64 x 32
-// and of 128 x 64 (9.4) 6.2 and 6.9.  Nearer to one tile a
-// warp the waits are short and end late with 256 ns: 768 x 256 (0.98) 9.5 us at
-// 64, 10.2 at 256; from 1024 x 256 on there is no difference.
+// 11.6 -> 9.7, 512 x 256 (0.70 of the warps) 9.6 -> 8.7; batches of four lattices
+// of 64 x 32 7.1 -> 6.2, of 128 x 64 9.4 -> 6.9.  Nearer to one tile a warp the
+// waits are short and end late with 256 ns: 768 x 256 (0.98) 9.5 us at 64, 10.2
+// at 256; from 1024 x 256 on there is no difference.
 unsigned sweep_poll_ns(int nitems, int resident) { return 4ll * nitems <= 3ll * resident ? 256u : 64u; }
 
 void sweep_plan(int store, int nx, int ny, int *nstrips, int *seg_h) {
