@@ -419,10 +419,15 @@ void set_tiles(lb_handle *h, int nstrips, int seg_h) {
 
 int ntiles(const lb_handle *h) { return h->tile_cols * h->tile_nseg; }
 
+// A tile writes its record without a bound of its own: every tiling that a
+// kernel runs must have passed this.
+size_t record_bytes(const lb_handle *h) { return 4 * sizeof(double) * (size_t)ntiles(h); }
+bool records_fit(const lb_handle *h) { return record_bytes(h) <= h->cta_bytes; }
+
 // Grow the per-tile record array to hold the current tiling's records.
 cudaError_t ensure_records(lb_handle *h) {
-  const size_t need = 4 * sizeof(double) * (size_t)ntiles(h);
-  if (need <= h->cta_bytes) return cudaSuccess;
+  if (records_fit(h)) return cudaSuccess;
+  const size_t need = record_bytes(h);
   double *p = nullptr;
   cudaError_t e = cudaStreamSynchronize(h->st);
   if (e == cudaSuccess) e = cudaMalloc((void **)&p, need);
@@ -645,7 +650,7 @@ int lb_create(const lb_params *p, lb_handle **out) {
   if (e == cudaSuccess) e = cudaMalloc((void **)&h->d_err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(h->d_err, 0, sizeof(int));
   if (e == cudaSuccess && h->sweep) {
-    h->cta_bytes = 4 * sizeof(double) * (size_t)ntiles(h);
+    h->cta_bytes = record_bytes(h);
     e = cudaMalloc((void **)&h->d_cta, h->cta_bytes);
     if (e == cudaSuccess) e = lbk::sweep_prepare(h->store, tau1(h), &h->sweep_smem);
     for (int b = 0; b < 2 && e == cudaSuccess; b++)
@@ -1328,11 +1333,14 @@ int lb_batch_create(const lb_params *ps, int32_t count, lb_batch **out) {
   for (const lb_handle *h : b->hs) tall = std::max(tall, (int)h->p.ny);
   for (const lb_handle *h : b->hs) cols += (double)h->tile_cols * h->p.ny / tall;
   const int want = lbk::sweep_seg_rule(cols, tall, resident_warps(b->store, b->tau1));
+  cudaError_t e = cudaSuccess;
   for (lb_handle *h : b->hs) {
+    // (a lattice that fills the device by itself is cut lower here than alone:
+    // more tiles, so more records than lb_create made room for)
     h->want_rows = std::min(want, (int)h->p.ny);
-    set_tiles(h, h->sweep_nstrips, h->sweep_seg);
+    if (e == cudaSuccess) e = change_tiles(h, h->sweep_nstrips, h->sweep_seg);
   }
-  cudaError_t e = lbk::sweep_prepare(b->store, b->tau1, &b->smem);
+  if (e == cudaSuccess) e = lbk::sweep_prepare(b->store, b->tau1, &b->smem);
   if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_args, 2 * (size_t)count * sizeof(lbk::SweepArgs));
   if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_maps, 4 * (size_t)count * sizeof(CUtensorMap));
   if (e != cudaSuccess) {
