@@ -467,11 +467,15 @@ cudaError_t ensure_deps(lb_handle *h) {
   h->d_dep = nullptr;
   h->d_done = nullptr;
   h->deps_gen = -1;
+  // Filled on the handle's stream: a stream of the program's own need not wait
+  // for the default one, and the next launch reads both.
   e = cudaMalloc((void **)&h->d_dep, csr.size() * sizeof(int));
-  if (e == cudaSuccess) e = cudaMemcpy(h->d_dep, csr.data(), csr.size() * sizeof(int), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc((void **)&h->d_done, (size_t)ntiles * sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMemset(h->d_done, 0, (size_t)ntiles * sizeof(unsigned));
   if (e == cudaSuccess && !h->d_ticket) e = cudaMalloc((void **)&h->d_ticket, sizeof(unsigned));
+  if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_dep, csr.data(), csr.size() * sizeof(int), cudaMemcpyHostToDevice, h->st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->d_done, 0, (size_t)ntiles * sizeof(unsigned), h->st);
+  const cudaError_t copied = cudaStreamSynchronize(h->st);  // csr goes out of scope
+  if (e == cudaSuccess) e = copied;
   if (e != cudaSuccess) return e;
   h->deps_ntiles = ntiles;
   h->epoch = 0;
