@@ -1193,6 +1193,9 @@ int fno_create(const fno_config *cfg, fno_handle **out) {
     for (cudaEvent_t *v : {&h->ev_dz, &h->ev_sums, &h->ev_dw[0], &h->ev_dw[1]})
       if (e == cudaSuccess) e = cudaEventCreateWithFlags(v, cudaEventDisableTiming);
   }
+  // The clears went to the default stream, for which a stream of the program's
+  // own need not wait.
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
   if (e != cudaSuccess) {
     std::string m = std::string("fno_create: ") + cudaGetErrorString(e);
     fno_destroy(h);

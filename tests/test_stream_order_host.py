@@ -55,6 +55,29 @@ def _steps(fake):
     return out
 
 
+def _create(fake):
+    """New handles, until the call returns."""
+    import paper_1307_6703_gb300 as lbm
+    from paper_1307_6703_gb300 import fno
+    out = {}
+    for what, nx, prec in (("fp64", 33, 0), ("fp32", 64, 1), ("odd", 57, 1), ("bf16", 64, 2)):
+        fake.clear()
+        lbm.lb_create(_params(lbm, nx, 32, prec))
+        out[what] = _unordered(fake.calls)
+    fake.clear()
+    lbm.Batch([_params(lbm, 64, 32, 1)] * 2, stream=STREAM)
+    out["batch"] = _unordered(fake.calls)
+    fake.clear()
+    fno.Fno(nx_max=64, ny_max=32, stream=STREAM)
+    out["network"] = _unordered(fake.calls)
+    return out
+
+
+def test_a_new_handle_is_cleared_when_its_call_returns(tmp_path):
+    out = host_call(__file__, "_create", tmp_path)
+    assert out == {k: [] for k in ("fp64", "fp32", "odd", "bf16", "batch", "network")}
+
+
 def test_dependency_lists_are_filled_on_the_handles_stream(tmp_path):
     assert host_call(__file__, "_steps", tmp_path) == {"fp32": [], "bf16": [], "odd": [], "batch": []}
 
