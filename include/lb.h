@@ -187,6 +187,14 @@ int lb_reduce_async(lb_handle *h, double *out);
  * address), LB_ERR_CUDA, LB_ERR_OOM.                                       */
 int lb_monitor(lb_handle *h, double *host_ring, int32_t capacity);
 
+/* Failure detection, for tests: every wait of the sweep kernels is bounded.
+ * Sets how many looks at a copy's barrier a wait of the launches of one step
+ * takes before it gives up (2^22 from the start; 0: every wait gives up).  A
+ * launch in which a wait gave up stops early, keeps every access in bounds and
+ * leaves no valid state or sums; lb_reduce then returns LB_ERR_TIMEOUT, for as
+ * long as the handle lives.  Errors: LB_ERR_ARG (instances of a batch).     */
+int lb_set_wait_limit(lb_handle *h, uint32_t looks);
+
 /* Checkpoint: copy the stored populations to the HOST buffer buf:
  * [9][ny][nx] elements of the storage precision (double for LB_FP64, float
  * for LB_FP32); for 16-bit storage the float rest plane [ny][nx] followed by

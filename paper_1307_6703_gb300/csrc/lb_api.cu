@@ -71,6 +71,7 @@ struct lb_handle {
   unsigned *d_mon_arr = nullptr; // their arrival counters (zero between launches)
   int mon_tiles = 0;             // tiles the slots were sized for
   bool in_batch = false;         // instance of an lb_batch
+  unsigned wait_limit = lbk::kSweepWaitLimit;  // of single steps (lb_set_wait_limit)
   int red_blocks = 0;
   int64_t step = 0;
   bool initialised = false;
@@ -385,6 +386,7 @@ lbk::SweepArgs sweep_args(const lb_handle *h, int in) {
   A.fdev = planes16(h->f[in ^ 1]);
   A.partials = h->d_cta;
   A.records = 1;
+  A.wait_limit = h->wait_limit;
   A.err = h->d_err;
   A.total = nullptr;
   A.arrivals = nullptr;
@@ -916,6 +918,13 @@ int lb_monitor(lb_handle *h, double *host_ring, int32_t capacity) {
   LB_CUDA(h, ensure_mon_slots(h, ntiles(h)));
   h->mon_ring = static_cast<double *>(dev);
   h->mon_cap = capacity;
+  return LB_OK;
+}
+
+int lb_set_wait_limit(lb_handle *h, uint32_t looks) {
+  if (!h) return LB_ERR_ARG;
+  if (h->in_batch) return fail(h, LB_ERR_ARG, "lb_set_wait_limit: only outside a batch");
+  h->wait_limit = looks;
   return LB_OK;
 }
 

@@ -53,6 +53,7 @@ struct SweepArgs {
   void *fdev;
   double *partials;            // 4 doubles per CTA: mass, J_x, J_y, bad-site flag
   int records;                 // write the per-CTA records (0: skip them)
+  unsigned wait_limit;         // looks at a copy's barrier before a wait of a single step gives up
   int *err;                    // set when a bounded wait gave up
   // Non-null (single-lattice launches with records only): the last CTA to
   // finish sums every CTA's record in a fixed order into total[0..4] --
@@ -65,6 +66,9 @@ struct SweepArgs {
   double *monitor;
   double mon_step;
 };
+
+// Looks at a barrier or a counter before a wait of the sweep kernels gives up.
+constexpr unsigned kSweepWaitLimit = 1u << 22;
 
 // Storage formats of the sweep kernel (values of lb_precision).
 constexpr int kStoreF32 = 1, kStoreBF16 = 2, kStoreFP16 = 3;

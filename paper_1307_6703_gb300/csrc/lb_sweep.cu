@@ -101,7 +101,6 @@ static_assert(kCols == kSweepWindow, "the dependency lists cover the window");
 constexpr int kTileW = kCols - 8;           // widest tile
 constexpr int kThreads = 32;
 constexpr unsigned kAll = 0xffffffffu;
-constexpr uint32_t kWaitLimit = 1u << 22;
 // Rows of a tile where the tiling's segments would leave warps idle: about
 // kTilesPerWarp tiles of a step per resident warp, so that a tile's neighbours
 // have finished the previous step by the time its ticket is drawn; a multiple
@@ -688,7 +687,8 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
     for (int p = 0; p < issued; ++p) request(p, p);
   }
   __syncwarp();
-  bool ok = mbar_wait(smem_u32(&S.full[0]), 0, kWaitLimit);
+  const uint32_t limit = kMulti ? kSweepWaitLimit : A.wait_limit;
+  bool ok = mbar_wait(smem_u32(&S.full[0]), 0, limit);
   // What the stages carry from one iteration to the next (rows relative to
   // the next iteration's a).
   const float2 zero = make_float2(0.f, 0.f);
@@ -715,7 +715,7 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
     const int s1 = s0 == kPairs - 1 ? 0 : s0 + 1;
     // newest pair needed: k+1.  After a wait that gave up a lane waits no more
     // and goes on with whatever is there (in bounds) to the tile's end.
-    ok = mbar_wait(smem_u32(&S.full[s1]), par, ok ? kWaitLimit : 1u) && ok;
+    ok = mbar_wait(smem_u32(&S.full[s1]), par, ok ? limit : 1u) && ok;
     __syncwarp();
     if (s1 == kPairs - 1) par ^= 1u;
     const int a = ya - 3 + 2 * k;
@@ -996,7 +996,7 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
     // lands in shared memory after the warp has moved on, then stop.
     if (t == 0) {
       for (int p = max(0, issued - kPairs); p < issued; ++p)
-        (void)mbar_wait(smem_u32(&S.full[p % kPairs]), (uint32_t)((p / kPairs) & 1), kWaitLimit);
+        (void)mbar_wait(smem_u32(&S.full[p % kPairs]), (uint32_t)((p / kPairs) & 1), kSweepWaitLimit);
     }
     __syncwarp();
     return false;
@@ -1083,8 +1083,10 @@ sweep_step_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant
                   const __grid_constant__ SweepArgs A) {
   const StepIO O{A.fin, A.fdin, A.fout, A.fdev, A.partials, gridDim.x * gridDim.y, A.total ? A.arrivals : nullptr,
                  A.total, A.monitor, A.mon_step};
-  (void)sweep_body<St, kTau1>(&tin, &tdev, A, A.k, O, blockIdx.x, blockIdx.y,
-                       A.partials + 4 * ((size_t)blockIdx.y * gridDim.x + blockIdx.x), A.records != 0);
+  if (!sweep_body<St, kTau1>(&tin, &tdev, A, A.k, O, blockIdx.x, blockIdx.y,
+                             A.partials + 4 * ((size_t)blockIdx.y * gridDim.x + blockIdx.x), A.records != 0)) {
+    if (threadIdx.x == 0 && A.total) A.total[4] = 1.0;  // the sums of this launch will not be written
+  }
 }
 
 // A lattice's arguments into shared memory (constants read by every lane).
@@ -1198,13 +1200,13 @@ __device__ __forceinline__ bool wait_deps(const MultiArgs &P, int i, unsigned ta
   uint32_t n = 0;
   for (int d = P.dep_ofs[i] + (int)threadIdx.x; d < d1; d += kThreads) {
     const unsigned *f = P.done + P.dep_idx[d];
-    while ((int)(ld_acquire_gpu(f) - target) < 0 && n < kWaitLimit) {
-      n = (n & 1023u) == 1023u && __ldcg(err) != 0 ? kWaitLimit : n + 1;
+    while ((int)(ld_acquire_gpu(f) - target) < 0 && n < kSweepWaitLimit) {
+      n = (n & 1023u) == 1023u && __ldcg(err) != 0 ? kSweepWaitLimit : n + 1;
       __nanosleep(P.poll_ns);
     }
   }
   __syncwarp();
-  if (__any_sync(kAll, n >= kWaitLimit)) {
+  if (__any_sync(kAll, n >= kSweepWaitLimit)) {
     if (threadIdx.x == 0) atomicOr(err, 4);
     return false;
   }

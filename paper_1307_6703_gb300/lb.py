@@ -72,6 +72,7 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
         lib.lb_reduce.argtypes = [P, C.POINTER(C.c_double)]
         lib.lb_reduce_async.argtypes = [P, P]
         lib.lb_monitor.argtypes = [P, P, C.c_int32]
+        lib.lb_set_wait_limit.argtypes = [P, C.c_uint32]
         lib.lb_get_state.argtypes = [P, P, C.POINTER(C.c_size_t)]
         lib.lb_set_state.argtypes = [P, P, C.c_size_t, C.c_int64]
         lib.lb_get_step.argtypes = [P, C.POINTER(C.c_int64)]
@@ -177,6 +178,11 @@ def lb_monitor(h, ring=None, capacity: int = 0) -> None:
     if ring is not None and capacity == 0:
         capacity = int(ring.numel() if hasattr(ring, "numel") else ring.size) // 6
     _check(load_library().lb_monitor(h, _addr(ring), capacity if ring is not None else 0), h)
+
+
+def lb_set_wait_limit(h, looks: int) -> None:
+    """Looks at a copy's barrier before a wait of single steps gives up."""
+    _check(load_library().lb_set_wait_limit(h, looks), h)
 
 
 def lb_get_state(h, buf=None) -> int:
