@@ -42,6 +42,16 @@ namespace {
 constexpr int kThreads = 128;
 constexpr int C = kWidth;
 
+// The tile of a block: tiles of a row in turn, then rows, all along the grid's
+// x (its y ends at 65,535: fewer than a field's rows may be), fields along z.
+struct Tile {
+  int x, y, b;
+};
+__device__ __forceinline__ Tile tile_of(int nx) {
+  const unsigned across = (unsigned)(nx + tc::kBM - 1) / tc::kBM, y = blockIdx.x / across;
+  return {(int)(blockIdx.x - y * across) * tc::kBM, (int)y, (int)blockIdx.z};
+}
+
 // Operand tiles of a layer kernel; kK: K columns of a tile (32 where 2 modes_x
 // allows, with 64-byte swizzle rows: half the shared memory, twice the CTAs).
 template <int kK>
@@ -177,7 +187,8 @@ layer_kernel(const __grid_constant__ CUtensorMap ma1, const __grid_constant__ CU
   using Sm = LayerSmem<kK>;
   Sm &S = *reinterpret_cast<Sm *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int xt = blockIdx.x * tc::kBM, y = blockIdx.y, b = blockIdx.z;
+  const Tile T = tile_of(p.nx);
+  const int xt = T.x, y = T.y, b = T.b;
   const uint32_t tmem = setup(&S.tmem, 64, &S.full, 2);
   if (t == 0) {
     const uint32_t bar = tc::smem_u32(&S.full);
@@ -259,7 +270,8 @@ lift_kernel(int nx, int ny, const float *__restrict__ prm, const float *__restri
   for (int i = threadIdx.x; i < C * kFeat; i += kThreads) Ps[i] = P[i];
   if (threadIdx.x < C) ps[threadIdx.x] = pb[threadIdx.x];
   __syncthreads();
-  const int x = blockIdx.x * kThreads + threadIdx.x, y = blockIdx.y, b = blockIdx.z;
+  const Tile T = tile_of(nx);
+  const int x = T.x + threadIdx.x, y = T.y, b = T.b;
   if (x >= nx) return;
   const long long sites = (long long)nx * ny, s = (long long)y * nx + x;
   float f[kFeat];
@@ -316,7 +328,8 @@ project_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ C
   using Sm = ProjSmem<H>;
   Sm &S = *reinterpret_cast<Sm *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int xt = blockIdx.x * tc::kBM, y = blockIdx.y, b = blockIdx.z;
+  const Tile T = tile_of(p.nx);
+  const int xt = T.x, y = T.y, b = T.b;
   constexpr uint32_t kCols = kBack ? 128 : H;  // accumulators: H, then C (a power of two in all)
   for (int i = t; i < H; i += kThreads) S.q1[i] = p.q1[i];
   for (int i = t; i < p.O * H; i += kThreads) S.Q2[i] = p.Q2[i];
@@ -446,7 +459,7 @@ project_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ C
       S.red[warp][base + p.O] = tail[kMaxO];
     }
     __syncthreads();
-    double *part = p.part + (((long long)b * gridDim.y + y) * gridDim.x + blockIdx.x) * n;
+    double *part = p.part + ((long long)b * gridDim.x + blockIdx.x) * n;
     for (int i = t; i < n; i += kThreads) part[i] = ((S.red[0][i] + S.red[1][i]) + S.red[2][i]) + S.red[3][i];
   }
   release_tmem(tmem, kCols);
@@ -504,7 +517,9 @@ __global__ void finish_kernel(const double *__restrict__ part2, int nval, SumOut
   if (e == 0) *loss = r / count;
 }
 
-dim3 tile_grid(const Shape &s) { return dim3((unsigned)((s.nx + tc::kBM - 1) / tc::kBM), (unsigned)s.ny, (unsigned)s.B); }
+dim3 tile_grid(const Shape &s) {
+  return dim3((unsigned)((s.nx + tc::kBM - 1) / tc::kBM) * (unsigned)s.ny, 1, (unsigned)s.B);
+}
 
 template <class K>
 cudaError_t allow_smem(K kernel, size_t bytes) {

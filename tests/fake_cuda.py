@@ -42,6 +42,11 @@ class Fake:
         """Bytes of device memory from p on (0: not device memory)."""
         return self.rt.fake_room(p)
 
+    def device(self, nbytes):
+        p = C.c_void_p()
+        assert self.rt.cudaMalloc(C.byref(p), C.c_size_t(nbytes)) == 0
+        return p.value
+
     def names(self):
         return [c[0] for c in self.calls]
 
