@@ -15,11 +15,18 @@ from paper_1307_6703_gb300.workloads import C2  # noqa: E402
 
 @pytest.mark.parametrize("prec,nx,ny", [(LB_FP32, 64, 32), (LB_FP32, 512, 256), (LB_BF16DEV, 64, 32), (LB_FP32, 57, 20)])
 @pytest.mark.parametrize("tau", [1.0, 2.0])
-def test_a_single_step_that_gives_up_is_reported(prec, nx, ny, tau):
+@pytest.mark.parametrize("monitored", [False, True])  # (then the last tile adds the records up)
+def test_a_single_step_that_gives_up_is_reported(prec, nx, ny, tau, monitored):
+    if monitored and nx % 4:
+        pytest.skip("no monitoring of these widths")
     import torch
     w = C2(0.05).with_(nx=nx, ny=ny, tau=tau, lam=32.0)
     make = (lambda: solver_for(w, prec)) if prec == LB_FP32 else (lambda: dev16_solver(w, prec, 1.0))
-    s = make().init_noise(1, 1.0, 0.01).step(1)
+    s = make().init_noise(1, 1.0, 0.01)
+    if monitored:
+        ring = torch.zeros((16, 6), dtype=torch.float64).pin_memory()
+        s.monitor(ring)
+    s.step(1)
     assert s.reduce()[0] == 0
     lb_set_wait_limit(s.h, 0)
     s.step(1)

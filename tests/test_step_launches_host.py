@@ -1,0 +1,47 @@
+"""What lb_step enqueues (host logic, on a CUDA runtime without a GPU)."""
+import ctypes as C
+import json
+import os
+import sys
+
+import pytest
+
+from fake_cuda import STREAM, Fake, host_call
+
+
+def _handle(lbm, nx, ny, prec=1, tau=1.0):
+    h = lbm.lb_create(lbm.lb_params(nx, ny, 1, prec, 0.375, 1 / 3, 0.3, 0.1, tau, 1e-4, 32.0, 0.0, 0.0, 0.3, 2.0, 0.0,
+                                    STREAM))
+    lbm.lb_init(h, 0, 1, 1.0, 0.01)
+    return h
+
+
+def _single_step_sums(fake):
+    """Device pointers of a single step's arguments."""
+    import paper_1307_6703_gb300 as lbm
+    out = []
+
+    def on_launch(name, grid, args):
+        words = (C.c_uint64 * 60).from_address(args[2])
+        out.append(len({w for w in words if fake.room(w)}))
+    for prec in (1, 2):
+        h = _handle(lbm, 512, 256, prec)
+        fake.on_launch = on_launch
+        lbm.lb_step(h, 1)
+        fake.on_launch = None
+        fake.clear()
+        lbm.lb_reduce(h, [0.0] * 3)
+        out.append([n for n in ("reduce_cta", "reduce_pass1") if any(n in c for c in fake.names())])
+    return out
+
+
+def test_single_steps_leave_the_records_to_the_reduction(tmp_path):
+    """sinx, the two states (and their 16-bit planes), records and error flag:
+    no arrival counter and no sums, which the last tile would add up in one warp
+    after the step; lb_reduce adds the records."""
+    assert host_call(__file__, "_single_step_sums", tmp_path) == [5, ["reduce_cta"], 7, ["reduce_cta"]]
+
+
+if __name__ == "__main__":
+    os.makedirs(sys.argv[2], exist_ok=True)
+    print(json.dumps(globals()[sys.argv[1]](Fake(sys.argv[2]))))
