@@ -453,8 +453,11 @@ cudaError_t change_tiles(lb_handle *h, int nstrips, int seg_h) {
 }
 
 // Dependency lists and counters of the multi-step kernel for the current
-// tiling (rebuilt when the tiling changes; counters then restart at 0).
-cudaError_t ensure_deps(lb_handle *h) {
+// tiling (rebuilt when the tiling changes; counters then restart at 0), filled
+// on stream st: the handle's -- a stream of the program's own need not wait for
+// the default one, and the next launch reads both -- or, before the handle is
+// in use, the default stream.
+cudaError_t ensure_deps(lb_handle *h, cudaStream_t st) {
   if (h->deps_gen == h->plan_gen) return cudaSuccess;
   std::vector<int> ofs, idx;
   lbk::sweep_deps(h->store, h->p.nx, h->p.ny, h->p.walls, h->tile_cols, h->tile_base, h->tile_extra, h->tile_rows,
@@ -462,21 +465,19 @@ cudaError_t ensure_deps(lb_handle *h) {
   const int ntiles = h->tile_cols * h->tile_nseg;
   std::vector<int> csr(ofs);
   csr.insert(csr.end(), idx.begin(), idx.end());
-  cudaError_t e = cudaStreamSynchronize(h->st);  // no launch may still use the old lists
+  cudaError_t e = cudaStreamSynchronize(st);  // no launch may still use the old lists
   if (e != cudaSuccess) return e;
   cudaFree(h->d_dep);
   cudaFree(h->d_done);
   h->d_dep = nullptr;
   h->d_done = nullptr;
   h->deps_gen = -1;
-  // Filled on the handle's stream: a stream of the program's own need not wait
-  // for the default one, and the next launch reads both.
   e = cudaMalloc((void **)&h->d_dep, csr.size() * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc((void **)&h->d_done, (size_t)ntiles * sizeof(unsigned));
   if (e == cudaSuccess && !h->d_ticket) e = cudaMalloc((void **)&h->d_ticket, sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_dep, csr.data(), csr.size() * sizeof(int), cudaMemcpyHostToDevice, h->st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->d_done, 0, (size_t)ntiles * sizeof(unsigned), h->st);
-  const cudaError_t copied = cudaStreamSynchronize(h->st);  // csr goes out of scope
+  if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_dep, csr.data(), csr.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->d_done, 0, (size_t)ntiles * sizeof(unsigned), st);
+  const cudaError_t copied = cudaStreamSynchronize(st);  // csr goes out of scope
   if (e == cudaSuccess) e = copied;
   if (e != cudaSuccess) return e;
   h->deps_ntiles = ntiles;
@@ -518,7 +519,7 @@ cudaError_t ensure_mon_slots(lb_handle *h, int ntiles) {
 
 // nsteps >= 2 steps of a strip-sweep handle in multi-step launches.
 int multi_steps(lb_handle *h, int64_t nsteps) {
-  LB_CUDA(h, ensure_deps(h));
+  LB_CUDA(h, ensure_deps(h, h->st));
   const int ntiles = h->deps_ntiles;
   const lbk::SweepArgs A = sweep_args(h, h->cur);
   lbk::MultiOut Q{};
@@ -570,19 +571,19 @@ int multi_steps(lb_handle *h, int64_t nsteps) {
 }
 
 // Whether lb_step may use multi-step launches.  Lattices of odd widths can be
-// stepped inside a stream capture and without memory of their own (their steps
-// were independent launches, which a graph may replay): there they keep single
-// steps.
+// stepped inside a stream capture, without memory of their own and without a
+// synchronisation (their steps were independent launches, which a graph may
+// replay): their dependency lists are made by lb_create, where there is memory
+// for them, and inside a capture, or without lists, they keep single steps.
 bool multi_allowed(lb_handle *h) {
   if (!h->odd) return true;
+  if (h->deps_gen != h->plan_gen) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(h->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+  if (cudaStreamIsCapturing(h->st, &cap) != cudaSuccess) {
     (void)cudaGetLastError();
     return false;
   }
-  if (ensure_deps(h) == cudaSuccess) return true;
-  (void)cudaGetLastError();
-  return false;
+  return cap == cudaStreamCaptureStatusNone;
 }
 
 }  // namespace
@@ -684,6 +685,7 @@ int lb_create(const lb_params *p, lb_handle **out) {
       free(tab);
     }
   }
+  if (e == cudaSuccess && h->odd && ensure_deps(h, nullptr) != cudaSuccess) (void)cudaGetLastError();  // (see multi_allowed)
   // The clears and the copy went to the default stream, for which a stream of
   // the program's own need not wait.
   if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);

@@ -17,7 +17,8 @@ typedef void (*report_fn)(const char *call, void *stream, void *ptr, size_t byte
 enum { kOk = 0, kNoMemory = 2, kMaxAllocs = 4096, kMaxKernels = 512 };
 
 static report_fn g_report;
-static int g_sms = 152, g_capturing, g_fail_over;
+static int g_sms = 152, g_capturing;
+static size_t g_fail_at;
 static struct { char *p; size_t n; } g_alloc[kMaxAllocs];
 static struct { const void *host; const char *name; } g_kernel[kMaxKernels];
 static int g_nkernels;
@@ -26,8 +27,8 @@ static launch_config g_pushed;
 void fake_report(report_fn f) { g_report = f; }
 void fake_sms(int n) { g_sms = n; }
 void fake_capturing(int on) { g_capturing = on; }
-/* Allocations of more than n bytes fail (0: none does). */
-void fake_fail_over(int n) { g_fail_over = n; }
+/* Allocations of exactly n bytes fail (0: none does). */
+void fake_fail_at(int n) { g_fail_at = (size_t)n; }
 /* Bytes from p to the end of its allocation, 0 outside all of them. */
 size_t fake_room(const char *p) {
   for (int i = 0; i < kMaxAllocs; ++i)
@@ -42,7 +43,7 @@ static int say(const char *call, void *stream, void *ptr, size_t n) {
 
 int cudaMalloc(void **p, size_t n) {
   say("cudaMalloc", NULL, NULL, n);
-  if (g_fail_over && n > (size_t)g_fail_over) return kNoMemory;
+  if (g_fail_at && n == g_fail_at) return kNoMemory;
   for (int i = 0; i < kMaxAllocs; ++i) {
     if (g_alloc[i].p) continue;
     void *m = mmap(NULL, n ? n : 1, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
