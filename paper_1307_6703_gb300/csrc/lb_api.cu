@@ -570,6 +570,16 @@ int multi_steps(lb_handle *h, int64_t nsteps) {
   return LB_OK;
 }
 
+// Whether many steps of a lattice of odd width are faster in one launch: where a
+// step has more tiles than the device holds warps.  Below that the tiles of
+// single steps, launched as programmatic dependents, all start at once, without
+// tickets and counters.  Measured per step, single / multi-step (the tile kernel
+// of compact planes before): 33 x 33 6.0 / 6.8 us (8.4), 57 x 64 6.0 / 8.9 (8.4),
+// 2049 x 33 6.4 / 12.8 (10.5), 4095 x 16 6.7 / 12.4 (10.5), 509 x 256 (1280 tiles
+// of 1824 warps) 7.8 / 12.4 (14.5); 15 x 4000 (2000 tiles) 12.4 / 9.1 (12.6), 4093
+// x 1024 (2368) 68 / 54 (243).
+bool odd_multi(const lb_handle *h) { return ntiles(h) > h->resident; }
+
 // Whether lb_step may use multi-step launches.  Lattices of odd widths can be
 // stepped inside a stream capture, without memory of their own and without a
 // synchronisation (their steps were independent launches, which a graph may
@@ -685,7 +695,8 @@ int lb_create(const lb_params *p, lb_handle **out) {
       free(tab);
     }
   }
-  if (e == cudaSuccess && h->odd && ensure_deps(h, nullptr) != cudaSuccess) (void)cudaGetLastError();  // (see multi_allowed)
+  if (e == cudaSuccess && h->odd && odd_multi(h) && ensure_deps(h, nullptr) != cudaSuccess)
+    (void)cudaGetLastError();  // (see multi_allowed)
   // The clears and the copy went to the default stream, for which a stream of
   // the program's own need not wait.
   if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);

@@ -75,7 +75,7 @@ def test_steps_of_odd_widths_only_enqueue(tmp_path):
     """[multi-step launches, single steps, calls that allocate or wait]"""
     out = host_call(__file__, "_odd", tmp_path)
     assert all(v[2] == [] for v in out.values()), out
-    assert out["large"][:2] == [2, 0]
+    assert out["small"][:2] == [0, 8] and out["large"][:2] == [2, 0]
     assert out["no_memory"][:2] == [0, 8] and out["capture"][:2] == [0, 8]
 
 
