@@ -79,6 +79,29 @@ def test_steps_of_odd_widths_only_enqueue(tmp_path):
     assert out["no_memory"][:2] == [0, 8] and out["capture"][:2] == [0, 8]
 
 
+def _state(fake):
+    """Strided copies of a state read and set, with and without memory for the
+    staging buffer."""
+    import numpy as np
+    import paper_1307_6703_gb300 as lbm
+    out = []
+    for prec, nx in ((1, 57), (1, 64), (2, 64)):
+        for room in (True, False):
+            h = _handle(lbm, nx, 32, prec)
+            f = np.zeros(lbm.lb_get_state(h), dtype=np.uint8)
+            fake.rt.fake_fail_at(0 if room else f.nbytes)
+            fake.clear()
+            lbm.lb_get_state(h, f)
+            lbm.lb_set_state(h, f)
+            fake.rt.fake_fail_at(0)
+            out.append(fake.names().count("cudaMemcpy2DAsync"))
+    return out
+
+
+def test_states_are_copied_in_one_piece(tmp_path):
+    assert host_call(__file__, "_state", tmp_path) == [0, 18] * 3
+
+
 if __name__ == "__main__":
     os.makedirs(sys.argv[2], exist_ok=True)
     print(json.dumps(globals()[sys.argv[1]](Fake(sys.argv[2]))))
