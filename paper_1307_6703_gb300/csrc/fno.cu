@@ -865,9 +865,9 @@ constexpr int kWSplit = 8;
 // gemm_tc.h for the argument layout.
 cudaError_t tcg(fno_handle *h, const __nv_bfloat16 *X, int ldx, long long sX, const __nv_bfloat16 *Y, int ldy,
                 long long sY, float *C, long long cm, long long cn, long long sC, int M, int N, int K, int batch,
-                int ksplit, float beta, bool side = false) {
+                int ksplit, float beta, cudaStream_t st = nullptr) {
   return tc::gemm_tn_bf16(X, ldx, sX, Y, ldy, sY, C, cm, cn, sC, M, N, K, batch, ksplit, beta, h->gerr,
-                          side ? h->side : h->st);
+                          st ? st : h->st);
 }
 
 // SIMT product (FP32 mode): C(m, n) = sum_k A(m, k) B(k, n), general strides.
@@ -877,7 +877,6 @@ cudaError_t sg(fno_handle *h, const float *A, long long am, long long ak, long l
   return tc::gemm_f32(A, am, ak, sA, B, bk, bn, sB, C, cm, cn, sC, M, N, K, batch, beta, h->st);
 }
 
-// Site-major copy of a [B][rows][S] BF16 activation: out[b][s][row].
 // Dynamic shared memory of the spectral kernels (bytes).
 // kx of a block of ydft_kernel.
 int ydft_group(int lines, int mx) { return lines >= 128 ? mx : std::min(mx, 4); }
@@ -886,12 +885,26 @@ size_t iy_smem(int mx, int my) { return (size_t)(2 * my * mx + 2 * my * kYChunk)
 dim3 iy_grid(int lines, int ny) { return dim3((unsigned)lines, (unsigned)((ny + kYChunk - 1) / kYChunk)); }
 size_t mix_smem(int B, int C, bool back) { return (size_t)((back ? 4 : 2) * B * C + 2 * C * C) * sizeof(float); }
 
+// The mixing kernels: one block per mode, fewer than SMs, and their time grows
+// with the fields.  Scheduled early, as dependents of the y-transform, the blocks
+// crowd onto the SMs that have room first; from kMixEarly fields on that costs
+// more than the gap before the grid (training steps of 64 fields of 32 x 16: 1391
+// us early, 738 not, of 64 x 64 2075 and 1425; of 24 fields 448 and 417; of 8
+// fields, early is the faster by 10 us).
+constexpr int kMixEarly = 24;
+template <class K, class... A>
+void launch_mix(int B, K kernel, int modes, size_t smem, cudaStream_t st, A... args) {
+  if (B < kMixEarly) (void)pdl::launch(kernel, modes, kThreads, smem, st, args...);
+  else kernel<<<modes, kThreads, smem, st>>>(args...);
+}
+
 void ydft(fno_handle *h, const float *A, int lines, int ny, float *Sh) {
   const int mx = h->c.modes_x, my = h->c.modes_y, gx = ydft_group(lines, mx);
   (void)pdl::launch(ydft_kernel, dim3((unsigned)lines, (unsigned)((mx + gx - 1) / gx)), kThreads, ydft_smem(gx, my),
                     h->st, A, h->Ty, ny, mx, my, gx, Sh);
 }
 
+// Site-major copy of a [B][rows][S] BF16 activation: out[b][s][row].
 void site_major(fno_handle *h, const __nv_bfloat16 *in, int B, int rows, long long S, __nv_bfloat16 *out) {
   const dim3 grid((unsigned)((rows + 31) / 32), (unsigned)((S + 63) / 64), (unsigned)B);
   if (rows % 32 == 0 && S % 8 == 0)
@@ -1048,7 +1061,7 @@ int forward_fused(fno_handle *h, int B, int nx, int ny, const float *params_dev,
   for (int l = 0; l < L; l++) {
     FNO_GEMM(h, tcg(h, h->Vb[l], nx, 0, h->FxTb, nx, 0, h->A, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 1, 0.f));
     ydft(h, h->A, B * c.width, ny, h->Sh[l]);
-    (void)pdl::launch(mix_kernel, my * mx, kThreads, mix_smem(B, c.width, false), st,
+    launch_mix(B, mix_kernel, my * mx, mix_smem(B, c.width, false), st,
                       h->Sh[l], P + h->o.Rr[l], P + h->o.Ri[l], B, c.width, my * mx, h->dY);
     (void)pdl::launch(iy_kernel, iy_grid(B * c.width, ny), kThreads, iy_smem(mx, my), st,
                       h->dY, h->Ty, ny, mx, my, nullptr, h->Gb);
@@ -1091,6 +1104,16 @@ struct SideJoin {
 // spectral path and the layer below: a training step of 8 fields of 512 x 128
 // 1650 -> 1414 us, of 16 fields of 256 x 64 1066 -> 963 us.
 //
+//
+// That is so while they leave room: each of their CTAs (one per field and K
+// share) holds 80 KB of shared memory.  Up to kBesideParts of them they run
+// beside, above in turn, measured at 32 x 16, 64 x 64 and 256 x 64 (us a training
+// step, beside / in turn, mixing launched as launch_mix says): 16 fields 383 / 366,
+// 570 / 582 and 772 / 845, 24 fields 438 / 417, 720 / 716 and 1070 / 1099, 32 fields
+// 700 / 474, 944 / 835 and 1356 / 1310, 64 fields 1027 / 738, 2006 / 1425 and 2963 /
+// 2416 (separate kernels: 964, 1865 and 4857).
+constexpr int kBesideParts = 24 * kWSplit;
+
 // Backward pass on the fused kernels.
 int backward_fused(fno_handle *h, const float *target, double *loss) {
   const fno_config &c = h->c;
@@ -1108,6 +1131,8 @@ int backward_fused(fno_handle *h, const float *target, double *loss) {
   // written when the first layer is, after dW of the second.
   __nv_bfloat16 *const dz[2] = {h->dZb, reinterpret_cast<__nv_bfloat16 *>(h->dV)};
   SideJoin join{h};
+  const bool beside = parts <= kBesideParts;
+  cudaStream_t sd = beside ? h->side : st;
   FNO_GEMM(h, fno::project_backward(sh, h->VbT[L], h->prmb + o.Q1, P + o.q1, P + o.Q2, h->wTb + (size_t)L * C * C,
                                     h->out, target, h->dhpb, dz[(L - 1) & 1], h->dZT, h->quads, h->fpart, h->gerr, st));
   const int nval = fno::project_back_sums(sh);
@@ -1117,22 +1142,22 @@ int backward_fused(fno_handle *h, const float *target, double *loss) {
     const __nv_bfloat16 *dzl = dz[l & 1];
     // on the side: dw = sum dz, dW = sum_b dz[b] v[b]^T (and of the projection
     // dQ1 = sum_b dhp[b] v_L[b]^T)
-    FNO_CUDA(h, join.fork());
-    quad_reduce(h, h->quads, B, C, S, g + o.w[l], h->side);
-    FNO_CUDA(h, cudaEventRecord(h->ev_sums, h->side));
+    if (beside) FNO_CUDA(h, join.fork());
+    quad_reduce(h, h->quads, B, C, S, g + o.w[l], sd);
+    if (beside) FNO_CUDA(h, cudaEventRecord(h->ev_sums, sd));
     FNO_GEMM(h, tcg(h, dzl, (int)S, CS, h->Vb[l], (int)S, CS, h->wpart, C, 1, (long long)C * C, C, C, (int)S, B,
-                    kWSplit, 0.f, true));
-    (void)pdl::launch(sum_fields_kernel, (C * C + 31) / 32, kThreads, 0, h->side, h->wpart, parts, C * C, g + o.W[l]);
-    FNO_CUDA(h, cudaEventRecord(h->ev_dw[l & 1], h->side));
+                    kWSplit, 0.f, sd));
+    (void)pdl::launch(sum_fields_kernel, (C * C + 31) / 32, kThreads, 0, sd, h->wpart, parts, C * C, g + o.W[l]);
+    if (beside) FNO_CUDA(h, cudaEventRecord(h->ev_dw[l & 1], sd));
     if (l == L - 1) {
       FNO_GEMM(h, tcg(h, h->dhpb, (int)S, HS, h->Vb[L], (int)S, CS, h->wpart, C, 1, (long long)H * C, H, C, (int)S, B,
-                      kWSplit, 0.f, true));
-      (void)pdl::launch(sum_fields_kernel, (H * C + 31) / 32, kThreads, 0, h->side, h->wpart, parts, H * C, g + o.Q1);
+                      kWSplit, 0.f, sd));
+      (void)pdl::launch(sum_fields_kernel, (H * C + 31) / 32, kThreads, 0, sd, h->wpart, parts, H * C, g + o.Q1);
     }
     // spectral path: dG = dz Fxi^T, the adjoints of the mixing and of the y-transforms
     FNO_GEMM(h, tcg(h, dzl, nx, 0, h->Fxib, nx, 0, h->dG, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 1, 0.f));
     ydft(h, h->dG, B * C, ny, h->dY);
-    (void)pdl::launch(mix_back_kernel, my * mx, kThreads, mix_smem(B, C, true), st,
+    launch_mix(B, mix_back_kernel, my * mx, mix_smem(B, C, true), st,
                       h->dY, h->Sh[l], P + o.Rr[l], P + o.Ri[l], B, C, my * mx, h->dS, g + o.Rr[l], g + o.Ri[l]);
     (void)pdl::launch(iy_kernel, iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st,
                       h->dS, h->Ty, ny, mx, my, nullptr, h->dAb);
@@ -1140,12 +1165,12 @@ int backward_fused(fno_handle *h, const float *target, double *loss) {
     // everything per site: dv, through the activation below (the site-major
     // copy in place: a tile reads and writes its own sites), when the channel
     // sums are read and dW of the layer above no longer reads the other buffer
-    FNO_CUDA(h, cudaStreamWaitEvent(st, h->ev_sums, 0));
-    if (l + 1 < L) FNO_CUDA(h, cudaStreamWaitEvent(st, h->ev_dw[(l + 1) & 1], 0));
+    if (beside) FNO_CUDA(h, cudaStreamWaitEvent(st, h->ev_sums, 0));
+    if (beside && l + 1 < L) FNO_CUDA(h, cudaStreamWaitEvent(st, h->ev_dw[(l + 1) & 1], 0));
     FNO_GEMM(h, fno::layer_backward(sh, h->dZT, h->wTb + (size_t)l * C * C, h->dAb, h->Fxb, l > 0 ? h->Z[l - 1] : nullptr,
                                     dz[(l + 1) & 1], h->dZT, h->quads, h->dV, h->gerr, st));
   }
-  FNO_CUDA(h, join.now());
+  if (beside) FNO_CUDA(h, join.now());
   // lift: dp = sum dv0, dP[o, c] = sum dv0[b, o, s] x0[b, c, s]
   chan_reduce(h, h->dV, B, C, S, g + o.p);
   outer_reduce<8, kFeatures, false>(h, h->dV, h->x0, B, C, kFeatures, S, g + o.P);
@@ -1267,7 +1292,7 @@ int fno_forward(fno_handle *h, int32_t B, int32_t nx, int32_t ny, const float *p
       FNO_GEMM(h, sg(h, h->V[l], nx, 1, 0, h->Fx, 2 * mx, 1, 0, h->A, 2 * mx, 1, 0, R, 2 * mx, nx, 1, 0.f));
     // y-transform, per-mode mixing (into the dY scratch), inverse y-transform
     ydft(h, h->A, B * C, ny, h->Sh[l]);
-    (void)pdl::launch(mix_kernel, my * mx, kThreads, mix_smem(B, C, false), st,
+    launch_mix(B, mix_kernel, my * mx, mix_smem(B, C, false), st,
                       h->Sh[l], P + h->o.Rr[l], P + h->o.Ri[l], B, C, my * mx, h->dY);
     (void)pdl::launch(iy_kernel, iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st,
                       h->dY, h->Ty, ny, mx, my, h->G, h->Gb);
@@ -1366,7 +1391,7 @@ int fno_backward(fno_handle *h, const float *target, double *loss) {
     // adjoints: of the inverse y-transform (a y-transform), of the mixing
     // (with the weights' gradient), of the y-transform (an inverse one)
     ydft(h, h->dG, B * C, ny, h->dY);
-    (void)pdl::launch(mix_back_kernel, my * mx, kThreads, mix_smem(B, C, true), st,
+    launch_mix(B, mix_back_kernel, my * mx, mix_smem(B, C, true), st,
                       h->dY, h->Sh[l], P + o.Rr[l], P + o.Ri[l], B, C, my * mx, h->dS, g + o.Rr[l], g + o.Ri[l]);
     (void)pdl::launch(iy_kernel, iy_grid(B * C, ny), kThreads, iy_smem(mx, my), st,
                       h->dS, h->Ty, ny, mx, my, h->dA, h->dAb);
