@@ -1428,7 +1428,7 @@ int lb_batch_create(const lb_params *ps, int32_t count, lb_batch **out) {
   int tall = 1;
   for (const lb_handle *h : b->hs) tall = std::max(tall, (int)h->p.ny);
   for (const lb_handle *h : b->hs) cols += (double)h->tile_cols * h->p.ny / tall;
-  const int want = lbk::sweep_seg_rule(cols, tall, resident_warps(b->store, b->tau1));
+  const int want = lbk::sweep_seg_rule(cols, tall, resident_warps(b->store, b->tau1), true);
   cudaError_t e = cudaSuccess;
   for (lb_handle *h : b->hs) {
     // (a lattice that fills the device by itself is cut lower here than alone:

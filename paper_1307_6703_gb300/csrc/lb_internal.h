@@ -90,7 +90,7 @@ int sweep_tile_cols(int store, int nx, int nstrips);
 // Segment height that gives about as many tiles in all as `resident` warps
 // want, for lattices of `cols` tile columns over ny rows (cols may sum over
 // several lattices).
-int sweep_seg_rule(double cols, int ny, int resident);
+int sweep_seg_rule(double cols, int ny, int resident, bool batch = false);
 // Sleep (ns) between two looks at a dependency in a launch of nitems tiles a
 // step on a device that holds `resident` warps.
 unsigned sweep_poll_ns(int nitems, int resident);

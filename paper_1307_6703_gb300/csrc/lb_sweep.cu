@@ -111,6 +111,12 @@ constexpr unsigned kAll = 0xffffffffu;
 // 32).
 constexpr int kSegMax = 64;
 constexpr double kTilesPerWarp = 1.3;
+// Fewer in a batch: its lattices do not wait for one another.  Per step at 1.3 /
+// 1.1, tau 1: 512 lattices of 64 x 32 FP32 37.2 / 31.7 us, bf16 45.6 / 41.5, 256 of
+// 128 x 64 48.7 / 45.3 and 61.6 / 57.5, 300 of 96 x 48 33.8 / 31.1 and 43.2 / 42.0, 64
+// uneven ones of up to 1024 x 256 85.4 / 85.8 and 88.0 / 87.0, 16 of 1024 x 256 53.9 /
+// 54.9 and 58.5 / 59.4.
+constexpr double kTilesPerWarpBatch = 1.1;
 
 // A storage policy describes one slot of the ring (two rows of the window)
 // and how a lane reads its two columns 2t, 2t + 1 of plane q: mid() is those
@@ -655,8 +661,8 @@ __device__ __forceinline__ void tile_columns(const SweepArgs &A, int i, int &x0,
 // mass/momentum record goes to rec.  Returns false when a copy wait gave up
 // (the warp then stopped and drained the copies still in flight).
 // kMulti: called once per tile by the multi-step kernel, which does not
-// hand its SM slots to a dependent grid early.
-template <class St, bool kTau1, bool kMulti = false, class Wait = WaitGrid, class Done = NoDone, class Mom = NoMoments>
+// hand its SM slots to a dependent grid early.  kLow: for low tiles.
+template <class St, bool kTau1, bool kMulti = false, bool kLow = false, class Wait = WaitGrid, class Done = NoDone, class Mom = NoMoments>
 __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtensorMap *tdev, const SweepArgs &A, const SweepConsts &K,
                                            const StepIO &O, const int strip, const int seg, double *rec,
                                            const bool records, const Wait &wait = Wait{}, const Done &done = Done{},
@@ -1009,16 +1015,38 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
   auto ceil2 = [](int v) { return (v + 1) >> 1; };  // ceil(v / 2), any sign
   const int klo = max(3, ceil2((walls ? 7 : 10) - ya));
   const int khi = min(min(kmax + 1, ceil2(yb - ya + 5)), walls ? ((ny - ya) >> 1) + 1 : ceil2(ny - ya - 2));
-  int k = 0;
-  for (; k < min(klo, kmax + 1); ++k) iteration(k, std::false_type{});
   // Two steady iterations per turn: what one carries to the next then needs no
   // register moves (an odd last one goes the general way).
+  int k = 0;
+  if constexpr (!kLow) {
+    for (; k < min(klo, kmax + 1); ++k) iteration(k, std::false_type{});
 #pragma unroll 1
-  for (; k + 1 < khi; k += 2) {
-    iteration(k, std::true_type{});
-    iteration(k + 1, std::true_type{});
+    for (; k + 1 < khi; k += 2) {
+      iteration(k, std::true_type{});
+      iteration(k + 1, std::true_type{});
+    }
+    for (; k <= kmax; ++k) iteration(k, std::false_type{});
+  } else {
+    // The same with one copy of the general iteration's code.  Where tiles are
+    // low, the warps of an SM are spread over all of it, and wait for
+    // instructions (7.2 of 11.8 cycles between two of a warp's): per step of 512
+    // lattices of 64 x 32, tau 1 and 2, FP32 37.8 -> 37.2 and 43.0 -> 42.4 us, bf16
+    // 49.3 -> 45.9 and 59.2 -> 51.1, of 256 of 128 x 64 FP32 56.3 -> 49.0 and 60.2
+    // -> 55.0.  It costs registers: single lattices of 4096 x 1024 50.4 -> 50.6, and
+    // up to 10 % in launches of one step.
+#pragma unroll 1
+    while (k <= kmax) {
+      iteration(k, std::false_type{});
+      ++k;
+      if (k >= klo) {
+#pragma unroll 1
+        for (; k + 1 < khi; k += 2) {
+          iteration(k, std::true_type{});
+          iteration(k + 1, std::true_type{});
+        }
+      }
+    }
   }
-  for (; k <= kmax; ++k) iteration(k, std::false_type{});
   if (!__all_sync(kAll, ok)) {
     if (t == 0) atomicOr(A.err, 1);
     // A copy wait gave up: wait (again bounded) for every copy this warp may
@@ -1278,9 +1306,9 @@ sweep_batch_multi_kernel(const BatchItem *__restrict__ items, const SweepArgs *_
     asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(m + 1) : "memory");
   }
   const StepIO O{A.fin, A.fdin, A.fout, A.fdev, A.partials, 0u, nullptr, nullptr, nullptr, 0.0};
-  (void)sweep_body<St, kTau1, true>(m, m + 1, A, K, O, it.strip, it.seg, A.partials + 4 * (size_t)it.rec,
-                                    k == P.nsteps - 1, [&] { return wait_deps(P, i, target, A.err); },
-                                    [&] { release_item(P, i, target + 1u); });
+  (void)sweep_body<St, kTau1, true, true>(m, m + 1, A, K, O, it.strip, it.seg, A.partials + 4 * (size_t)it.rec,
+                                          k == P.nsteps - 1, [&] { return wait_deps(P, i, target, A.err); },
+                                          [&] { release_item(P, i, target + 1u); });
 }
 
 // Single-lattice form: item i is tile i (tile column i % nstrips, segment
@@ -1464,8 +1492,8 @@ int sweep_warps_per_sm(int store, bool tau1) {
                             : (tau1 ? Form<StoreF32, true>::kMinBlocks : Form<StoreF32, false>::kMinBlocks);
 }
 
-int sweep_seg_rule(double cols, int ny, int resident) {
-  const double rows = ny * cols / (kTilesPerWarp * std::max(resident, 1));
+int sweep_seg_rule(double cols, int ny, int resident, bool batch) {
+  const double rows = ny * cols / ((batch ? kTilesPerWarpBatch : kTilesPerWarp) * std::max(resident, 1));
   const int h = rows < 3.0 ? 2 : std::min(kSegMax, 4 * std::max(1, (int)(rows / 4.0 + 0.5)));
   return std::min(ny, h);
 }
