@@ -6,13 +6,14 @@
 // The equilibrium is evaluated in double-FP32 arithmetic (a value as the sum of
 // two floats; error-free transformations of Dekker, Numer. Math. 18 (1971) 224,
 // and Knuth, TAOCP 2, 4.2.2), good to 2^-43 for densities and velocities within
-// the bounds below.  A site whose result lies so close to the middle of two
-// floats that this does not decide the rounding (one value in 2^18), or whose
-// fields are outside the bounds -- infinities and NaN among them -- is evaluated
-// in FP64.  FP64 itself runs at 1/64 of the FP32 rate on this part and bound
+// the bounds below.  A population that lies so close to the middle of two floats
+// that this does not decide its rounding (one in 2^17), and a site whose fields
+// are outside the bounds -- infinities and NaN among them -- are evaluated in
+// FP64.  FP64 for every site runs at 1/64 of the FP32 rate on this part and bound
 // the kernel: 4096 x 1024 from noise 174 us, 2048 x 512 from density and velocity
 // 850 us.  Now bound by memory: 36 (FP32) or 20 (16-bit) bytes written a site, and
-// 8 bytes read per field given.
+// 8 bytes read per field given; 4096 x 1024 FP32 from noise 24.9 us, from a density
+// 44.7, with one velocity 77 (25.5, 45.0 and 71 if nothing were decided again).
 #include <algorithm>
 #include <cmath>
 
@@ -48,10 +49,11 @@ __device__ __forceinline__ Ff ff_mul(Ff a, Ff b) {
   const float p = __fmul_rn(a.h, b.h);
   return {p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)))};
 }
-// a, known to within d, as a float; `sure` becomes false where that leaves two.
-__device__ __forceinline__ float ff_round(Ff a, float d, bool &sure) {
+// a, known to within d, as a float; where that leaves two, `links` are marked
+// undecided.
+__device__ __forceinline__ float ff_round(Ff a, float d, unsigned links, unsigned &open) {
   const float lo = __fadd_rn(a.h, __fsub_rn(a.l, d)), hi = __fadd_rn(a.h, __fadd_rn(a.l, d));
-  sure = sure && lo == hi;
+  if (lo != hi) open |= links;
   return lo;
 }
 
@@ -86,13 +88,14 @@ struct InitArgs {
   float ref_ax, ref_dg;
   // FP64 forms, and the error of the double-FP32 ones: each population is known
   // to within `slack` times its class's w_i n
-  double rho64, amp64, T, iso64[3];
+  double rho64, amp64, t3[3];
   float slack;
 };
 
 // Where the double-FP32 arithmetic is good to `slack`: densities that leave room
 // for the low parts, velocities at which no sum cancels (terms of at most 0.75
 // beside the rest factor's 1 or so).
+constexpr unsigned kLinks = 0x1ff;  // all nine
 constexpr float kMinN = 0x1p-60f, kMaxN = 0x1p+60f, kMaxU = 0.125f;
 
 // Noise of site s: x = 2 U - 1 with U the top 53 bits of SplitMix64, exact up
@@ -102,25 +105,25 @@ __device__ __forceinline__ Ff noise_at(uint64_t seed, uint64_t s) {
   return {(float)(int)(j >> 29) * 0x1p-23f, (float)(unsigned)(j & 0x1fffffff) * 0x1p-52f};
 }
 
-// Equilibrium of one moving site in FP64, rounded once.
-__device__ __noinline__ void equilibrium64(double n, double u, double v, double T, float *f) {
-  double t3[3], fe[9];
-  isotropic3(T, t3);
-  feq9<double>(n, u, v, t3, fe);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) f[i] = (float)fe[i];
+// Population of link q of a moving site in FP64 (feq9's expressions), rounded
+// once.
+__device__ __noinline__ float link64(double cu, double n, double u, double v, double w, double t3) {
+  constexpr double T0 = Consts<double>::T0, c2 = 2.0 * T0 * T0;
+  const double t1 = div_const(cu, T0, 1.0 / T0), t2 = div_const(cu * cu - T0 * (u * u + v * v), c2, 1.0 / c2);
+  return (float)(w * n * (((1.0 + t1) + t2) + t3));
 }
 
-// Equilibrium of one site.  Class 0: rest, 1: axes, 2: diagonals.  False where
-// a rounding is not decided.
+// Equilibrium of one site.  Class 0: rest, 1: axes, 2: diagonals.  Returns the
+// links whose rounding is not decided.
 template <bool kMoving>
-__device__ __forceinline__ bool equilibrium(const InitArgs &A, Ff n, Ff u, Ff v, float *f) {
-  bool sure = fabsf(n.h) >= kMinN && fabsf(n.h) <= kMaxN && fabsf(u.h) <= kMaxU && fabsf(v.h) <= kMaxU;
+__device__ __forceinline__ unsigned equilibrium(const InitArgs &A, Ff n, Ff u, Ff v, float *f) {
+  unsigned open = 0;
+  if (!(fabsf(n.h) >= kMinN && fabsf(n.h) <= kMaxN && fabsf(u.h) <= kMaxU && fabsf(v.h) <= kMaxU)) open = kLinks;
   if constexpr (!kMoving) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const Ff p = ff_mul(A.wiso[c], n);
-      const float e = ff_round(p, __fmul_rn(fabsf(p.h), A.slack), sure);
+      const float e = ff_round(p, __fmul_rn(fabsf(p.h), A.slack), kLinks, open);
 #pragma unroll
       for (int i = 0; i < 9; ++i)
         if (cx(i) * cx(i) + cy(i) * cy(i) == c) f[i] = e;
@@ -135,20 +138,20 @@ __device__ __forceinline__ bool equilibrium(const InitArgs &A, Ff n, Ff u, Ff v,
       base[c] = ff_add(A.iso[c], uu);
       wn[c] = ff_mul(A.w[c], n);
     }
-    f[0] = ff_round(ff_mul(wn[0], base[0]), __fmul_rn(fabsf(wn[0].h), A.slack), sure);
+    f[0] = ff_round(ff_mul(wn[0], base[0]), __fmul_rn(fabsf(wn[0].h), A.slack), 1u, open);
     // the four directions and their opposites
     auto pair = [&](int i, int j, int c, Ff cu) {
       const Ff even = ff_add(base[c], ff_mul(nine2, ff_mul(cu, cu))), odd = ff_mul(three, cu);
       const float d = __fmul_rn(fabsf(wn[c].h), A.slack);
-      f[i] = ff_round(ff_mul(wn[c], ff_add(even, odd)), d, sure);
-      f[j] = ff_round(ff_mul(wn[c], ff_add(even, ff_neg(odd))), d, sure);
+      f[i] = ff_round(ff_mul(wn[c], ff_add(even, odd)), d, 1u << i, open);
+      f[j] = ff_round(ff_mul(wn[c], ff_add(even, ff_neg(odd))), d, 1u << j, open);
     };
     pair(1, 3, 1, u);
     pair(2, 4, 1, v);
     pair(5, 7, 2, ff_add(u, v));
     pair(6, 8, 2, ff_add(v, ff_neg(u)));
   }
-  return sure;
+  return open;
 }
 
 // Storage: nine float planes, or the float rest plane and eight 16-bit planes
@@ -215,7 +218,7 @@ __device__ __forceinline__ float PutDev<__half>::dec(__half v) { return __half2f
 // Threads along x (kCols columns each: 2 where the layout keeps pairs of
 // columns aligned), blocks strided over rows.
 template <class Put, int kCols, bool kMoving>
-__global__ void __launch_bounds__(256, kMoving ? 1 : 8) init_f32_kernel(Put put, const __grid_constant__ InitArgs A) {
+__global__ void __launch_bounds__(256, kMoving ? 4 : 8) init_f32_kernel(Put put, const __grid_constant__ InitArgs A) {
   pdl::begin();
   const int cols = A.nx / kCols;
   for (int y = blockIdx.y; y < A.ny; y += gridDim.y) {
@@ -243,17 +246,16 @@ __global__ void __launch_bounds__(256, kMoving ? 1 : 8) init_f32_kernel(Put put,
 #pragma unroll
       for (int j = 0; j < kCols; ++j) {
         const Ff n = A.n0 == nullptr ? ff_add(A.rho, ff_mul(A.amp, noise_at(A.seed, s + j))) : ff_of(n0[j]);
-        if (!equilibrium<kMoving>(A, n, ff_of(u0[j]), ff_of(v0[j]), f[j])) {
-          if constexpr (kMoving) {
-            float g[9];
-            equilibrium64(n0[j], u0[j], v0[j], A.T, g);
+        const unsigned open = equilibrium<kMoving>(A, n, ff_of(u0[j]), ff_of(v0[j]), f[j]);
+        if (open != 0) {
+          const double U = (double)(splitmix64_at(A.seed, s + j) >> 11) * 0x1.0p-53;
+          const double m = A.n0 == nullptr ? A.rho64 + A.amp64 * (2.0 * U - 1.0) : n0[j];
 #pragma unroll
-            for (int q = 0; q < 9; ++q) f[j][q] = g[q];
-          } else {
-            const double U = (double)(splitmix64_at(A.seed, s + j) >> 11) * 0x1.0p-53;
-            const double m = A.n0 == nullptr ? A.rho64 + A.amp64 * (2.0 * U - 1.0) : n0[j];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) f[j][q] = (float)(Consts<double>::w(q) * m * A.iso64[cx(q) * cx(q) + cy(q) * cy(q)]);
+          for (int q = 0; q < 9; ++q) {
+            const double w = Consts<double>::w(q), t3 = A.t3[cx(q) * cx(q) + cy(q) * cy(q)];
+            if (!(open >> q & 1u)) continue;
+            if constexpr (kMoving) f[j][q] = link64(cx(q) * u0[j] + cy(q) * v0[j], m, u0[j], v0[j], w, t3);
+            else f[j][q] = (float)(w * m * (1.0 + t3));
           }
         }
       }
@@ -309,12 +311,11 @@ cudaError_t launch_init_f32(int store, void *buf, const InitState &I, cudaStream
   A.ref_dg = I.ref_dg;
   A.rho64 = I.rho_mean;
   A.amp64 = I.amp;
-  A.T = I.T;
   const double T0 = 1.0 / 3.0, w[3] = {4.0 / 9.0, 1.0 / 9.0, 1.0 / 36.0};
   for (int c = 0; c < 3; ++c) {
-    const double iso = 1.0 + (I.T - T0) * ((double)c - 2.0 * T0) / (2.0 * T0 * T0);
+    const double t3 = (I.T - T0) * ((double)c - 2.0 * T0) / (2.0 * T0 * T0), iso = 1.0 + t3;
     A.iso[c] = ff_host(iso);
-    A.iso64[c] = iso;
+    A.t3[c] = t3;
     A.w[c] = ff_host(w[c]);
     A.wiso[c] = ff_host(w[c] * iso);
     A.slack = std::max(A.slack, (float)(0x1p-43 * (1.0 + std::abs(iso))));
