@@ -912,7 +912,8 @@ int lb_moments(lb_handle *h, void *rho, void *ux, void *uy, int dtype, int on_de
     e = lbk::launch_moments((const double *)h->f[h->cur], make_args<double>(h), dn, du, dv, dtype, h->st);
   } else if (h->sweep) {
     lbk::SweepArgs A = sweep_args(h, h->cur);
-    if (!on_device && !(staged[0] || staged[1] || staged[2])) {
+    const bool host = !on_device && !(staged[0] || staged[1] || staged[2]);
+    if (host) {
       // Written over the host link: tiles of 32 columns, so that a warp writes
       // whole 128-byte lines (4096 x 1024 in 285 us; 332 with tiles of 56).
       A.nstrips = (h->p.nx + 31) / 32;
@@ -922,7 +923,7 @@ int lb_moments(lb_handle *h, void *rho, void *ux, void *uy, int dtype, int on_de
     // lattices into higher ones: 30 us for one of them, against 6)
     A.seg_h = lbk::sweep_seg_rule(A.nstrips, h->p.ny, h->resident);
     A.nseg = (h->p.ny + A.seg_h - 1) / A.seg_h;
-    e = lbk::launch_sweep_moments(h->store, h->tmap[h->cur][0], h->tmap[h->cur][1], A, dn, du, dv, dtype, h->st);
+    e = lbk::launch_sweep_moments(h->store, h->tmap[h->cur][0], h->tmap[h->cur][1], A, dn, du, dv, dtype, host, h->st);
   } else {
     e = lbk::launch_moments((const float *)h->f[h->cur], make_args<float>(h), dn, du, dv, dtype, h->st);
   }

@@ -112,9 +112,10 @@ cudaError_t launch_sweep(int store, bool tau1, const CUtensorMap &m0, const CUte
                          size_t smem, cudaStream_t st);
 
 // Density and velocity u* of the state A.fin describes (maps m0, m1) into
-// compact arrays n, ux, uy (each may be null; dtype 0 = double, 1 = float).
+// compact arrays n, ux, uy (each may be null; dtype 0 = double, 1 = float; host:
+// they are page-locked host memory).
 cudaError_t launch_sweep_moments(int store, const CUtensorMap &m0, const CUtensorMap &m1, const SweepArgs &A, void *n,
-                                 void *ux, void *uy, int dtype, cudaStream_t st);
+                                 void *ux, void *uy, int dtype, bool host, cudaStream_t st);
 
 // Dependency lists of the tiles (CSR): tile a waits for the tiles
 // idx[ofs[a] .. ofs[a+1]) before each step.  Tile = column + ncol * segment;

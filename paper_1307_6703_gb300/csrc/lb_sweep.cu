@@ -622,12 +622,16 @@ struct WaitGrid {
 
 // Where a moments launch writes: compact [ny][nx] arrays (null: not wanted)
 // of T; a lane's two columns in one store where the arrays are aligned for it.
+// kRows (host arrays of odd widths): 32 consecutive columns of a row in one store
+// of the warp instead of every other one in two, which cross the link in twice
+// as many pieces (doubles, 509 x 256 52 -> 44 us, 4093 x 1024 736 -> 696; device
+// arrays take 18 us longer that way).
 struct NoMoments {
-  static constexpr bool kOn = false;
+  static constexpr bool kOn = false, kRows = false;
 };
-template <class T>
+template <class T, bool kByRows = false>
 struct Moments {
-  static constexpr bool kOn = true;
+  static constexpr bool kOn = true, kRows = kByRows;
   T *n, *ux, *uy;
   int pairs;
   __device__ __forceinline__ void put(T *p, size_t s, float2 v, bool half) const {
@@ -642,6 +646,18 @@ struct Moments {
     } else {
       p[s] = (T)v.x;
       p[s + 1] = (T)v.y;
+    }
+  }
+  // The values v of a row of a tile of W columns whose first is element s; the
+  // whole warp.
+  __device__ __forceinline__ void put_row(T *p, size_t s, int W, float2 v) const {
+    if (p == nullptr) return;
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {  // the tile's column 32 r + t, the window's 4 + 32 r + t
+      const int c = 32 * r + t, lane = ((4 + c) >> 1) & 31;
+      const float x = __shfl_sync(kAll, v.x, lane), y = __shfl_sync(kAll, v.y, lane);
+      if (c < W) p[s + c] = (T)(t & 1 ? y : x);
     }
   }
 };
@@ -856,8 +872,19 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const int y = a - 2 + j;
-        if (!(actD || half) || y < ya || y >= yb) continue;
         const float2 n = j ? N1.c : N0.c;
+        if constexpr (Mom::kRows) {
+          if (y < ya || y >= yb) continue;
+          auto over_n = [&](float2 J) {  // (halo values may be anything: no quotients of them)
+            return actD || half ? make_float2(__fdiv_rn(J.x, n.x), __fdiv_rn(J.y, n.y)) : zero;
+          };
+          const size_t s = (size_t)y * nx + x0;
+          mom.put_row(mom.n, s, W, n);
+          mom.put_row(mom.ux, s, W, over_n(JxC[j]));
+          mom.put_row(mom.uy, s, W, over_n(JyC[j]));
+          continue;
+        }
+        if (!(actD || half) || y < ya || y >= yb) continue;
         const size_t s = (size_t)y * nx + x;
         mom.put(mom.n, s, n, half);
         if (mom.ux != nullptr) mom.put(mom.ux, s, make_float2(__fdiv_rn(JxC[j].x, n.x), __fdiv_rn(JxC[j].y, n.y)), half);
@@ -1181,10 +1208,10 @@ __device__ __forceinline__ SweepConsts lattice_consts(const SweepConsts &own, co
 
 // Density and velocity of a state: the same sweep, stages A to C only.  Reads
 // the populations once (36 or 20 bytes a site) and writes the three fields.
-template <class St, class T>
+template <class St, class Mom>
 __global__ void __launch_bounds__(kThreads, Form<St, true>::kMinBlocks)
 sweep_moments_kernel(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tdev,
-                     const __grid_constant__ SweepArgs A, const Moments<T> M) {
+                     const __grid_constant__ SweepArgs A, const Mom M) {
   const StepIO O{A.fin, A.fdin, nullptr, nullptr, nullptr, 0u, nullptr, nullptr, nullptr, 0.0};
   (void)sweep_body<St, true>(&tin, &tdev, A, A.k, O, blockIdx.x, blockIdx.y, nullptr, false, WaitGrid{}, NoDone{}, M);
 }
@@ -1437,15 +1464,16 @@ cudaError_t launch_multi_one(const CUtensorMap (&m)[2][2], const SweepArgs &A, c
   return cudaLaunchKernelEx(&cfg, sweep_multi_kernel<St, kTau1>, m[0][0], m[0][1], m[1][0], m[1][1], A, P, Q);
 }
 
-template <class St, class T>
+template <class St, class T, bool kRows = false>
 cudaError_t launch_moments_one(const CUtensorMap &m0, const CUtensorMap &m1, const SweepArgs &A, void *n, void *ux,
                                void *uy, cudaStream_t st) {
   const int smem = (int)sizeof(SmemOf<St, true>);
-  cudaError_t e = cudaFuncSetAttribute(sweep_moments_kernel<St, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  using Mom = Moments<T, kRows>;
+  cudaError_t e = cudaFuncSetAttribute(sweep_moments_kernel<St, Mom>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const uintptr_t all = (uintptr_t)n | (uintptr_t)ux | (uintptr_t)uy;  // (even nx: rows keep the alignment)
-  const Moments<T> M{(T *)n, (T *)ux, (T *)uy, all % (2 * sizeof(T)) == 0 && A.nx % 2 == 0};
-  return pdl::launch(sweep_moments_kernel<St, T>, dim3((unsigned)A.nstrips, (unsigned)A.nseg), kThreads, (size_t)smem,
+  const Mom M{(T *)n, (T *)ux, (T *)uy, all % (2 * sizeof(T)) == 0 && A.nx % 2 == 0};
+  return pdl::launch(sweep_moments_kernel<St, Mom>, dim3((unsigned)A.nstrips, (unsigned)A.nseg), kThreads, (size_t)smem,
                      st, m0, m1, A, M);
 }
 
@@ -1543,7 +1571,10 @@ cudaError_t launch_sweep(int store, bool tau1, const CUtensorMap &m0, const CUte
 }
 
 cudaError_t launch_sweep_moments(int store, const CUtensorMap &m0, const CUtensorMap &m1, const SweepArgs &A, void *n,
-                                 void *ux, void *uy, int dtype, cudaStream_t st) {
+                                 void *ux, void *uy, int dtype, bool host, cudaStream_t st) {
+  if (host && store == kStoreF32Odd)
+    return dtype == 0 ? launch_moments_one<StoreF32Odd, double, true>(m0, m1, A, n, ux, uy, st)
+                      : launch_moments_one<StoreF32Odd, float, true>(m0, m1, A, n, ux, uy, st);
   switch (store) {
     case kStoreF32:
       return dtype == 0 ? launch_moments_one<StoreF32, double>(m0, m1, A, n, ux, uy, st)
