@@ -105,9 +105,15 @@ int cudaGetLastError(void) { return kOk; }
 const char *cudaGetErrorString(int e) { return e == kNoMemory ? "out of memory" : "error"; }
 int cudaGetSymbolAddress(void **p, const void *sym) { *p = (void *)sym; return kOk; }
 
-/* The two driver functions the library asks for: descriptors are left empty,
- * and every pointer counts as pageable memory. */
-static int encode_tiled(void *map) { memset(map, 0, 128); return 0; }
+/* The two driver functions the library asks for: a descriptor holds the box it
+ * was made for, and every pointer counts as pageable memory. */
+static int encode_tiled(void *map, int type, unsigned rank, void *base, const uint64_t *dims, const uint64_t *strides,
+                        const uint32_t *box) {
+  (void)type; (void)base; (void)dims; (void)strides;
+  memset(map, 0, 128);
+  memcpy(map, box, rank * sizeof(*box));
+  return 0;
+}
 static int pointer_attribute(void *v, int attr, uint64_t p) { (void)v; (void)attr; (void)p; return 1; }
 int cudaGetDriverEntryPointByVersion(const char *name, void **fn, unsigned version, unsigned long long flags, int *q) {
   (void)version;
