@@ -681,12 +681,14 @@ __device__ __forceinline__ void tile_columns(const SweepArgs &A, int i, int &x0,
 template <class St, bool kTau1, bool kMulti = false, bool kLow = false, class Wait = WaitGrid, class Done = NoDone, class Mom = NoMoments>
 __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtensorMap *tdev, const SweepArgs &A, const SweepConsts &K,
                                            const StepIO &O, const int strip, const int seg, double *rec,
-                                           const bool records, const Wait &wait = Wait{}, const Done &done = Done{},
+                                           const bool want_records, const Wait &wait = Wait{}, const Done &done = Done{},
                                            const Mom &mom = Mom{}) {
   using Row = typename St::Row;
   using Smem = SmemOf<St, kTau1>;
   using V = V2;
   constexpr int kPairs = Form<St, kTau1>::kPairs;
+  // (not of odd widths: half a pair would count a ghost column)
+  const bool records = !St::kOdd && want_records;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   Smem &S = *reinterpret_cast<Smem *>(smem_raw);
 
