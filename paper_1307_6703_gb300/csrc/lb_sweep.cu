@@ -101,6 +101,8 @@ static_assert(kCols == kSweepWindow, "the dependency lists cover the window");
 constexpr int kTileW = kCols - 8;           // widest tile
 constexpr int kThreads = 32;
 constexpr unsigned kAll = 0xffffffffu;
+constexpr uint32_t kWaitLimit = 1u << 22;
+static_assert(kWaitLimit == kSweepWaitLimit, "what lb_set_wait_limit starts from");
 // Rows of a tile where the tiling's segments would leave warps idle: about
 // kTilesPerWarp tiles of a step per resident warp, so that a tile's neighbours
 // have finished the previous step by the time its ticket is drawn; a multiple
@@ -734,7 +736,7 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
     for (int p = 0; p < issued; ++p) request(p, p);
   }
   __syncwarp();
-  const uint32_t limit = kMulti ? kSweepWaitLimit : A.wait_limit;
+  const uint32_t limit = kMulti ? kWaitLimit : A.wait_limit;
   bool ok = mbar_wait(smem_u32(&S.full[0]), 0, limit);
   // What the stages carry from one iteration to the next (rows relative to
   // the next iteration's a).
@@ -1083,7 +1085,7 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
     // lands in shared memory after the warp has moved on, then stop.
     if (t == 0) {
       for (int p = max(0, issued - kPairs); p < issued; ++p)
-        (void)mbar_wait(smem_u32(&S.full[p % kPairs]), (uint32_t)((p / kPairs) & 1), kSweepWaitLimit);
+        (void)mbar_wait(smem_u32(&S.full[p % kPairs]), (uint32_t)((p / kPairs) & 1), kWaitLimit);
     }
     __syncwarp();
     return false;
@@ -1287,13 +1289,13 @@ __device__ __forceinline__ bool wait_deps(const MultiArgs &P, int i, unsigned ta
   uint32_t n = 0;
   for (int d = P.dep_ofs[i] + (int)threadIdx.x; d < d1; d += kThreads) {
     const unsigned *f = P.done + P.dep_idx[d];
-    while ((int)(ld_acquire_gpu(f) - target) < 0 && n < kSweepWaitLimit) {
-      n = (n & 1023u) == 1023u && __ldcg(err) != 0 ? kSweepWaitLimit : n + 1;
+    while ((int)(ld_acquire_gpu(f) - target) < 0 && n < kWaitLimit) {
+      n = (n & 1023u) == 1023u && __ldcg(err) != 0 ? kWaitLimit : n + 1;
       __nanosleep(P.poll_ns);
     }
   }
   __syncwarp();
-  if (__any_sync(kAll, n >= kSweepWaitLimit)) {
+  if (__any_sync(kAll, n >= kWaitLimit)) {
     if (threadIdx.x == 0) atomicOr(err, 4);
     return false;
   }
