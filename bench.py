@@ -10,7 +10,7 @@ arithmetic).  Prints one JSON line (rank 0).
                   [--precision fp32|bf16dev|fp16dev]
                   [--workload single|batch|warmstart|precision|network|next4]
 
-`value`: K steps in one lb_step call (one persistent launch), CUDA events
+`value`: K steps in one lb_step call (one multi-step launch), CUDA events
 on the solver's stream, inputs resident in HBM.  `e2e`: the same K steps
 through the C ABI with host buffers -- lb_init from a page-locked FP64
 density field, every step's record written into a page-locked ring by the
@@ -467,7 +467,7 @@ def run_batch(args):
     seq = sites * k_seq / (seq_ms * 1e-3) / 1e6
     peak, peak_kind = measured_peaks()
     # one lb_batch_step call is one launch: a single step-kernel launch, or
-    # one persistent launch (its chunks hold 2^30 / items steps, over a
+    # one multi-step launch (its chunks hold 2^30 / items steps, over a
     # million for this ensemble's few hundred items)
     launches = 1
     kernel = "lbk::sweep_batch_kernel" if args.steps == 1 else "lbk::sweep_batch_multi_kernel"

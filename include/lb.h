@@ -134,7 +134,10 @@ int lb_init(lb_handle *h, int mode, uint64_t seed, double rho_mean,
  * (periodicforce), wall rule, u* of Eq. (newvel), equilibrium Eq.
  * (eqfunc), forcing Eqs. (forceterm, coeff), BGK collision -- in one fused
  * kernel (strip-sweep handles: one launch for many steps), enqueued on the
- * handle's stream without synchronising.  Errors: LB_ERR_STATE (not initialised), LB_ERR_CUDA.     */
+ * handle's stream without synchronising.  (The first launch of many steps of a
+ * tiling builds the dependency lists of its tiles: it allocates and waits for the
+ * stream.  FP32 lattices whose nx is not a multiple of 4 have theirs from
+ * lb_create.)  Errors: LB_ERR_STATE (not initialised), LB_ERR_CUDA, LB_ERR_OOM. */
 int lb_step(lb_handle *h, int64_t nsteps);
 
 /* Density n (n-hat on wall rows) and physical velocity u* of Eq. (newvel)
@@ -182,7 +185,8 @@ int lb_reduce_async(lb_handle *h, double *out);
  * tiling (synchronising the stream when it replaces smaller ones); while
  * monitoring, lb_step launches at most min(capacity, 64) steps at a time,
  * so each ring record is written once per launch and in step order.
- * Strip-sweep handles only (FP32 and 16-bit storage, not inside a batch).
+ * FP32 with nx a multiple of 4 and 16-bit storage, nx, ny >= 8, not inside a
+ * batch.
  * Errors: LB_ERR_ARG (other handles, capacity < 0, memory the device cannot
  * address), LB_ERR_CUDA, LB_ERR_OOM.                                       */
 int lb_monitor(lb_handle *h, double *host_ring, int32_t capacity);
@@ -216,8 +220,8 @@ int lb_set_state(lb_handle *h, const void *buf, size_t bytes, int64_t step);
  * repeated warm-up rows) that gives other tiles than the ones before, times
  * the three fastest twice more and keeps the one with
  * the smallest of its three timings for later lb_step calls, and writes its
- * segment height to *seg_h (may be NULL; 0 when the handle uses the tile
- * kernel, which has no tiling choice; lb_get_tiling gives both).  The state and the step counter are restored
+ * segment height to *seg_h (may be NULL; 0 for handles without a tiling
+ * choice, see lb_get_tiling, which gives both).    The state and the step counter are restored
  * afterwards: the trajectory is the same as without the call.  Needs one
  * extra state buffer of device memory while it runs; synchronises the
  * stream.  Errors: LB_ERR_ARG (steps < 1), LB_ERR_STATE, LB_ERR_CUDA,
@@ -230,13 +234,15 @@ int lb_autotune(lb_handle *h, int steps, int32_t *seg_h);
  * strip wider than a tile can be (56 columns) is replaced by the fewest
  * narrower ones, and segments that would leave the GPU partly idle are cut
  * into lower tiles.  The trajectory does not depend on it beyond FP32 rounding
- * order.  No-op (LB_OK) for a handle on the tile kernel.  Host-side only
+ * order.  No-op (LB_OK) for a handle without a tiling choice.  Host-side only
  * (may grow the per-tile record array).  Errors: LB_ERR_ARG (seg_h < 1),
  * LB_ERR_CUDA, LB_ERR_OOM.                                                 */
 int lb_set_seg_h(lb_handle *h, int32_t seg_h);
 
-/* The strip-sweep tiling in use: number of column strips and segment
- * height (both 0 for a handle on the tile kernel).  A performance control
+/* The strip-sweep tiling that was chosen or set: number of column strips and
+ * segment height (both 0 for handles without a tiling choice: FP64, and FP32
+ * lattices whose nx is not a multiple of 4 or with nx or ny < 8).  The tiles
+ * that run may be narrower and lower, see lb_set_seg_h.  A performance control
  * of this library; the paper has no counterpart.  Errors: LB_ERR_ARG (NULL
  * outputs).                                                                */
 int lb_get_tiling(const lb_handle *h, int32_t *nstrips, int32_t *seg_h);
@@ -248,8 +254,8 @@ int lb_get_tiling(const lb_handle *h, int32_t *nstrips, int32_t *seg_h);
  * for 16-bit storage); seg_h as lb_set_seg_h.  Strip s starts at column
  * s base + quantum min(s, extra) and is base or base + quantum wide (the
  * first `extra` strips wider), base = quantum floor(nx / (quantum nstrips)).
- * The trajectory is the same bit for bit for every tiling.  No-op for the
- * tile kernel.  Errors: LB_ERR_ARG (out of range), LB_ERR_CUDA, LB_ERR_OOM. */
+ * The trajectory is the same bit for bit for every tiling.  No-op for handles
+ * without a tiling choice.  Errors: LB_ERR_ARG (out of range), LB_ERR_CUDA, LB_ERR_OOM. */
 int lb_set_tiling(lb_handle *h, int32_t nstrips, int32_t seg_h);
 
 /* Dependency lists of the multi-step sweep, for inspection and tests (host
@@ -294,8 +300,10 @@ int lb_batch_create(const lb_params *ps, int32_t count, lb_batch **out);
  * i is out of range.                                                       */
 lb_handle *lb_batch_handle(lb_batch *b, int32_t i);
 
-/* Advance every instance by nsteps >= 0 steps (asynchronous on the stream).
- * Afterwards lb_reduce of each instance costs one small kernel.
+/* Advance every instance by nsteps >= 0 steps (asynchronous on the stream, but
+ * for the first call after a change of an instance's tiling or buffers, which
+ * rebuilds the work list).  Afterwards lb_reduce of each instance costs one small
+ * kernel, as after a single step of a lattice of its own.
  * Errors: LB_ERR_STATE (an instance not initialised), LB_ERR_CUDA.         */
 int lb_batch_step(lb_batch *b, int64_t nsteps);
 

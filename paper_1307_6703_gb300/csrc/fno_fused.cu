@@ -2,7 +2,10 @@
 // (include/fno.h) as fused tensor-core kernels, for the width the warm start
 // uses (32 channels, 32 or 64 hidden).
 //
-// A tile is 128 sites of one lattice row: the rows of an MMA.  Per site the
+// A tile is 128 sites of one lattice row: the rows of an MMA.  (Rows that leave
+// part of the last tile empty, 64 or 136 sites, leave that part of the
+// accumulators and of the epilogue's lanes idle; the kernels are the faster ones
+// all the same, see below.)  Per site the
 // layer is two products with K <= 64 -- the channel mixing (the site-major
 // BF16 copy of v against W) and the inverse x-transform (the table FxiT[x][j]
 // against the 2 modes_x transformed values of each channel at this y) -- so one
@@ -23,9 +26,10 @@
 // (each product in its own accumulator, then added, then the bias), so a
 // layer's values are the same bits.  Bound by the activations (normcdff) and
 // by memory about equally.  Measured: training step of 16 fields of 256 x 64
-// 1.61 -> 1.07 ms, of 8 fields of 512 x 128 2.74 -> 1.65 ms (0.90 and 1.34 with
-// the weight gradients beside them and launches overlapped); warm start of a
-// 2048 x 512 lattice (forward pass, fields, initial state) 2.36 -> 0.84 ms.
+// 1.61 -> 1.07 ms, of 8 fields of 512 x 128 2.74 -> 1.65 ms (0.86 and 1.27 with
+// the weight gradients beside them and launches overlapped), of 16 fields of 64 x
+// 64 0.86 -> 0.57 and of 32 x 16 0.61 -> 0.39; warm start of a 2048 x 512 lattice
+// (forward pass, fields, initial state) 2.36 -> 0.83 ms.
 #include "fno_fused.h"
 
 #include <algorithm>

@@ -33,9 +33,10 @@
 // nothing is recomputed.
 //
 // Why this split.  One warp per tile needs no barrier, and two columns per lane
-// halve the instructions: 237 -> about 140 thread instructions a site against
-// 320 in the form before (a CTA of 124 threads, one column each, all stages
-// exchanging through shared memory between four CTA barriers an iteration).
+// take fewer instructions: 187 a site and thread (FP32, warm-ups and waits
+// included) against 320 in the form before (a CTA of 124 threads, one column each,
+// all stages exchanging through shared memory between four CTA barriers an
+// iteration).
 // What bounds it now is memory for FP32 (72 algorithmic bytes a site) and, for
 // 16-bit storage, the issue rate and the latency of 12 warps an SM.  Measured
 // per step of 4096 x 1024, tau = 1, 20 steps a launch: FP32 58.7 -> 51.9 us
@@ -69,9 +70,10 @@
 //
 // On the last step of a call (or every step while a monitoring ring is set)
 // every CTA also writes FP64 partial sums of mass and momentum of the state
-// it stored, and a flag for non-finite or out-of-range sites; the CTA that
-// finishes last adds them up, so the global sums of the new state need no
-// further kernel.
+// it stored, and a flag for non-finite or out-of-range sites.  In a multi-step
+// launch, and while monitoring, the CTA that finishes last adds them up, so the
+// global sums of the new state need no further kernel; after a single step a
+// block does when they are asked for (one warp takes 34 us for 2368 records).
 //
 // Initial state, single steps and moments are programmatic dependent launches
 // (pdl.cuh): a step's successor may be scheduled once every CTA of the step has
@@ -158,8 +160,8 @@ struct StoreF32 {
 // column of tiles is narrower, its last pair of columns may be half outside,
 // and periodic images are stored one column at a time (nx odd shifts them by
 // half a pair).  (These lattices used the tile kernel, whose tiles of 32 x 16
-// sites pull every population three times from L1/L2: 25 us a step for 1021 x
-// 509, now 20.)
+// sites pull every population three times from L1/L2: 20 steps of 1021 x 509
+// 990 us a pass, now 394.)
 struct StoreF32Odd : StoreF32 {
   static constexpr bool kOdd = true;
 };
@@ -418,10 +420,6 @@ struct StepIO {
   double *monitor;
   double mon_step;
 };
-// x-derivative, y-derivative and Laplacian stencils of Eqs. (xstencil,
-// laplstencil).  Every operation is rounded as written (explicit intrinsics,
-// no contraction), so a site's value does not depend on the tile that
-// computed it.
 // One row of a quantity as a lane sees it: its two columns c and the columns
 // on their left and right.
 struct Nbr {
@@ -431,6 +429,11 @@ struct Nbr {
 __device__ __forceinline__ Nbr spread(float2 c) {
   return {c, __shfl_up_sync(kAll, c.y, 1), __shfl_down_sync(kAll, c.x, 1)};
 }
+// x-derivative, y-derivative and Laplacian stencils of Eqs. (xstencil,
+// laplstencil).  Every operation is rounded as written (explicit intrinsics,
+// no contraction), so a site's value does not depend on the tile that
+// computed it.
+//
 // right - left neighbour, right + left neighbour
 __device__ __forceinline__ float2 xdiff(const Nbr &v) {
   return make_float2(__fsub_rn(v.c.y, v.l), __fsub_rn(v.r, v.c.x));
@@ -705,7 +708,7 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
   const bool actD = 2 * t >= 4 && 2 * t + 1 < W + 4;         // both columns in the tile
   const bool half = St::kOdd && 2 * t >= 4 && 2 * t == W + 3;  // the first one only
   const int kmax = (yb - ya + 5) >> 1;  // last iteration
-  const int npairs = kmax + 2;          // rows ya-4 .. ya+2*kmax+3
+  const int npairs = kmax + 2;          // rows ya-4 .. ya+2*kmax-1, at most yb+4
   const int pitch = A.pitch, plane = (int)A.plane;
   auto image = [&](int c) { return c < 4 ? nx : (c >= nx - 4 ? -nx : 0); };
   const int im0 = image(x), im1 = St::kOdd ? image(x + 1) : im0;  // to the periodic image columns
@@ -1092,7 +1095,7 @@ __device__ __forceinline__ bool sweep_body(const CUtensorMap *tin, const CUtenso
   }
   // The next step may be scheduled now (it waits for this grid to finish).
   if constexpr (!kMulti) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // Every lane is here: the tile's stores are done.  A persistent caller
+  // Every lane is here: the tile's stores are done.  A multi-step caller
   // publishes its completion now -- the records below touch only the record
   // slots, so dependent tiles need not wait.
   done();
