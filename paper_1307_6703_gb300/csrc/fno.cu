@@ -1220,7 +1220,7 @@ int fno_create(const fno_config *cfg, fno_handle **out) {
   }
   // The clears went to the default stream, for which a stream of the program's
   // own need not wait.
-  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+  if (e == cudaSuccess && h->st != nullptr) e = cudaStreamSynchronize(nullptr);
   if (e != cudaSuccess) {
     std::string m = std::string("fno_create: ") + cudaGetErrorString(e);
     fno_destroy(h);

@@ -780,7 +780,7 @@ int lb_create(const lb_params *p, lb_handle **out) {
     (void)cudaGetLastError();  // (see multi_allowed)
   // The clears and the copy went to the default stream, for which a stream of
   // the program's own need not wait.
-  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+  if (e == cudaSuccess && h->st != nullptr) e = cudaStreamSynchronize(nullptr);
   if (e != cudaSuccess) {
     std::string m = std::string("lb_create: ") + cudaGetErrorString(e);
     int code = (e == cudaErrorMemoryAllocation) ? LB_ERR_OOM : LB_ERR_CUDA;
